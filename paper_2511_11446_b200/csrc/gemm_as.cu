@@ -224,7 +224,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   // ---- teardown ----
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // neither CTA frees tensor memory or exits while the other may still touch it
+  cluster_sync_relaxed();  // neither CTA frees tensor memory or exits while the other may still touch it
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, TCOLS);

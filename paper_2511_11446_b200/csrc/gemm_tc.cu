@@ -315,7 +315,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   // ---- teardown ----
   tc_fence_before();
   __syncthreads();
-  if constexpr (CG == 2) cluster_sync();  // neither CTA frees tensor memory or exits while the other may still touch it
+  if constexpr (CG == 2) cluster_sync_relaxed();  // neither CTA frees tensor memory or exits while the other may still touch it
   if (warp == 1) {
     tc_fence_after();
     if constexpr (CG == 2) tmem_dealloc_pair(tmem_base, TCOLS);
