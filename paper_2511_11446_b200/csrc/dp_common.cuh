@@ -165,24 +165,31 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   // arriving thread for ~1400 cycles per call
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// Non-blocking phase test whose acquire covers arrivals made by the other CTA of the pair. (The
-// suspending try_wait form was measured to sleep through remote arrivals for ~0.5 us at a time.)
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+// Non-blocking phase test for a single polling thread. (The suspending try_wait form was measured to
+// sleep through arrivals from the other CTA of a pair for ~0.5 us at a time.) Its acquire is the default
+// CTA-scope one, also where the other CTA arrives: what such a barrier guards (operand stages, tensor
+// memory) is written and read by the asynchronous proxies or ordered by tcgen05 fences, and an
+// acquire at cluster scope cost the thread ~250 cycles per successful poll, more than the k-block it
+// waited for.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
       : "r"(smem_u32(bar)), "r"(parity)
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
+// Spinning (non-suspending), bounded wait for one polling thread: lowest wake-up latency. The clock is
+// read only once a wait has turned out long.
+__device__ __forceinline__ bool mbar_spin_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  for (int i = 0; i < 256; ++i)
+    if (mbar_test_wait(bar, parity)) return true;
   const long long t0 = clock64();
   uint32_t polls = 0;
-  while (!mbar_try_wait_cluster(bar, parity)) {
-    if ((++polls & 63u) == 0) {
+  while (!mbar_test_wait(bar, parity)) {
+    if ((++polls & 255u) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > kWaitBudgetCycles) {
         *abort_flag = 1;
@@ -235,21 +242,6 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, in
 // arrive + expect_tx on an mbarrier that may live in the pair's other CTA.
 __device__ __forceinline__ void mbar_arrive_expect_tx_cluster(uint32_t cluster_bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_bar), "r"(bytes) : "memory");
-}
-// Spinning (non-suspending) wait for one polling thread: lowest wake-up latency.
-__device__ __forceinline__ bool mbar_spin_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  const long long t0 = clock64();
-  uint32_t polls = 0;
-  while (!mbar_try_wait_cluster(bar, parity)) {
-    if ((++polls & 255u) == 0) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > kWaitBudgetCycles) {
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-  return true;
 }
 // Untiled bulk copy global -> shared (both addresses 16-byte aligned, size a multiple of 16 bytes),
 // completion counted in bytes on an mbarrier of this CTA.

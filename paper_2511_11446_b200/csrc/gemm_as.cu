@@ -100,7 +100,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
   if (warp == 0) {
     // ================= TMA producer =================
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st;
       bool ok = true;
       bool open = !p.early_w;  // false until griddepcontrol.wait has been executed
@@ -126,7 +126,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         const int m_row = strip * (2 * BM) + static_cast<int>(rank) * BM;
         if (new_strip) {
           // the resident strip may be overwritten once every MMA reading it has completed
-          if (strips > 0 && !(ok = mbar_wait_cluster(a_free, (strips - 1) & 1u, abort_flag))) break;
+          if (strips > 0 && !(ok = mbar_spin_wait(a_free, (strips - 1) & 1u, abort_flag))) break;
           cur_strip = strip;
           ++strips;
         }
@@ -158,7 +158,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       // ================= MMA issuer (leader) =================
       const uint32_t idesc = idesc_i8(2 * BM, ap.bns);
       const uint64_t a_desc0 = smem_desc_sw128(smem_u32(sA));
@@ -176,7 +176,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
         for (int sub = 0; sub < ap.nsub && ok; ++sub, ++g) {
           const int buf = g & 1;
-          if (!(ok = mbar_wait_cluster(&acc_empty[buf], ((g >> 1) & 1u) ^ 1u, abort_flag))) break;
+          if (!(ok = mbar_spin_wait(&acc_empty[buf], ((g >> 1) & 1u) ^ 1u, abort_flag))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + buf * (TCOLS / 2);
           for (int kb = 0; kb < KB; ++kb) {

@@ -94,17 +94,20 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   pdl_wait();  // the activations may come from the preceding kernel on the stream
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st;
-      bool ok = true;
+      bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
         const int n_blk = tile % p.n_tiles, m_row = (tile / p.n_tiles) * BM;
         for (int kb = 0; kb < KB; ++kb) {
-          if (!(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          Ring nx = st;
+          nx.next(NS);
+          free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);  // one k-block ahead
           mbar_arrive_expect_tx(&full[st.s], A_BYTES + B_BYTES);
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, kb * kBfBK, m_row, &full[st.s]);
           tma_load_2d(sB + st.s * B_BYTES, &tmap_w, kb * kBfBK, n_blk * BN, &full[st.s]);
-          st.next(NS);
+          st = nx;
         }
       }
       if (!ok) {  // give copies still in flight a bounded time to land before the CTA exits
@@ -114,10 +117,11 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       constexpr uint32_t idesc = idesc_bf16(BM, BN);
+      const uint64_t adesc0 = smem_desc_sw128(smem_u32(sA)), bdesc0 = smem_desc_sw128(smem_u32(sB));
       Ring st;
-      bool ok = true;
+      bool ok = true, full_next = mbar_test_wait(&full[0], 0u);
       int tcount = 0;
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
         const int buf = tcount & 1;
@@ -125,15 +129,18 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * (TCOLS / 2);
         for (int kb = 0; kb < KB; ++kb) {
-          if (!(ok = mbar_spin_wait(&full[st.s], st.ph, abort_flag))) break;
+          if (!full_next && !(ok = mbar_spin_wait(&full[st.s], st.ph, abort_flag))) break;
           tc_fence_after();
-          const uint64_t adesc = smem_desc_sw128(smem_u32(sA + st.s * A_BYTES));
-          const uint64_t bdesc = smem_desc_sw128(smem_u32(sB + st.s * B_BYTES));
+          Ring nx = st;
+          nx.next(NS);
+          full_next = mbar_test_wait(&full[nx.s], nx.ph);
+          const uint64_t adesc = adesc0 + static_cast<uint64_t>(st.s * (A_BYTES >> 4));
+          const uint64_t bdesc = bdesc0 + static_cast<uint64_t>(st.s * (B_BYTES >> 4));
 #pragma unroll
           for (int k4 = 0; k4 < kBfBK / 32; ++k4)  // 16 bf16 = 32 bytes of K per instruction
             mma_bf16_ss(d_tmem, adesc + 2 * k4, bdesc + 2 * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
           mma_commit(&empty[st.s]);
-          st.next(NS);
+          st = nx;
         }
         if (ok) mma_commit(&acc_full[buf]);
       }

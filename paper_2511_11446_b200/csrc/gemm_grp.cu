@@ -90,13 +90,16 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   pdl_wait();  // activations, scales and the int8 weight copy come from the preceding kernels on the stream
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st;
-      bool ok = true;
+      bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
         const int n_blk = tile % p.n_tiles, m_row = (tile / p.n_tiles) * BM;
         for (int kb = 0; kb < KB; ++kb) {
-          if (!(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          Ring nx = st;
+          nx.next(NS);
+          free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);  // one k-block ahead
           mbar_arrive_expect_tx(&full[st.s], A_BYTES + B_BYTES);
           int c0, c1;
           if (p.a_tiled) {
@@ -108,7 +111,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           }
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, c0, c1, &full[st.s]);
           tma_load_2d(sB + st.s * B_BYTES, &tmap_w, kb * BK, n_blk * kGrpBN, &full[st.s]);
-          st.next(NS);
+          st = nx;
         }
       }
       if (!ok) {
@@ -118,7 +121,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       constexpr uint32_t idesc = idesc_i8(BM, kGrpBN);
       Ring st;
       bool ok = true;

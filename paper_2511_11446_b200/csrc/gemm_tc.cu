@@ -67,16 +67,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const int total_tiles = p.m_tiles * p.n_tiles;
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;  // 0 = leader of the pair
   const int first_tile = blockIdx.x / CG, tile_stride = gridDim.x / CG;
-  // TMA loads of operand stages: in a pair both CTAs' bytes are counted on the leader's barrier
-  auto stage_expect = [&](uint64_t* bar, uint32_t bytes) {
-    if constexpr (CG == 2) mbar_arrive_expect_tx_cluster(map_to_cta(bar, 0), bytes);
-    else mbar_arrive_expect_tx(bar, bytes);
-  };
-  auto stage_load = [&](void* dst, const CUtensorMap* tm, int c0, int c1, uint64_t* bar) {
-    if constexpr (CG == 2) tma_load_2d_pair(dst, tm, c0, c1, map_to_cta(bar, 0));
-    else tma_load_2d(dst, tm, c0, c1, bar);
-  };
-
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&full_a[i], CG);  // pair: the leader's copy counts both CTAs' TMA loads
@@ -128,48 +118,82 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   // constants; unless early_w is set, everything waits here.
   if (!p.early_w) pdl_wait();
 
+  // The two single-thread roles run behind elect.sync, not a lane comparison: the compiler then knows
+  // that one thread is active and keeps descriptors, addresses and barriers in uniform registers. Behind
+  // `lane == 0` the four MMAs and the commit of a k-block took 317 cycles to issue and the two TMA
+  // loads 224, which set a pace of ~560 cycles per k-block at EVERY tile width (64 .. 256; the tensor
+  // core needs 128 .. 512); this way they take 100 and 127. A stage's barrier is polled one k-block
+  // ahead, before the current one's instructions, so the poll's ~75 cycles run under them.
   if (warp == 0) {
     // ================= TMA producer =================
-    if (lane == 0) {
+    if (elect_one()) {
       Ring st, ps;
       bool ok = true;
       bool a_open = !p.early_w || p.x != nullptr;  // false until griddepcontrol.wait has been executed
       int ready_tile = -1;                          // in-kernel DAQ: last 128-token tile seen complete
-      int deferred = 0;          // stages whose weight tile is in flight but whose A tile is not
-      int def_kb[NS], def_m[NS], def_s[NS];
+      // In a pair both CTAs' bytes are counted on the leader's barrier.
+      const uint32_t full0 = CG == 2 ? map_to_cta(&full_a[0], 0) : smem_u32(&full_a[0]);
+      auto expect = [&](int s, uint32_t bytes) {
+        if constexpr (CG == 2) mbar_arrive_expect_tx_cluster(full0 + 8u * s, bytes);
+        else mbar_arrive_expect_tx(&full_a[s], bytes);
+      };
+      auto load = [&](void* dst, const CUtensorMap* tm, int c0, int c1, int s) {
+        if constexpr (CG == 2) tma_load_2d_pair(dst, tm, c0, c1, full0 + 8u * s);
+        else tma_load_2d(dst, tm, c0, c1, &full_a[s]);
+      };
+      auto load_a = [&](int tile, int kb, int s) {
+        int c0, c1;
+        a_tile_coords(p, (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM, kb, c0, c1);
+        load(sA + s * A_BYTES, &tmap_a, c0, c1, s);
+      };
+      // Stages whose weight tile is in flight but whose activation tile is not (before a_open): they are
+      // the ring's first ones, in order, from (first_tile, k-block 0) on.
+      int deferred = 0;
+      auto open_a = [&]() {
+        pdl_wait();
+        a_open = true;
+        int t = first_tile, k = 0;
+        for (int d = 0; d < deferred; ++d) {
+          load_a(t, k, d);
+          if (++k == KB) {
+            k = 0;
+            t += tile_stride;
+          }
+        }
+      };
+      bool free_next = mbar_test_wait(&empty[0], 1u);
       for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
         const int n_blk = tile % p.n_tiles;  // column tiles of one row strip run together
         const int m_row = (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM;
         const int w_row = n_blk * BN + static_cast<int>(rank) * BNL;
         bool a_ready = p.x == nullptr || (m_row >> 7) == ready_tile;
-        for (int kb = 0; kb < KB; ++kb) {
+        int a0, a1;
+        a_tile_coords(p, m_row, 0, a0, a1);
+        const int a0_step = p.a_tiled ? 0 : BK, a1_step = p.a_tiled ? BM : 0;
+        for (int kb = 0; kb < KB; ++kb, a0 += a0_step, a1 += a1_step) {
           if constexpr (CG == 1 && BITS == 8) {
             // test hook: this stage gets no loads and no arrival, so its barrier never completes and
             // the bounded waits of the other roles run out
             if (kb == p.dbg_skip_kb && tile == first_tile) {
+              if (!a_open) open_a();
               st.next(NS);
+              free_next = false;
               continue;
             }
           }
-          if (!a_open && deferred == NS) {  // ring full of weight tiles: now wait for the activations
-            pdl_wait();
-            a_open = true;
-            for (int d = 0; d < deferred; ++d) {
-              int c0, c1;
-              a_tile_coords(p, def_m[d], def_kb[d], c0, c1);
-              stage_load(sA + def_s[d] * A_BYTES, &tmap_a, c0, c1, &full_a[def_s[d]]);
-            }
-            deferred = 0;
-          }
-          if (!(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          if (!a_open && deferred == NS) open_a();  // ring full of weight tiles: now wait for the activations
+          if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          Ring nx = st;
+          nx.next(NS);
+          free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
           if constexpr (BITS == 8) {
-            stage_expect(&full_a[st.s], A_BYTES + B_BYTES);
-            stage_load(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, &full_a[st.s]);
+            expect(st.s, A_BYTES + B_BYTES);
+            load(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, st.s);
           } else {
-            if (!(ok = mbar_wait(&pempty[ps.s], ps.ph ^ 1u, abort_flag))) break;
+            if (!(ok = mbar_spin_wait(&pempty[ps.s], ps.ph ^ 1u, abort_flag))) break;
             mbar_arrive_expect_tx(&pfull[ps.s], P_BYTES);
             tma_load_2d(sP + ps.s * P_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[ps.s]);
-            stage_expect(&full_a[st.s], A_BYTES);
+            expect(st.s, A_BYTES);
             ps.next(NP);
           }
           if (a_open) {
@@ -180,26 +204,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               ready_tile = m_row >> 7;
               a_ready = true;
             }
-            int c0, c1;
-            a_tile_coords(p, m_row, kb, c0, c1);
-            stage_load(sA + st.s * A_BYTES, &tmap_a, c0, c1, &full_a[st.s]);
+            load(sA + st.s * A_BYTES, &tmap_a, a0, a1, st.s);
           } else {
-            def_kb[deferred] = kb;
-            def_m[deferred] = m_row;
-            def_s[deferred] = st.s;
             ++deferred;
           }
-          st.next(NS);
+          st = nx;
         }
       }
-      if (!a_open) {  // fewer k-blocks than stages in the whole CTA
-        pdl_wait();
-        for (int d = 0; d < deferred; ++d) {
-          int c0, c1;
-          a_tile_coords(p, def_m[d], def_kb[d], c0, c1);
-          stage_load(sA + def_s[d] * A_BYTES, &tmap_a, c0, c1, &full_a[def_s[d]]);
-        }
-      }
+      if (!a_open) open_a();  // fewer k-blocks than stages in the whole CTA
       if (!ok) {
         // drain: give copies still in flight a bounded time to land before the CTA exits
         const long long t0 = clock64();
@@ -208,7 +220,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       if (CG == 2 && rank != 0) {
         // ================= pair follower: report each expanded weight stage to the leader =================
         // (TMA loads of both CTAs are counted on the leader's barrier directly)
@@ -217,7 +229,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           bool ok = true;
           for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
             for (int kb = 0; kb < KB; ++kb) {
-              if (!(ok = mbar_wait(&bready[st.s], st.ph, abort_flag))) break;
+              if (!(ok = mbar_spin_wait(&bready[st.s], st.ph, abort_flag))) break;
               mbar_arrive_cluster(map_to_cta(&peer_ready[st.s], 0));
               st.next(NS);
             }
@@ -226,28 +238,31 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       } else {
         // ================= MMA issuer =================
         constexpr uint32_t idesc = idesc_i8(BM * CG, BN);
+        const uint64_t adesc0 = smem_desc_sw128(smem_u32(sA)), bdesc0 = smem_desc_sw128(smem_u32(sB));
         Ring st;
         bool ok = true;
         int tcount = 0;
+        bool full_next = mbar_test_wait(&full_a[0], 0u);
         for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride, ++tcount) {
           const int buf = tcount & 1;
           const uint32_t aph = (tcount >> 1) & 1;
-          if (!(ok = CG == 2 ? mbar_wait_cluster(&acc_empty[buf], aph ^ 1u, abort_flag)
-                             : mbar_wait(&acc_empty[buf], aph ^ 1u, abort_flag)))
-            break;
+          if (!(ok = mbar_spin_wait(&acc_empty[buf], aph ^ 1u, abort_flag))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + buf * (TCOLS / 2);
           for (int kb = 0; kb < KB; ++kb) {
-            if (!(ok = mbar_spin_wait(&full_a[st.s], st.ph, abort_flag))) break;
+            if (!full_next && !(ok = mbar_spin_wait(&full_a[st.s], st.ph, abort_flag))) break;
             if constexpr (BITS != 8) {
-              if (!(ok = mbar_wait(&bready[st.s], st.ph, abort_flag))) break;
+              if (!(ok = mbar_spin_wait(&bready[st.s], st.ph, abort_flag))) break;
               if constexpr (CG == 2) {
-                if (!(ok = mbar_wait_cluster(&peer_ready[st.s], st.ph, abort_flag))) break;
+                if (!(ok = mbar_spin_wait(&peer_ready[st.s], st.ph, abort_flag))) break;
               }
             }
             tc_fence_after();
-            const uint64_t adesc = smem_desc_sw128(smem_u32(sA + st.s * A_BYTES));
-            const uint64_t bdesc = smem_desc_sw128(smem_u32(sB + st.s * B_BYTES));
+            Ring nx = st;
+            nx.next(NS);
+            full_next = mbar_test_wait(&full_a[nx.s], nx.ph);
+            const uint64_t adesc = adesc0 + static_cast<uint64_t>(st.s * (A_BYTES >> 4));
+            const uint64_t bdesc = bdesc0 + static_cast<uint64_t>(st.s * (B_BYTES >> 4));
 #pragma unroll
             for (int k4 = 0; k4 < BK / 32; ++k4) {  // 32 bytes of K per instruction: +2 in 16-byte units
               if constexpr (CG == 2)
@@ -257,7 +272,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             }
             if constexpr (CG == 2) mma_commit_pair(&empty[st.s]);
             else mma_commit(&empty[st.s]);
-            st.next(NS);
+            st = nx;
           }
           if (ok) {
             if constexpr (CG == 2) mma_commit_pair(&acc_full[buf]);

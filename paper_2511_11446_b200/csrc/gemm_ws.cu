@@ -98,10 +98,11 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
   if (warp == 0) {
     // ================= TMA producer =================
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st, pr;
       bool ok = true, a_open = !p.early_w || p.x != nullptr;
       int cur_strip = -1, strips = 0, ready_tile = -1;
+      const uint32_t full0 = map_to_cta(&full_a[0], 0);
       for (int item = item0; item < item1 && ok; ++item) {
         const int strip = strip_of(item);
         if (strip != cur_strip) {
@@ -141,15 +142,19 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           if (!(ok = wait_tile_quantized(p, m_row >> 7, abort_flag))) break;
           ready_tile = m_row >> 7;
         }
+        bool free_next = mbar_test_wait(&empty[st.s], st.ph ^ 1u);  // polled one k-block ahead, as in gemm_tc.cu
         for (int kb = 0; kb < KB; ++kb) {
-          if (!(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          Ring nx = st;
+          nx.next(NS);
+          free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
           // both CTAs' activation tiles are counted on the LEADER's barrier: the MMA thread waits once
-          const uint32_t bar = map_to_cta(&full_a[st.s], 0);
+          const uint32_t bar = full0 + 8u * static_cast<uint32_t>(st.s);
           mbar_arrive_expect_tx_cluster(bar, A_BYTES);
           int c0, c1;
           a_tile_coords(p, m_row, kb, c0, c1);
           tma_load_2d_pair(sA + st.s * A_BYTES, &tmap_a, c0, c1, bar);
-          st.next(NS);
+          st = nx;
         }
       }
       if (!ok) {
@@ -159,7 +164,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       if (rank != 0) {
         // ================= pair follower: report each resident strip to the leader =================
         bool ok = true;
@@ -176,31 +181,35 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       } else {
         // ================= MMA issuer =================
         constexpr uint32_t idesc = idesc_i8(BM * CG, BN);
+        const uint64_t adesc0 = smem_desc_sw128(smem_u32(sA)), bdesc0 = smem_desc_sw128(smem_u32(sW));
         Ring st;
-        bool ok = true;
+        bool ok = true, full_next = false;
         int tcount = 0, cur_strip = -1, strips = 0;
         for (int item = item0; item < item1 && ok; ++item, ++tcount) {
           if (strip_of(item) != cur_strip) {
             if (!(ok = mbar_wait(w_full, strips & 1u, abort_flag))) break;
-            if (!(ok = mbar_wait_cluster(w_peer, strips & 1u, abort_flag))) break;
+            if (!(ok = mbar_spin_wait(w_peer, strips & 1u, abort_flag))) break;
             cur_strip = strip_of(item);
             ++strips;
           }
           const int buf = tcount & 1;
           const uint32_t aph = (tcount >> 1) & 1;
-          if (!(ok = mbar_wait_cluster(&acc_empty[buf], aph ^ 1u, abort_flag))) break;
+          if (!(ok = mbar_spin_wait(&acc_empty[buf], aph ^ 1u, abort_flag))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + buf * (TCOLS / 2);
           for (int kb = 0; kb < KB; ++kb) {
-            if (!(ok = mbar_spin_wait(&full_a[st.s], st.ph, abort_flag))) break;  // both CTAs' tiles landed
+            if (!full_next && !(ok = mbar_spin_wait(&full_a[st.s], st.ph, abort_flag))) break;  // both CTAs' tiles landed
             tc_fence_after();
-            const uint64_t adesc = smem_desc_sw128(smem_u32(sA + st.s * A_BYTES));
-            const uint64_t bdesc = smem_desc_sw128(smem_u32(sW + kb * B_BYTES));
+            Ring nx = st;
+            nx.next(NS);
+            full_next = mbar_test_wait(&full_a[nx.s], nx.ph);
+            const uint64_t adesc = adesc0 + static_cast<uint64_t>(st.s * (A_BYTES >> 4));
+            const uint64_t bdesc = bdesc0 + static_cast<uint64_t>(kb * (B_BYTES >> 4));
 #pragma unroll
             for (int k4 = 0; k4 < BK / 32; ++k4)
               mma_i8_ss_pair(d_tmem, adesc + 2 * k4, bdesc + 2 * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
             mma_commit_pair(&empty[st.s]);
-            st.next(NS);
+            st = nx;
           }
           if (!ok) break;
           mma_commit_pair(&acc_full[buf]);
