@@ -125,12 +125,15 @@ def lib():
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()  # every pointer parameter is declared c_void_p: an int is enough
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    # The handle alone: building a torch.cuda.Stream object for the current stream took 3.2 us of the
+    # 6 us that a call spent in Python (a launch itself takes 2.3), the raw lookup takes 0.2.
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _check(st, where):
@@ -173,7 +176,7 @@ def dp_daq_quantize_robust(x, M, K, ldx, q, ldq, s_a, rank, act_bits=8, rowsum=N
 
 def dp_wq_linear(w: dp_weight, x, ldx, s_a_in, M, y, ldy, workspace, dbg: dp_debug | None = None,
                  device_status=None, flags=0, stream=None):
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    ws_bytes = 0 if workspace is None else workspace.nbytes
     _check(lib().dp_wq_linear(C.byref(w), _ptr(x), ldx, _ptr(s_a_in), M, _ptr(y), ldy, _ptr(workspace),
                               ws_bytes, None if dbg is None else C.byref(dbg), _ptr(device_status),
                               flags, _stream(stream)), "dp_wq_linear")
@@ -267,7 +270,7 @@ def dp_plan_run(plan, steps, start_index, x_ptrs, y_ptrs, workspace, device_stat
     """x_ptrs / y_ptrs: ctypes arrays of device addresses (see ptr_array)."""
     st = (C.c_int32 * len(steps))(*steps)
     _check(lib().dp_plan_run(plan, st, len(steps), start_index, x_ptrs, y_ptrs, _ptr(workspace),
-                             workspace.numel() * workspace.element_size(), _ptr(device_status), flags,
+                             workspace.nbytes, _ptr(device_status), flags,
                              _stream(stream)), "dp_plan_run")
 
 
@@ -275,8 +278,8 @@ def dp_plan_run_host(plan, steps, x_host, x_stage, y_dev, d2h_layer, y_host, wor
                      device_status=None, flags=0, stream=None):
     st = (C.c_int32 * len(steps))(*steps)
     _check(lib().dp_plan_run_host(plan, st, len(steps), x_host, _ptr(x_stage),
-                                  x_stage.numel() * x_stage.element_size(), y_dev, d2h_layer, y_host,
-                                  _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                  x_stage.nbytes, y_dev, d2h_layer, y_host,
+                                  _ptr(workspace), workspace.nbytes,
                                   _ptr(device_status), flags, _stream(stream)), "dp_plan_run_host")
 
 
