@@ -238,18 +238,19 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     float* wsa = reinterpret_cast<float*>(ws8 + align256(scratch_q_bytes(M, w->K)));
     size_t off = align256(scratch_q_bytes(M, w->K)) + align256(sizeof(float) * static_cast<size_t>(M));
     const int8_t* w8 = static_cast<const int8_t*>(w->qweight);
-    UnpackJob job{nullptr, nullptr, 0, 0, 0};
+    UnpackJob job{nullptr, nullptr, 0, 0, 0, chained && pdl};
     if (w->bits < 8) {
       int8_t* dst = reinterpret_cast<int8_t*>(ws8 + off);
       off += align256(static_cast<size_t>(w->N) * w->K);
-      job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0};
+      job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0,
+                    chained && pdl};
       w8 = dst;
     }
     int32_t* rowsum = w->zeros != nullptr ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
     int st = robust ? launch_daq_robust(x, M, w->K, ldx, wq, w->K, wsa, nullptr, daq_rank, daq_bits, true, stream, pdl,
-                                        w->bits < 8 ? &job : nullptr)
+                                        &job)
                     : launch_daq(x, M, w->K, ldx, wq, w->K, wsa, nullptr, KORDER_NATURAL, true, stream, pdl,
-                                 w->bits < 8 ? &job : nullptr);
+                                 &job);
     if (st != DP_OK) return st;
     return launch_gemm_grp(wq, w->K, true, wsa, w8, w->bits, w->group_size, w->s_w, static_cast<const uint8_t*>(w->zeros),
                            static_cast<const uint16_t*>(w->bias), rowsum, M, w->N, w->K, static_cast<uint16_t*>(y), ldy,
@@ -305,11 +306,12 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   }
   const bool unpack_first = pre > 0 && w->bits < 8;
   dp_weight w8 = *w;
-  UnpackJob job{nullptr, nullptr, 0, 0, 0};
+  UnpackJob job{nullptr, nullptr, 0, 0, 0, chained && pdl};
   if (unpack_first) {
     int8_t* dst = reinterpret_cast<int8_t*>(static_cast<uint8_t*>(workspace) + align256(scratch_q_bytes(M, w->K)) +
                                             align256(sizeof(float) * static_cast<size_t>(M)));
-    job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0};
+    job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0,
+                    chained && pdl};
     w8.bits = 8;
     w8.qweight = dst;
     w = &w8;
@@ -324,11 +326,11 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     korder = gemm_korder(w->bits);
     if (robust) {
       int st = launch_daq_robust(x, M, w->K, ldx, wq, w->K, wsa, nullptr, daq_rank, daq_bits, true, stream, pdl,
-                                 unpack_first ? &job : nullptr);
+                                 &job);
       if (st != DP_OK) return st;
     } else if (!fused) {
       int st = launch_daq(x, M, w->K, ldx, wq, w->K, wsa, nullptr, korder, true, stream, pdl,
-                          unpack_first ? &job : nullptr);
+                          &job);
       if (st != DP_OK) return st;
     }
     q = wq;

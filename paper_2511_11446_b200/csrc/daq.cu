@@ -11,28 +11,41 @@
 namespace dp {
 
 constexpr int kDaqWarps = 8;
+constexpr int kDaqThreads = 128;  // CTA of the register-resident kernel
 
-// MAXV = 16-byte vectors held per lane (row of up to 256*MAXV elements in registers).
-template <int MAXV, bool EO>
-__global__ void __launch_bounds__(kDaqWarps * 32)
+// The first launch of a call lets its dependents start only once everything before the call has
+// finished (they may read the layers' constants ahead of their own wait, and those may have been written by
+// the kernel before the call); later ones let them start at once.
+__device__ __forceinline__ void daq_begin(const UnpackJob& job) {
+  if (!job.early) pdl_wait();
+  pdl_launch_dependents();
+}
+
+// RW warps share a row: MAXV = 16-byte vectors held per lane (a row of up to 256 * RW * MAXV elements in
+// registers). SUM: also the row's code sum.
+template <int RW, int MAXV, bool EO, bool SUM>
+__global__ void __launch_bounds__(kDaqThreads)
 daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
                 int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
                 int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
-  pdl_launch_dependents();
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kDaqWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  pdl_wait();
+  constexpr int kRows = kDaqThreads / 32 / RW;  // rows of a CTA
+  constexpr int TPR = 32 * RW;
+  __shared__ uint32_t part[kDaqThreads / 32];
+  daq_begin(job);
   if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
-  if (row >= M) return;
-  const int nvec = K >> 3;
+  pdl_wait();
+  const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;  // row of the CTA, position in the row
+  const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + rw;
+  const bool live = row < M;
+  const int nvec = live ? K >> 3 : 0;
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
   uint4 v[MAXV];
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
+    const int idx = lane + TPR * i;
     if (idx < nvec) ld_nc_u32x4(xr + idx, v[i]);
     else v[i] = make_uint4(0, 0, 0, 0);
   }
@@ -45,24 +58,41 @@ daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
     m = absmax_bits2(m, v[i].w);
   }
   m = warp_max_u32(max(m & 0xFFFFu, m >> 16));
+  if constexpr (RW > 1) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < RW; ++w) m = max(m, part[rw * RW + w]);
+  }
+  if (RW == 1 && !live) return;
   float sc, inv;
   token_scale(m, sc, inv);
   const QRow qr(q, row, ldq, tiled_kb);
   int sum = 0;
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
+    const int idx = lane + TPR * i;
     if (idx < nvec) {
       uint2 o = quant_vec<EO>(v[i], inv);
       qr.store(idx, o);
-      sum = __dp4a(static_cast<int>(o.x), 0x01010101, sum);
-      sum = __dp4a(static_cast<int>(o.y), 0x01010101, sum);
+      if constexpr (SUM) {
+        sum = __dp4a(static_cast<int>(o.x), 0x01010101, sum);
+        sum = __dp4a(static_cast<int>(o.y), 0x01010101, sum);
+      }
     }
   }
-  if (lane == 0) s_a[row] = sc;
-  if (rowsum != nullptr) {
+  if (lane == 0 && live) s_a[row] = sc;
+  if constexpr (SUM) {
     sum = warp_sum_i32(sum);
-    if (lane == 0) rowsum[row] = sum;
+    if constexpr (RW > 1) {
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = static_cast<uint32_t>(sum);
+      __syncthreads();
+      sum = 0;
+#pragma unroll
+      for (int w = 0; w < RW; ++w) sum += static_cast<int>(part[rw * RW + w]);
+    }
+    if (lane == 0 && live) rowsum[row] = sum;
   }
 }
 
@@ -72,14 +102,14 @@ __global__ void __launch_bounds__(kDaqWarps * 32)
 daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
                       int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
                       int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
-  pdl_launch_dependents();
+  daq_begin(job);
   const int64_t row = static_cast<int64_t>(blockIdx.x) * kDaqWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  pdl_wait();
   if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
+  pdl_wait();
   if (row >= M) return;
   const int nvec = K >> 3;
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
@@ -112,14 +142,14 @@ __global__ void __launch_bounds__(kDaqWarps * 32, MAXV <= 5 ? 3 : 2)  // registe
 daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx, int8_t* __restrict__ q,
                        int64_t ldq, float* __restrict__ s_a, int32_t* __restrict__ rowsum, int clip_rank,
                        float qmax, int tiled_kb, const UnpackJob job) {
-  pdl_launch_dependents();
+  daq_begin(job);
   const int64_t row = static_cast<int64_t>(blockIdx.x) * kDaqWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  pdl_wait();
   if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
+  pdl_wait();
   if (row >= M) return;
   const QRow qr(q, row, ldq, tiled_kb);
   float sc;
@@ -134,27 +164,41 @@ daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t
 
 __global__ void __launch_bounds__(kDaqWarps * 32)
 unpack_kernel(const UnpackJob job) {
-  pdl_launch_dependents();
-  pdl_wait();
+  daq_begin(job);
   unpack_units(job, blockIdx.x);
 }
 
-template <bool EO>
+static unsigned unpack_blocks(const UnpackJob& job, int threads) {
+  return static_cast<unsigned>((job.units + threads - 1) / threads);
+}
+
+template <int RW, int MAXV, bool EO, bool SUM, typename... A>
+static cudaError_t launch_rows(int64_t M, UnpackJob job, cudaStream_t stream, bool pdl, A... a) {
+  constexpr int kRows = kDaqThreads / 32 / RW;
+  const unsigned daq_blocks = static_cast<unsigned>((M + kRows - 1) / kRows);
+  job.first_block = static_cast<int32_t>(daq_blocks);
+  const dim3 grid(daq_blocks + unpack_blocks(job, kDaqThreads));
+  return launch(daq_rows_kernel<RW, MAXV, EO, SUM>, grid, dim3(kDaqThreads), 0, stream, pdl, a..., job);
+}
+
+template <bool EO, bool SUM>
 static cudaError_t launch_daq_t(const uint16_t* xp, int64_t M, int k, int64_t ldx, int8_t* q, int64_t ldq,
                                 float* s_a, int32_t* rowsum, int tiled_kb, cudaStream_t stream, bool pdl,
                                 UnpackJob job) {
+#define DP_ROWS(RW, MAXV) launch_rows<RW, MAXV, EO, SUM>(M, job, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb)
+  // As many warps to a row as leave a lane at most five vectors: a row of 4608 held by one warp (18 vectors,
+  // ~90 registers) left one CTA beside a running GEMM and a long serial chain per warp. Whole 8-bit layer,
+  // K = 4608, N = 1152, M = 256 / 2048 / 32768: one warp 12.1 / 18.8 / 182.5 us, two 12.3 / 17.6 / 182.5,
+  // four 12.1 / 17.4 / 181.7. Shorter rows want one: K = 1152 whole layer (N = 1152), M = 2048 / 32768: one
+  // 8.8 / 56.8 us, two 9.2 / 58.1, four 8.8 / 70.3 (their warps spend longer starting than working).
+  if (k <= 256 * 5) return DP_ROWS(1, 5);
+  if (k <= 512 * 5) return DP_ROWS(2, 5);
+  if (k <= 1024 * 5) return DP_ROWS(4, 5);
+#undef DP_ROWS
   const unsigned daq_blocks = static_cast<unsigned>((M + kDaqWarps - 1) / kDaqWarps);
   job.first_block = static_cast<int32_t>(daq_blocks);
-  const unsigned extra = static_cast<unsigned>((job.units + kDaqWarps * 32 - 1) / (kDaqWarps * 32));
-  const dim3 grid(daq_blocks + extra);
-  const dim3 block(kDaqWarps * 32);
-  if (k <= 256 * 5)
-    return launch(daq_rows_kernel<5, EO>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, job);
-  if (k <= 256 * 9)
-    return launch(daq_rows_kernel<9, EO>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, job);
-  if (k <= 256 * 18)
-    return launch(daq_rows_kernel<18, EO>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, job);
-  return launch(daq_rows_2pass_kernel<EO>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, job);
+  return launch(daq_rows_2pass_kernel<EO>, dim3(daq_blocks + unpack_blocks(job, kDaqWarps * 32)), dim3(kDaqWarps * 32), 0,
+                stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, job);
 }
 
 int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq,
@@ -164,11 +208,13 @@ int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int6
   const uint16_t* xp = static_cast<const uint16_t*>(x);
   const int k = static_cast<int>(K);
   const int tiled_kb = tiled ? k / 128 : 0;
-  UnpackJob job{nullptr, nullptr, 0, 0, 0};
+  UnpackJob job{nullptr, nullptr, 0, 0, 0, 0};
   if (unpack != nullptr) job = *unpack;
   const cudaError_t e = korder == KORDER_EVEN_ODD
-                            ? launch_daq_t<true>(xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, stream, pdl, job)
-                            : launch_daq_t<false>(xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, stream, pdl, job);
+                            ? launch_daq_t<true, false>(xp, M, k, ldx, q, ldq, s_a, nullptr, tiled_kb, stream, pdl, job)
+                        : rowsum != nullptr
+                            ? launch_daq_t<false, true>(xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, stream, pdl, job)
+                            : launch_daq_t<false, false>(xp, M, k, ldx, q, ldq, s_a, rowsum, tiled_kb, stream, pdl, job);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "DAQ launch failed: %s", cudaGetErrorString(e));
   return DP_OK;
 }
@@ -181,12 +227,11 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
   const int k = static_cast<int>(K);
   const int tiled_kb = tiled ? k / 128 : 0;
   const float qmax = static_cast<float>((1 << (act_bits - 1)) - 1);
-  UnpackJob job{nullptr, nullptr, 0, 0, 0};
+  UnpackJob job{nullptr, nullptr, 0, 0, 0, 0};
   if (unpack != nullptr) job = *unpack;
   const unsigned daq_blocks = static_cast<unsigned>((M + kDaqWarps - 1) / kDaqWarps);
   job.first_block = static_cast<int32_t>(daq_blocks);
-  const unsigned extra = static_cast<unsigned>((job.units + kDaqWarps * 32 - 1) / (kDaqWarps * 32));
-  const dim3 grid(daq_blocks + extra), block(kDaqWarps * 32);
+  const dim3 grid(daq_blocks + unpack_blocks(job, kDaqWarps * 32)), block(kDaqWarps * 32);
   cudaError_t e;
   if (k <= 256 * 5)
     e = launch(daq_rows_robust_kernel<5>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank,
@@ -203,7 +248,7 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
 
 int launch_unpack(const UnpackJob& job, cudaStream_t stream, bool pdl) {
   if (job.units == 0) return DP_OK;
-  const dim3 grid(static_cast<unsigned>((job.units + kDaqWarps * 32 - 1) / (kDaqWarps * 32)));
+  const dim3 grid(unpack_blocks(job, kDaqWarps * 32));
   const cudaError_t e = launch(unpack_kernel, grid, dim3(kDaqWarps * 32), 0, stream, pdl, job);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "weight expansion launch failed: %s", cudaGetErrorString(e));
   return DP_OK;

@@ -287,21 +287,27 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t
   }
 }
 
-// CTA `block` of an unpack job: one thread per unit of 32 codes (12 or 16 bytes in, 32 bytes out).
+// CTA `block` of an unpack job: one thread per unit of 32 codes (12 or 16 bytes in, 32 bytes out). Executes
+// griddepcontrol.wait before it writes (the destination may still be read by the preceding kernel) and,
+// unless job.early, before it reads.
 __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int block) {
   const int64_t u = static_cast<int64_t>(block) * blockDim.x + threadIdx.x;
-  if (u >= job.units) return;
+  if (!job.early) pdl_wait();
   uint32_t w[8];
-  if (job.bits == 4) {
-    const uint4 v = reinterpret_cast<const uint4*>(job.packed)[u];
-    const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
-    expand_unit<4>(pk, w);
-  } else {
-    const uint32_t* p = job.packed + u * 3;
-    const uint32_t pk[3] = {p[0], p[1], p[2]};
-    expand_unit<3>(pk, w);
+  if (u < job.units) {
+    if (job.bits == 4) {
+      const uint4 v = reinterpret_cast<const uint4*>(job.packed)[u];
+      const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
+      expand_unit<4>(pk, w);
+    } else {
+      const uint32_t* p = job.packed + u * 3;
+      const uint32_t pk[3] = {p[0], p[1], p[2]};
+      expand_unit<3>(pk, w);
+    }
   }
-  st_global_v8(reinterpret_cast<uint4*>(job.out) + u * 2, w);  // 32 bytes, read next by the GEMM through L2
+  if (job.early) pdl_wait();
+  if (u < job.units)
+    st_global_v8(reinterpret_cast<uint4*>(job.out) + u * 2, w);  // 32 bytes, read next by the GEMM through L2
 }
 
 }  // namespace dp

@@ -26,6 +26,7 @@ struct UnpackJob {
   int64_t units;
   int32_t bits;         // 3 or 4
   int32_t first_block;  // filled by the launcher: CTAs from here on unpack
+  int32_t early;        // the preceding kernel on the stream cannot be writing `packed`: read before it has finished
 };
 int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq,
                float* s_a, int32_t* rowsum, int korder, bool tiled, cudaStream_t stream, bool pdl,
@@ -136,7 +137,7 @@ int gemm_encode_w(CUtensorMap* out, const void* qweight, int32_t N, int32_t K, i
 int launch_gemm(const GemmProblem& p, cudaStream_t stream, bool pdl);
 void gemm_debug_skip_stage_load(int32_t kb);  // see dp_debug_skip_stage_load
 // Two ranges (a plan's next layer's packed weights and its bf16 input) that the calling thread's next
-// launch_gemm sends on their way into L2 while it runs; cleared by that launch. Hints: any valid
+// tensor-core launch sends on their way into L2 while it runs; cleared by that launch. Hints: any valid
 // device ranges of the caller's, or nullptr.
 void gemm_set_next_reads(const void* w, size_t w_bytes, const void* x, size_t x_bytes);
 

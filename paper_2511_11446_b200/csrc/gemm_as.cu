@@ -97,6 +97,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const uint32_t tmem_base = *tmem_slot;
 
   pdl_launch_dependents();
+  if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
 
   if (warp == 0) {
     // ================= TMA producer =================
@@ -323,6 +324,7 @@ int launch_gemm_as(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   const int stage_bytes = (bns / 2) * BK;
   ap.stages = kAsRingBytes / stage_bytes > kAsMaxStages ? kAsMaxStages : kAsRingBytes / stage_bytes;
   const dim3 grid(static_cast<unsigned>(2 * ((ap.units + ap.units_per_pair - 1) / ap.units_per_pair)));
+  p.next = take_next_reads(grid.x);
   const cudaError_t e = launch_cluster(gemm_as_kernel, grid, dim3(kAsThreads), as_smem_bytes(), stream, pdl, 2u,
                                        g.tmap_a, g.tmap_w, p, ap);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "activation-stationary GEMM launch failed: %s", cudaGetErrorString(e));

@@ -39,6 +39,7 @@ struct BfParams {
   int32_t N, K;
   int32_t m_tiles, n_tiles;
   int32_t* status;
+  NextReads next;
 };
 
 __host__ __device__ constexpr int bf_stages(int bn) { return (200 * 1024) / ((BM + bn) * kBfBK); }
@@ -91,6 +92,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   const uint32_t tmem_base = *tmem_slot;
 
   pdl_launch_dependents();
+  if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
   pdl_wait();  // the activations may come from the preceding kernel on the stream
 
   if (warp == 0) {
@@ -258,6 +260,7 @@ int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* 
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   const int sms = num_sms() > 0 ? num_sms() : 148;
   const dim3 grid(static_cast<unsigned>(tiles < sms ? tiles : sms)), block(kBfThreads);
+  p.next = take_next_reads(grid.x);
   cudaError_t e;
   if (bn == 256) e = launch(gemm_bf16_kernel<256>, grid, block, bf_smem_bytes<256>(), stream, pdl, ta, tw, p);
   else if (bn == 128) e = launch(gemm_bf16_kernel<128>, grid, block, bf_smem_bytes<128>(), stream, pdl, ta, tw, p);

@@ -30,6 +30,28 @@ __host__ __device__ constexpr int num_stages(int bn, int bits) {
 }
 __host__ __device__ constexpr int tmem_cols(int bn) { return bn <= 64 ? 128 : bn <= 128 ? 256 : 512; }
 
+// Two ranges a later launch will read soon (a plan's next layer's packed weights and its bf16 input):
+// each CTA sends its slices on the way into L2 while this kernel, which leaves HBM mostly idle at a
+// few thousand tokens, runs. Hints only (L2 is the point of coherence: a range rewritten after the
+// hint is simply current when it is read); nullptr: none.
+struct NextReads {
+  const uint8_t* ptr[2] = {nullptr, nullptr};
+  uint32_t bytes[2] = {0, 0}, slice[2] = {0, 0};
+};
+// One thread of each CTA.
+__device__ __forceinline__ void prefetch_next_reads(const NextReads& n) {
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const uint32_t off = blockIdx.x * n.slice[r];
+    if (n.ptr[r] != nullptr && off < n.bytes[r]) {
+      const uint32_t len = min(n.slice[r], n.bytes[r] - off);
+      for (uint32_t o = 0; o < len; o += 32768u) bulk_prefetch_l2(n.ptr[r] + off + o, min(32768u, len - o));
+    }
+  }
+}
+// The ranges given to gemm_set_next_reads by the calling thread, cut into slices for `ctas` CTAs; consumed.
+NextReads take_next_reads(unsigned ctas);
+
 struct GemmParams {
   const float* s_a;
   const float* s_w;
@@ -61,12 +83,7 @@ struct GemmParams {
   int32_t a_tiled;  // activations are stored as contiguous 128 x 128 tiles
   int32_t early_w;  // weights may be fetched before the preceding kernel on the stream has finished
   int32_t* status;
-  // Two ranges a later launch will read soon (a plan's next layer's packed weights and its bf16 input):
-  // each CTA sends its slices on the way into L2 while this kernel, which leaves HBM mostly idle at a
-  // few thousand tokens, runs. Hints only (L2 is the point of coherence: a range rewritten after the
-  // hint is simply current when it is read); nullptr: none.
-  const uint8_t* pf[2] = {nullptr, nullptr};
-  uint32_t pf_bytes[2] = {0, 0}, pf_slice[2] = {0, 0};
+  NextReads next;
   int32_t dbg_skip_kb = -1;  // test hook (dp_debug_skip_stage_load): k-block whose loads are left out, or -1
 };
 

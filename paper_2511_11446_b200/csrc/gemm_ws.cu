@@ -94,6 +94,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const uint32_t tmem_base = *tmem_slot;
 
   pdl_launch_dependents();
+  if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
   if (!p.early_w) pdl_wait();
 
   if (warp == 0) {
@@ -364,6 +365,7 @@ int launch_gemm_ws(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   const int64_t pairs = gemm_max_pairs() > 0 ? gemm_max_pairs() : num_sms() / 2;
   const int per_pair = static_cast<int>((items + pairs - 1) / pairs);
   const dim3 grid(static_cast<unsigned>(2 * ((items + per_pair - 1) / per_pair)));
+  p.next = take_next_reads(grid.x);
   const cudaError_t e = g.bn == 256 ? ws_launch_bn<256>(g, p, per_pair, grid, stream, pdl)
                                     : ws_launch_bn<192>(g, p, per_pair, grid, stream, pdl);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "weight-stationary GEMM launch failed: %s", cudaGetErrorString(e));

@@ -36,6 +36,18 @@ def test_daq_matches_oracle(M, K):
     assert np.array_equal(rs, ors)
 
 
+@pytest.mark.parametrize("rowsum", [True, False])
+@pytest.mark.parametrize("M,K", [(1, 1280), (6, 1288), (3, 2560), (5, 2568), (2, 4616), (3, 5120), (2, 5128)])
+def test_daq_rows_shared_by_warps(M, K, rowsum):
+    """Row lengths on both sides of every change in the number of warps that share a row."""
+    x = synth.activations(synth.BASE_SEED, 4, 2, M, K, 1.0, n_out=max(1, K // 100))
+    q, s_a, rs = _run(x, ldq=(K + 15) // 16 * 16, rowsum=rowsum)
+    oq, osa, ors = oracle.daq(x)
+    assert np.array_equal(s_a.view(np.uint32), osa.view(np.uint32))
+    assert np.array_equal(q[:, :K], oq)
+    assert not rowsum or np.array_equal(rs, ors)
+
+
 def test_daq_edge_rows_and_pitch():
     K = 1152
     rng = np.random.default_rng(0)
