@@ -232,27 +232,36 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   const bool robust = s_a_in == nullptr && (daq_rank > 1 || daq_bits < 8);
   if (w->group_size > 0) {
     // Group-wise scales: DAQ into the tiled scratch (packed weights expanded to int8 by the same
-    // launch), the per-group code sums when there are zero-points, then the folding GEMM.
+    // launch, which takes their zero-points off: u - z fits a byte up to 4 bits), the per-group code sums
+    // when 8-bit codes have zero-points, then the folding GEMM.
+    const uint8_t* zeros = static_cast<const uint8_t*>(w->zeros);
     uint8_t* ws8 = static_cast<uint8_t*>(workspace);
     int8_t* wq = static_cast<int8_t*>(workspace);
     float* wsa = reinterpret_cast<float*>(ws8 + align256(scratch_q_bytes(M, w->K)));
     size_t off = align256(scratch_q_bytes(M, w->K)) + align256(sizeof(float) * static_cast<size_t>(M));
     const int8_t* w8 = static_cast<const int8_t*>(w->qweight);
-    UnpackJob job{nullptr, nullptr, 0, 0, 0, chained && pdl};
+    UnpackJob job;
+    job.early = chained && pdl;
     if (w->bits < 8) {
       int8_t* dst = reinterpret_cast<int8_t*>(ws8 + off);
       off += align256(static_cast<size_t>(w->N) * w->K);
-      job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0,
-                    chained && pdl};
+      job.packed = static_cast<const uint32_t*>(w->qweight);
+      job.out = dst;
+      job.units = static_cast<int64_t>(w->N) * w->K / 32;
+      job.bits = w->bits;
+      job.zeros = zeros;
+      job.row_units = w->K / 32;
+      job.group_units = w->group_size / 32;
+      zeros = nullptr;
       w8 = dst;
     }
-    int32_t* rowsum = w->zeros != nullptr ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
+    int32_t* rowsum = zeros != nullptr ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
     int st = robust ? launch_daq_robust(x, M, w->K, ldx, wq, w->K, wsa, nullptr, daq_rank, daq_bits, true, stream, pdl,
                                         &job)
                     : launch_daq(x, M, w->K, ldx, wq, w->K, wsa, nullptr, KORDER_NATURAL, true, stream, pdl,
                                  &job);
     if (st != DP_OK) return st;
-    return launch_gemm_grp(wq, w->K, true, wsa, w8, w->bits, w->group_size, w->s_w, static_cast<const uint8_t*>(w->zeros),
+    return launch_gemm_grp(wq, w->K, true, wsa, w8, w->bits, w->group_size, w->s_w, zeros,
                            static_cast<const uint16_t*>(w->bias), rowsum, M, w->N, w->K, static_cast<uint16_t*>(y), ldy,
                            status, stream, pdl);
   }
@@ -306,12 +315,15 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   }
   const bool unpack_first = pre > 0 && w->bits < 8;
   dp_weight w8 = *w;
-  UnpackJob job{nullptr, nullptr, 0, 0, 0, chained && pdl};
+  UnpackJob job;
+  job.early = chained && pdl;
   if (unpack_first) {
     int8_t* dst = reinterpret_cast<int8_t*>(static_cast<uint8_t*>(workspace) + align256(scratch_q_bytes(M, w->K)) +
                                             align256(sizeof(float) * static_cast<size_t>(M)));
-    job = UnpackJob{static_cast<const uint32_t*>(w->qweight), dst, static_cast<int64_t>(w->N) * w->K / 32, w->bits, 0,
-                    chained && pdl};
+    job.packed = static_cast<const uint32_t*>(w->qweight);
+    job.out = dst;
+    job.units = static_cast<int64_t>(w->N) * w->K / 32;
+    job.bits = w->bits;
     w8.bits = 8;
     w8.qweight = dst;
     w = &w8;

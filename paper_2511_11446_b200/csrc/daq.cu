@@ -208,7 +208,7 @@ int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int6
   const uint16_t* xp = static_cast<const uint16_t*>(x);
   const int k = static_cast<int>(K);
   const int tiled_kb = tiled ? k / 128 : 0;
-  UnpackJob job{nullptr, nullptr, 0, 0, 0, 0};
+  UnpackJob job;
   if (unpack != nullptr) job = *unpack;
   const cudaError_t e = korder == KORDER_EVEN_ODD
                             ? launch_daq_t<true, false>(xp, M, k, ldx, q, ldq, s_a, nullptr, tiled_kb, stream, pdl, job)
@@ -227,7 +227,7 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
   const int k = static_cast<int>(K);
   const int tiled_kb = tiled ? k / 128 : 0;
   const float qmax = static_cast<float>((1 << (act_bits - 1)) - 1);
-  UnpackJob job{nullptr, nullptr, 0, 0, 0, 0};
+  UnpackJob job;
   if (unpack != nullptr) job = *unpack;
   const unsigned daq_blocks = static_cast<unsigned>((M + kDaqWarps - 1) / kDaqWarps);
   job.first_block = static_cast<int32_t>(daq_blocks);

@@ -261,18 +261,21 @@ __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K
   }
 }
 
-// Packed unit -> 8 words of 4 int8 (true values, k ascending).
+// Packed unit -> 8 words of 4 int8 (u - z of the stored codes u, k ascending). z in [0, 2^BITS): the
+// zero-point in use, 2^(BITS-1) for symmetric layers. u + 128 - z stays inside its byte, and flipping the
+// byte's top bit takes the 128 off again.
 template <int BITS>
-__device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t (&w)[8]) {
-  if constexpr (BITS == 8) {
+__device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t (&w)[8], uint32_t z) {
+  const uint32_t up = 0x80808080u - z * 0x01010101u;
+  if constexpr (BITS == 8) {  // stored as they are
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = pk[i];
   } else if constexpr (BITS == 4) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint32_t lo = pk[i] & 0x0F0F0F0Fu, hi = (pk[i] >> 4) & 0x0F0F0F0Fu;
-      w[2 * i] = __vsub4(__byte_perm(lo, hi, 0x5140), 0x08080808u);
-      w[2 * i + 1] = __vsub4(__byte_perm(lo, hi, 0x7362), 0x08080808u);
+      w[2 * i] = (__byte_perm(lo, hi, 0x5140) + up) ^ 0x80808080u;
+      w[2 * i + 1] = (__byte_perm(lo, hi, 0x7362) + up) ^ 0x80808080u;
     }
   } else {
     const uint64_t lo64 = (static_cast<uint64_t>(pk[1]) << 32) | pk[0];
@@ -282,7 +285,7 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t
       const int bit = 12 * j;
       const uint32_t x = static_cast<uint32_t>(bit < 32 ? (lo64 >> bit) : (hi64 >> (bit - 32))) & 0xFFFu;
       const uint32_t o = (x & 7u) | ((x & 0x38u) << 5) | ((x & 0x1C0u) << 10) | ((x & 0xE00u) << 15);
-      w[j] = __vsub4(o, 0x04040404u);
+      w[j] = (o + up) ^ 0x80808080u;
     }
   }
 }
@@ -295,14 +298,19 @@ __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int blo
   if (!job.early) pdl_wait();
   uint32_t w[8];
   if (u < job.units) {
+    uint32_t z = 1u << (job.bits - 1);
+    if (job.zeros != nullptr) {  // one zero-point per channel and group (a multiple of 32 codes)
+      const int64_t n = u / job.row_units;
+      z = job.zeros[n * (job.row_units / job.group_units) + (u - n * job.row_units) / job.group_units];
+    }
     if (job.bits == 4) {
       const uint4 v = reinterpret_cast<const uint4*>(job.packed)[u];
       const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
-      expand_unit<4>(pk, w);
+      expand_unit<4>(pk, w, z);
     } else {
       const uint32_t* p = job.packed + u * 3;
       const uint32_t pk[3] = {p[0], p[1], p[2]};
-      expand_unit<3>(pk, w);
+      expand_unit<3>(pk, w, z);
     }
   }
   if (job.early) pdl_wait();

@@ -12,13 +12,19 @@
 // weight tiles, 128 bytes of K per stage). Warp 1: MMA issuer: tcgen05.mma kind::i8 in steps of 32
 // bytes of K; the steps of one group accumulate in one of FOUR 128-column tensor-memory buffers, the
 // next group starts in the next buffer (group boundaries need not fall on stage boundaries: g = 192
-// or 288 span one and a half or two and a quarter stages). Warps 2-9: fold and epilogue, one token
-// per thread and 64 columns per warp: per group tcgen05.ld, the zero-point correction
-// (2^(b-1) - z[n,G]) * rowsum_G[m] in int32 (the tensor core multiplies by u - 2^(b-1)), one fma into
-// 64 fp32 partial outputs held in registers, then the buffer goes back to the MMA issuer; after the
-// last group the token scale, bias, bf16 rounding and 32-byte stores.
-// The fold costs two instructions per output and group, so this kernel is bound by the fold, not the
-// tensor core, the more so the smaller g is.
+// or 288 span one and a half or two and a quarter stages). Warp 2: brings each group's 128 scales into
+// the buffer's slot in shared memory, four groups ahead in registers (they lie ng apart in memory, a
+// trip to L2 each; fetched by the folding warps one group ahead they set the pace). Warps 4-19: fold and
+// epilogue, one token per thread and 32 columns per warp: per group one tcgen05.ld, int32 -> fp32 and a
+// packed fma into 32 fp32 partial outputs held in registers, then the buffer goes back to the MMA
+// issuer; after the last group the token scale, bias, bf16 rounding and 32-byte stores.
+// Zero-points of 3- and 4-bit layers are taken off when the packed weights are expanded to int8. For 8-bit
+// codes u - z does not fit a byte: the tensor core multiplies by u - 128 and (128 - z[n,G]) * rowsum_G[m] is
+// added in int32 before the conversion (form ZP, with rowsum from a kernel of its own).
+// The fold is what bounds this kernel: 1.5 instructions per output and group, the conversion at 64 per
+// clock and SM, 256 clocks per 128 x 128 x g step against 256 of MMA at g = 128. Sixteen warps keep both busy
+// (eight, 64 columns each, left them waiting on each other): block of 4-bit layers with zero-points, g = 128,
+// M = 2048: 173 -> 110 us.
 #include "gemm_device.cuh"
 
 namespace dp {
@@ -26,7 +32,10 @@ namespace dp {
 constexpr int kGrpBN = 128;
 constexpr int kGrpBufs = 4;
 constexpr int kGrpStages = 6;
-constexpr int kGrpThreads = kUnpackWarp0 * 32;
+constexpr int kGrpFoldWarp0 = 4, kGrpFoldWarps = 16;  // (warp & 3) is the tensor-memory quadrant
+constexpr int kGrpCols = kGrpBN / (kGrpFoldWarps / 4);  // columns of a fold warp
+constexpr int kGrpThreads = (kGrpFoldWarp0 + kGrpFoldWarps) * 32;
+constexpr int kGrpScaleWords = 2 * kGrpBufs * kGrpBN + kGrpFoldWarps * kGrpCols;  // scales, zero-point terms, biases
 
 struct GrpParams {
   const float* s_a;       // [M]
@@ -42,6 +51,7 @@ struct GrpParams {
   int32_t* status;
 };
 
+template <bool ZP>
 __global__ void __launch_bounds__(kGrpThreads, 1)
 gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                 const GrpParams p) {
@@ -50,8 +60,10 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = sA + NS * A_BYTES;
-  float* s_scale = reinterpret_cast<float*>(sB + NS * B_BYTES);  // per warp: [2][64] group scales, [2][64] zero-point terms, [64] biases
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_scale + kEpiWarps * 320);
+  float* s_scale = reinterpret_cast<float*>(sB + NS * B_BYTES);               // [buffer][column] of the group in it
+  int32_t* s_dz = reinterpret_cast<int32_t*>(s_scale + kGrpBufs * kGrpBN);    // the same, 2^(b-1) - z
+  float* s_bias = reinterpret_cast<float*>(s_dz + kGrpBufs * kGrpBN);         // per fold warp: its columns'
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_scale + kGrpScaleWords);
   uint64_t* empty = full + NS;
   uint64_t* grp_full = empty + NS;
   uint64_t* grp_empty = grp_full + kGrpBufs;
@@ -69,8 +81,8 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < kGrpBufs; ++i) {
-      mbar_init(&grp_full[i], 1);
-      mbar_init(&grp_empty[i], kEpiWarps);
+      mbar_init(&grp_full[i], 2);  // the group's MMAs, its scales
+      mbar_init(&grp_empty[i], kGrpFoldWarps);
     }
     *abort_flag = 0;
     fence_barrier_init();
@@ -136,7 +148,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           for (int k4 = 0; k4 < BK / 32; ++k4) {
             const uint32_t buf = gcount % kGrpBufs;
             if (pos == 0) {  // a new group: its buffer must have been folded
-              if (!(ok = mbar_wait(&grp_empty[buf], ((gcount / kGrpBufs) & 1u) ^ 1u, abort_flag))) break;
+              if (!(ok = mbar_spin_wait(&grp_empty[buf], ((gcount / kGrpBufs) & 1u) ^ 1u, abort_flag))) break;
               tc_fence_after();
             }
             mma_i8_ss(tmem_base + buf * kGrpBN, adesc + 2 * k4, bdesc + 2 * k4, idesc, pos != 0 ? 1u : 0u);
@@ -151,15 +163,63 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         }
       }
     }
-  } else {
-    // ================= fold + epilogue: quadrant (warp & 3), column half (ew >> 2) =================
-    const int ew = warp - kEpiWarp0, qd = warp & 3;
-    const int col0 = (ew >> 2) * 64;
-    float* wsc = s_scale + ew * 320;                            // [2][64] scales of the current / next group
-    int32_t* wdz = reinterpret_cast<int32_t*>(wsc + 128);       // [2][64] (2^(b-1) - z) of the same groups
-    float* wb = wsc + 256;                                      // [64] biases
+  } else if (warp == 2) {
+    // ================= scales of each group, columns lane, lane + 32, .. =================
+    constexpr int AHEAD = 4, C = kGrpBN / 32;
+    bool ok = true;
+    uint32_t gcount = 0;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      const int64_t n0 = (tile % p.n_tiles) * kGrpBN + lane;
+      float nx[AHEAD][C];
+      int nz[AHEAD][C];
+      auto fetch = [&](int G0) {
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const int64_t at = (n0 + 32 * c) * p.ng + G0 + i;
+            if (G0 + i < p.ng) {
+              nx[i][c] = __ldg(p.s_w + at);
+              if constexpr (ZP) nz[i][c] = __ldg(p.zeros + at);
+            }
+          }
+      };
+      fetch(0);
+      for (int G0 = 0; G0 < p.ng && ok; G0 += AHEAD) {
+        float sc[AHEAD][C];
+        int dz[AHEAD][C];
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            sc[i][c] = nx[i][c];
+            if constexpr (ZP) dz[i][c] = p.half - nz[i][c];
+          }
+        fetch(G0 + AHEAD);
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) {
+          if (G0 + i >= p.ng) break;
+          const uint32_t buf = gcount % kGrpBufs;
+          ok = mbar_wait(&grp_empty[buf], ((gcount / kGrpBufs) & 1u) ^ 1u, abort_flag);
+          ok = __all_sync(0xFFFFFFFFu, ok);
+          if (!ok) break;
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            s_scale[buf * kGrpBN + lane + 32 * c] = sc[i][c];
+            if constexpr (ZP) s_dz[buf * kGrpBN + lane + 32 * c] = dz[i][c];
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&grp_full[buf]);
+          ++gcount;
+        }
+      }
+    }
+  } else if (warp >= kGrpFoldWarp0) {
+    // ================= fold + epilogue: quadrant (warp & 3), column quarter (fw >> 2) =================
+    const int fw = warp - kGrpFoldWarp0, qd = warp & 3;
+    const int col0 = (fw >> 2) * kGrpCols;
+    float* wb = s_bias + fw * kGrpCols;
     const bool wide = ((reinterpret_cast<uintptr_t>(p.y) | static_cast<uintptr_t>(p.ldy * 2)) & 31u) == 0;
-    const bool zp = p.zeros != nullptr;
     bool ok = true;
     uint32_t gcount = 0;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
@@ -167,91 +227,57 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       const int64_t row = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + lane;
       const bool live = row < p.M;
       const float sa = live ? __ldg(p.s_a + row) : 0.0f;
-      // this lane stages columns lane and lane + 32 of the warp's 64
-      const float* swp = p.s_w + static_cast<int64_t>(n0 + lane) * p.ng;
-      const uint8_t* zpp = zp ? p.zeros + static_cast<int64_t>(n0 + lane) * p.ng : nullptr;
-      const int64_t hop = static_cast<int64_t>(32) * p.ng;
       __syncwarp();
       wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
-      wb[lane + 32] =
-          p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane + 32)) << 16) : 0.0f;
-      float s0 = __ldg(swp), s1 = __ldg(swp + hop);  // group 0
-      int z0 = zp ? p.half - static_cast<int>(__ldg(zpp)) : 0, z1 = zp ? p.half - static_cast<int>(__ldg(zpp + hop)) : 0;
-      int rs = (zp && live) ? __ldg(p.rowsum + row * p.ng) : 0;
-      float t[64];
+      int rs = (ZP && live) ? __ldg(p.rowsum + row * p.ng) : 0;
+      uint64_t t[kGrpCols / 2];  // pairs of fp32 partial outputs
 #pragma unroll
-      for (int i = 0; i < 64; ++i) t[i] = 0.0f;
-      for (int G = 0; G < p.ng && ok; ++G, ++gcount) {
-        const int par = G & 1;
-        wsc[par * 64 + lane] = s0;
-        wsc[par * 64 + lane + 32] = s1;
-        wdz[par * 64 + lane] = z0;
-        wdz[par * 64 + lane + 32] = z1;
-        __syncwarp();
-        const int rs_g = rs;
-        if (G + 1 < p.ng) {  // the next group's scales fly while this one is folded
-          s0 = __ldg(swp + G + 1);
-          s1 = __ldg(swp + hop + G + 1);
-          if (zp) {
-            z0 = p.half - static_cast<int>(__ldg(zpp + G + 1));
-            z1 = p.half - static_cast<int>(__ldg(zpp + hop + G + 1));
-            if (live) rs = __ldg(p.rowsum + row * p.ng + G + 1);
-          }
-        }
+      for (int i = 0; i < kGrpCols / 2; ++i) t[i] = 0;
+      for (int G = 0; G < p.ng; ++G, ++gcount) {
         const uint32_t buf = gcount % kGrpBufs;
+        const int rs_g = rs;
+        if (ZP && live && G + 1 < p.ng) rs = __ldg(p.rowsum + row * p.ng + G + 1);
         ok = mbar_wait(&grp_full[buf], (gcount / kGrpBufs) & 1u, abort_flag);
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + buf * kGrpBN + col0;
-        const float4* sc4 = reinterpret_cast<const float4*>(wsc + par * 64);
-        const int4* dz4 = reinterpret_cast<const int4*>(wdz + par * 64);
-        uint32_t ra[16];
-        tmem_ld_32x16(t_addr, ra);
+        uint32_t a[kGrpCols];
+        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + buf * kGrpBN + col0, a);
+        const float4* sc4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0);
+        const int4* dz4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0);
+        tmem_ld_wait();
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          tmem_ld_wait();
-          uint32_t a[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) a[i] = ra[i];
-          if (c + 1 < 4) {
-            tmem_ld_32x16(t_addr + (c + 1) * 16, ra);
-          } else {  // the group's accumulators are in registers: the buffer may take the next group
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&grp_empty[buf]);
+        for (int q = 0; q < kGrpCols / 4; ++q) {
+          const float4 sc = sc4[q];
+          int a0 = static_cast<int>(a[4 * q]), a1 = static_cast<int>(a[4 * q + 1]);
+          int a2 = static_cast<int>(a[4 * q + 2]), a3 = static_cast<int>(a[4 * q + 3]);
+          if constexpr (ZP) {
+            const int4 dz = dz4[q];
+            a0 += dz.x * rs_g;
+            a1 += dz.y * rs_g;
+            a2 += dz.z * rs_g;
+            a3 += dz.w * rs_g;
           }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float4 sc = sc4[c * 4 + q];
-            int a0 = static_cast<int>(a[4 * q]), a1 = static_cast<int>(a[4 * q + 1]);
-            int a2 = static_cast<int>(a[4 * q + 2]), a3 = static_cast<int>(a[4 * q + 3]);
-            if (zp) {
-              const int4 dz = dz4[c * 4 + q];
-              a0 += dz.x * rs_g;
-              a1 += dz.y * rs_g;
-              a2 += dz.z * rs_g;
-              a3 += dz.w * rs_g;
-            }
-            float* tt = t + c * 16 + 4 * q;
-            tt[0] = __fmaf_rn(__int2float_rn(a0), sc.x, tt[0]);
-            tt[1] = __fmaf_rn(__int2float_rn(a1), sc.y, tt[1]);
-            tt[2] = __fmaf_rn(__int2float_rn(a2), sc.z, tt[2]);
-            tt[3] = __fmaf_rn(__int2float_rn(a3), sc.w, tt[3]);
-          }
+          t[2 * q] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)), f32x2_pack(sc.x, sc.y), t[2 * q]);
+          t[2 * q + 1] = f32x2_fma(f32x2_pack(__int2float_rn(a2), __int2float_rn(a3)), f32x2_pack(sc.z, sc.w), t[2 * q + 1]);
         }
+        tc_fence_before();  // accumulators and scales are in registers: the buffer may take another group
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&grp_empty[buf]);
       }
       if (!ok) break;
       if (live) {
         uint16_t* yrow = p.y + row * p.ldy + n0;
+        const uint64_t sa2 = f32x2_pack(sa, sa);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < kGrpCols / 16; ++c) {
           uint32_t w[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             const float2 bb = *reinterpret_cast<const float2*>(wb + c * 16 + 2 * q);
-            const __nv_bfloat162 v = __floats2bfloat162_rn(__fmaf_rn(t[c * 16 + 2 * q], sa, bb.x),
-                                                           __fmaf_rn(t[c * 16 + 2 * q + 1], sa, bb.y));
+            float y0, y1;
+            f32x2_unpack(f32x2_fma(t[c * 8 + q], sa2, f32x2_pack(bb.x, bb.y)), y0, y1);
+            const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
             w[q] = *reinterpret_cast<const uint32_t*>(&v);
           }
           if (wide) {
@@ -307,18 +333,20 @@ group_rowsum_kernel(const int8_t* __restrict__ q, int64_t M, int K, int64_t ldq,
 
 // ---- host side -------------------------------------------------------------------------------------
 constexpr size_t grp_smem_bytes() {
-  return 1024 + static_cast<size_t>(kGrpStages) * (BM + kGrpBN) * BK + kEpiWarps * 320 * 4 +
+  return 1024 + static_cast<size_t>(kGrpStages) * (BM + kGrpBN) * BK + kGrpScaleWords * 4 +
          (2 * kGrpStages + 2 * kGrpBufs + 1) * 8 + 64;
 }
 
 int gemm_grp_init_device() {
-  DP_CUDA_OK(cudaFuncSetAttribute(gemm_grp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  DP_CUDA_OK(cudaFuncSetAttribute(gemm_grp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(grp_smem_bytes())));
+  DP_CUDA_OK(cudaFuncSetAttribute(gemm_grp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(grp_smem_bytes())));
   return DP_OK;
 }
 
-// q / s_a: the quantized activations (tiled scratch when a_tiled); w8: int8 [N][K] (true values
-// u - 2^(bits-1)); rowsum: scratch int32 [M][K/g], used (and filled here) only with zero-points.
+// q / s_a: the quantized activations (tiled scratch when a_tiled); w8: int8 [N][K] (codes less their
+// zero-point; with `zeros`, which 8-bit layers pass, u - 2^(bits-1)); rowsum: scratch int32 [M][K/g], used (and filled here) only with zero-points.
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
                     int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,
                     int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl) {
@@ -358,7 +386,7 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   p.status = status;
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   const int sms = num_sms() > 0 ? num_sms() : 148;
-  const cudaError_t e = launch(gemm_grp_kernel, dim3(static_cast<unsigned>(tiles < sms ? tiles : sms)), dim3(kGrpThreads),
+  const cudaError_t e = launch(zeros != nullptr ? gemm_grp_kernel<true> : gemm_grp_kernel<false>, dim3(static_cast<unsigned>(tiles < sms ? tiles : sms)), dim3(kGrpThreads),
                                grp_smem_bytes(), stream, pdl, ta, tw, p);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "group-wise GEMM launch failed: %s", cudaGetErrorString(e));
   return DP_OK;

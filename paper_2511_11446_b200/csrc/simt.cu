@@ -224,7 +224,7 @@ __device__ __forceinline__ void simt_linear_body(const SimtArgs& a, const int bl
       const int u = base + sub + kSimtLanesPerCh * i;
       if (n_ok && u < units) {
         uint32_t w[8];
-        expand_unit<BITS>(pk[i], w);
+        expand_unit<BITS>(pk[i], w, 1u << (BITS - 1));
 #pragma unroll
         for (int m = 0; m < kSimtRows; ++m) {
           const uint4* qp = reinterpret_cast<const uint4*>(sq + m * K + u * 32);
