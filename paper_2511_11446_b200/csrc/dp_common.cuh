@@ -230,6 +230,21 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int c0,
         "r"(smem_u32(bar))
       : "memory");
 }
+// 5-D load of weight rows through a map of gemm_encode_w_rows: byte c0 of the rows w_row (a multiple of 32) on.
+__device__ __forceinline__ void tma_load_w(void* dst, const void* tmap, int c0, int w_row, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %4, %4, %4, %3}], [%5];"
+      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(w_row >> 5), "r"(0), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_w_pair(void* dst, const void* tmap, int c0, int w_row, uint32_t cluster_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %4, %4, %4, %3}], [%5];"
+      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(w_row >> 5), "r"(0), "r"(cluster_bar)
+      : "memory");
+}
 // CTA-pair form: the copy lands in THIS CTA's shared memory but its bytes are counted on an mbarrier
 // that may live in the pair's other CTA (`cluster_bar` from map_to_cta). No multicast.
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, int c0, int c1, uint32_t cluster_bar) {
@@ -411,6 +426,12 @@ __device__ __forceinline__ uint4 ld_global_v4(const void* p) {
 __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&w)[8]) {
   asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]),
                "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+
+// 16-byte form, for output rows in pieces of 8 channels.
+__device__ __forceinline__ void st_global_v4(void* p, const uint32_t (&w)[4]) {
+  asm volatile("st.global.L1::no_allocate.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
                : "memory");
 }
 

@@ -165,6 +165,8 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
 // gemm_bf16.cu -- pass-through linear of 16-bit layers (bf16 x bf16 -> fp32 -> bf16, tcgen05 kind::f16).
 int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* bias, int64_t M, int32_t N, int32_t K,
                      uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl);
+int gemm_encode_w_rows(CUtensorMap* out, const void* base, uint64_t row_bytes, uint64_t rows, uint32_t box_inner,
+                       uint32_t box_rows, bool swizzle128);
 int gemm_encode_bytes_2d(CUtensorMap* out, const void* base, uint64_t inner_bytes, uint64_t rows, uint64_t pitch_bytes,
                          uint32_t box_inner, uint32_t box_rows);
 

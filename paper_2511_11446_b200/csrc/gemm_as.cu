@@ -18,8 +18,7 @@
 // consecutive units of a pair share the strip and the resident activations are kept.
 //
 // Warp roles: warp 0 TMA producer (one thread), warp 1 MMA issuer (one thread of the pair's leader),
-// warps 2-9 epilogue (two per 32-token quadrant of tensor memory, half of the sub-block's columns each;
-// one token per thread).
+// warps 2-9 epilogue (two per 32-token quadrant of tensor memory, half of the sub-block's columns each).
 // All loads are plain (non-multicast) TMA loads; both CTAs' bytes are counted on the leader's
 // barriers; tcgen05.commit frees ring stages in both CTAs.
 #include "gemm_device.cuh"
@@ -111,7 +110,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       auto load_w = [&](int kb, int w_row) {
         const uint32_t bar = w_full0 + 8u * static_cast<uint32_t>(st.s);
         mbar_arrive_expect_tx_cluster(bar, static_cast<uint32_t>(B_BYTES));
-        tma_load_2d_pair(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, bar);
+        tma_load_w_pair(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, bar);
         st.next(NS);
       };
       auto load_a = [&](int kb, int m_row) {

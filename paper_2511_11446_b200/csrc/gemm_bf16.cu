@@ -8,8 +8,8 @@
 // One persistent CTA per SM walks 128 x BN output tiles (column tiles of a row strip together). Warp 0:
 // TMA producer (activation and weight tiles of 64 bf16 = 128-byte rows, 128-byte swizzle, straight
 // from the caller's row-major matrices); warp 1: MMA issuer (tcgen05.mma kind::f16 with bf16 operands,
-// fp32 accumulators in tensor memory, two buffers); warps 2-9: epilogue, one token per thread:
-// tcgen05.ld -> + bias -> bf16 -> one 32-byte store per 16 columns.
+// fp32 accumulators in tensor memory, two buffers); warps 2-9: epilogue:
+// tcgen05.ld -> + bias -> bf16 -> 16-byte stores.
 #include "gemm_device.cuh"
 
 namespace dp {
@@ -108,7 +108,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
           free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);  // one k-block ahead
           mbar_arrive_expect_tx(&full[st.s], A_BYTES + B_BYTES);
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, kb * kBfBK, m_row, &full[st.s]);
-          tma_load_2d(sB + st.s * B_BYTES, &tmap_w, kb * kBfBK, n_blk * BN, &full[st.s]);
+          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * kBfBK, n_blk * BN, &full[st.s]);
           st = nx;
         }
       }
@@ -153,13 +153,13 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     constexpr int NCOLS = BN >= 64 ? BN / 2 : BN;  // columns per warp
     const int col0 = (ew >> 2) * NCOLS;
     float* tb = s_bias + ew * 128;
-    const bool wide = ((reinterpret_cast<uintptr_t>(p.y) | static_cast<uintptr_t>(p.ldy * 2)) & 31u) == 0;
+    const int tc = (lane & 3) * 8;  // this lane's channels of a round of 32 (see RowEpilogue)
     bool ok = true;
     int tcount = 0, staged = -1;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
       const int buf = tcount & 1;
       const int n0 = (tile % p.n_tiles) * BN + col0;
-      const int64_t row = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + lane;
+      const int64_t row0 = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + (lane >> 2);
       if (n0 != staged) {
         __syncwarp();
         for (int c = lane; c < NCOLS; c += 32)
@@ -172,38 +172,38 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
       if (!ok) break;
       tc_fence_after();
       const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + buf * (TCOLS / 2) + col0;
-      uint16_t* yrow = p.y + row * p.ldy + n0;
-      uint32_t ra[16];
-      tmem_ld_32x16(t_addr, ra);
-      for (int c = 0; c < NCOLS / 16; ++c) {
-        tmem_ld_wait();
-        uint32_t a[16];
+      uint16_t* yrow = p.y + row0 * p.ldy + n0 + tc;
+      uint32_t lo[16], hi[16];
+      float bb[8];
+      auto emit = [&](const uint32_t (&a)[16], int c, int i0) {  // tokens row0 + 8 * i0, + 8 more
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[i] = ra[i];
-        if (c + 1 < NCOLS / 16) {
-          tmem_ld_32x16(t_addr + (c + 1) * 16, ra);
+        for (int k = 0; k < 2; ++k) {
+          uint32_t w[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(__fadd_rn(__uint_as_float(a[4 * j + 2 * k]), bb[2 * j]),
+                                                           __fadd_rn(__uint_as_float(a[4 * j + 2 * k + 1]), bb[2 * j + 1]));
+            w[j] = *reinterpret_cast<const uint32_t*>(&v);
+          }
+          if (row0 + 8 * (i0 + k) < p.M) st_global_v4(yrow + 8 * (i0 + k) * p.ldy + c * 32, w);
+        }
+      };
+      tmem_ld_16x256b_x4(t_addr, lo);
+      for (int c = 0; c < NCOLS / 32; ++c) {
+        *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(tb + c * 32 + tc);
+        *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(tb + c * 32 + tc + 4);
+        tmem_ld_wait();
+        tmem_ld_16x256b_x4(t_addr + (16u << 16) + c * 32, hi);
+        emit(lo, c, 0);
+        tmem_ld_wait();
+        if (c + 1 < NCOLS / 32) {
+          tmem_ld_16x256b_x4(t_addr + (c + 1) * 32, lo);
         } else {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
-        uint32_t w[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float2 bb = *reinterpret_cast<const float2*>(tb + c * 16 + 2 * q);
-          const __nv_bfloat162 v = __floats2bfloat162_rn(__fadd_rn(__uint_as_float(a[2 * q]), bb.x),
-                                                         __fadd_rn(__uint_as_float(a[2 * q + 1]), bb.y));
-          w[q] = *reinterpret_cast<const uint32_t*>(&v);
-        }
-        if (row < p.M) {
-          if (wide) {
-            st_global_v8(yrow + c * 16, w);
-          } else {
-            uint4* y4 = reinterpret_cast<uint4*>(yrow + c * 16);
-            y4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            y4[1] = make_uint4(w[4], w[5], w[6], w[7]);
-          }
-        }
+        emit(hi, c, 2);
       }
     }
   }
@@ -244,8 +244,7 @@ int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* 
   int st = gemm_encode_bytes_2d(&ta, x, static_cast<uint64_t>(K) * 2, static_cast<uint64_t>(M),
                                 static_cast<uint64_t>(ldx) * 2, kBfBK, BM);
   if (st != DP_OK) return st;
-  st = gemm_encode_bytes_2d(&tw, w, static_cast<uint64_t>(K) * 2, static_cast<uint64_t>(N), static_cast<uint64_t>(K) * 2,
-                            kBfBK, bn);
+  st = gemm_encode_w_rows(&tw, w, static_cast<uint64_t>(K) * 2, static_cast<uint64_t>(N), kBfBK, bn, true);
   if (st != DP_OK) return st;
   BfParams p;
   p.bias = bias;

@@ -1,6 +1,6 @@
 // Device-side pieces shared by the tensor-core GEMM kernels of libdiffpro: tile constants, kernel
 // parameters, the in-shared-memory expansion of packed 3/4-bit weight tiles, and the dequant
-// epilogue of one warp (tcgen05.ld -> fp32 sequence -> bf16 -> 32-byte stores, one token per thread).
+// epilogue of one warp (tcgen05.ld -> fp32 sequence -> bf16 -> 16-byte stores).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -228,26 +228,28 @@ __device__ __forceinline__ void unpack3_tile(const uint8_t* P, uint8_t* B, int t
   }
 }
 
-// ---- epilogue with one token per thread ---------------------------------------------------------------
-// A warp serves its tensor-memory quadrant (32 tokens, one per thread) over a range of accumulator
-// columns in rounds of 16: tcgen05.ld.32x32b.x16 (the next round's read is in flight while this one
-// is converted), the fp32 sequence of Step 5 on packed pairs (two independent IEEE operations per
-// instruction: int32 -> fp32, sc = s_a * s_w[n], fma(t, sc, bias[n]), bf16 round-to-nearest-even),
-// and ONE 32-byte global store per thread and round (st.global.v8: a full sector of the token's
-// output row), so nothing is staged in shared memory and no warp-level synchronisation sits between
-// the arithmetic and the stores. Weight scales and biases come from a private fp32 copy in shared
-// memory, read as broadcast 16-byte loads: global loads in this loop, even of a few cached KB, cost
-// a trip to L2 per round with only ten warps on the SM to hide it. What bounds an epilogue on B200
-// is the chip's store throughput (4.4 TB/s measured: about 15 bytes per clock and SM), then
-// instruction issue; arithmetic does not.
+// ---- epilogue ---------------------------------------------------------------------------------------
+// A warp serves its tensor-memory quadrant (32 tokens) over a range of accumulator columns in rounds of 32
+// columns x 16 tokens: tcgen05.ld.16x256b.x4 leaves lane (r, t) = (lane / 4, lane % 4) the tokens r and
+// r + 8 at columns 8j + 2t + e (j < 4, e < 2), which are the channels 8t .. 8t + 7 of the round, because the
+// weight rows were brought in in that order (gemm_encode_w_rows). The next round's read is in flight while
+// this one is converted: the fp32 sequence of Step 5 on packed pairs (two independent IEEE operations per
+// instruction: int32 -> fp32, sc = s_a * s_w[n], fma(t, sc, bias[n]), bf16 round-to-nearest-even) and one
+// 16-byte store per token, a quad covering 64 contiguous bytes of the token's row. Nothing is staged in
+// shared memory.
+// Why fragments and not one token per thread: a lane needs 8 scales and 8 biases per 4 tokens, four 16-byte
+// shared-memory reads, where one token per thread needs sixteen. Such a read, even a broadcast, takes four
+// clocks of the 128-byte port that the tensor core's operand reads (and TMA's writes) already keep busy:
+// whole 8-bit layers, K = 1152, N = 4608, M = 4096 / 8192: 23.1 / 43.8 us with one token per thread, 20.9 /
+// 39.8 this way; K = 384, N = 1536, M = 32768: 44.7 -> 38.0; K = 1152, N = 1152, M = 64: 6.8 -> 6.3.
 template <int SHIFT>
 struct RowEpilogue {
-  static constexpr int CW = 16;         // columns per round
+  static constexpr int CW = 32;         // columns per round
   static constexpr int kMaxCols = 128;  // columns a warp may own (its private copy of scales and biases)
   static constexpr int kScaleBytes = 2 * kMaxCols * 4;
   int qd, lane, staged_col;
   float *tsw, *tbias;
-  uint32_t acc_empty_addr[2];
+  uint32_t acc_empty_addr0, acc_empty_addr1;
 
   __device__ __forceinline__ void init(int warp, int lane_, float* scale_copy, uint32_t acc_empty0,
                                        uint32_t acc_empty1) {
@@ -255,12 +257,12 @@ struct RowEpilogue {
     qd = warp & 3;
     tsw = scale_copy;
     tbias = scale_copy + kMaxCols;
-    acc_empty_addr[0] = acc_empty0;
-    acc_empty_addr[1] = acc_empty1;
+    acc_empty_addr0 = acc_empty0;
+    acc_empty_addr1 = acc_empty1;
     staged_col = -1;
   }
 
-  // Output columns col .. col + ncols - 1 (col and ncols multiples of 16, ncols at most 128), this
+  // Output columns col .. col + ncols - 1 (col and ncols multiples of 32, ncols at most 128), this
   // CTA's tokens cta_row0 .. +127; their accumulators start at tensor-memory column t_col (buffer
   // `buf`, published on acc_full with phase aph). False if the wait was aborted.
   // RES: the kernel takes the residual (and gate) of GemmParams into the output; without it those
@@ -269,9 +271,14 @@ struct RowEpilogue {
   __device__ __forceinline__ bool tile(const GemmParams& p, int col, int ncols, int cta_row0, uint32_t tmem_base,
                                        uint32_t t_col, uint64_t* acc_full, uint32_t aph, int buf,
                                        volatile int* abort_flag) {
-    const int64_t row = static_cast<int64_t>(cta_row0) + qd * 32 + lane;
-    float sa = 0.0f;
-    if (p.x == nullptr && row < p.M) sa = __ldg(p.s_a + row);  // from an earlier kernel: fetched while waiting
+    // this lane's tokens: row0 + 8 * i, i < 4; its channels of a round: col + 32 * round + tc .. + 7
+    const int64_t row0 = static_cast<int64_t>(cta_row0) + qd * 32 + (lane >> 2);
+    const int tc = (lane & 3) * 8;
+    const int live = row0 >= p.M ? 0 : static_cast<int>(p.M - row0 > 24 ? 4 : (p.M - row0 + 7) >> 3);  // tokens inside M
+    float sa[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)  // from an earlier kernel: fetched while waiting
+      sa[i] = (p.x == nullptr && i < live) ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
     if (col != staged_col) {
       float sv[4], bv[4];
 #pragma unroll
@@ -291,21 +298,27 @@ struct RowEpilogue {
       __syncwarp();
       staged_col = col;
     }
-    // Residual and gate of this thread's token, fetched one round ahead of their use (plain loads: the
-    // residual may be the output buffer, whose 32 bytes this thread reads before it overwrites them).
-    const bool has_res = RES && p.res != nullptr && row < p.M;
+    // Residual and gate of this lane's tokens, fetched one round of 32 columns ahead of their use (plain loads:
+    // the residual may be the output buffer, whose bytes this thread reads before it overwrites them).
+    const bool has_res = RES && p.res != nullptr;
     const bool has_gate = has_res && p.gate != nullptr;
-    const uint16_t* rrow = has_res ? p.res + row * p.ldr + col : nullptr;
-    const uint16_t* grow = has_gate ? p.gate + (row / p.rows_per_gate) * p.N + col : nullptr;
-    uint4 rn0 = make_uint4(0, 0, 0, 0), rn1 = rn0, gn0 = rn0, gn1 = rn0;
-    if (has_res) {  // the later rounds' lines on their way into L2 while the accumulators are still being summed
-      for (int b = 128; b < ncols * 2; b += 128) prefetch_l2(reinterpret_cast<const uint8_t*>(rrow) + b);
-      rn0 = ld_global_v4(rrow);
-      rn1 = ld_global_v4(rrow + 8);
-    }
-    if (has_gate) {
-      gn0 = ld_global_v4(grow);
-      gn1 = ld_global_v4(grow + 8);
+    const uint16_t* rrow = has_res ? p.res + row0 * p.ldr + col + tc : nullptr;
+    uint4 rn[4], gn[4];
+    auto fetch_res = [&](int c) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        rn[i] = gn[i] = make_uint4(0, 0, 0, 0);
+        if (has_res && i < live) rn[i] = ld_global_v4(rrow + 8 * i * p.ldr + c * CW);
+        if (has_gate && i < live) gn[i] = ld_global_v4(p.gate + ((row0 + 8 * i) / p.rows_per_gate) * p.N + col + tc + c * CW);
+      }
+    };
+    if constexpr (RES) {
+      // the later rounds' lines on their way into L2 while the accumulators are still being summed
+      const int64_t prow = static_cast<int64_t>(cta_row0) + qd * 32 + lane;
+      if (has_res && prow < p.M)
+        for (int b = 128; b < ncols * 2; b += 128)
+          prefetch_l2(reinterpret_cast<const uint8_t*>(p.res + prow * p.ldr + col) + b);
+      fetch_res(0);
     }
     bool ok = mbar_wait(acc_full, aph, abort_flag);
     ok = __all_sync(0xFFFFFFFFu, ok);
@@ -313,94 +326,87 @@ struct RowEpilogue {
     tc_fence_after();
     if (p.x != nullptr) {  // scales written by other CTAs of this kernel: their tile is complete by now
       (void)ld_acquire_gpu(p.sync + (cta_row0 >> 7));
-      if (row < p.M) sa = *reinterpret_cast<const volatile float*>(p.s_a + row);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < live) sa[i] = *reinterpret_cast<const volatile float*>(p.s_a + row0 + 8 * i);
     }
-    const uint64_t sa2 = f32x2_pack(sa, sa);
     const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + t_col;
-    const float4* sw4 = reinterpret_cast<const float4*>(tsw);
-    const float4* tb4 = reinterpret_cast<const float4*>(tbias);
-    uint16_t* yrow = p.y + row * p.ldy + col;
-    // 32-byte stores need the token's row segment 32-byte aligned; else two 16-byte stores
-    const bool wide = ((reinterpret_cast<uintptr_t>(p.y) | static_cast<uintptr_t>(p.ldy * 2)) & 31u) == 0;
+    uint16_t* yrow = p.y + row0 * p.ldy + col + tc;
     const int rounds = ncols / CW;
-    uint32_t ra[16];
-    tmem_ld_32x16(t_addr, ra);
-    for (int c = 0; c < rounds; ++c) {
-      const uint32_t rr[8] = {rn0.x, rn0.y, rn0.z, rn0.w, rn1.x, rn1.y, rn1.z, rn1.w};
-      const uint32_t gg[8] = {gn0.x, gn0.y, gn0.z, gn0.w, gn1.x, gn1.y, gn1.z, gn1.w};
-      if (RES && c + 1 < rounds) {
-        if (has_res) {
-          rn0 = ld_global_v4(rrow + (c + 1) * CW);
-          rn1 = ld_global_v4(rrow + (c + 1) * CW + 8);
+    uint32_t lo[16], hi[16];  // tokens 0, 1 and 2, 3 of a round
+    float s[8], b[8];
+    auto emit = [&](const uint32_t (&a)[16], int c, int i0, const uint4* rr4, const uint4* gg4) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int i = i0 + k;
+        const uint64_t sa2 = f32x2_pack(sa[i], sa[i]);
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {  // channels tc + 2j, tc + 2j + 1
+          uint64_t t = f32x2_pack(__int2float_rn(static_cast<int>(a[4 * j + 2 * k])),
+                                  __int2float_rn(static_cast<int>(a[4 * j + 2 * k + 1])));
+          if constexpr (SHIFT != 0)  // exact: the accumulator is a multiple of 2^SHIFT
+            t = f32x2_mul(t, f32x2_pack(1.0f / (1 << SHIFT), 1.0f / (1 << SHIFT)));
+          float y0, y1;
+          f32x2_unpack(f32x2_fma(t, f32x2_mul(sa2, f32x2_pack(s[2 * j], s[2 * j + 1])), f32x2_pack(b[2 * j], b[2 * j + 1])),
+                       y0, y1);
+          if (RES && has_res) {  // uniform over the grid
+            const uint32_t r = reinterpret_cast<const uint32_t*>(&rr4[i])[j];
+            const float r0 = __uint_as_float(r << 16), r1 = __uint_as_float(r & 0xFFFF0000u);
+            if (has_gate) {
+              const uint32_t g = reinterpret_cast<const uint32_t*>(&gg4[i])[j];
+              y0 = fmaf(__uint_as_float(g << 16), y0, r0);
+              y1 = fmaf(__uint_as_float(g & 0xFFFF0000u), y1, r1);
+            } else {
+              y0 = __fadd_rn(y0, r0);
+              y1 = __fadd_rn(y1, r1);
+            }
+          }
+          const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
+          w[j] = *reinterpret_cast<const uint32_t*>(&v);
         }
-        if (has_gate) {
-          gn0 = ld_global_v4(grow + (c + 1) * CW);
-          gn1 = ld_global_v4(grow + (c + 1) * CW + 8);
+        if (i < live) {
+          if (p.dbg_acc != nullptr) {
+            int32_t* arow = p.dbg_acc + (row0 + 8 * i) * p.dbg_ldacc + col + c * CW + tc;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              arow[2 * j] = static_cast<int>(a[4 * j + 2 * k]) >> SHIFT;
+              arow[2 * j + 1] = static_cast<int>(a[4 * j + 2 * k + 1]) >> SHIFT;
+            }
+          }
+          st_global_v4(yrow + 8 * i * p.ldy + c * CW, w);
         }
       }
-      tmem_ld_wait();
-      uint32_t a[16];
+    };
+    tmem_ld_16x256b_x4(t_addr, lo);
+    for (int c = 0; c < rounds; ++c) {
+      const float4* s4 = reinterpret_cast<const float4*>(tsw + c * CW + tc);
+      const float4* b4 = reinterpret_cast<const float4*>(tbias + c * CW + tc);
+      *reinterpret_cast<float4*>(s) = s4[0];
+      *reinterpret_cast<float4*>(s + 4) = s4[1];
+      *reinterpret_cast<float4*>(b) = b4[0];
+      *reinterpret_cast<float4*>(b + 4) = b4[1];
+      uint4 rr[4], gg[4];
+      if constexpr (RES) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) a[i] = ra[i];
+        for (int i = 0; i < 4; ++i) {
+          rr[i] = rn[i];
+          gg[i] = gn[i];
+        }
+        if (c + 1 < rounds) fetch_res(c + 1);
+      }
+      tmem_ld_wait();
+      tmem_ld_16x256b_x4(t_addr + (16u << 16) + c * CW, hi);
+      emit(lo, c, 0, rr, gg);
+      tmem_ld_wait();
       if (c + 1 < rounds) {
-        tmem_ld_32x16(t_addr + (c + 1) * CW, ra);
+        tmem_ld_16x256b_x4(t_addr + (c + 1) * CW, lo);
       } else {  // this warp's last accumulators are in registers: hand the buffer back
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(acc_empty_addr[buf]);
+        if (lane == 0) mbar_arrive_cluster(buf ? acc_empty_addr1 : acc_empty_addr0);
       }
-      uint32_t w[8];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {  // four columns at a time
-        const float4 sw = sw4[c * 4 + q];
-        const float4 bb = tb4[c * 4 + q];
-        uint64_t t01 = f32x2_pack(__int2float_rn(static_cast<int>(a[4 * q])),
-                                  __int2float_rn(static_cast<int>(a[4 * q + 1])));
-        uint64_t t23 = f32x2_pack(__int2float_rn(static_cast<int>(a[4 * q + 2])),
-                                  __int2float_rn(static_cast<int>(a[4 * q + 3])));
-        if constexpr (SHIFT != 0) {  // exact: the accumulator is a multiple of 2^SHIFT
-          const uint64_t down = f32x2_pack(1.0f / (1 << SHIFT), 1.0f / (1 << SHIFT));
-          t01 = f32x2_mul(t01, down);
-          t23 = f32x2_mul(t23, down);
-        }
-        const uint64_t y01 = f32x2_fma(t01, f32x2_mul(sa2, f32x2_pack(sw.x, sw.y)), f32x2_pack(bb.x, bb.y));
-        const uint64_t y23 = f32x2_fma(t23, f32x2_mul(sa2, f32x2_pack(sw.z, sw.w)), f32x2_pack(bb.z, bb.w));
-        float y0, y1, y2, y3;
-        f32x2_unpack(y01, y0, y1);
-        f32x2_unpack(y23, y2, y3);
-        if (RES && p.res != nullptr) {  // uniform over the grid
-          const float r0 = __uint_as_float(rr[2 * q] << 16), r1 = __uint_as_float(rr[2 * q] & 0xFFFF0000u);
-          const float r2 = __uint_as_float(rr[2 * q + 1] << 16), r3 = __uint_as_float(rr[2 * q + 1] & 0xFFFF0000u);
-          if (p.gate != nullptr) {
-            y0 = fmaf(__uint_as_float(gg[2 * q] << 16), y0, r0);
-            y1 = fmaf(__uint_as_float(gg[2 * q] & 0xFFFF0000u), y1, r1);
-            y2 = fmaf(__uint_as_float(gg[2 * q + 1] << 16), y2, r2);
-            y3 = fmaf(__uint_as_float(gg[2 * q + 1] & 0xFFFF0000u), y3, r3);
-          } else {
-            y0 = __fadd_rn(y0, r0);
-            y1 = __fadd_rn(y1, r1);
-            y2 = __fadd_rn(y2, r2);
-            y3 = __fadd_rn(y3, r3);
-          }
-        }
-        const __nv_bfloat162 v01 = __floats2bfloat162_rn(y0, y1), v23 = __floats2bfloat162_rn(y2, y3);
-        w[2 * q] = *reinterpret_cast<const uint32_t*>(&v01);
-        w[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&v23);
-      }
-      if (row < p.M) {
-        if (p.dbg_acc != nullptr) {
-          int32_t* arow = p.dbg_acc + row * p.dbg_ldacc + col + c * CW;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) arow[i] = static_cast<int>(a[i]) >> SHIFT;
-        }
-        if (wide) {
-          st_global_v8(yrow + c * CW, w);
-        } else {
-          uint4* y4 = reinterpret_cast<uint4*>(yrow + c * CW);
-          y4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-          y4[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        }
-      }
+      emit(hi, c, 2, rr, gg);
     }
     return true;
   }

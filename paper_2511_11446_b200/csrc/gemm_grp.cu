@@ -12,8 +12,8 @@
 // weight tiles, 128 bytes of K per stage). Warp 1: MMA issuer: tcgen05.mma kind::i8 in steps of 32
 // bytes of K; the steps of one group accumulate in one of FOUR 128-column tensor-memory buffers, the
 // next group starts in the next buffer (group boundaries need not fall on stage boundaries: g = 192
-// or 288 span one and a half or two and a quarter stages). Warp 2: brings each group's 128 scales into
-// the buffer's slot in shared memory, four groups ahead in registers (they lie ng apart in memory, a
+// or 288 span one and a half or two and a quarter stages). Warps 2 and 3 bring each group's 128 scales
+// into the buffer's slot in shared memory, eight groups ahead in registers (they lie ng apart in memory, a
 // trip to L2 each; fetched by the folding warps one group ahead they set the pace). Warps 4-19: fold and
 // epilogue, one token per thread and 32 columns per warp: per group one tcgen05.ld, int32 -> fp32 and a
 // packed fma into 32 fp32 partial outputs held in registers, then the buffer goes back to the MMA
@@ -33,6 +33,7 @@ constexpr int kGrpBN = 128;
 constexpr int kGrpBufs = 4;
 constexpr int kGrpStages = 6;
 constexpr int kGrpFoldWarp0 = 4, kGrpFoldWarps = 16;  // (warp & 3) is the tensor-memory quadrant
+constexpr int kGrpLoadWarps = 2;                         // warps 2 and 3
 constexpr int kGrpCols = kGrpBN / (kGrpFoldWarps / 4);  // columns of a fold warp
 constexpr int kGrpThreads = (kGrpFoldWarp0 + kGrpFoldWarps) * 32;
 constexpr int kGrpScaleWords = 2 * kGrpBufs * kGrpBN + kGrpFoldWarps * kGrpCols;  // scales, zero-point terms, biases
@@ -50,6 +51,52 @@ struct GrpParams {
   int32_t m_tiles, n_tiles, a_tiled;
   int32_t* status;
 };
+
+// The MMA issuer's whole run over this CTA's tiles (one thread).
+template <int U>
+__device__ __forceinline__ void grp_issue(const GrpParams& p, const uint8_t* sA, const uint8_t* sB, uint64_t* full,
+                                          uint64_t* empty, uint64_t* grp_full, uint64_t* grp_empty, uint32_t tmem_base,
+                                          volatile int* abort_flag) {
+  constexpr uint32_t idesc = idesc_i8(BM, kGrpBN);
+  constexpr int NS = kGrpStages;
+  const uint64_t adesc0 = smem_desc_sw128(smem_u32(sA)), bdesc0 = smem_desc_sw128(smem_u32(sB));
+  const int KB = p.K / BK, total_tiles = p.m_tiles * p.n_tiles;
+  const int rpg = (p.g >> 5) / U;  // runs per group
+  Ring st, gb;                     // operand stage; group buffer
+  // both polled ahead: the next stage, the next group's buffer
+  bool full_next = mbar_test_wait(&full[0], 0u), room_next = true;
+  for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
+    int pos = 0;  // run inside the current group
+    for (int kb = 0; kb < KB; ++kb) {
+      if (!full_next && !mbar_spin_wait(&full[st.s], st.ph, abort_flag)) return;
+      tc_fence_after();
+      Ring nx = st;
+      nx.next(NS);
+      full_next = mbar_test_wait(&full[nx.s], nx.ph);
+      const uint64_t adesc = adesc0 + static_cast<uint64_t>(st.s * ((BM * BK) >> 4));
+      const uint64_t bdesc = bdesc0 + static_cast<uint64_t>(st.s * ((kGrpBN * BK) >> 4));
+#pragma unroll
+      for (int u = 0; u < BK / 32 / U; ++u) {
+        if (pos == 0) {  // a new group: its buffer must have been folded
+          if (!room_next && !mbar_spin_wait(&grp_empty[gb.s], gb.ph ^ 1u, abort_flag)) return;
+          tc_fence_after();
+        }
+        const uint32_t d_tmem = tmem_base + gb.s * kGrpBN;
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+          mma_i8_ss(d_tmem, adesc + 2 * (u * U + j), bdesc + 2 * (u * U + j), idesc, (pos | j) != 0 ? 1u : 0u);
+        if (++pos == rpg) {
+          mma_commit(&grp_full[gb.s]);
+          pos = 0;
+          gb.next(kGrpBufs);
+          room_next = mbar_test_wait(&grp_empty[gb.s], gb.ph ^ 1u);
+        }
+      }
+      mma_commit(&empty[st.s]);
+      st = nx;
+    }
+  }
+}
 
 template <bool ZP>
 __global__ void __launch_bounds__(kGrpThreads, 1)
@@ -81,7 +128,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < kGrpBufs; ++i) {
-      mbar_init(&grp_full[i], 2);  // the group's MMAs, its scales
+      mbar_init(&grp_full[i], 1 + kGrpLoadWarps);  // the group's MMAs, its scales
       mbar_init(&grp_empty[i], kGrpFoldWarps);
     }
     *abort_flag = 0;
@@ -122,7 +169,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             c1 = m_row;
           }
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, c0, c1, &full[st.s]);
-          tma_load_2d(sB + st.s * B_BYTES, &tmap_w, kb * BK, n_blk * kGrpBN, &full[st.s]);
+          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, n_blk * kGrpBN, &full[st.s]);
           st = nx;
         }
       }
@@ -134,42 +181,21 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     }
   } else if (warp == 1) {
     if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
-      constexpr uint32_t idesc = idesc_i8(BM, kGrpBN);
-      Ring st;
-      bool ok = true;
-      uint32_t gcount = 0;  // groups issued so far: buffer = gcount % 4
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        int pos = 0;  // step inside the current group
-        for (int kb = 0; kb < KB && ok; ++kb) {
-          if (!(ok = mbar_spin_wait(&full[st.s], st.ph, abort_flag))) break;
-          tc_fence_after();
-          const uint64_t adesc = smem_desc_sw128(smem_u32(sA + st.s * A_BYTES));
-          const uint64_t bdesc = smem_desc_sw128(smem_u32(sB + st.s * B_BYTES));
-          for (int k4 = 0; k4 < BK / 32; ++k4) {
-            const uint32_t buf = gcount % kGrpBufs;
-            if (pos == 0) {  // a new group: its buffer must have been folded
-              if (!(ok = mbar_spin_wait(&grp_empty[buf], ((gcount / kGrpBufs) & 1u) ^ 1u, abort_flag))) break;
-              tc_fence_after();
-            }
-            mma_i8_ss(tmem_base + buf * kGrpBN, adesc + 2 * k4, bdesc + 2 * k4, idesc, pos != 0 ? 1u : 0u);
-            if (++pos == spg) {
-              mma_commit(&grp_full[buf]);
-              pos = 0;
-              ++gcount;
-            }
-          }
-          if (ok) mma_commit(&empty[st.s]);
-          st.next(NS);
-        }
-      }
+      // Steps are issued in straight-line runs of U, the largest power of two up to a stage's four that
+      // divides a group: group bookkeeping between single steps kept the issuing thread busy for 570-930
+      // cycles per k-block (a run of four takes ~100), which was the pace of the whole kernel.
+      if (spg % 4 == 0) grp_issue<4>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
+      else if (spg % 2 == 0) grp_issue<2>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
+      else grp_issue<1>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
     }
-  } else if (warp == 2) {
-    // ================= scales of each group, columns lane, lane + 32, .. =================
-    constexpr int AHEAD = 4, C = kGrpBN / 32;
+  } else if (warp < kGrpFoldWarp0) {
+    // ================= scales of each group: this warp's columns lane, lane + 32 =================
+    constexpr int AHEAD = 8, C = kGrpBN / 32 / kGrpLoadWarps;
+    const int c0 = (warp - 2) * 32 * C + lane;
     bool ok = true;
     uint32_t gcount = 0;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int64_t n0 = (tile % p.n_tiles) * kGrpBN + lane;
+      const int64_t n0 = (tile % p.n_tiles) * kGrpBN + c0;
       float nx[AHEAD][C];
       int nz[AHEAD][C];
       auto fetch = [&](int G0) {
@@ -205,8 +231,8 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           if (!ok) break;
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            s_scale[buf * kGrpBN + lane + 32 * c] = sc[i][c];
-            if constexpr (ZP) s_dz[buf * kGrpBN + lane + 32 * c] = dz[i][c];
+            s_scale[buf * kGrpBN + c0 + 32 * c] = sc[i][c];
+            if constexpr (ZP) s_dz[buf * kGrpBN + c0 + 32 * c] = dz[i][c];
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&grp_full[buf]);
@@ -214,80 +240,104 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         }
       }
     }
-  } else if (warp >= kGrpFoldWarp0) {
+  } else {
     // ================= fold + epilogue: quadrant (warp & 3), column quarter (fw >> 2) =================
     const int fw = warp - kGrpFoldWarp0, qd = warp & 3;
     const int col0 = (fw >> 2) * kGrpCols;
+    const int tc = (lane & 3) * 8;  // this lane's channels of the warp's 32 (see RowEpilogue)
     float* wb = s_bias + fw * kGrpCols;
-    const bool wide = ((reinterpret_cast<uintptr_t>(p.y) | static_cast<uintptr_t>(p.ldy * 2)) & 31u) == 0;
     bool ok = true;
     uint32_t gcount = 0;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int n0 = (tile % p.n_tiles) * kGrpBN + col0;
-      const int64_t row = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + lane;
-      const bool live = row < p.M;
-      const float sa = live ? __ldg(p.s_a + row) : 0.0f;
+      const int64_t row0 = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + (lane >> 2);
+      bool live[4];
+      float sa[4];
+      int rs[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        live[i] = row0 + 8 * i < p.M;
+        sa[i] = live[i] ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
+        rs[i] = (ZP && live[i]) ? __ldg(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
+      }
       __syncwarp();
       wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
-      int rs = (ZP && live) ? __ldg(p.rowsum + row * p.ng) : 0;
-      uint64_t t[kGrpCols / 2];  // pairs of fp32 partial outputs
+      uint64_t t[4][4];  // fp32 partial outputs: token row0 + 8 * i, channels tc + 2j, tc + 2j + 1
 #pragma unroll
-      for (int i = 0; i < kGrpCols / 2; ++i) t[i] = 0;
+      for (int i = 0; i < 16; ++i) t[i >> 2][i & 3] = 0;
+      // A group is folded in two halves of 16 tokens, each read while the other is computed, the first
+      // half of the next group under the second of this one.
+      const uint32_t t_row = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + col0;
+      auto wait_group = [&](uint32_t g) {
+        ok = mbar_wait(&grp_full[g % kGrpBufs], (g / kGrpBufs) & 1u, abort_flag);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        tc_fence_after();
+      };
+      float sc[8];
+      int dz[8];
+      auto fold = [&](const uint32_t (&a)[16], int i0, const int* rs_g) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            int a0 = static_cast<int>(a[4 * j + 2 * k]), a1 = static_cast<int>(a[4 * j + 2 * k + 1]);
+            if constexpr (ZP) {
+              a0 += dz[2 * j] * rs_g[i0 + k];
+              a1 += dz[2 * j + 1] * rs_g[i0 + k];
+            }
+            t[i0 + k][j] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)),
+                                     f32x2_pack(sc[2 * j], sc[2 * j + 1]), t[i0 + k][j]);
+          }
+      };
+      uint32_t lo[16], hi[16];
+      wait_group(gcount);
+      if (!ok) break;
+      tmem_ld_16x256b_x4(t_row + (gcount % kGrpBufs) * kGrpBN, lo);
       for (int G = 0; G < p.ng; ++G, ++gcount) {
         const uint32_t buf = gcount % kGrpBufs;
-        const int rs_g = rs;
-        if (ZP && live && G + 1 < p.ng) rs = __ldg(p.rowsum + row * p.ng + G + 1);
-        ok = mbar_wait(&grp_full[buf], (gcount / kGrpBufs) & 1u, abort_flag);
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t a[kGrpCols];
-        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + buf * kGrpBN + col0, a);
-        const float4* sc4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0);
-        const int4* dz4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0);
-        tmem_ld_wait();
+        const float4* s4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0 + tc);
+        *reinterpret_cast<float4*>(sc) = s4[0];
+        *reinterpret_cast<float4*>(sc + 4) = s4[1];
+        int rs_g[4];
+        if constexpr (ZP) {
+          const int4* d4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0 + tc);
+          *reinterpret_cast<int4*>(dz) = d4[0];
+          *reinterpret_cast<int4*>(dz + 4) = d4[1];
 #pragma unroll
-        for (int q = 0; q < kGrpCols / 4; ++q) {
-          const float4 sc = sc4[q];
-          int a0 = static_cast<int>(a[4 * q]), a1 = static_cast<int>(a[4 * q + 1]);
-          int a2 = static_cast<int>(a[4 * q + 2]), a3 = static_cast<int>(a[4 * q + 3]);
-          if constexpr (ZP) {
-            const int4 dz = dz4[q];
-            a0 += dz.x * rs_g;
-            a1 += dz.y * rs_g;
-            a2 += dz.z * rs_g;
-            a3 += dz.w * rs_g;
+          for (int i = 0; i < 4; ++i) {
+            rs_g[i] = rs[i];
+            if (live[i] && G + 1 < p.ng) rs[i] = __ldg(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
           }
-          t[2 * q] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)), f32x2_pack(sc.x, sc.y), t[2 * q]);
-          t[2 * q + 1] = f32x2_fma(f32x2_pack(__int2float_rn(a2), __int2float_rn(a3)), f32x2_pack(sc.z, sc.w), t[2 * q + 1]);
         }
+        tmem_ld_wait();
+        tmem_ld_16x256b_x4(t_row + (16u << 16) + buf * kGrpBN, hi);
+        fold(lo, 0, rs_g);
+        tmem_ld_wait();
         tc_fence_before();  // accumulators and scales are in registers: the buffer may take another group
         __syncwarp();
         if (lane == 0) mbar_arrive(&grp_empty[buf]);
+        if (G + 1 < p.ng) {
+          wait_group(gcount + 1);
+          if (!ok) break;
+          tmem_ld_16x256b_x4(t_row + ((gcount + 1) % kGrpBufs) * kGrpBN, lo);
+        }
+        fold(hi, 2, rs_g);
       }
       if (!ok) break;
-      if (live) {
-        uint16_t* yrow = p.y + row * p.ldy + n0;
-        const uint64_t sa2 = f32x2_pack(sa, sa);
+      float bb[8];
+      *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(wb + tc);
+      *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(wb + tc + 4);
 #pragma unroll
-        for (int c = 0; c < kGrpCols / 16; ++c) {
-          uint32_t w[8];
+      for (int i = 0; i < 4; ++i) {
+        uint32_t w[4];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float2 bb = *reinterpret_cast<const float2*>(wb + c * 16 + 2 * q);
-            float y0, y1;
-            f32x2_unpack(f32x2_fma(t[c * 8 + q], sa2, f32x2_pack(bb.x, bb.y)), y0, y1);
-            const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
-            w[q] = *reinterpret_cast<const uint32_t*>(&v);
-          }
-          if (wide) {
-            st_global_v8(yrow + c * 16, w);
-          } else {
-            uint4* y4 = reinterpret_cast<uint4*>(yrow + c * 16);
-            y4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            y4[1] = make_uint4(w[4], w[5], w[6], w[7]);
-          }
+        for (int j = 0; j < 4; ++j) {
+          float y0, y1;
+          f32x2_unpack(f32x2_fma(t[i][j], f32x2_pack(sa[i], sa[i]), f32x2_pack(bb[2 * j], bb[2 * j + 1])), y0, y1);
+          const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
+          w[j] = *reinterpret_cast<const uint32_t*>(&v);
         }
+        if (live[i]) st_global_v4(p.y + (row0 + 8 * i) * p.ldy + n0 + tc, w);
       }
     }
   }

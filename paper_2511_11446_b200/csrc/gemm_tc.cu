@@ -14,8 +14,7 @@
 //   warp 1      MMA issuer: tcgen05.mma kind::i8, int32 accumulators in tensor memory (two
 //               accumulator buffers, so a tile's epilogue overlaps the next tile's mainloop)
 //   warps 2-9   epilogue: tcgen05.ld -> (float)acc * s_a[m]*s_w[n] + bias -> bf16 -> global; two warps
-//               per 32-token TMEM quadrant, each taking half of the tile's columns, one token per
-//               thread and one 32-byte store per 16 columns
+//               per 32-token TMEM quadrant, each taking half of the tile's columns
 //   warps 10-17 unpack (3/4-bit only): packed tile in smem -> int8 operand tile in smem, written in
 //               the swizzled layout the MMA descriptor expects, then fence.proxy.async
 //
@@ -128,14 +127,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         if constexpr (CG == 2) mbar_arrive_expect_tx_cluster(full0 + 8u * s, bytes);
         else mbar_arrive_expect_tx(&full_a[s], bytes);
       };
-      auto load = [&](void* dst, const CUtensorMap* tm, int c0, int c1, int s) {
-        if constexpr (CG == 2) tma_load_2d_pair(dst, tm, c0, c1, full0 + 8u * s);
-        else tma_load_2d(dst, tm, c0, c1, &full_a[s]);
+      auto load_tokens = [&](int s, int c0, int c1) {
+        if constexpr (CG == 2) tma_load_2d_pair(sA + s * A_BYTES, &tmap_a, c0, c1, full0 + 8u * s);
+        else tma_load_2d(sA + s * A_BYTES, &tmap_a, c0, c1, &full_a[s]);
       };
       auto load_a = [&](int tile, int kb, int s) {
         int c0, c1;
         a_tile_coords(p, (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM, kb, c0, c1);
-        load(sA + s * A_BYTES, &tmap_a, c0, c1, s);
+        load_tokens(s, c0, c1);
       };
       // Stages whose weight tile is in flight but whose activation tile is not (before a_open): they are
       // the ring's first ones, in order, from (first_tile, k-block 0) on.
@@ -179,11 +178,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
           if constexpr (BITS == 8) {
             expect(st.s, A_BYTES + B_BYTES);
-            load(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, st.s);
+            if constexpr (CG == 2) tma_load_w_pair(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, full0 + 8u * st.s);
+            else tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, &full_a[st.s]);
           } else {
             if (!(ok = mbar_spin_wait(&pempty[ps.s], ps.ph ^ 1u, abort_flag))) break;
             mbar_arrive_expect_tx(&pfull[ps.s], P_BYTES);
-            tma_load_2d(sP + ps.s * P_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[ps.s]);
+            tma_load_w(sP + ps.s * P_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[ps.s]);
             expect(st.s, A_BYTES);
             ps.next(NP);
           }
@@ -195,7 +195,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               ready_tile = m_row >> 7;
               a_ready = true;
             }
-            load(sA + st.s * A_BYTES, &tmap_a, a0, a1, st.s);
+            load_tokens(st.s, a0, a1);
           } else {
             ++deferred;
           }
@@ -423,6 +423,24 @@ static int encode_2d(CUtensorMap* out, const void* base, uint64_t inner_bytes, u
   return DP_OK;
 }
 
+// Rows of a row-major weight matrix of row_bytes bytes, `rows` a multiple of 32, in the order the epilogues
+// want their accumulator columns in: within every 32 rows, row 8t + 2j + e of the matrix becomes row
+// 8j + 2t + e of the tile (t, j < 4, e < 2). The accumulator-fragment read of tensor memory gives lane t of a
+// quad columns 8j + 2t + e, which are then 8 consecutive output channels: one 16-byte store per token.
+int gemm_encode_w_rows(CUtensorMap* out, const void* base, uint64_t row_bytes, uint64_t rows, uint32_t box_inner,
+                       uint32_t box_rows, bool swizzle128) {
+  const cuuint64_t dims[5] = {row_bytes, 2, 4, 4, rows / 32};
+  const cuuint64_t strides[4] = {row_bytes, 8 * row_bytes, 2 * row_bytes, 32 * row_bytes};
+  const cuuint32_t box[5] = {box_inner, 2, 4, 4, box_rows / 32};
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(DP_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+  return DP_OK;
+}
+
 // Any row-major matrix seen as bytes: rows of inner_bytes at pitch_bytes, boxes of box_inner x box_rows
 // bytes, 128-byte swizzle.
 int gemm_encode_bytes_2d(CUtensorMap* out, const void* base, uint64_t inner_bytes, uint64_t rows, uint64_t pitch_bytes,
@@ -442,7 +460,7 @@ int gemm_encode_a_tiled(CUtensorMap* out, const int8_t* q, int64_t M, int64_t K)
 int gemm_encode_w(CUtensorMap* out, const void* qweight, int32_t N, int32_t K, int32_t bits,
                   int32_t bn, int32_t cg) {
   const uint64_t row_bytes = static_cast<uint64_t>(K) * bits / 8;
-  return encode_2d(out, qweight, row_bytes, N, row_bytes, BK * bits / 8, bn / cg, bits == 8);
+  return gemm_encode_w_rows(out, qweight, row_bytes, N, BK * bits / 8, bn / cg, bits == 8);
 }
 
 // Tile shape: width from {256, 192, 128, 64} dividing N, rows 128 (one CTA) or 256 (a CTA pair),

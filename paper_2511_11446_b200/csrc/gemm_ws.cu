@@ -113,12 +113,12 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           const int w_row = strip * BN + static_cast<int>(rank) * BNL;
           if constexpr (BITS == 8) {
             mbar_arrive_expect_tx(w_full, KB * B_BYTES);
-            for (int kb = 0; kb < KB; ++kb) tma_load_2d(sW + kb * B_BYTES, &tmap_w, kb * BK, w_row, w_full);
+            for (int kb = 0; kb < KB; ++kb) tma_load_w(sW + kb * B_BYTES, &tmap_w, kb * BK, w_row, w_full);
           } else {
             for (int kb = 0; kb < KB && ok; ++kb) {
               if (!(ok = mbar_wait(&pempty[pr.s], pr.ph ^ 1u, abort_flag))) break;
               mbar_arrive_expect_tx(&pfull[pr.s], P_BYTES);
-              tma_load_2d(sA + pr.s * A_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[pr.s]);
+              tma_load_w(sA + pr.s * A_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[pr.s]);
               pr.next(NS);
             }
             // activation tiles reuse these slots: wait until the expansion warps have read them all
