@@ -261,6 +261,23 @@ __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K
   }
 }
 
+// 32 codes of 3 bits (a little-endian stream in s0, s1, s2) -> 8 words of 4 bytes, byte i of the table t_hi:t_lo
+// for code i. Eight codes at a time: their 24 bits are opened up to one code per nibble in three halvings
+// (a field that moves up by n bits is added 2^n - 1 times more), and a nibble is what a byte permute selects
+// by: 11 instructions per eight codes, against 20 with a shift and a mask per code.
+__device__ __forceinline__ void expand3(uint32_t s0, uint32_t s1, uint32_t s2, uint32_t t_lo, uint32_t t_hi,
+                                        uint32_t (&w)[8]) {
+  const uint32_t v[4] = {s0, __funnelshift_r(s0, s1, 24), __funnelshift_r(s1, s2, 16), s2 >> 8};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t a = (v[i] & 0xFFFu) + (v[i] & 0xFFF000u) * 16u;  // 4 codes per half word
+    const uint32_t b = a + (a & 0x0FC00FC0u) * 3u;                  // 2 codes per byte
+    const uint32_t c = b + (b & 0x38383838u);                       // 1 code per nibble
+    w[2 * i] = __byte_perm(t_lo, t_hi, c);
+    w[2 * i + 1] = __byte_perm(t_lo, t_hi, c >> 16);
+  }
+}
+
 // Packed unit -> 8 words of 4 int8 (u - z of the stored codes u, k ascending). z in [0, 2^BITS): the
 // zero-point in use, 2^(BITS-1) for symmetric layers. u + 128 - z stays inside its byte, and flipping the
 // byte's top bit takes the 128 off again.
@@ -278,15 +295,7 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t
       w[2 * i + 1] = (__byte_perm(lo, hi, 0x7362) + up) ^ 0x80808080u;
     }
   } else {
-    const uint64_t lo64 = (static_cast<uint64_t>(pk[1]) << 32) | pk[0];
-    const uint64_t hi64 = (static_cast<uint64_t>(pk[2]) << 32) | pk[1];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int bit = 12 * j;
-      const uint32_t x = static_cast<uint32_t>(bit < 32 ? (lo64 >> bit) : (hi64 >> (bit - 32))) & 0xFFFu;
-      const uint32_t o = (x & 7u) | ((x & 0x38u) << 5) | ((x & 0x1C0u) << 10) | ((x & 0xE00u) << 15);
-      w[j] = (o + up) ^ 0x80808080u;
-    }
+    expand3(pk[0], pk[1], pk[2], (0x03020100u + up) ^ 0x80808080u, (0x07060504u + up) ^ 0x80808080u, w);
   }
 }
 

@@ -199,10 +199,6 @@ __device__ __forceinline__ void unpack4_tile(const uint8_t* P, uint8_t* B, int t
 }
 
 // 3-bit: tile P is [BN][48 bytes]; each thread expands 3 words (32 codes) into two 16-byte chunks.
-__device__ __forceinline__ uint32_t spread3(uint32_t v) {  // 4 fields of 3 bits -> top 3 bits of 4 bytes
-  return (((v << 5) & 0x000000E0u) | ((v << 10) & 0x0000E000u) | ((v << 15) & 0x00E00000u) |
-          ((v << 20) & 0xE0000000u)) ^ 0x80808080u;
-}
 template <int BN>
 __device__ __forceinline__ void unpack3_tile(const uint8_t* P, uint8_t* B, int tid) {
 #pragma unroll
@@ -211,20 +207,12 @@ __device__ __forceinline__ void unpack3_tile(const uint8_t* P, uint8_t* B, int t
     if (BN * 4 % kUnpackThreads != 0 && idx >= BN * 4) break;
     const int row = idx >> 2, g = idx & 3;
     const uint32_t* src = reinterpret_cast<const uint32_t*>(P + row * 48 + g * 12);
-    const uint32_t s0 = src[0], s1 = src[1], s2 = src[2];
-    uint4 o0, o1;
-    o0.x = spread3(s0);                               // stream bits  0..11
-    o0.y = spread3(s0 >> 12);                         //             12..23
-    o0.z = spread3(__funnelshift_r(s0, s1, 24));      //             24..35
-    o0.w = spread3(s1 >> 4);                          //             36..47
-    o1.x = spread3(s1 >> 16);                         //             48..59
-    o1.y = spread3(__funnelshift_r(s1, s2, 28));      //             60..71
-    o1.z = spread3(s2 >> 8);                          //             72..83
-    o1.w = spread3(s2 >> 20);                         //             84..95
+    uint32_t w[8];
+    expand3(src[0], src[1], src[2], 0xE0C0A080u, 0x60402000u, w);  // (u - 4) * 32
     uint8_t* brow = B + row * 128;
     const int sw = row & 7;
-    *reinterpret_cast<uint4*>(brow + (((2 * g) ^ sw) << 4)) = o0;
-    *reinterpret_cast<uint4*>(brow + (((2 * g + 1) ^ sw) << 4)) = o1;
+    *reinterpret_cast<uint4*>(brow + (((2 * g) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(brow + (((2 * g + 1) ^ sw) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
   }
 }
 
