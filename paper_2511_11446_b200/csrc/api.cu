@@ -524,7 +524,7 @@ extern "C" int dp_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t l
   int st = check_device();
   if (st != DP_OK) return st;
   return launch_ln_modulate_daq(x, M, K, ldx, shift, scale, shift ? rows_per_sample : 1, eps, q, ldq, s_a,
-                                static_cast<cudaStream_t>(stream), false);
+                                static_cast<cudaStream_t>(stream), true);
 }
 
 extern "C" int dp_wq_linear_residual(const dp_weight* w, const void* x_bf16, int64_t ldx, int64_t M,

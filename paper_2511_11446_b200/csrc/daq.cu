@@ -271,7 +271,7 @@ extern "C" int dp_daq_quantize(const void* x_bf16, int64_t M, int64_t K, int64_t
   int st = check_device();
   if (st != DP_OK) return st;
   return launch_daq(x_bf16, M, K, ldx, q, ldq, s_a, rowsum, KORDER_NATURAL, false,
-                    static_cast<cudaStream_t>(stream), false);
+                    static_cast<cudaStream_t>(stream), true);
 }
 
 extern "C" int dp_daq_quantize_robust(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, int8_t* q,
@@ -293,5 +293,5 @@ extern "C" int dp_daq_quantize_robust(const void* x_bf16, int64_t M, int64_t K, 
   int st = check_device();
   if (st != DP_OK) return st;
   return launch_daq_robust(x_bf16, M, K, ldx, q, ldq, s_a, rowsum, clip_rank, act_bits, false,
-                           static_cast<cudaStream_t>(stream), false, nullptr);
+                           static_cast<cudaStream_t>(stream), true, nullptr);
 }
