@@ -159,6 +159,13 @@ __device__ __forceinline__ void daq_sync_exit(const GemmParams& p) {
   }
 }
 
+// A producer that gave up: copies still in flight get a bounded time to land before the CTA exits.
+__device__ __forceinline__ void producer_drain() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < (1ll << 22)) {
+  }
+}
+
 struct Ring {  // stage index + phase bit of a circular buffer
   int s = 0;
   uint32_t ph = 0;

@@ -10,7 +10,8 @@
 // memory, and each CTA ends up with its 128 x BN accumulator in its own tensor memory. Per CTA this
 // halves the weight bytes fetched, expanded and read by the tensor core for the same MACs.
 // Warp roles:
-//   warp 0      TMA producer: int8 activation tiles (128-byte-swizzled) and packed weight tiles
+//   warp 0      TMA producer: int8 activation tiles (128-byte-swizzled)
+//   last warp   TMA producer: (packed) weight tiles
 //   warp 1      MMA issuer: tcgen05.mma kind::i8, int32 accumulators in tensor memory (two
 //               accumulator buffers, so a tile's epilogue overlaps the next tile's mainloop)
 //   warps 2-9   epilogue: tcgen05.ld -> (float)acc * s_a[m]*s_w[n] + bias -> bf16 -> global; two warps
@@ -32,9 +33,12 @@
 
 namespace dp {
 
+// One warp more than the shared roles: the weights' TMA producer.
+__host__ __device__ constexpr int tc_threads(int bits) { return gemm_threads(bits) + 32; }
+
 // ---- the kernel ----------------------------------------------------------------------------------
 template <int BN, int BITS, bool PERM, int CG, bool RES = false>
-__global__ void __launch_bounds__(gemm_threads(BITS), 1)
+__global__ void __launch_bounds__(tc_threads(BITS), 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                const GemmParams p) {
   constexpr int BNL = BN / CG;  // weight rows held by this CTA
@@ -42,6 +46,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   constexpr int NP = kPStages;
   constexpr int A_BYTES = BM * BK, B_BYTES = BNL * BK, P_BYTES = p_stage_bytes(BNL, BITS);
   constexpr int TCOLS = tmem_cols(BN);
+  constexpr int kWeightWarp = gemm_threads(BITS) / 32;
   constexpr int SHIFT = 8 - BITS;  // accumulator carries a factor 2^SHIFT
 
   extern __shared__ uint8_t smem_raw[];
@@ -68,7 +73,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const int first_tile = blockIdx.x / CG, tile_stride = gridDim.x / CG;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
-      mbar_init(&full_a[i], CG);  // pair: the leader's copy counts both CTAs' TMA loads
+      mbar_init(&full_a[i], (BITS == 8 ? 2 : 1) * CG);  // one arrival per producer; pair: the leader's copy counts both CTAs'
       mbar_init(&bready[i], kUnpackThreads);
       mbar_init(&empty[i], 1);
       mbar_init(&peer_ready[i], 1);
@@ -108,55 +113,30 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   // constants; unless early_w is set, everything waits here.
   if (!p.early_w) pdl_wait();
 
-  // The two single-thread roles run behind elect.sync, not a lane comparison: the compiler then knows
+  // The single-thread roles run behind elect.sync, not a lane comparison: the compiler then knows
   // that one thread is active and keeps descriptors, addresses and barriers in uniform registers. Behind
   // `lane == 0` the four MMAs and the commit of a k-block took 317 cycles to issue and the two TMA
   // loads 224, which set a pace of ~560 cycles per k-block at EVERY tile width (64 .. 256; the tensor
   // core needs 128 .. 512); this way they take 100 and 127. A stage's barrier is polled one k-block
-  // ahead, before the current one's instructions, so the poll's ~75 cycles run under them.
+  // ahead, before the current one's instructions, so the poll's ~75 cycles run under them. Activations and
+  // weights are brought in by two threads: one issuing both set a pace of 390 cycles per k-block, which tiles
+  // up to 128 wide feel (whole 8-bit layers K = 1152, N = 1152, M = 64 / 1024: 6.4 / 7.4 us with one producer, 5.2 /
+  // 6.7 with two; K = 4608, N = 1152, M = 256: 12.0 -> 11.3).
   if (warp == 0) {
-    // ================= TMA producer =================
+    // ================= TMA producer: activations =================
     if (elect_one()) {
-      Ring st, ps;
-      bool ok = true;
-      bool a_open = !p.early_w || p.x != nullptr;  // false until griddepcontrol.wait has been executed
-      int ready_tile = -1;                          // in-kernel DAQ: last 128-token tile seen complete
+      Ring st;
+      bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
+      int ready_tile = -1;  // in-kernel DAQ: last 128-token tile seen complete
       // In a pair both CTAs' bytes are counted on the leader's barrier.
       const uint32_t full0 = CG == 2 ? map_to_cta(&full_a[0], 0) : smem_u32(&full_a[0]);
-      auto expect = [&](int s, uint32_t bytes) {
-        if constexpr (CG == 2) mbar_arrive_expect_tx_cluster(full0 + 8u * s, bytes);
-        else mbar_arrive_expect_tx(&full_a[s], bytes);
-      };
-      auto load_tokens = [&](int s, int c0, int c1) {
-        if constexpr (CG == 2) tma_load_2d_pair(sA + s * A_BYTES, &tmap_a, c0, c1, full0 + 8u * s);
-        else tma_load_2d(sA + s * A_BYTES, &tmap_a, c0, c1, &full_a[s]);
-      };
-      auto load_a = [&](int tile, int kb, int s) {
-        int c0, c1;
-        a_tile_coords(p, (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM, kb, c0, c1);
-        load_tokens(s, c0, c1);
-      };
-      // Stages whose weight tile is in flight but whose activation tile is not (before a_open): they are
-      // the ring's first ones, in order, from (first_tile, k-block 0) on.
-      int deferred = 0;
-      auto open_a = [&]() {
-        pdl_wait();
-        a_open = true;
-        int t = first_tile, k = 0;
-        for (int d = 0; d < deferred; ++d) {
-          load_a(t, k, d);
-          if (++k == KB) {
-            k = 0;
-            t += tile_stride;
-          }
-        }
-      };
-      bool free_next = mbar_test_wait(&empty[0], 1u);
+      if (p.early_w) pdl_wait();
       for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
-        const int n_blk = tile % p.n_tiles;  // column tiles of one row strip run together
         const int m_row = (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM;
-        const int w_row = n_blk * BN + static_cast<int>(rank) * BNL;
-        bool a_ready = p.x == nullptr || (m_row >> 7) == ready_tile;
+        if (p.x != nullptr && (m_row >> 7) != ready_tile) {
+          if (!(ok = wait_tile_quantized(p, m_row >> 7, abort_flag))) break;
+          ready_tile = m_row >> 7;
+        }
         int a0, a1;
         a_tile_coords(p, m_row, 0, a0, a1);
         const int a0_step = p.a_tiled ? 0 : BK, a1_step = p.a_tiled ? BM : 0;
@@ -165,50 +145,72 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             // test hook: this stage gets no loads and no arrival, so its barrier never completes and
             // the bounded waits of the other roles run out
             if (kb == p.dbg_skip_kb && tile == first_tile) {
-              if (!a_open) open_a();
               st.next(NS);
               free_next = false;
               continue;
             }
           }
-          if (!a_open && deferred == NS) open_a();  // ring full of weight tiles: now wait for the activations
           if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
           Ring nx = st;
           nx.next(NS);
           free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
-          if constexpr (BITS == 8) {
-            expect(st.s, A_BYTES + B_BYTES);
-            if constexpr (CG == 2) tma_load_w_pair(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, full0 + 8u * st.s);
-            else tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, &full_a[st.s]);
+          if constexpr (CG == 2) {
+            mbar_arrive_expect_tx_cluster(full0 + 8u * st.s, A_BYTES);
+            tma_load_2d_pair(sA + st.s * A_BYTES, &tmap_a, a0, a1, full0 + 8u * st.s);
           } else {
-            if (!(ok = mbar_spin_wait(&pempty[ps.s], ps.ph ^ 1u, abort_flag))) break;
-            mbar_arrive_expect_tx(&pfull[ps.s], P_BYTES);
-            tma_load_w(sP + ps.s * P_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[ps.s]);
-            expect(st.s, A_BYTES);
-            ps.next(NP);
-          }
-          if (a_open) {
-            if (!a_ready) {  // weights of this stage are already in flight; now the tile's tokens
-              if (p.early_w && ready_tile < 0) pdl_wait();  // until the preceding kernel has exited the
-                                                           // counters still hold ITS tiles' counts
-              if (!(ok = wait_tile_quantized(p, m_row >> 7, abort_flag))) break;
-              ready_tile = m_row >> 7;
-              a_ready = true;
-            }
-            load_tokens(st.s, a0, a1);
-          } else {
-            ++deferred;
+            mbar_arrive_expect_tx(&full_a[st.s], A_BYTES);
+            tma_load_2d(sA + st.s * A_BYTES, &tmap_a, a0, a1, &full_a[st.s]);
           }
           st = nx;
         }
       }
-      if (!a_open) open_a();  // fewer k-blocks than stages in the whole CTA
-      if (!ok) {
-        // drain: give copies still in flight a bounded time to land before the CTA exits
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) {
+      if (!ok) producer_drain();
+    }
+  } else if (warp == kWeightWarp) {
+    // ================= TMA producer: weights (constants: with early_w it does not wait for the preceding
+    // kernel) =================
+    if (elect_one()) {
+      Ring st;
+      bool ok = true;
+      if constexpr (BITS == 8) {
+        bool free_next = mbar_test_wait(&empty[0], 1u);
+        const uint32_t full0 = CG == 2 ? map_to_cta(&full_a[0], 0) : smem_u32(&full_a[0]);
+        for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
+          const int w_row = (tile % p.n_tiles) * BN + static_cast<int>(rank) * BNL;
+          for (int kb = 0; kb < KB; ++kb) {
+            if constexpr (CG == 1) {
+              if (kb == p.dbg_skip_kb && tile == first_tile) {
+                st.next(NS);
+                free_next = false;
+                continue;
+              }
+            }
+            if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+            Ring nx = st;
+            nx.next(NS);
+            free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
+            if constexpr (CG == 2) {
+              mbar_arrive_expect_tx_cluster(full0 + 8u * st.s, B_BYTES);
+              tma_load_w_pair(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, full0 + 8u * st.s);
+            } else {
+              mbar_arrive_expect_tx(&full_a[st.s], B_BYTES);
+              tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, &full_a[st.s]);
+            }
+            st = nx;
+          }
+        }
+      } else {
+        for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
+          const int w_row = (tile % p.n_tiles) * BN + static_cast<int>(rank) * BNL;
+          for (int kb = 0; kb < KB; ++kb) {
+            if (!(ok = mbar_spin_wait(&pempty[st.s], st.ph ^ 1u, abort_flag))) break;
+            mbar_arrive_expect_tx(&pfull[st.s], P_BYTES);
+            tma_load_w(sP + st.s * P_BYTES, &tmap_w, kb * (BK * BITS / 8), w_row, &pfull[st.s]);
+            st.next(NP);
+          }
         }
       }
+      if (!ok) producer_drain();
     }
   } else if (warp == 1) {
     if (elect_one()) {
@@ -384,7 +386,7 @@ int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out) {
   {  // how many CTA pairs fit on the device at once (one CTA per SM)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(sms & ~1));
-    cfg.blockDim = dim3(gemm_threads(4));
+    cfg.blockDim = dim3(tc_threads(4));
     cfg.dynamicSmemBytes = gemm_smem_bytes<256, 4, 2>();
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -467,7 +469,7 @@ int gemm_encode_w(CUtensorMap* out, const void* qweight, int32_t N, int32_t K, i
 // 8-bit operands: a fixed cost (prologue, first loads, last epilogue) plus, per wave of tiles over the SMs or
 // pairs, the larger of the k-blocks' time and the least time a tile takes (its epilogue, when K is short). The
 // constants, in us, are a least-squares fit to 88 shapes (K = 384 .. 4608, N = 768 .. 4608, 48 .. 32768 tokens)
-// timed at every width: the choice is 0.5 % from the fastest on average, 8 % at worst. Fixed costs alone
+// timed at every width: the choice is 0.4 % from the fastest on average, 6 % at worst. Fixed costs alone
 // say: narrow single tiles while a layer is one wave, wide pairs beyond.
 // Packed operands (expanded in the kernel): waves times width, pairs, which expand half, preferred.
 void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int* bn_out, int* cg_out) {
@@ -477,9 +479,9 @@ void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allo
     int bn, cg;
     double fixed, per_kb, min_tile;
   };
-  static const Form forms[] = {{256, 2, 1.88, 0.23, 1.18}, {192, 2, 1.40, 0.20, 1.05}, {128, 2, 1.12, 0.17, 0.90},
-                               {256, 1, 0.99, 0.34, 1.61}, {192, 1, 0.82, 0.26, 1.30}, {128, 1, 0.69, 0.21, 1.02},
-                               {64, 1, 0.31, 0.20, 0.82}};
+  static const Form forms[] = {{256, 2, 2.39, 0.211, 1.16}, {192, 2, 1.91, 0.179, 1.03}, {128, 2, 1.47, 0.139, 0.89},
+                               {256, 1, 1.71, 0.313, 1.52}, {192, 1, 1.45, 0.235, 1.21}, {128, 1, 1.14, 0.182, 0.98},
+                               {64, 1, 0.86, 0.152, 0.76}};
   int best_bn = 0, best_cg = 1;
   double best_cost = 1e30;
   for (const Form& f : forms) {
@@ -502,7 +504,7 @@ void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allo
 template <int BN, int CG>
 static cudaError_t launch_bn(const GemmProblem& g, const GemmParams& p, dim3 grid, cudaStream_t stream,
                              bool pdl) {
-  const dim3 block(gemm_threads(g.bits));
+  const dim3 block(tc_threads(g.bits));
   switch (g.bits) {
     case 8:
       if (g.res != nullptr)
