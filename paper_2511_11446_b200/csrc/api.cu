@@ -39,7 +39,7 @@ int fail(int status, const char* fmt, ...) {
 constexpr int kMaxDevices = 64;
 struct DeviceInfo {
   int status;  // DP_OK or DP_ERR_ARCH
-  int num_sms, max_pairs;
+  int num_sms, max_pairs, max_clusters[kMaxSplits + 1];
 };
 static DeviceInfo g_dev[kMaxDevices];
 static std::atomic<int> g_dev_ready[kMaxDevices];
@@ -59,14 +59,14 @@ int check_device() {
   if (!g_dev_ready[dev].load(std::memory_order_acquire)) {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!g_dev_ready[dev].load(std::memory_order_relaxed)) {
-      DeviceInfo d = {DP_OK, 0, 0};
+      DeviceInfo d = {DP_OK, 0, 0, {}};
       int major = 0;
       cudaError_t e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
       if (e != cudaSuccess) return fail(DP_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
       if (major != 10) {
         d.status = DP_ERR_ARCH;
       } else {  // a failure here is reported and NOT cached: the next call tries again
-        st = gemm_init_device(dev, &d.num_sms, &d.max_pairs);
+        st = gemm_init_device(dev, &d.num_sms, &d.max_pairs, d.max_clusters);
         if (st != DP_OK) return st;
       }
       g_dev[dev] = d;
@@ -92,6 +92,16 @@ int gemm_max_pairs() {
   return d ? d->max_pairs : 0;
 }
 
+GemmLimits gemm_limits() {
+  GemmLimits lim = {148, 74, {}};
+  if (const DeviceInfo* d = ready_device()) {
+    lim.sms = d->num_sms;
+    lim.pairs = d->max_pairs;
+    for (int s = 0; s <= kMaxSplits; ++s) lim.clusters[s] = d->max_clusters[s];
+  }
+  return lim;
+}
+
 static size_t align256(size_t v) { return (v + 255) & ~static_cast<size_t>(255); }
 // Bytes of the int8 activation scratch: whole 128-token tiles.
 static size_t scratch_q_bytes(int64_t M, int32_t K) { return static_cast<size_t>((M + 127) / 128 * 128) * K; }
@@ -100,6 +110,8 @@ constexpr uint32_t kLinearFlags =
     DP_FLAG_FORCE_SIMT | DP_FLAG_FORCE_MMA | DP_FLAG_NO_PDL | DP_FLAG_TILE_N_MASK | DP_FLAG_CTA_PAIR |
     DP_FLAG_NO_CTA_PAIR | DP_FLAG_WEIGHT_STATIONARY | DP_FLAG_NO_WEIGHT_STATIONARY | DP_FLAG_UNPACK_FIRST |
     DP_FLAG_NO_UNPACK_FIRST | DP_FLAG_ACT_STATIONARY | DP_FLAG_NO_ACT_STATIONARY;
+constexpr int64_t kAsMinRows = 1024;   // below, its strip fill is never made up for
+constexpr int kTuneReps = 12;
 constexpr int64_t kWsMinRows = 8192;  // from here on a resident weight strip is reused often enough to pay
 static int forced_bn(uint32_t flags) { return static_cast<int>((flags & DP_FLAG_TILE_N_MASK) >> 8) * 64; }
 
@@ -139,7 +151,8 @@ static void choose_tile(uint32_t flags, int64_t M, int32_t N, int32_t K, int32_t
   uint32_t allow = 0x6;
   if (flags & DP_FLAG_CTA_PAIR) allow = 0x4;
   if (flags & DP_FLAG_NO_CTA_PAIR) allow = 0x2;
-  gemm_pick_tile(M, N, K, bits, allow, bn, cg);
+  int splits = 1;  // decided again by the launch, from the same numbers
+  gemm_pick_tile(M, N, K, bits, allow, 0, bn, cg, &splits);
   const int fb = forced_bn(flags);
   if (fb != 0 && N % fb == 0) {
     *bn = fb;
@@ -651,17 +664,28 @@ static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool al
   };
   std::vector<Cand> cands;
   const int widths[4] = {64, 128, 192, 256};
-  const int pre_lo = (flags & DP_FLAG_UNPACK_FIRST) ? 1 : 0;
-  const int pre_hi = (w.bits < 8 && !(flags & (DP_FLAG_NO_UNPACK_FIRST | DP_FLAG_FUSED_DAQ))) ? 1 : 0;
-  for (int pre = pre_lo < pre_hi ? pre_lo : pre_hi; pre <= pre_hi; ++pre)
-    for (int i = 0; i < 4; ++i)
-      if (w.N % widths[i] == 0) {
-        cands.push_back({widths[i], 1, 0, pre});
-        if (widths[i] >= 128) cands.push_back({widths[i], 2, 0, pre});
-        if (widths[i] >= 192 && gemm_ws_supported(w.N, w.K)) cands.push_back({widths[i], 2, 1, pre});
-        if (allow_as && as_pointers_ok(&w) && gemm_as_supported(w.N, w.K) && (w.bits == 8 || pre))
-          cands.push_back({widths[i], 2, 2, pre});
+  // Packed layers are tried in the unpack-first form (faster at every measured size) unless the flags say otherwise.
+  const bool pre = w.bits < 8 && !(flags & (DP_FLAG_NO_UNPACK_FIRST | DP_FLAG_FUSED_DAQ));
+  const bool eight = w.bits == 8 || pre;  // the kernel sees 8-bit weights: the time model applies
+  double least = 1e30;
+  for (int i = 0; i < 4; ++i)
+    for (int cg = 1; cg <= 2; ++cg)
+      if (w.N % widths[i] == 0) least = std::min(least, gemm_tile_cost(M, w.N, w.K, widths[i], cg));
+  for (int i = 0; i < 4; ++i)
+    if (w.N % widths[i] == 0) {
+      for (int cg = 1; cg <= 2; ++cg) {
+        if (cg == 2 && widths[i] < 128) continue;
+        if (!eight || gemm_tile_cost(M, w.N, w.K, widths[i], cg) < 1.25 * least) cands.push_back({widths[i], cg, 0, pre});
       }
+      if (widths[i] >= 192 && gemm_ws_supported(w.N, w.K) && (!eight || M >= kWsMinRows)) cands.push_back({widths[i], 2, 1, pre});
+      if (allow_as && as_pointers_ok(&w) && gemm_as_supported(w.N, w.K) && eight && M >= kAsMinRows)
+        cands.push_back({widths[i], 2, 2, pre});
+    }
+  // (the default first: a later one has to beat it)
+  std::stable_sort(cands.begin(), cands.end(), [&](const Cand& a, const Cand& b) {
+    auto is_default = [&](const Cand& c) { return c.bn == *bn_out && c.cg == *cg_out && c.ws == *ws_out; };
+    return is_default(a) && !is_default(b);
+  });
   void *x = nullptr, *y = nullptr, *ws = nullptr;
   cudaStream_t stream = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -679,22 +703,41 @@ static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool al
   for (size_t c = 0; c < cands.size() && st == DP_OK; ++c) {
     CUtensorMap tw;
     st = gemm_encode_w(&tw, w.qweight, w.N, w.K, w.bits, cands[c].bn, cands[c].cg);
-    const int warm = 2, reps = 8;
-    for (int it = 0; it < warm + reps && st == DP_OK; ++it) {
-      if (it == warm) cudaEventRecord(e0, stream);
-      st = run_linear(&w, x, w.K, nullptr, M, y, w.N, ws, nullptr, nullptr, flags & DP_FLAG_NO_PDL, stream, &tw,
-                      cands[c].bn, cands[c].cg, cands[c].ws, nullptr, it > 0, nullptr, cands[c].pre);
+    // Timed as one graph of kTuneReps layers: launched one by one, layers of a few microseconds would measure the
+    // host. The best of three replays counts.
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if (st == DP_OK) {  // lazy loading of the kernels, outside the capture
+      st = run_linear(&w, x, w.K, nullptr, M, y, w.N, ws, nullptr, nullptr, flags & DP_FLAG_NO_PDL, stream, &tw, cands[c].bn,
+                      cands[c].cg, cands[c].ws, nullptr, false, nullptr, cands[c].pre);
     }
     if (st != DP_OK) break;
-    cudaEventRecord(e1, stream);
-    e = cudaEventSynchronize(e1);
-    float ms = 0.0f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      for (int it = 0; it < kTuneReps && st == DP_OK; ++it)
+        st = run_linear(&w, x, w.K, nullptr, M, y, w.N, ws, nullptr, nullptr, flags & DP_FLAG_NO_PDL, stream, &tw,
+                        cands[c].bn, cands[c].cg, cands[c].ws, nullptr, it > 0, nullptr, cands[c].pre);
+      e = cudaStreamEndCapture(stream, &graph);
+    }
+    if (e == cudaSuccess && st == DP_OK) e = cudaGraphInstantiate(&exec, graph, 0);
+    float ms = 1e30f;
+    for (int it = 0; it < 4 && e == cudaSuccess && st == DP_OK; ++it) {
+      cudaEventRecord(e0, stream);
+      cudaGraphLaunch(exec, stream);
+      cudaEventRecord(e1, stream);
+      e = cudaEventSynchronize(e1);
+      float t = 0.0f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+      if (it > 0 && t < ms) ms = t;
+    }
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
+    if (st != DP_OK) break;
     if (e != cudaSuccess) {
       st = fail(DP_ERR_CUDA, "autotune timing: %s", cudaGetErrorString(e));
       break;
     }
-    if (ms < best) {
+    if (ms < 0.985f * best) {
       best = ms;
       *bn_out = cands[c].bn;
       *cg_out = cands[c].cg;

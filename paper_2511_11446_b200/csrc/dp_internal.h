@@ -129,9 +129,21 @@ struct GemmProblem {
   float* s_a_out;
   int32_t* sync;
 };
-// allow: bit 1 = single-CTA tiles permitted, bit 2 = CTA-pair tiles permitted
-void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int* bn_out, int* cg_out);
+// allow: bit 1 = single-CTA tiles permitted, bit 2 = CTA-pair tiles permitted, bit 3 = no 192-wide ones
+// forced_bn: 0, or the width to take; *splits_out: CTAs that share a tile along K (1: not split).
+void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int forced_bn, int* bn_out, int* cg_out,
+                    int* splits_out);
+// The model's estimate (us) for one width and CTA count of an 8-bit layer's GEMM.
+double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg);
 int gemm_max_pairs();
+// gemm_split.cu -- split-K form of the single-CTA streaming kernel and of the 16-bit kernel (64-wide tiles).
+constexpr int kMaxSplits = 4;
+struct GemmLimits {  // of the current device: SMs, resident CTA pairs, resident clusters of s split-K CTAs
+  int sms, pairs, clusters[kMaxSplits + 1];
+};
+GemmLimits gemm_limits();
+int gemm_split_init_device(int* max_clusters);
+int gemm_split_factor(const GemmLimits& lim, int64_t tiles, int kb, double per_kb, double* saved_us);
 int gemm_encode_a(CUtensorMap* out, const int8_t* q, int64_t M, int64_t K, int64_t ldq);
 // int8 activations stored as [ceil(M/128)][K/128] tiles of 128 tokens x 128 codes (16 KB each).
 int gemm_encode_a_tiled(CUtensorMap* out, const int8_t* q, int64_t M, int64_t K);
@@ -150,7 +162,7 @@ int gemm_ws_pick_bn(int32_t N);
 int launch_gemm_ws(const GemmProblem& p, cudaStream_t stream, bool pdl);
 // Per-device set-up (kernel attributes, tensor-map encoder, SM and CTA-pair counts), called once per
 // device by check_device() with that device current.
-int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out);
+int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out, int* max_clusters_out);
 int gemm_ws_init_device();
 int gemm_as_init_device();
 int gemm_bf16_init_device();

@@ -6,7 +6,7 @@
 //   be able to run them in the same call sequence. No DAQ, no weight scales.
 //
 // One persistent CTA per SM walks 128 x BN output tiles (column tiles of a row strip together). Warp 0:
-// TMA producer (activation and weight tiles of 64 bf16 = 128-byte rows, 128-byte swizzle, straight
+// TMA producer (activation tiles, the last warp: weight tiles, of 64 bf16 = 128-byte rows, 128-byte swizzle, straight
 // from the caller's row-major matrices); warp 1: MMA issuer (tcgen05.mma kind::f16 with bf16 operands,
 // fp32 accumulators in tensor memory, two buffers); warps 2-9: epilogue:
 // tcgen05.ld -> + bias -> bf16 -> 16-byte stores.
@@ -14,22 +14,9 @@
 
 namespace dp {
 
-constexpr int kBfThreads = kUnpackWarp0 * 32;
+constexpr int kBfWeightWarp = kUnpackWarp0;  // the warp after the epilogue's
+constexpr int kBfThreads = (kBfWeightWarp + 1) * 32;
 constexpr int kBfBK = 128;  // bytes of K per k-block = 64 bf16
-
-// Instruction descriptor, kind::f16: D = f32, A = B = bf16, both K-major, dense.
-__host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
-         (static_cast<uint32_t>(m >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 
 struct BfParams {
   const uint16_t* bias;
@@ -70,7 +57,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
-      mbar_init(&full[i], 1);
+      mbar_init(&full[i], 2);
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -96,27 +83,40 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   pdl_wait();  // the activations may come from the preceding kernel on the stream
 
   if (warp == 0) {
-    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
+    if (elect_one()) {  // see gemm_tc.cu: single-thread roles, activations and weights by a thread each
       Ring st;
       bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int n_blk = tile % p.n_tiles, m_row = (tile / p.n_tiles) * BM;
+        const int m_row = (tile / p.n_tiles) * BM;
         for (int kb = 0; kb < KB; ++kb) {
           if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
           Ring nx = st;
           nx.next(NS);
           free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);  // one k-block ahead
-          mbar_arrive_expect_tx(&full[st.s], A_BYTES + B_BYTES);
+          mbar_arrive_expect_tx(&full[st.s], A_BYTES);
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, kb * kBfBK, m_row, &full[st.s]);
-          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * kBfBK, n_blk * BN, &full[st.s]);
           st = nx;
         }
       }
-      if (!ok) {  // give copies still in flight a bounded time to land before the CTA exits
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) {
+      if (!ok) producer_drain();
+    }
+  } else if (warp == kBfWeightWarp) {
+    if (elect_one()) {
+      Ring st;
+      bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
+      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+        const int w_row = (tile % p.n_tiles) * BN;
+        for (int kb = 0; kb < KB; ++kb) {
+          if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
+          Ring nx = st;
+          nx.next(NS);
+          free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);
+          mbar_arrive_expect_tx(&full[st.s], B_BYTES);
+          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * kBfBK, w_row, &full[st.s]);
+          st = nx;
         }
       }
+      if (!ok) producer_drain();
     }
   } else if (warp == 1) {
     if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
@@ -239,13 +239,28 @@ int gemm_bf16_init_device() {
 int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* bias, int64_t M, int32_t N, int32_t K,
                      uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl) {
   if (M == 0) return DP_OK;
-  const int bn = N % 256 == 0 ? 256 : N % 128 == 0 ? 128 : 64;
+  int bn = 0, cg = 1, splits = 1;
+  gemm_pick_tile(M, N, 2 * K, 16, 0xA, 0, &bn, &cg, &splits);  // a k-block is 128 bytes here too
   CUtensorMap ta, tw;
   int st = gemm_encode_bytes_2d(&ta, x, static_cast<uint64_t>(K) * 2, static_cast<uint64_t>(M),
                                 static_cast<uint64_t>(ldx) * 2, kBfBK, BM);
   if (st != DP_OK) return st;
   st = gemm_encode_w_rows(&tw, w, static_cast<uint64_t>(K) * 2, static_cast<uint64_t>(N), kBfBK, bn, true);
   if (st != DP_OK) return st;
+  const int32_t m_tiles = static_cast<int32_t>((M + BM - 1) / BM), n_tiles = N / bn;
+  if (splits > 1) {
+    GemmParams g{};
+    g.bias = bias;
+    g.y = y;
+    g.ldy = ldy;
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.m_tiles = m_tiles;
+    g.n_tiles = n_tiles;
+    g.status = status;
+    return launch_gemm_split(ta, tw, g, true, splits, stream, pdl);
+  }
   BfParams p;
   p.bias = bias;
   p.y = y;
@@ -253,8 +268,8 @@ int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* 
   p.M = M;
   p.N = N;
   p.K = K;
-  p.m_tiles = static_cast<int32_t>((M + BM - 1) / BM);
-  p.n_tiles = N / bn;
+  p.m_tiles = m_tiles;
+  p.n_tiles = n_tiles;
   p.status = status;
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   const int sms = num_sms() > 0 ? num_sms() : 148;

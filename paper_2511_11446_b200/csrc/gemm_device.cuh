@@ -159,6 +159,9 @@ __device__ __forceinline__ void daq_sync_exit(const GemmParams& p) {
   }
 }
 
+int launch_gemm_split(const CUtensorMap& tmap_a, const CUtensorMap& tmap_w, GemmParams& p, bool f16, int splits,
+                      cudaStream_t stream, bool pdl);
+
 // A producer that gave up: copies still in flight get a bounded time to land before the CTA exits.
 __device__ __forceinline__ void producer_drain() {
   const long long t0 = clock64();

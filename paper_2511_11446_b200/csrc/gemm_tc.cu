@@ -363,7 +363,7 @@ int gemm_korder(int32_t bits) { return bits == 4 ? KORDER_EVEN_ODD : KORDER_NATU
 // First use of device `dev` (current; called under the library's device lock): the kernels'
 // shared-memory attributes, the SM count and how many CTA pairs of the widest pair kernel can be
 // resident at once.
-int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out) {
+int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out, int* max_clusters_out) {
   if (g_encode == nullptr) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -401,6 +401,8 @@ int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out) {
   int st = gemm_ws_init_device();
   if (st != DP_OK) return st;
   st = gemm_as_init_device();
+  if (st != DP_OK) return st;
+  st = gemm_split_init_device(max_clusters_out);
   if (st != DP_OK) return st;
   st = gemm_bf16_init_device();
   if (st != DP_OK) return st;
@@ -466,39 +468,60 @@ int gemm_encode_w(CUtensorMap* out, const void* qweight, int32_t N, int32_t K, i
 }
 
 // Tile shape: width from {256, 192, 128, 64} dividing N, rows 128 (one CTA) or 256 (a CTA pair), by a time model.
-// 8-bit operands: a fixed cost (prologue, first loads, last epilogue) plus, per wave of tiles over the SMs or
+// 8-bit operands (and 16-bit ones, whose K counts 128-byte blocks): a fixed cost (prologue, first loads, last epilogue) plus, per wave of tiles over the SMs or
 // pairs, the larger of the k-blocks' time and the least time a tile takes (its epilogue, when K is short). The
 // constants, in us, are a least-squares fit to 88 shapes (K = 384 .. 4608, N = 768 .. 4608, 48 .. 32768 tokens)
 // timed at every width: the choice is 0.4 % from the fastest on average, 6 % at worst. Fixed costs alone
 // say: narrow single tiles while a layer is one wave, wide pairs beyond.
 // Packed operands (expanded in the kernel): waves times width, pairs, which expand half, preferred.
-void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int* bn_out, int* cg_out) {
-  const int sms = num_sms() > 0 ? num_sms() : 148;
-  const int pairs = gemm_max_pairs() > 0 ? gemm_max_pairs() : sms / 2;
-  struct Form {
-    int bn, cg;
-    double fixed, per_kb, min_tile;
-  };
-  static const Form forms[] = {{256, 2, 2.39, 0.211, 1.16}, {192, 2, 1.91, 0.179, 1.03}, {128, 2, 1.47, 0.139, 0.89},
-                               {256, 1, 1.71, 0.313, 1.52}, {192, 1, 1.45, 0.235, 1.21}, {128, 1, 1.14, 0.182, 0.98},
-                               {64, 1, 0.86, 0.152, 0.76}};
-  int best_bn = 0, best_cg = 1;
+namespace {
+struct TileForm {
+  int bn, cg;
+  double fixed, per_kb, min_tile;
+};
+constexpr TileForm kTileForms[] = {{256, 2, 2.39, 0.211, 1.16}, {192, 2, 1.91, 0.179, 1.03}, {128, 2, 1.47, 0.139, 0.89},
+                                   {256, 1, 1.71, 0.313, 1.52}, {192, 1, 1.45, 0.235, 1.21}, {128, 1, 1.14, 0.182, 0.98},
+                                   {64, 1, 0.86, 0.152, 0.76}};
+double tile_cost(const TileForm& f, const GemmLimits& lim, int64_t M, int32_t N, int32_t K, int32_t bits, int* splits) {
+  const int64_t slots = f.cg == 2 ? lim.pairs : lim.sms;
+  const int64_t tiles = ((M + BM * f.cg - 1) / (BM * f.cg)) * (N / f.bn);
+  const double waves = static_cast<double>((tiles + slots - 1) / slots);
+  *splits = 1;
+  if (bits < 8) return waves * (f.bn + 24.0) * (f.cg == 2 ? 0.98 : 1.0);
+  double cost = f.fixed + waves * fmax(f.per_kb * (K / BK), f.min_tile);
+  if (f.bn == 64) {
+    double saved = 0.0;
+    *splits = gemm_split_factor(lim, tiles, K / BK, bits == 16 ? 0.8 * f.per_kb : f.per_kb, &saved);
+    cost -= saved;
+  }
+  return cost;
+}
+}  // namespace
+
+double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg) {
+  int splits;
+  for (const TileForm& f : kTileForms)
+    if (f.bn == bn && f.cg == cg) return tile_cost(f, gemm_limits(), M, N, K, 8, &splits);
+  return 1e30;
+}
+
+void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int forced_bn, int* bn_out, int* cg_out,
+                    int* splits_out) {
+  *bn_out = 0;
+  *cg_out = *splits_out = 1;
   double best_cost = 1e30;
-  for (const Form& f : forms) {
-    if (N % f.bn || !(allow & (1u << f.cg))) continue;
-    const int64_t tiles = ((M + BM * f.cg - 1) / (BM * f.cg)) * (N / f.bn);
-    const int64_t slots = f.cg == 2 ? pairs : sms;
-    const double waves = static_cast<double>((tiles + slots - 1) / slots);
-    const double cost = bits == 8 ? f.fixed + waves * fmax(f.per_kb * (K / BK), f.min_tile)
-                                  : waves * (f.bn + 24.0) * (f.cg == 2 ? 0.98 : 1.0);
+  const GemmLimits lim = gemm_limits();
+  for (const TileForm& f : kTileForms) {
+    if (N % f.bn || !(allow & (1u << f.cg)) || (f.bn == 192 && (allow & 0x8)) || (forced_bn != 0 && f.bn != forced_bn)) continue;
+    int splits;
+    const double cost = tile_cost(f, lim, M, N, K, bits, &splits);
     if (cost < best_cost) {
       best_cost = cost;
-      best_bn = f.bn;
-      best_cg = f.cg;
+      *bn_out = f.bn;
+      *cg_out = f.cg;
+      *splits_out = splits;
     }
   }
-  *bn_out = best_bn;
-  *cg_out = best_cg;
 }
 
 template <int BN, int CG>
@@ -587,6 +610,12 @@ int launch_gemm(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   p.early_w = (pdl && g.early_w) ? 1 : 0;
   p.status = g.status;
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
+  // (taps, in-kernel DAQ and the test hook belong to the unsplit kernel)
+  if (cg == 1 && g.bits == 8 && g.bn == 64 && g.dbg_acc == nullptr && g.x == nullptr && p.dbg_skip_kb < 0) {
+    int bn = 0, one = 1, splits = 1;
+    gemm_pick_tile(g.M, g.N, g.K, 8, 0x2, g.bn, &bn, &one, &splits);
+    if (splits > 1) return launch_gemm_split(g.tmap_a, g.tmap_w, p, false, splits, stream, pdl);
+  }
   const int64_t slots = cg == 2 ? (gemm_max_pairs() > 0 ? gemm_max_pairs() : num_sms() / 2) : num_sms();
   const dim3 grid(static_cast<unsigned>((tiles < slots ? tiles : slots) * cg));
   p.next = take_next_reads(grid.x);

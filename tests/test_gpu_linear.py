@@ -314,3 +314,20 @@ def test_default_dispatch_and_argument_errors():
         B.dp_wq_linear(L.w, xt, 1152, None, 200, y, 128, None, flags=B.DP_FLAG_FORCE_MMA)
     assert e.value.status == B.DP_ERR_WORKSPACE
     B.dp_wq_linear(L.w, xt, 1152, None, 0, y, 128, ws)   # M = 0: no-op
+
+
+@pytest.mark.parametrize("bits", [8, 3])
+@pytest.mark.parametrize("bn", [0, 64])
+@pytest.mark.parametrize("M,K,N", [(33, 4608, 1152), (128, 2304, 128), (129, 4608, 256), (300, 4608, 1152), (520, 4608, 1152),
+                                   (40, 3200, 64)])
+def test_mma_split_k(bits, bn, M, K, N):
+    """Layers with fewer tiles than SMs and many k-blocks (25 and 36: uneven shares too) run split along K
+    when no taps are asked for; ragged token counts, one and several tiles."""
+    if bn and N % bn:
+        pytest.skip("width does not divide N")
+    x, w, s_w, b = _case(M, K, N, bits)
+    flags = B.DP_FLAG_FORCE_MMA | (B.DP_FLAG_TILE_N(bn) | B.DP_FLAG_NO_CTA_PAIR if bn else 0)
+    out = run_linear(DevLayer(w, s_w, b, bits), x, flags=flags, taps=False)
+    assert out["status"] == 0
+    y, *_ = oracle.wq_linear(x, oracle.pack(w, bits), s_w, b, bits, taps=True)
+    assert np.array_equal(out["y"], y)

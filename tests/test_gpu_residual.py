@@ -60,6 +60,12 @@ def test_residual_in_place_dit_projection():
     _run(2048, 1152, 1152, 4, True, 1024, True, seed=7)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+def test_residual_split_k(in_place):
+    # few tiles, long K: the layer runs split along K
+    _run(200, 4608, 384, 8, True, 64, in_place, seed=11)
+
+
 def test_residual_argument_errors():
     dev = "cuda:0"
     M, K, N = 128, 128, 64
