@@ -1,4 +1,5 @@
-"""ctypes binding of libdiffpro.so — argument marshalling only.
+"""Binding of libdiffpro.so — argument marshalling only: ctypes, and for the per-layer calls, whose Python cost
+would show beside a kernel of a few microseconds, a small extension module (csrc/call.c).
 
 Every function has the name and argument order of its C entry point in ``include/diffpro.h``.
 torch tensors supply device memory and the current CUDA stream; every step of the quantized
@@ -136,6 +137,25 @@ def _stream(stream=None):
     return stream.cuda_stream
 
 
+_call = None
+
+
+def _calls():
+    """The extension module with the per-layer calls, bound to the library."""
+    global _call
+    if _call is None:
+        L = lib()
+        try:
+            from . import _call as m
+        except ImportError as e:
+            raise RuntimeError("the call module is missing: build it with `python -m paper_2511_11446_b200.build`") from e
+        addr = lambda f: C.cast(f, C.c_void_p).value
+        m.bind(addr(L.dp_wq_linear), addr(L.dp_wq_linear_residual), addr(L.dp_daq_quantize), addr(L.dp_ln_modulate_daq),
+               torch.cuda.current_device, torch._C._cuda_getCurrentRawStream)
+        _call = m
+    return _call
+
+
 def _check(st, where):
     if st != DP_OK:
         raise DiffproError(st, where)
@@ -148,8 +168,7 @@ def make_weight(qweight: torch.Tensor, s_w: torch.Tensor, bias, N: int, K: int, 
 
 
 def dp_daq_quantize(x, M, K, ldx, q, ldq, s_a, rowsum=None, stream=None):
-    _check(lib().dp_daq_quantize(_ptr(x), M, K, ldx, _ptr(q), ldq, _ptr(s_a), _ptr(rowsum),
-                                 _stream(stream)), "dp_daq_quantize")
+    _check((_call or _calls()).daq_quantize(x, M, K, ldx, q, ldq, s_a, rowsum, stream), "dp_daq_quantize")
 
 
 def dp_wq_linear_workspace(M, N, K, bits, flags=0) -> int:
@@ -176,16 +195,15 @@ def dp_daq_quantize_robust(x, M, K, ldx, q, ldq, s_a, rank, act_bits=8, rowsum=N
 
 def dp_wq_linear(w: dp_weight, x, ldx, s_a_in, M, y, ldy, workspace, dbg: dp_debug | None = None,
                  device_status=None, flags=0, stream=None):
-    ws_bytes = 0 if workspace is None else workspace.nbytes
-    _check(lib().dp_wq_linear(C.byref(w), _ptr(x), ldx, _ptr(s_a_in), M, _ptr(y), ldy, _ptr(workspace),
-                              ws_bytes, None if dbg is None else C.byref(dbg), _ptr(device_status),
-                              flags, _stream(stream)), "dp_wq_linear")
+    _check((_call or _calls()).wq_linear(C.addressof(w), x, ldx, s_a_in, M, y, ldy, workspace,
+                                         0 if dbg is None else C.addressof(dbg), device_status, flags, stream),
+           "dp_wq_linear")
 
 
 def dp_ln_modulate_daq(x, M, K, ldx, shift, scale, rows_per_sample, eps, q, ldq, s_a, stream=None):
     """LayerNorm + adaLN modulation + DAQ of bf16 tokens in one pass (shift, scale may both be None)."""
-    _check(lib().dp_ln_modulate_daq(_ptr(x), M, K, ldx, _ptr(shift), _ptr(scale), rows_per_sample, eps, _ptr(q), ldq,
-                                    _ptr(s_a), _stream(stream)), "dp_ln_modulate_daq")
+    _check((_call or _calls()).ln_modulate_daq(x, M, K, ldx, shift, scale, rows_per_sample, eps, q, ldq, s_a, stream),
+           "dp_ln_modulate_daq")
 
 
 class dp_residual(C.Structure):
@@ -196,9 +214,9 @@ def dp_wq_linear_residual(w: dp_weight, x, ldx, M, residual, ldr, gate, rows_per
                           device_status=None, flags=0, stream=None):
     """dp_wq_linear on bf16 activations with y = bf16(gate * lin + residual) (gate None: lin + residual)
     in the epilogue; residual may be y."""
-    r = dp_residual(residual.data_ptr(), ldr, None if gate is None else gate.data_ptr(), rows_per_gate)
-    _check(lib().dp_wq_linear_residual(C.byref(w), _ptr(x), ldx, M, C.byref(r), _ptr(y), ldy, _ptr(workspace),
-                                       ws_bytes, _ptr(device_status), flags, _stream(stream)), "dp_wq_linear_residual")
+    _check((_call or _calls()).wq_linear_residual(C.addressof(w), x, ldx, M, residual, ldr, gate, rows_per_gate, y, ldy,
+                                                  workspace, ws_bytes, device_status, flags, stream),
+           "dp_wq_linear_residual")
 
 
 def dp_wq_linear_static(w: dp_weight, x, ldx, M, y, ldy, device_status=None, flags=0, stream=None):

@@ -1,4 +1,5 @@
-"""Builds libdiffpro.so (and the input-generator and measurement-probe libraries) in-tree with nvcc for sm_100a.
+"""Builds libdiffpro.so (and the input-generator and measurement-probe libraries) in-tree with nvcc for sm_100a, and
+the binding's call module with the host compiler.
 
     python -m paper_2511_11446_b200.build [--force] [--verbose]
 
@@ -9,6 +10,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -23,6 +25,9 @@ SOURCES = ["api.cu", "daq.cu", "simt.cu", "gemm_tc.cu", "gemm_ws.cu", "gemm_as.c
 SYNTH_SOURCES = ["synth_cuda.cu"]
 PROBE_LIB = os.path.join(HERE, "libdpprobe.so")
 PROBE_SOURCES = ["peak.cu"]
+CALL_LIB = os.path.join(HERE, "_call.so")
+CALL_SOURCE = os.path.join(CSRC, "call.c")
+CC = os.environ.get("CC", "gcc")
 
 
 def _deps():
@@ -63,13 +68,22 @@ def _link(lib, sources, verbose):
     return lib
 
 
+def _call_module():
+    if _stale(CALL_LIB, [CALL_SOURCE] + _deps()):
+        subprocess.check_call([CC, "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], "-o",
+                               CALL_LIB, CALL_SOURCE])
+    return CALL_LIB
+
+
 def build(force: bool = False, verbose: bool = False):
     os.makedirs(OBJ, exist_ok=True)
     if force:
         for f in os.listdir(OBJ):
             os.remove(os.path.join(OBJ, f))
+        if os.path.exists(CALL_LIB):
+            os.remove(CALL_LIB)
     return (_link(LIB, SOURCES, verbose), _link(SYNTH_LIB, SYNTH_SOURCES, verbose),
-            _link(PROBE_LIB, PROBE_SOURCES, verbose))
+            _link(PROBE_LIB, PROBE_SOURCES, verbose), _call_module())
 
 
 if __name__ == "__main__":
