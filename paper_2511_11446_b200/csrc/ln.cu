@@ -15,16 +15,17 @@
 // h = fma(n, 1 + scale, shift) in fp32; DAQ of h as for bf16 inputs (absmax / 127, one rounding of
 // the exact product with fl(127 / absmax), half to even).
 //
-// One warp owns one token; the row stays in registers as bf16 (16-byte loads); h is recomputed for
-// the quantization pass only when the row is too long to keep it (same operations, same bits). Moves
-// DAQ's bytes (2 read + 1 written per element) but is bound by the double-precision additions of the
-// statistics (two per element; building the doubles with integer operations instead of the
-// conversion instruction was slower): 34 us at M = 32768, K = 1152 against 19 us for DAQ alone.
+// One to four warps own a token; the row stays in registers as bf16 (16-byte loads), then as fp32 h. Moves
+// DAQ's bytes (2 read + 1 written per element) but is bound by the double precision of the statistics: the
+// conversions (16 per clock and SM; building the doubles with integer operations was slower), two additions
+// per element, a division and a root per token. M = 2048, K = 1152 / 2304 / 4608: 4.6 / 9.0 / 15.1 us with one
+// warp, a single chain of additions and the modulation read after the statistics, 4.4 / 7.0 / 11.5 this way;
+// M = 32768, K = 1152: 42 -> 38 us against 19 for DAQ alone.
 #include "daq_device.cuh"
 
 namespace dp {
 
-constexpr int kLnWarps = 8;
+constexpr int kLnThreads = 128;
 
 struct LnArgs {
   const uint16_t* x;
@@ -57,41 +58,75 @@ __device__ __forceinline__ uint64_t ln_pair(uint32_t w, uint32_t sw, uint32_t hw
   return h;
 }
 
-template <int MAXV, bool MOD>
-__global__ void __launch_bounds__(kLnWarps * 32) ln_modulate_daq_kernel(const LnArgs a) {
+// RW warps share a row, MAXV = 16-byte vectors held per lane.
+template <int RW, int MAXV, bool MOD>
+__global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArgs a) {
+  constexpr int kRows = kLnThreads / 32 / RW, TPR = 32 * RW;
+  __shared__ double part1[kLnThreads / 32], part2[kLnThreads / 32];
+  __shared__ uint32_t part3[kLnThreads / 32];
   pdl_launch_dependents();
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kLnWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;  // row of the CTA, position in the row
+  const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + rw;
+  const bool live = row < a.M;
+  const int nvec = live ? a.K >> 3 : 0;
   pdl_wait();
-  if (row >= a.M) return;
-  const int nvec = a.K >> 3;
   const uint4* xr = reinterpret_cast<const uint4*>(a.x + row * a.ldx);
-  uint4 v[MAXV];
-#pragma unroll
-  for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
-    if (idx < nvec) ld_nc_u32x4(xr + idx, v[i]);
-    else v[i] = make_uint4(0, 0, 0, 0);
+  const uint4* shr = nullptr;
+  const uint4* scr = nullptr;
+  if constexpr (MOD) {
+    const int64_t sample = live ? row / a.rows_per_sample : 0;
+    shr = reinterpret_cast<const uint4*>(a.shift + sample * a.K);
+    scr = reinterpret_cast<const uint4*>(a.scale + sample * a.K);
   }
-  // ---- token statistics in double ----
-  double s1 = 0.0, s2 = 0.0;
+  uint4 v[MAXV], sh[MAXV], sc[MAXV];  // the modulation's vectors fly beside the row's
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    if (lane + 32 * i >= nvec) continue;  // (padding vectors are zero: nothing to add)
+    const int idx = lane + TPR * i;
+    v[i] = sh[i] = sc[i] = make_uint4(0, 0, 0, 0);
+    if (idx < nvec) {
+      ld_nc_u32x4(xr + idx, v[i]);
+      if constexpr (MOD) {
+        sh[i] = __ldg(shr + idx);
+        sc[i] = __ldg(scr + idx);
+      }
+    }
+  }
+  // ---- token statistics in double, even and odd elements apart (two chains of additions each) ----
+  double s1 = 0.0, s2 = 0.0, s1b = 0.0, s2b = 0.0;
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) {
+    if (lane + TPR * i >= nvec) continue;  // (padding vectors are zero: nothing to add)
     const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const double lo = static_cast<double>(bf16_lo(w[j])), hi = static_cast<double>(bf16_hi(w[j]));
       s1 = __dadd_rn(s1, lo);
-      s1 = __dadd_rn(s1, hi);
+      s1b = __dadd_rn(s1b, hi);
       s2 = __fma_rn(lo, lo, s2);
-      s2 = __fma_rn(hi, hi, s2);
+      s2b = __fma_rn(hi, hi, s2b);
     }
   }
+  s1 = __dadd_rn(s1, s1b);
+  s2 = __dadd_rn(s2, s2b);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     s1 = __dadd_rn(s1, __shfl_xor_sync(0xFFFFFFFFu, s1, o));
     s2 = __dadd_rn(s2, __shfl_xor_sync(0xFFFFFFFFu, s2, o));
+  }
+  if constexpr (RW > 1) {
+    if ((threadIdx.x & 31) == 0) {
+      part1[warp] = s1;
+      part2[warp] = s2;
+    }
+    __syncthreads();
+    s1 = part1[rw * RW];
+    s2 = part2[rw * RW];
+#pragma unroll
+    for (int w = 1; w < RW; ++w) {
+      s1 = __dadd_rn(s1, part1[rw * RW + w]);
+      s2 = __dadd_rn(s2, part2[rw * RW + w]);
+    }
   }
   const double kd = static_cast<double>(a.K);
   const double mean_d = __ddiv_rn(s1, kd);
@@ -99,44 +134,31 @@ __global__ void __launch_bounds__(kLnWarps * 32) ln_modulate_daq_kernel(const Ln
   if (var_d < 0.0) var_d = 0.0;
   const float mean = __double2float_rn(mean_d);
   const float rstd = __double2float_rn(__ddiv_rn(1.0, __dsqrt_rn(__dadd_rn(var_d, static_cast<double>(a.eps)))));
-  // ---- h and its absmax (kept in registers when the row is short enough, else recomputed below) ----
-  constexpr bool KEEP = MAXV <= 5;
-  const uint4* shr = nullptr;
-  const uint4* scr = nullptr;
-  if constexpr (MOD) {
-    const int64_t sample = row / a.rows_per_sample;
-    shr = reinterpret_cast<const uint4*>(a.shift + sample * a.K);
-    scr = reinterpret_cast<const uint4*>(a.scale + sample * a.K);
-  }
+  // ---- h and its absmax ----
   const uint64_t nmean2 = f32x2_pack(-mean, -mean), rstd2 = f32x2_pack(rstd, rstd), one2 = f32x2_pack(1.0f, 1.0f);
-  uint64_t hk[KEEP ? MAXV * 4 : 1];
-  auto h_of = [&](const int i, const int idx, uint64_t (&h)[4]) {
-    uint4 sh = make_uint4(0, 0, 0, 0), sc = sh;
-    if constexpr (MOD) {
-      sh = __ldg(shr + idx);
-      sc = __ldg(scr + idx);
-    }
-    h[0] = ln_pair<MOD>(v[i].x, sc.x, sh.x, nmean2, rstd2, one2);
-    h[1] = ln_pair<MOD>(v[i].y, sc.y, sh.y, nmean2, rstd2, one2);
-    h[2] = ln_pair<MOD>(v[i].z, sc.z, sh.z, nmean2, rstd2, one2);
-    h[3] = ln_pair<MOD>(v[i].w, sc.w, sh.w, nmean2, rstd2, one2);
-  };
+  uint64_t h[MAXV][4];
   uint32_t amax_bits = 0;  // |h| as an integer: ordered like the value for finite h
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
-    if (idx < nvec) {
-      uint64_t h[4];
-      h_of(i, idx, h);
+    if (lane + TPR * i >= nvec) continue;
+    h[i][0] = ln_pair<MOD>(v[i].x, sc[i].x, sh[i].x, nmean2, rstd2, one2);
+    h[i][1] = ln_pair<MOD>(v[i].y, sc[i].y, sh[i].y, nmean2, rstd2, one2);
+    h[i][2] = ln_pair<MOD>(v[i].z, sc[i].z, sh[i].z, nmean2, rstd2, one2);
+    h[i][3] = ln_pair<MOD>(v[i].w, sc[i].w, sh[i].w, nmean2, rstd2, one2);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        amax_bits = max(amax_bits, static_cast<uint32_t>(h[j]) & 0x7FFFFFFFu);
-        amax_bits = max(amax_bits, static_cast<uint32_t>(h[j] >> 32) & 0x7FFFFFFFu);
-        if constexpr (KEEP) hk[4 * i + j] = h[j];
-      }
+    for (int j = 0; j < 4; ++j) {
+      amax_bits = max(amax_bits, static_cast<uint32_t>(h[i][j]) & 0x7FFFFFFFu);
+      amax_bits = max(amax_bits, static_cast<uint32_t>(h[i][j] >> 32) & 0x7FFFFFFFu);
     }
   }
   amax_bits = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
+  if constexpr (RW > 1) {
+    if ((threadIdx.x & 31) == 0) part3[warp] = amax_bits;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < RW; ++w) amax_bits = max(amax_bits, part3[rw * RW + w]);
+  }
+  if (!live) return;
   const float amax = __uint_as_float(amax_bits);
   float sa = 0.0f, inv = 0.0f;
   if (!(amax < 7.888609052210118e-31f)) {  // 2^-100: below it the token is all-zero, as in the bf16 form
@@ -148,19 +170,12 @@ __global__ void __launch_bounds__(kLnWarps * 32) ln_modulate_daq_kernel(const Ln
   uint2* qrow = reinterpret_cast<uint2*>(a.q + row * a.ldq);
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
+    const int idx = lane + TPR * i;
     if (idx < nvec) {
-      uint64_t h[4];
-      if constexpr (KEEP) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = hk[4 * i + j];
-      } else {
-        h_of(i, idx, h);
-      }
       uint32_t p[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const uint64_t r = f32x2_fma(h[j], inv2, magic2);
+        const uint64_t r = f32x2_fma(h[i][j], inv2, magic2);
         p[j] = __byte_perm(static_cast<uint32_t>(r), static_cast<uint32_t>(r >> 32), 0x0040);  // two codes in the low bytes
       }
       qrow[idx] = make_uint2(__byte_perm(p[0], p[1], 0x5410), __byte_perm(p[2], p[3], 0x5410));
@@ -169,10 +184,12 @@ __global__ void __launch_bounds__(kLnWarps * 32) ln_modulate_daq_kernel(const Ln
   if (lane == 0) a.s_a[row] = sa;
 }
 
-template <int MAXV>
-static cudaError_t launch_ln_v(const LnArgs& a, dim3 grid, cudaStream_t stream, bool pdl) {
-  if (a.shift != nullptr) return launch(ln_modulate_daq_kernel<MAXV, true>, grid, dim3(kLnWarps * 32), 0, stream, pdl, a);
-  return launch(ln_modulate_daq_kernel<MAXV, false>, grid, dim3(kLnWarps * 32), 0, stream, pdl, a);
+template <int RW, int MAXV>
+static cudaError_t launch_ln_v(const LnArgs& a, cudaStream_t stream, bool pdl) {
+  constexpr int kRows = kLnThreads / 32 / RW;
+  const dim3 grid(static_cast<unsigned>((a.M + kRows - 1) / kRows));
+  if (a.shift != nullptr) return launch(ln_modulate_daq_kernel<RW, MAXV, true>, grid, dim3(kLnThreads), 0, stream, pdl, a);
+  return launch(ln_modulate_daq_kernel<RW, MAXV, false>, grid, dim3(kLnThreads), 0, stream, pdl, a);
 }
 
 int launch_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t ldx, const void* shift, const void* scale,
@@ -181,8 +198,14 @@ int launch_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t ldx, con
   if (M == 0) return DP_OK;
   LnArgs a{static_cast<const uint16_t*>(x), M, ldx, static_cast<int>(K), static_cast<const uint16_t*>(shift),
            static_cast<const uint16_t*>(scale), rows_per_sample, eps, q, ldq, s_a};
-  const dim3 grid(static_cast<unsigned>((M + kLnWarps - 1) / kLnWarps));
-  cudaError_t e = K <= 256 * 5 ? launch_ln_v<5>(a, grid, stream, pdl) : launch_ln_v<18>(a, grid, stream, pdl);
+  // As many warps to a row as leave a lane at most five vectors, one more thing than in plain quantization
+  // speaking for few: every warp of a row repeats the statistics' division and root in double. K = 1152, M = 64 /
+  // 2056 / 32768: one warp 2.4 / 4.5 / 38 us, two 2.3 / 4.4 / 46, four 2.0 / 5.4 / 62.
+  const cudaError_t e = M <= 512 && K <= 2048 ? launch_ln_v<4, 2>(a, stream, pdl)
+                        : K <= 256 * 5        ? launch_ln_v<1, 5>(a, stream, pdl)
+                        : K <= 512 * 3        ? launch_ln_v<2, 3>(a, stream, pdl)
+                        : K <= 1024 * 3       ? launch_ln_v<4, 3>(a, stream, pdl)
+                                              : launch_ln_v<4, 5>(a, stream, pdl);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "LayerNorm + DAQ launch failed: %s", cudaGetErrorString(e));
   return DP_OK;
 }

@@ -35,7 +35,9 @@ def _run(x, shift, scale, rps, ldq=None):
     return q.cpu().numpy(), sa.cpu().numpy(), (q, sa)
 
 
-@pytest.mark.parametrize("M,K,rps", [(2048, 1152, 256), (300, 1152, 77), (9, 64, 4), (1000, 4608, 256), (37, 1280, 1)])
+@pytest.mark.parametrize("M,K,rps", [(2048, 1152, 256), (300, 1152, 77), (9, 64, 4), (1000, 4608, 256), (37, 1280, 1),
+                                     (3, 2048, 2), (5, 2064, 2), (515, 1296, 64), (514, 1536, 64),
+                                     (513, 1552, 64), (6, 3088, 3)])
 @pytest.mark.parametrize("mod", [True, False])
 def test_codes_and_scales_match_the_oracle(M, K, rps, mod):
     x, shift, scale = _inputs(M, K, K % 97 + M % 13, rps)
