@@ -48,6 +48,7 @@ struct SimtArgs {
   const void* x;        // bf16 [M][ldx] or int8 [M][ldx] when s_a_in != nullptr
   int64_t ldx;
   const float* s_a_in;  // nullptr -> DAQ inside the kernel
+  int rows;  // tokens per CTA of the matrix-instruction form, 8 or 16 (set by the launch)
   int64_t M;
   int32_t N, K, bits;
   const void* qweight;

@@ -13,8 +13,7 @@
 // instructions (m16n8k32 with the tokens as the 16 rows and 8 output channels as the columns), and
 // the weights reach the SM as bulk asynchronous copies: eight consecutive weight rows are one
 // contiguous run of the packed matrix, which each warp streams through a private ring of
-// shared-memory stages (3- and 4-bit: one copy of eight whole rows per stage; 8-bit: one copy per
-// row and third of K; completion counted in bytes on the stage's mbarrier), so
+// shared-memory stages, one copy to a stage (completion counted in bytes on its mbarrier), so
 // HBM sees a few thousand long sequential streams and the bytes in flight do not depend on
 // registers. Lane (g, t) = (lane / 4, lane % 4) reads the units 4j + t of row g from the stage and
 // feeds them as B fragments: 8-bit codes as they are; packed 3- and 4-bit codes as UNSIGNED bytes
@@ -24,6 +23,14 @@
 // visit k in any order as long as both operands agree, the A fragments are the same units of tokens
 // g and g + 8 from shared memory, staged in the k order the masks produce (row pitch K + 16 keeps
 // those 128-bit reads conflict-free).
+//
+// A single layer of few tokens is a chain of latencies (launch, token, DAQ, contraction, store), not a stream: a
+// launch in a chain takes 2.3 us for K = 128, N = 64. K = 1152, N = 6912, one token: 4.7 -> 2.75 us at 4 bits,
+// 5.0 -> 3.1 at 3, 6.0 -> 3.0 at 8 (weights alone 0.5 to 1.2 at the copy rate); 16 tokens 8.5 -> 3.8, 32 tokens 9.0 -> 5.2.
+// Of that, with 4 bits and one token: the loads of a token all at once 4.7 -> 3.7 (load_token), blocks dealt out
+// to all SMs before a second warp of one takes any 3.7 -> 2.8; with 8 bits, one copy to a stage instead of 24
+// short ones 4.0 -> 3.0. Short code matters as well: a CTA runs it once, from a cold instruction cache (the
+// contraction as a loop of three units instead of nine written out: K = 128 2.5 -> 2.3 us).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -39,17 +46,13 @@ constexpr int kSimtLanesPerCh = 8;  // lanes sharing one output channel
 constexpr int kSimtChPerCta = kSimtWarps * (32 / kSimtLanesPerCh);
 constexpr int kSimtSlots = 5;       // units a lane holds per pass (K = 1152: 36 units / 8 lanes)
 // Matrix-instruction form (K <= kMmaMaxK).
-constexpr int kMmaMaxK = 1152;
+constexpr int kMmaMaxK = 1152;         // a token is kTokVec vectors a lane or fewer
 constexpr int kMmaWarps = 8;
 constexpr int kMmaRows = 16;          // tokens per CTA (the M of m16n8k32)
 constexpr int kMmaCh = 8;             // output channels per block (the N of m16n8k32)
 constexpr int kMmaMaxStages = 8;
 constexpr int kMmaRingBytes = 9600;   // per warp
-// 128-k steps per ring stage. Low-bit rows are short enough for a stage to hold eight whole rows,
-// which are contiguous in the packed matrix: one copy per stage. 8-bit rows go in thirds, one copy
-// per row, 16 bytes of padding per staged row so that the lanes' reads spread over all banks.
-template <int BITS> __host__ __device__ constexpr int mma_chunk_j() { return BITS == 8 ? 3 : 9; }
-constexpr int kMmaPitch8 = 3 * 128 + 16;
+constexpr int kMmaUnits = kMmaMaxK / 128;  // 32-code units of a row per lane, at most
 
 // Packed form of one unit (32 consecutive k of one weight row): BITS words.
 template <int BITS>
@@ -85,96 +88,117 @@ __device__ __forceinline__ void fetch_unit(const uint32_t* __restrict__ row, int
 //                  (3-bit: the fields at the same place of the four 3-byte periods of a packed unit).
 enum { ORDER_NATURAL = 0, ORDER_NIBBLE = 1, ORDER_PERIOD = 2 };
 
+// Codes 8i .. 8i + 7 of a token, put in that order: the eight bytes to store at 8i. Every lane takes part, lane l
+// with an i of l (mod 4): ORDER_PERIOD transposes bytes among the four lanes of a unit (codes 8p .. 8p + 7 go to
+// byte p of its eight words; byte stores in place of the two shuffles ran into two-way bank conflicts, 80 cycles
+// of the store port for a token of 1152).
 template <int ORDER>
-__device__ __forceinline__ void store_codes(int8_t* row, const int i, const uint2 v) {
+__device__ __forceinline__ uint2 arrange_codes(const uint2 v, const int lane) {
   if constexpr (ORDER == ORDER_NATURAL) {
-    reinterpret_cast<uint2*>(row)[i] = v;
+    return v;
   } else if constexpr (ORDER == ORDER_NIBBLE) {
-    reinterpret_cast<uint2*>(row)[i] = make_uint2(__byte_perm(v.x, v.y, 0x6420), __byte_perm(v.x, v.y, 0x7531));
-  } else {  // codes 8p .. 8p + 7 of a unit go to byte p of its eight words
-    uint8_t* unit = reinterpret_cast<uint8_t*>(row) + (i >> 2) * 32 + (i & 3);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      unit[4 * c] = static_cast<uint8_t>(v.x >> (8 * c));
-      unit[4 * (c + 4)] = static_cast<uint8_t>(v.y >> (8 * c));
-    }
+    return make_uint2(__byte_perm(v.x, v.y, 0x6420), __byte_perm(v.x, v.y, 0x7531));
+  } else {
+    const bool up = (lane & 2) != 0, odd = (lane & 1) != 0;
+    // lanes 0, 1 of the unit collect the first words of all four lanes, 2, 3 the second words
+    const uint32_t own = up ? v.y : v.x, got = __shfl_xor_sync(0xFFFFFFFFu, up ? v.x : v.y, 2);
+    const uint32_t lo = up ? got : own, hi = up ? own : got;  // of lanes (lane & 1) and (lane & 1) + 2
+    // even lanes the lower halves, odd lanes the upper ones
+    const uint32_t keep = __byte_perm(lo, hi, odd ? 0x7632 : 0x5410);
+    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, __byte_perm(lo, hi, odd ? 0x5410 : 0x7632), 1);
+    const uint32_t e = odd ? other : keep, o = odd ? keep : other;  // lanes 0 and 2, lanes 1 and 3
+    return make_uint2(__byte_perm(e, o, 0x6240), __byte_perm(e, o, 0x7351));
   }
 }
 
-// Token `warp` of this CTA -> int8 in shared memory, by one warp (rows `pitch` bytes apart), its
-// scale and (srs != nullptr) the sum of its codes: DAQ here (Step 3, Eq. "daq"), or a copy when the
-// caller passes quantized tokens.
-template <int ORDER = ORDER_NATURAL>
-__device__ __forceinline__ void stage_tokens(const SimtArgs& a, const int64_t m0, const int block_x,
-                                             int8_t* sq, const int pitch, float* ssa, const int warp,
-                                             int* srs = nullptr) {
+// Vectors base + lane + 32 j (eight elements each) of a token, zeros beyond its end and for rows that are not
+// there. The loads are predicated, not looped over the row: a loop leaves the lanes that have one vector fewer to a
+// remainder of one load at a time, and for K = 1152 those four round trips through L2 were the longest phase of
+// the kernel (K = 1152, N = 6912, 4-bit, a launch in a chain: M = 1 4.7 -> 3.7 us, M = 16 8.5 -> 5.8).
+constexpr int kTokVec = 5;
+__device__ __forceinline__ void load_token(const SimtArgs& a, const int64_t row, const int base,
+                                           uint4 (&v)[kTokVec]) {
+  const int first = base + (threadIdx.x & 31);
+  const int left = row < a.M ? (a.K >> 3) - first : 0;
+  if (a.s_a_in != nullptr) {
+    const uint2* src = reinterpret_cast<const uint2*>(static_cast<const int8_t*>(a.x) + row * a.ldx) + first;
+#pragma unroll
+    for (int j = 0; j < kTokVec; ++j) {
+      const uint2 c = 32 * j < left ? src[32 * j] : make_uint2(0, 0);
+      v[j].x = c.x;
+      v[j].y = c.y;
+    }
+  } else {
+    const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.x) + row * a.ldx) + first;
+#pragma unroll
+    for (int j = 0; j < kTokVec; ++j) v[j] = 32 * j < left ? src[32 * j] : make_uint4(0, 0, 0, 0);
+  }
+}
+
+// Token `slot` of this CTA (row m0 + slot) -> int8 in shared memory, by one warp (rows `pitch` bytes apart), its
+// scale and (srs != nullptr) the sum of its codes: DAQ here (Step 3, Eq. "daq"), or the codes as they are when the
+// caller passes quantized tokens. v: its first vectors (load_token), all there is of a token unless LONG.
+template <int ORDER, bool LONG>
+__device__ __forceinline__ void stage_token(const SimtArgs& a, const int64_t m0, const int block_x, int8_t* sq,
+                                            const int pitch, float* ssa, const int slot, uint4 (&v)[kTokVec],
+                                            int* srs = nullptr) {
   const int lane = threadIdx.x & 31;
-  const int K = a.K;
-  {
-    const int64_t row = m0 + warp;
-    int8_t* dst = sq + warp * pitch;
-    const int nvec = K >> 3;
-    const bool tap_q = block_x == 0 && row < a.M && a.dbg_q != nullptr;  // optional taps, written once per token
-    uint2* dq = tap_q ? reinterpret_cast<uint2*>(a.dbg_q + row * a.dbg_ldq) : nullptr;
-    int sum = 0;
-    if (row >= a.M) {
-      for (int i = lane; i < nvec; i += 32) reinterpret_cast<uint2*>(dst)[i] = make_uint2(0, 0);
-      if (lane == 0) ssa[warp] = 0.0f;
-    } else if (a.s_a_in != nullptr) {
-      const uint2* src = reinterpret_cast<const uint2*>(static_cast<const int8_t*>(a.x) + row * a.ldx);
-      for (int i = lane; i < nvec; i += 32) {
-        const uint2 v = src[i];
-        sum = __dp4a(static_cast<int>(v.x), 0x01010101, __dp4a(static_cast<int>(v.y), 0x01010101, sum));
-        store_codes<ORDER>(dst, i, v);
-        if (tap_q) dq[i] = v;
-      }
-      if (lane == 0) ssa[warp] = a.s_a_in[row];
-    } else {
-      const uint4* xr = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.x) + row * a.ldx);
-      uint32_t mx = 0;
-#pragma unroll 5
-      for (int i = lane; i < nvec; i += 32) {
-        uint4 v = xr[i];
-        mx = __vmaxu2(mx, v.x & 0x7FFF7FFFu);
-        mx = __vmaxu2(mx, v.y & 0x7FFF7FFFu);
-        mx = __vmaxu2(mx, v.z & 0x7FFF7FFFu);
-        mx = __vmaxu2(mx, v.w & 0x7FFF7FFFu);
-      }
-      mx = max(mx & 0xFFFFu, mx >> 16);
+  const int64_t row = m0 + slot;
+  const int nvec = a.K >> 3;
+  uint2* dst = reinterpret_cast<uint2*>(sq + slot * pitch);
+  if (row >= a.M) {
+    for (int i = lane; i < nvec; i += 32) dst[i] = make_uint2(0, 0);
+    if (lane == 0) {
+      ssa[slot] = 0.0f;
+      if (srs != nullptr) srs[slot] = 0;
+    }
+    return;
+  }
+  const bool codes = a.s_a_in != nullptr;
+  const bool tap_q = block_x == 0 && a.dbg_q != nullptr;  // optional taps, written once per token
+  uint2* dq = tap_q ? reinterpret_cast<uint2*>(a.dbg_q + row * a.dbg_ldq) : nullptr;
+  float sc, inv = 0.0f;
+  if (codes) {
+    sc = a.s_a_in[row];
+  } else {
+    uint32_t mx = 0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-      const float amax = __uint_as_float(mx << 16);
-      float sc = 0.0f, inv = 0.0f;
-      if (!(amax < 7.888609052210118e-31f)) {  // 2^-100
-        sc = __fdiv_rn(amax, 127.0f);
-        inv = __fdiv_rn(127.0f, amax);
-      }
-      const float magic = 12582912.0f;
-#pragma unroll 5
-      for (int i = lane; i < nvec; i += 32) {
-        uint4 v = xr[i];
-        const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-        uint32_t b[8];
+    for (int j = 0; j < kTokVec; ++j)
+      mx = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(mx, v[j].x), v[j].y), v[j].z), v[j].w);
+    if constexpr (LONG) {
+      for (int base = 32 * kTokVec; base < nvec; base += 32 * kTokVec) {
+        uint4 u[kTokVec];
+        load_token(a, row, base, u);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          b[2 * j] = __float_as_uint(__fmaf_rn(__uint_as_float(in[j] << 16), inv, magic)) & 0xFFu;
-          b[2 * j + 1] =
-              __float_as_uint(__fmaf_rn(__uint_as_float(in[j] & 0xFFFF0000u), inv, magic)) & 0xFFu;
-        }
-        const uint2 w = make_uint2(b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24),
-                                   b[4] | (b[5] << 8) | (b[6] << 16) | (b[7] << 24));
-        sum = __dp4a(static_cast<int>(w.x), 0x01010101, __dp4a(static_cast<int>(w.y), 0x01010101, sum));
-        store_codes<ORDER>(dst, i, w);
+        for (int j = 0; j < kTokVec; ++j)
+          mx = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(mx, u[j].x), u[j].y), u[j].z), u[j].w);
+      }
+    }
+    token_scale(__reduce_max_sync(0xFFFFFFFFu, max(mx & 0xFFFFu, mx >> 16)), sc, inv);
+  }
+  int sum = 0;
+  for (int base = 0;;) {
+#pragma unroll
+    for (int j = 0; j < kTokVec; ++j) {
+      const int i = base + lane + 32 * j;
+      const uint2 w = codes ? make_uint2(v[j].x, v[j].y) : quant_vec<false>(v[j], inv);
+      sum = __dp4a(static_cast<int>(w.x), 0x01010101, __dp4a(static_cast<int>(w.y), 0x01010101, sum));
+      const uint2 o = arrange_codes<ORDER>(w, lane);
+      if (i < nvec) {
+        dst[i] = o;
         if (tap_q) dq[i] = w;
       }
-      if (lane == 0) ssa[warp] = sc;
     }
-    if (srs != nullptr) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-      if (lane == 0) srs[warp] = sum;
-    }
-    if (block_x == 0 && row < a.M && a.dbg_sa != nullptr && lane == 0) a.dbg_sa[row] = ssa[warp];
+    if constexpr (!LONG) break;
+    base += 32 * kTokVec;
+    if (base >= nvec) break;
+    load_token(a, row, base, v);
+  }
+  if (srs != nullptr) sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+  if (lane == 0) {
+    ssa[slot] = sc;
+    if (srs != nullptr) srs[slot] = sum;
+    if (block_x == 0 && a.dbg_sa != nullptr) a.dbg_sa[row] = sc;
   }
 }
 
@@ -204,7 +228,9 @@ __device__ __forceinline__ void simt_linear_body(const SimtArgs& a, const int bl
   }
   if (a.early_w) pdl_wait();  // the tokens come from the preceding kernel on the stream
 
-  stage_tokens(a, m0, block_x, sq, K, ssa, warp);
+  uint4 tok[kTokVec];
+  load_token(a, m0 + warp, 0, tok);
+  stage_token<ORDER_NATURAL, true>(a, m0, block_x, sq, K, ssa, warp, tok);
   __syncthreads();
 
   // ---- contraction: passes of kSimtSlots units per lane ----
@@ -294,13 +320,15 @@ __device__ __forceinline__ void mma_m16n8k32_s8u8(int (&c)[4], uint32_t a0, uint
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Packed unit `unit` of a staged weight row.
+// Packed unit `unit` of a staged weight row. 8-bit rows are a multiple of 128 bytes apart, so the lanes of an odd
+// row take the two halves of a unit in the other order: every eight lanes then cover all banks.
 template <int BITS>
-__device__ __forceinline__ void stage_unit(const uint8_t* row, int unit, uint32_t (&pk)[BITS]) {
+__device__ __forceinline__ void stage_unit(const uint8_t* row, int unit, const bool odd, uint32_t (&pk)[BITS]) {
   if constexpr (BITS == 8) {
-    const uint4 u = reinterpret_cast<const uint4*>(row)[unit * 2], v = reinterpret_cast<const uint4*>(row)[unit * 2 + 1];
-    pk[0] = u.x; pk[1] = u.y; pk[2] = u.z; pk[3] = u.w;
-    pk[4] = v.x; pk[5] = v.y; pk[6] = v.z; pk[7] = v.w;
+    const uint4* p = reinterpret_cast<const uint4*>(row) + unit * 2;
+    const uint4 u = p[odd ? 1 : 0], v = p[odd ? 0 : 1];
+    pk[0] = odd ? v.x : u.x; pk[1] = odd ? v.y : u.y; pk[2] = odd ? v.z : u.z; pk[3] = odd ? v.w : u.w;
+    pk[4] = odd ? u.x : v.x; pk[5] = odd ? u.y : v.y; pk[6] = odd ? u.z : v.z; pk[7] = odd ? u.w : v.w;
   } else if constexpr (BITS == 4) {
     const uint4 u = reinterpret_cast<const uint4*>(row)[unit];
     pk[0] = u.x; pk[1] = u.y; pk[2] = u.z; pk[3] = u.w;
@@ -337,24 +365,21 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   uint8_t* ring = reinterpret_cast<uint8_t*>(bars + kMmaWarps * kMmaMaxStages);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  const int64_t m0 = static_cast<int64_t>(block_y) * kMmaRows;
-  const bool two = a.M - m0 > 8;  // tokens g + 8 exist
-  constexpr int CJ = mma_chunk_j<BITS>();
-  const int64_t rowbytes = (static_cast<int64_t>(K) * BITS) >> 3;
-  const int pitch = BITS == 8 ? kMmaPitch8 : static_cast<int>(rowbytes);  // of a staged row
-  const int stage = kMmaCh * pitch;
+  const int64_t m0 = static_cast<int64_t>(block_y) * a.rows;
+  const bool two = a.rows > 8 && a.M - m0 > 8;  // tokens g + 8 exist
+  const int rowbytes = (K * BITS) >> 3;
+  const int stage = kMmaCh * rowbytes;
   const int S = min(kMmaMaxStages, kMmaRingBytes / stage);
   uint64_t* bar = bars + warp * kMmaMaxStages;
   uint8_t* myring = ring + warp * kMmaRingBytes;
   const uint8_t* wbase = static_cast<const uint8_t*>(a.qweight);
   const int kj = K >> 7;
-  const int nc = (kj + CJ - 1) / CJ;  // 1 for the low-bit forms (K <= kMmaMaxK)
-  // 8-channel blocks of this warp: blk0, blk0 + stride, ... The grid is sized to one wave, so a warp
-  // streams several blocks back to back.
+  // 8-channel blocks of this warp: blk0, blk0 + stride, ... Every CTA's first warp has one before any CTA's
+  // second warp, so that a layer of few blocks is spread over all SMs.
   const int nblocks = a.N / kMmaCh;
   const int stride = grid_x * kMmaWarps;
-  const int blk0 = block_x * kMmaWarps + warp;
-  const int total = blk0 < nblocks ? ((nblocks - blk0 + stride - 1) / stride) * nc : 0;
+  const int blk0 = warp * grid_x + block_x;
+  const int total = blk0 < nblocks ? (nblocks - blk0 + stride - 1) / stride : 0;
 
   if (threadIdx.x == 0) *abort_flag = 0;
   if (lane == 0) {
@@ -365,35 +390,34 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   pdl_launch_dependents();
   if (!a.early_w) pdl_wait();
 
-  // Producer side of the ring (lane 0): item = (block, chunk); the copy of item i lands in stage i % S.
-  int f_it = 0, f_c = 0, f_blk = blk0, f_s = 0;
+  // Producer side of the ring (lane 0): block i of this warp lands in stage i % S.
+  int f_it = 0, f_blk = blk0, f_s = 0;
   auto issue = [&]() {
     if (f_it < total) {
-      const uint8_t* src = wbase + static_cast<int64_t>(f_blk) * kMmaCh * rowbytes;
-      uint8_t* dst = myring + f_s * stage;
-      if constexpr (BITS < 8) {
-        if (lane == 0) {
-          const uint32_t bytes = static_cast<uint32_t>(kMmaCh * rowbytes);
-          mbar_arrive_expect_tx(&bar[f_s], bytes);
-          bulk_load_1d(dst, src, bytes, &bar[f_s]);
-        }
-      } else {
-        // one copy per row: issued by eight lanes at once (a bulk copy costs its issuing thread
-        // 115-280 cycles; in sequence that was the longest phase of an 8-bit stage)
-        const uint32_t bytes = static_cast<uint32_t>(min(CJ, kj - f_c * CJ) * 128);
-        if (lane == 0) mbar_arrive_expect_tx(&bar[f_s], kMmaCh * bytes);
-        __syncwarp();
-        if (lane < kMmaCh)
-          bulk_load_1d(dst + lane * kMmaPitch8, src + f_c * (CJ * 128) + lane * rowbytes, bytes, &bar[f_s]);
+      if (lane == 0) {
+        mbar_arrive_expect_tx(&bar[f_s], static_cast<uint32_t>(stage));
+        bulk_load_1d(myring + f_s * stage, wbase + static_cast<int64_t>(f_blk) * stage, static_cast<uint32_t>(stage),
+                     &bar[f_s]);
       }
       ++f_it;
       if (++f_s == S) f_s = 0;
-      if (++f_c == nc) { f_c = 0; f_blk += stride; }
+      f_blk += stride;
     }
   };
+  // Weights and tokens are both in flight before either is waited for; the tokens first where they may be read at
+  // once (theirs is the longer way: DAQ follows).
+  uint4 tok[kMmaRows / kMmaWarps][kTokVec];
+  auto load_tokens = [&]() {
+    load_token(a, m0 + warp, 0, tok[0]);
+    if (two) load_token(a, m0 + warp + kMmaWarps, 0, tok[1]);
+  };
+  if (!a.early_w) load_tokens();
 #pragma unroll 1
-  for (int s = 0; s < S; ++s) issue();  // in flight across the prologue
-  if (a.early_w) pdl_wait();
+  for (int s = 0; s < S; ++s) issue();
+  if (a.early_w) {
+    pdl_wait();
+    load_tokens();
+  }
   // Scale and bias of channels 2t, 2t + 1: of the current block, and fetched one block ahead for the
   // next (a load issued at the top of the block it is needed in came back, under a saturated memory
   // system, a couple of thousand cycles later, and its first use stalled the warp for that long).
@@ -419,8 +443,12 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   };
   constexpr int ORDER = BITS == 4 ? ORDER_NIBBLE : BITS == 3 ? ORDER_PERIOD : ORDER_NATURAL;
   fetch_scales(blk0);  // of the first block: back by the time the tokens are staged
-  for (int r = warp; r < (two ? kMmaRows : kMmaRows / 2); r += kMmaWarps)
-    stage_tokens<ORDER>(a, m0, block_x, sq, qpitch, ssa, r, srs);
+#pragma unroll 1
+  for (int slot = warp; slot < (two ? kMmaRows : kMmaRows / 2); slot += kMmaWarps) {
+    stage_token<ORDER, false>(a, m0, block_x, sq, qpitch, ssa, slot, tok[0], srs);
+#pragma unroll
+    for (int j = 0; j < kTokVec; ++j) tok[0][j] = tok[1][j];  // (one copy of the code: it is executed once)
+  }
   __syncthreads();
 
   // One accumulator set per matrix instruction of a unit: consecutive instructions never wait on each
@@ -430,7 +458,7 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   int c[NC][4];
 #pragma unroll
   for (int i = 0; i < NC; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0;
-  int c_c = 0, c_blk = blk0, st = 0;
+  int c_blk = blk0, st = 0;
   uint32_t ph = 0;
   const int8_t* qrow = sq + g * qpitch + t * 32;
   auto epilogue = [&]() {
@@ -441,7 +469,7 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
       for (int h = 0; h < 2; ++h) {
         const int tok = g + 8 * h;
         const int64_t row = m0 + tok;
-        if (row < a.M) {
+        if (row < a.M && (h == 0 || two)) {
           const int i = 2 * h + e;
           // Packed weights enter as unsigned fields u = w + 2^(BITS-1), each set carrying its power of
           // two (the shifts are exact), so the sum of the tokens' codes comes off at the end.
@@ -467,7 +495,7 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
       h1 = *reinterpret_cast<const uint4*>(qu + 8 * qpitch + 16);
     }
     uint32_t pk[BITS];
-    stage_unit<BITS>(srow, u, pk);
+    stage_unit<BITS>(srow, u, (g & 1) != 0, pk);
     if constexpr (BITS == 8) {
       mma_m16n8k32_s8(c[0], l0.x, h0.x, l0.y, h0.y, pk[0], pk[1]);
       mma_m16n8k32_s8(c[1], l0.z, h0.z, l0.w, h0.w, pk[2], pk[3]);
@@ -509,35 +537,34 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   };
   int it = 0;
   for (; it < total; ++it) {
-    if (c_c == 0) {
-      take_scales();
-      fetch_scales(c_blk + stride);
-    }
+    take_scales();
+    fetch_scales(c_blk + stride);
     if (!mbar_wait(&bar[st], ph, abort_flag)) break;
-    const int nj = min(CJ, kj - c_c * CJ);
-    const uint8_t* srow = myring + st * stage + g * pitch;
-    const int8_t* qc = qrow + c_c * (CJ * 128);
-    if (nj == CJ && !two) {  // the common case, free of per-unit tests
+    const uint8_t* srow = myring + st * stage + g * rowbytes;
+    auto contract = [&](auto two_tag) {
+      int jj = 0;
+#pragma unroll 1
+      for (; jj + 3 <= kj; jj += 3) {
 #pragma unroll
-      for (int jj = 0; jj < CJ; ++jj) unit_step(srow, qc + jj * 128, 4 * jj + t, std::false_type{});
-    } else if (two) {
+        for (int e = 0; e < 3; ++e) unit_step(srow, qrow + (jj + e) * 128, 4 * (jj + e) + t, two_tag);
+      }
+#pragma unroll 1
+      for (; jj < kj; ++jj) unit_step(srow, qrow + jj * 128, 4 * jj + t, two_tag);
+    };
+    if (two) {
+      contract(std::true_type{});
+    } else if (kj == kMmaUnits) {  // K = 1152, up to 8 tokens: written out, 2.90 -> 2.74 us
 #pragma unroll
-      for (int jj = 0; jj < CJ; ++jj)
-        if (jj < nj) unit_step(srow, qc + jj * 128, 4 * jj + t, std::true_type{});
+      for (int jj = 0; jj < kMmaUnits; ++jj) unit_step(srow, qrow + jj * 128, 4 * jj + t, std::false_type{});
     } else {
-#pragma unroll
-      for (int jj = 0; jj < CJ; ++jj)
-        if (jj < nj) unit_step(srow, qc + jj * 128, 4 * jj + t, std::false_type{});
+      contract(std::false_type{});
     }
     __syncwarp();  // every lane has consumed the stage: refill it
     issue();
-    if (++c_c == nc) {
-      epilogue();
+    epilogue();
 #pragma unroll
-      for (int i = 0; i < NC; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0;
-      c_c = 0;
-      c_blk += stride;
-    }
+    for (int i = 0; i < NC; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0;
+    c_blk += stride;
     if (++st == S) { st = 0; ph ^= 1u; }
   }
   // A warp that gave up lets the copies it still has in flight land before the CTA may exit.
@@ -611,6 +638,7 @@ simt_group_kernel(SimtGroupArgs g) {
     a.s_a_in = g.sa_scratch + static_cast<int64_t>(layer) * g.M;
   }
   a.M = g.M;
+  a.rows = kMmaRows;
   a.N = g.N;
   a.K = g.K;
   a.bits = L.bits;
@@ -644,19 +672,22 @@ static size_t simt_smem_bytes(int32_t K) {
          sizeof(uint64_t) * kMmaWarps * kMmaMaxStages + static_cast<size_t>(kMmaWarps) * kMmaRingBytes;
 }
 
-// grid.x of the matrix-instruction form: all CTAs of the launch resident at once (one wave), each
-// warp walking its strided share of the 8-channel blocks.
+// grid.x of the matrix-instruction form: one CTA per SM while that gives every block a warp of its own, else all
+// CTAs that are resident at once (one wave), each warp walking its strided share of the blocks.
 template <typename Kern>
 static int mma_grid_x(Kern kern, size_t smem, int32_t N, int64_t other_ctas) {
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
-  const int64_t slots = static_cast<int64_t>(num_sms()) * per_sm;
-  const int64_t full = (N / kMmaCh + kMmaWarps - 1) / kMmaWarps;
-  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(full, slots / std::max<int64_t>(1, other_ctas))));
+  const int64_t sms = num_sms();
+  const int64_t blocks = N / kMmaCh;
+  const int64_t room = std::max<int64_t>(1, (blocks * other_ctas <= sms * kMmaWarps ? sms : sms * per_sm) / std::max<int64_t>(1, other_ctas));
+  return static_cast<int>(std::max<int64_t>(1, std::min(blocks, room)));
 }
 
 static_assert(kMmaWarps == kSimtWarps, "both forms launch kSimtWarps warps");
+static_assert(kMmaRingBytes >= kMmaCh * kMmaMaxK, "a stage holds eight whole rows of any bit width");
+static_assert(kMmaRows == 2 * kMmaWarps && kMmaMaxK <= 256 * kTokVec, "a warp holds its two tokens in registers");
 
 size_t simt_max_k() { return 16384; }
 
@@ -691,8 +722,8 @@ int launch_simt_group(const SimtGroupArgs& g, cudaStream_t stream, bool pdl) {
   SimtGroupArgs args = g;
   if (mma) {
     // One wave: the resident-CTA slots are shared out in proportion to the time a CTA of each
-    // bit-width needs per channel block (measured: the 8-bit form is bound by its copies, the 3-bit
-    // form by the expansion arithmetic), every layer getting at least one CTA.
+    // bit-width needs per channel block, every layer getting at least one CTA (8-bit between 1.4 and
+    // 1.75 measures the same, 2.0 and above slower: plan of 64 tokens 829 -> 833 us).
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, smem) != cudaSuccess || per_sm < 1)
       per_sm = 1;
@@ -725,7 +756,10 @@ int launch_simt_linear(const SimtArgs& a, cudaStream_t stream, bool pdl) {
   if (a.M == 0) return DP_OK;
   const size_t smem = simt_smem_bytes(a.K);
   const bool mma = simt_use_mma(a.K);
-  const int rows = mma ? kMmaRows : kSimtRows;
+  // Tokens per CTA: 8 (one to a warp) while that leaves a warp for each (block, token group), else 16, so that the
+  // weights are read once for twice the tokens. N = K = 1152, 4-bit: M = 9 3.6 -> 2.4 us, M = 32 3.4 -> 2.5 with
+  // groups of 8; N = 6912 M = 16 3.8 either way, and above it the second reading of the weights shows.
+  const int rows = mma && a.N / kMmaCh * ((a.M + 7) / 8) > static_cast<int64_t>(num_sms()) * kMmaWarps ? kMmaRows : kSimtRows;
   const int64_t m_groups = (a.M + rows - 1) / rows;
   dim3 grid((a.N + kSimtChPerCta - 1) / kSimtChPerCta, static_cast<unsigned>(m_groups));
   const dim3 block(kSimtWarps * 32);
@@ -741,6 +775,7 @@ int launch_simt_linear(const SimtArgs& a, cudaStream_t stream, bool pdl) {
   }
   if (mma) grid.x = mma_grid_x(kern, smem, a.N, m_groups);
   SimtArgs args = a;
+  args.rows = rows;
   if (!pdl) args.early_w = 0;
   cudaError_t e = launch(kern, grid, block, smem, stream, pdl, args);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "simt launch failed: %s", cudaGetErrorString(e));

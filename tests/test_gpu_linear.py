@@ -54,6 +54,18 @@ def test_simt_path(bits, M, K, N):
     _check(run_linear(L, x, flags=B.DP_FLAG_FORCE_SIMT), x, w, s_w, b, bits)
 
 
+@pytest.mark.parametrize("bits", [3, 4, 8])
+@pytest.mark.parametrize("codes", [False, True], ids=["bf16", "prequantized"])
+@pytest.mark.parametrize("M,K", [(1, 128), (7, 1024), (9, 1152), (17, 640), (3, 1280), (9, 1408), (33, 2688)])
+def test_simt_token_lengths(bits, codes, M, K):
+    """Tokens of the small-M kernel around the 1280 elements a warp holds in registers (matrix-instruction
+    form up to K = 1152, more than one pass over the token above 1280), one and two tokens to a warp."""
+    x, w, s_w, b = _case(M, K, 96, bits, full_range=True)
+    L = DevLayer(w, s_w, b, bits)
+    pre = oracle.daq(x)[:2] if codes else None
+    _check(run_linear(L, x, flags=B.DP_FLAG_FORCE_SIMT, prequant=pre), x, w, s_w, b, bits)
+
+
 @pytest.mark.parametrize("bits", [8, 4, 3])
 @pytest.mark.parametrize("M,K,N", [(128, 128, 64), (128, 256, 128), (256, 1152, 1152),
                                    (300, 1152, 384), (1000, 4608, 1152), (77, 384, 192),
