@@ -165,6 +165,7 @@ int launch_gemm_ws(const GemmProblem& p, cudaStream_t stream, bool pdl);
 // device by check_device() with that device current.
 int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out, int* max_clusters_out);
 int gemm_ws_init_device();
+int simt_init_device();
 int gemm_as_init_device();
 int gemm_bf16_init_device();
 int gemm_grp_init_device();

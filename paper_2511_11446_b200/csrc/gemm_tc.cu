@@ -400,6 +400,8 @@ int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out, int* max_clu
   }
   int st = gemm_ws_init_device();
   if (st != DP_OK) return st;
+  st = simt_init_device();
+  if (st != DP_OK) return st;
   st = gemm_as_init_device();
   if (st != DP_OK) return st;
   st = gemm_split_init_device(max_clusters_out);

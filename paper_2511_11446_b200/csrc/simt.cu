@@ -52,6 +52,7 @@ constexpr int kMmaRows = 16;          // tokens per CTA (the M of m16n8k32)
 constexpr int kMmaCh = 8;             // output channels per block (the N of m16n8k32)
 constexpr int kMmaMaxStages = 8;
 constexpr int kMmaRingBytes = 9600;   // per warp
+constexpr int kMmaCtasPerSm = 2;      // by registers (launch bounds) and by the rings, for every K
 constexpr int kMmaUnits = kMmaMaxK / 128;  // 32-code units of a row per lane, at most
 
 // Packed form of one unit (32 consecutive k of one weight row): BITS words.
@@ -577,7 +578,7 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
 }
 
 template <int BITS, bool MMA>
-__global__ void __launch_bounds__(kSimtWarps * 32, MMA ? 2 : 0)
+__global__ void __launch_bounds__(kSimtWarps * 32, MMA ? kMmaCtasPerSm : 0)
 simt_linear_kernel(SimtArgs a) {
   if constexpr (MMA) simt_mma_body<BITS>(a, blockIdx.x, blockIdx.y, gridDim.x);
   else simt_linear_body<BITS>(a, blockIdx.x, blockIdx.y);
@@ -619,7 +620,7 @@ daq_group_robust_kernel(SimtGroupArgs g) {
 }
 
 template <bool MMA>
-__global__ void __launch_bounds__(kSimtWarps * 32, MMA ? 2 : 0)
+__global__ void __launch_bounds__(kSimtWarps * 32, MMA ? kMmaCtasPerSm : 0)
 simt_group_kernel(SimtGroupArgs g) {
   SimtArgs a;
   int layer = blockIdx.z, block_x = blockIdx.x, grid_x = gridDim.x;
@@ -674,22 +675,36 @@ static size_t simt_smem_bytes(int32_t K) {
 
 // grid.x of the matrix-instruction form: one CTA per SM while that gives every block a warp of its own, else all
 // CTAs that are resident at once (one wave), each warp walking its strided share of the blocks.
-template <typename Kern>
-static int mma_grid_x(Kern kern, size_t smem, int32_t N, int64_t other_ctas) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, smem) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
+static int mma_grid_x(int32_t N, int64_t other_ctas) {
   const int64_t sms = num_sms();
   const int64_t blocks = N / kMmaCh;
-  const int64_t room = std::max<int64_t>(1, (blocks * other_ctas <= sms * kMmaWarps ? sms : sms * per_sm) / std::max<int64_t>(1, other_ctas));
+  const int64_t room = std::max<int64_t>(1, (blocks * other_ctas <= sms * kMmaWarps ? sms : sms * kMmaCtasPerSm) /
+                                                std::max<int64_t>(1, other_ctas));
   return static_cast<int>(std::max<int64_t>(1, std::min(blocks, room)));
 }
 
-static_assert(kMmaWarps == kSimtWarps, "both forms launch kSimtWarps warps");
 static_assert(kMmaRingBytes >= kMmaCh * kMmaMaxK, "a stage holds eight whole rows of any bit width");
+static_assert(kMmaCtasPerSm * (kMmaWarps * kMmaRingBytes + kMmaRows * (kMmaMaxK + 16) + 2048) <= 227 * 1024,
+              "kMmaCtasPerSm CTAs fit an SM's shared memory");
 static_assert(kMmaRows == 2 * kMmaWarps && kMmaMaxK <= 256 * kTokVec, "a warp holds its two tokens in registers");
 
 size_t simt_max_k() { return 16384; }
+
+// Once per device: the shared-memory limits of the kernels (a launch that set its own, and asked for the
+// occupancy, spent 0.24 us of host time on it: 3.72 -> 3.48 us a call).
+int simt_init_device() {
+  const int mma = static_cast<int>(simt_smem_bytes(kMmaMaxK)), dp4a = 227 * 1024;
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<3, true>, attr, mma));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<4, true>, attr, mma));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<8, true>, attr, mma));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_group_kernel<true>, attr, mma));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<3, false>, attr, dp4a));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<4, false>, attr, dp4a));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<8, false>, attr, dp4a));
+  DP_CUDA_OK(cudaFuncSetAttribute(simt_group_kernel<false>, attr, dp4a));
+  return DP_OK;
+}
 
 size_t simt_group_scratch_bytes(int64_t M, int32_t K, int32_t n_layers) {
   const size_t q = (static_cast<size_t>(n_layers) * M * K + 255) & ~static_cast<size_t>(255);
@@ -714,20 +729,12 @@ int launch_simt_group(const SimtGroupArgs& g, cudaStream_t stream, bool pdl) {
             static_cast<unsigned>(g.n_layers));
   const dim3 block(kSimtWarps * 32);
   void (*kern)(SimtGroupArgs) = mma ? simt_group_kernel<true> : simt_group_kernel<false>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return fail(DP_ERR_CUDA, "simt smem attribute: %s", cudaGetErrorString(e));
-  }
   SimtGroupArgs args = g;
   if (mma) {
     // One wave: the resident-CTA slots are shared out in proportion to the time a CTA of each
     // bit-width needs per channel block, every layer getting at least one CTA (8-bit between 1.4 and
     // 1.75 measures the same, 2.0 and above slower: plan of 64 tokens 829 -> 833 us).
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, smem) != cudaSuccess || per_sm < 1)
-      per_sm = 1;
-    const int64_t slots = std::max<int64_t>(g.n_layers, static_cast<int64_t>(num_sms()) * per_sm / m_groups);
+    const int64_t slots = std::max<int64_t>(g.n_layers, static_cast<int64_t>(num_sms()) * kMmaCtasPerSm / m_groups);
     const int full = (g.N / kMmaCh + kMmaWarps - 1) / kMmaWarps;
     double cost[kSimtGroupMax], total = 0.0;
     for (int l = 0; l < g.n_layers; ++l) {
@@ -768,12 +775,7 @@ int launch_simt_linear(const SimtArgs& a, cudaStream_t stream, bool pdl) {
                                                                           : simt_linear_kernel<3, true>;
   else kern = a.bits == 8 ? simt_linear_kernel<8, false> : a.bits == 4 ? simt_linear_kernel<4, false>
                                                                        : simt_linear_kernel<3, false>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return fail(DP_ERR_CUDA, "simt smem attribute: %s", cudaGetErrorString(e));
-  }
-  if (mma) grid.x = mma_grid_x(kern, smem, a.N, m_groups);
+  if (mma) grid.x = mma_grid_x(a.N, m_groups);
   SimtArgs args = a;
   args.rows = rows;
   if (!pdl) args.early_w = 0;
