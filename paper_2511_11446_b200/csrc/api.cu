@@ -204,6 +204,12 @@ static bool use_simt(int64_t M, int32_t N, int32_t K, uint32_t flags) {
 // (kept for kernels with alignment needs beyond check_weight's; none at present)
 static bool as_pointers_ok(const dp_weight*) { return true; }
 
+// Whether two bf16 ranges share memory (lengths in elements).
+static bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + 2 * static_cast<uintptr_t>(nb) && y < x + 2 * static_cast<uintptr_t>(na);
+}
+
 static int check_weight(const dp_weight* w) {
   if (!w) return fail(DP_ERR_INVALID_ARG, "dp_weight is NULL");
   if (w->bits != 3 && w->bits != 4 && w->bits != 8 && w->bits != 16)
@@ -235,7 +241,8 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
                       void* y, int64_t ldy, void* workspace, const dp_debug* dbg, int32_t* status,
                       uint32_t flags, cudaStream_t stream, const CUtensorMap* tmap_w, int bn, int cg, int ws,
                       const CUtensorMap* tmap_a_cached, bool chained, int32_t* daq_sync = nullptr,
-                      int pre = -1, int daq_rank = 1, int daq_bits = 8, const dp_residual* res = nullptr) {
+                      int pre = -1, int daq_rank = 1, int daq_bits = 8, const dp_residual* res = nullptr,
+                      bool ahead = false) {
   const bool pdl = !(flags & DP_FLAG_NO_PDL);
   if (w->bits == 16)  // a layer the plan keeps in 16-bit precision: no DAQ, no scales (checked by the caller)
     return launch_gemm_bf16(x, ldx, w->qweight, static_cast<const uint16_t*>(w->bias), M, w->N, w->K,
@@ -329,6 +336,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   dp_weight w8 = *w;
   UnpackJob job;
   job.early = chained && pdl;
+  job.ahead = ahead && job.early;
   if (unpack_first) {
     int8_t* dst = reinterpret_cast<int8_t*>(static_cast<uint8_t*>(workspace) + align256(scratch_q_bytes(M, w->K)) +
                                             align256(sizeof(float) * static_cast<size_t>(M)));
@@ -638,6 +646,7 @@ struct dp_plan {
   std::vector<PlanLayer> layers;
   uint32_t flags;
   size_t workspace_bytes;
+  size_t half_bytes;  // of the two halves that consecutive layers take in turn
   size_t x_bytes;
   std::vector<TmapACache> a_cache;
   std::vector<std::vector<int>> groups;  // small-M layers of equal shape, run first in every step
@@ -648,6 +657,10 @@ struct dp_plan {
   int32_t daq_p_e3, daq_timesteps, daq_bits[3];
   cudaStream_t copy_stream;
   cudaEvent_t ev_copied[2], ev_consumed[2], ev_entry;
+  void need(size_t layer_bytes) {  // room for a layer of this scratch size
+    half_bytes = std::max(half_bytes, align256(layer_bytes));
+    workspace_bytes = std::max(workspace_bytes, 2 * half_bytes);
+  }
 };
 
 // Times every kernel variant that can run this layer shape (the whole layer: DAQ + GEMM, as the
@@ -773,6 +786,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   if (!p) return fail(DP_ERR_CUDA, "out of host memory");
   p->flags = flags;
   p->workspace_bytes = 256;
+  p->half_bytes = 0;
   p->x_bytes = 0;
   p->copy_stream = nullptr;
   p->daq_sync = nullptr;
@@ -839,7 +853,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
                           : dp_wq_linear_workspace(L.M, L.w.N, L.w.K, L.w.bits,
                                                    (flags & ~(DP_FLAG_UNPACK_FIRST | DP_FLAG_NO_UNPACK_FIRST)) |
                                                        (L.pre ? DP_FLAG_UNPACK_FIRST : DP_FLAG_NO_UNPACK_FIRST));
-    if (ws > p->workspace_bytes) p->workspace_bytes = ws;
+    p->need(ws);
 
     L.x_offset = p->x_bytes;
     p->x_bytes += align256(static_cast<size_t>(L.M) * L.w.K * 2);
@@ -904,7 +918,7 @@ extern "C" int dp_plan_set_daq(dp_plan* plan, int32_t clip_percentile_e3, int32_
   for (int b = 0; b < 3 && n_timesteps > 0; ++b)
     if (act_bits_by_bin[b] < 2 || act_bits_by_bin[b] > 8)
       return fail(DP_ERR_BITS, "dp_plan_set_daq: activation bits %d not in [2, 8]", act_bits_by_bin[b]);
-  size_t need = plan->workspace_bytes;
+  size_t need = plan->half_bytes;
   for (const PlanLayer& L : plan->layers) {
     if (L.M == 0 || L.w.bits == 16 || L.w.group_size > 0) continue;  // no DAQ / scratch already sized for any rule
     const int rank = clip_rank_of(clip_percentile_e3, L.w.K);
@@ -916,7 +930,7 @@ extern "C" int dp_plan_set_daq(dp_plan* plan, int32_t clip_percentile_e3, int32_
     if (!L.simt && L.w.bits < 8) ws += align256(static_cast<size_t>(L.w.N) * L.w.K);
     if (ws > need) need = ws;
   }
-  plan->workspace_bytes = need;
+  plan->need(need);
   plan->daq_p_e3 = clip_percentile_e3;
   plan->daq_timesteps = n_timesteps;
   for (int b = 0; b < 3; ++b) plan->daq_bits[b] = n_timesteps > 0 ? act_bits_by_bin[b] : 8;
@@ -950,7 +964,7 @@ extern "C" int dp_plan_set_layer_flags(dp_plan* plan, int32_t layer, uint32_t fl
   L = T;
   const size_t ws = dp_wq_linear_workspace(L.M, L.w.N, L.w.K, L.w.bits,
                                            L.pre ? DP_FLAG_UNPACK_FIRST : DP_FLAG_NO_UNPACK_FIRST);
-  if (ws > plan->workspace_bytes) plan->workspace_bytes = ws;
+  plan->need(ws);
   return DP_OK;
 }
 extern "C" int dp_plan_layer_unpack_first(const dp_plan* plan, int32_t layer, int32_t* unpack_first) {
@@ -1001,8 +1015,20 @@ static const CUtensorMap* cached_tmap_a(dp_plan* plan, const void* ws, int64_t M
   return &plan->a_cache.back().map;
 }
 
+// What a call has launched so far.
+struct PlanRun {
+  bool chained = false;  // something
+  int half = 0;          // half of the workspace that the next layer takes
+  const void* y = nullptr;  // outputs of the launch before, if that is a tensor-core GEMM: it may still be running when the
+  int64_t y_elems = 0;      // next launch starts, but then nothing before it is (it lets the next one start after its own wait)
+};
+
+// DAQ (and weight expansion) of a layer runs beside the GEMM of the layer before: it reads only the layer's own input
+// and weights and writes the half of the workspace that that GEMM does not read. Not so where the input overlaps that GEMM's
+// output. Steps of 28 DiT blocks, mixed bits, 256 / 2048 tokens: 915 -> 774 / 1559 -> 1350 us; 1024 tokens with
+// the percentile rule 1385 -> 1244.
 static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* const* ys, void* workspace,
-                         int32_t* status, cudaStream_t stream, bool* chained) {
+                         int32_t* status, cudaStream_t stream, PlanRun* run) {
   const int n = static_cast<int>(plan->layers.size());
   // DAQ policy of this step: the activation bits of the time bin t falls into (thirds of the range)
   int act_bits = 8;
@@ -1021,7 +1047,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     ga.N = G.w.N;
     ga.K = G.w.K;
     ga.n_layers = static_cast<int32_t>(grp.size());
-    ga.early_w = *chained ? 1 : 0;
+    ga.early_w = run->chained ? 1 : 0;
     ga.status = status;
     ga.daq_rank = robust ? clip_rank_of(plan->daq_p_e3, G.w.K) : 1;
     ga.daq_bits = act_bits;
@@ -1043,17 +1069,21 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     }
     int st = launch_simt_group(ga, stream, !(plan->flags & DP_FLAG_NO_PDL));
     if (st != DP_OK) return st;
-    *chained = true;
+    run->chained = true;
+    run->y = nullptr;
   }
   for (int l = 0; l < n; ++l) {
     const PlanLayer& L = plan->layers[l];
     if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
     if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", l);
     if (!aligned16(xs[l]) || !aligned16(ys[l])) return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", l);
+    uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->half * plan->half_bytes;
+    const bool ahead = run->y != nullptr && plan->daq_sync == nullptr &&
+                       !overlap(xs[l], L.M * L.w.K, run->y, run->y_elems);
     const CUtensorMap* ta = nullptr;
     if (!L.simt && L.w.bits != 16 && L.w.group_size == 0) {
       int st = DP_OK;
-      ta = cached_tmap_a(plan, workspace, L.M, L.w.K, &st);
+      ta = cached_tmap_a(plan, scratch, L.M, L.w.K, &st);
       if (st != DP_OK) return st;
     }
     // The next tensor-core layer's packed weights and its input start towards L2 while this layer's
@@ -1070,13 +1100,16 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
       if (!Nx.simt && xs[j] != nullptr) gemm_set_next_reads(Nx.w.qweight, wb, xb <= (32u << 20) ? xs[j] : nullptr, xb);
       break;
     }
-    int st = run_linear(&L.w, xs[l], L.w.K, nullptr, L.M, ys[l], L.w.N, workspace, nullptr, status,
-                        plan->flags, stream, L.simt ? nullptr : &L.tmap_w, L.bn, L.cg, L.ws, ta, *chained,
+    int st = run_linear(&L.w, xs[l], L.w.K, nullptr, L.M, ys[l], L.w.N, scratch, nullptr, status,
+                        plan->flags, stream, L.simt ? nullptr : &L.tmap_w, L.bn, L.cg, L.ws, ta, run->chained,
                         L.simt ? nullptr : plan->daq_sync, L.simt ? 0 : L.pre,
-                        robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits);
+                        robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead);
     gemm_set_next_reads(nullptr, 0, nullptr, 0);
     if (st != DP_OK) return st;
-    *chained = true;
+    run->chained = true;
+    run->half ^= 1;
+    run->y = !L.simt && L.w.group_size == 0 ? ys[l] : nullptr;
+    run->y_elems = L.M * L.w.N;
   }
   return DP_OK;
 }
@@ -1102,11 +1135,11 @@ extern "C" int dp_plan_run(const dp_plan* plan_c, const int32_t* steps, int32_t 
   if (st != DP_OK) return st;
   dp_plan* plan = const_cast<dp_plan*>(plan_c);
   const int64_t n = static_cast<int64_t>(plan->layers.size());
-  bool chained = false;
+  PlanRun run;
   for (int32_t i = n_steps - 1 - start_index; i >= 0; --i) {  // reverse(K*)
     const void* const* xs = x_ptrs + ((flags & DP_PLAN_SAME_X) ? 0 : i * n);
     void* const* ys = y_ptrs + ((flags & DP_PLAN_SAME_Y) ? 0 : i * n);
-    st = plan_run_step(plan, steps[i], xs, ys, workspace, device_status, static_cast<cudaStream_t>(stream), &chained);
+    st = plan_run_step(plan, steps[i], xs, ys, workspace, device_status, static_cast<cudaStream_t>(stream), &run);
     if (st != DP_OK) return st;
   }
   return DP_OK;
@@ -1149,8 +1182,8 @@ extern "C" int dp_plan_run_host(const dp_plan* plan_c, const int32_t* steps, int
     }
     DP_CUDA_OK(cudaEventRecord(plan->ev_copied[h], plan->copy_stream));
     DP_CUDA_OK(cudaStreamWaitEvent(stream, plan->ev_copied[h], 0));
-    bool chained = false;  // an event wait precedes every step's first launch
-    st = plan_run_step(plan, steps[i], xs.data(), y_dev, workspace, device_status, stream, &chained);
+    PlanRun run;  // an event wait precedes every step's first launch
+    st = plan_run_step(plan, steps[i], xs.data(), y_dev, workspace, device_status, stream, &run);
     if (st != DP_OK) return st;
     DP_CUDA_OK(cudaEventRecord(plan->ev_consumed[h], stream));
     if (d2h_layer >= 0) {

@@ -20,6 +20,10 @@ __device__ __forceinline__ void daq_begin(const UnpackJob& job) {
   if (!job.early) pdl_wait();
   pdl_launch_dependents();
 }
+// The end of a launch's first CTA.
+__device__ __forceinline__ void daq_end(const UnpackJob& job) {
+  if (job.ahead && blockIdx.x == 0) pdl_wait();
+}
 
 // RW warps share a row: MAXV = 16-byte vectors held per lane (a row of up to 256 * RW * MAXV elements in
 // registers). SUM: also the row's code sum.
@@ -36,7 +40,7 @@ daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
-  pdl_wait();
+  if (!job.ahead) pdl_wait();
   const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;  // row of the CTA, position in the row
   const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + rw;
   const bool live = row < M;
@@ -94,6 +98,7 @@ daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
     }
     if (lane == 0 && live) rowsum[row] = sum;
   }
+  daq_end(job);
 }
 
 // Any K (multiple of 8): two passes over the row, the second served by L1/L2.
@@ -109,7 +114,7 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
-  pdl_wait();
+  if (!job.ahead) pdl_wait();
   if (row >= M) return;
   const int nvec = K >> 3;
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
@@ -134,6 +139,7 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
     sum = warp_sum_i32(sum);
     if (lane == 0) rowsum[row] = sum;
   }
+  daq_end(job);
 }
 
 // ---- DAQ with a percentile clip and a-bit codes: robust_row in daq_device.cuh, one warp per token ----
@@ -149,7 +155,7 @@ daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
-  pdl_wait();
+  if (!job.ahead) pdl_wait();
   if (row >= M) return;
   const QRow qr(q, row, ldq, tiled_kb);
   float sc;
@@ -160,6 +166,7 @@ daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t
     sum = warp_sum_i32(sum);
     if (lane == 0) rowsum[row] = sum;
   }
+  daq_end(job);
 }
 
 __global__ void __launch_bounds__(kDaqWarps * 32)

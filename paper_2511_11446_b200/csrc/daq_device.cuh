@@ -300,8 +300,8 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t
 }
 
 // CTA `block` of an unpack job: one thread per unit of 32 codes (12 or 16 bytes in, 32 bytes out). Executes
-// griddepcontrol.wait before it writes (the destination may still be read by the preceding kernel) and,
-// unless job.early, before it reads.
+// griddepcontrol.wait before it writes (the destination may still be read by the preceding kernel; not with
+// job.ahead) and, unless job.early, before it reads.
 __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int block) {
   const int64_t u = static_cast<int64_t>(block) * blockDim.x + threadIdx.x;
   if (!job.early) pdl_wait();
@@ -322,7 +322,7 @@ __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int blo
       expand_unit<3>(pk, w, z);
     }
   }
-  if (job.early) pdl_wait();
+  if (job.early && !job.ahead) pdl_wait();
   if (u < job.units)
     st_global_v8(reinterpret_cast<uint4*>(job.out) + u * 2, w);  // 32 bytes, read next by the GEMM through L2
 }

@@ -28,6 +28,8 @@ struct UnpackJob {
   int32_t first_block = 0;  // filled by the launcher: CTAs from here on unpack
   int32_t early = 0;        // the preceding kernel on the stream is of the same call, so it cannot be writing
                             // `packed` or `zeros`: they are read before it has finished
+  int32_t ahead = 0;        // (with early) nor x, nor reading the destinations: the whole launch runs beside it. One CTA
+                            // stays until it has finished, so that whatever waits for this launch waits for both
   const uint8_t* zeros = nullptr;  // group-wise zero-points [N][row_units / group_units], or null (symmetric)
   int32_t row_units = 0, group_units = 0;
 };

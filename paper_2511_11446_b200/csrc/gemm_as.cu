@@ -95,7 +95,6 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  pdl_launch_dependents();
   if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
 
   if (warp == 0) {
@@ -210,6 +209,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     bool ok = true;
     int g = 0;
     pdl_wait();  // s_a is written by the preceding kernel
+    pdl_launch_dependents();  // as in gemm_tc.cu
     for (int u = unit0; u < unit1 && ok; ++u) {
       const int strip = u / ap.n_slices, slice = u - strip * ap.n_slices;
       for (int sub = 0; sub < ap.nsub && ok; ++sub, ++g) {

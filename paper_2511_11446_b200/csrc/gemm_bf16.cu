@@ -78,9 +78,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  pdl_launch_dependents();
   if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
   pdl_wait();  // the activations may come from the preceding kernel on the stream
+  pdl_launch_dependents();  // as in gemm_tc.cu
 
   if (warp == 0) {
     if (elect_one()) {  // see gemm_tc.cu: single-thread roles, activations and weights by a thread each

@@ -80,7 +80,6 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
   const uint32_t tmem_base = *tmem_slot;
   cluster_arrive_relaxed();  // this CTA has started; waited for before its shared memory is written from outside
 
-  pdl_launch_dependents();
   if (threadIdx.x == 96) prefetch_next_reads(p.next);
   if (!p.early_w) pdl_wait();
 
@@ -145,6 +144,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
       s_bias[et] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + et)) << 16) : 0.0f;
     }
     if (p.early_w) pdl_wait();  // s_a is written by the preceding kernel
+    pdl_launch_dependents();  // as in gemm_tc.cu
     if constexpr (!F16) {
       if (et >= 128) s_sa[et - 128] = m_row + et - 128 < p.M ? __ldg(p.s_a + m_row + et - 128) : 0.0f;
     }

@@ -106,7 +106,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  pdl_launch_dependents();
   if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);  // an epilogue thread: idle until the first accumulators
   // Activations and their scales come from the preceding kernel on the stream: the roles that read
   // them wait for it (griddepcontrol.wait) right before their first such read. Weights are
@@ -290,6 +289,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     bool ok = true;
     int tcount = 0;
     if (p.early_w && p.x == nullptr) pdl_wait();  // s_a is written by the preceding kernel
+    pdl_launch_dependents();  // only now that everything before this launch has finished: see plan_run_step
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride, ++tcount) {
       const int buf = tcount & 1;
       ok = epi.template tile<RES>(p, (tile % p.n_tiles) * BN + col0, NCOLS,

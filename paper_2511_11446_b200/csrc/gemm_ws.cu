@@ -93,7 +93,6 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  pdl_launch_dependents();
   if (threadIdx.x == kEpiWarp0 * 32) prefetch_next_reads(p.next);
   if (!p.early_w) pdl_wait();
 
@@ -233,6 +232,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     bool ok = true;
     int tcount = 0;
     if (p.early_w && p.x == nullptr) pdl_wait();  // s_a is written by the preceding kernel
+    pdl_launch_dependents();  // as in gemm_tc.cu
     for (int item = item0; item < item1 && ok; ++item, ++tcount) {
       const int buf = tcount & 1;
       ok = epi.tile(p, strip_of(item) * BN + col0, NCOLS, mtile_of(item) * (BM * CG) + static_cast<int>(rank) * BM,

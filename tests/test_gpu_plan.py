@@ -389,3 +389,56 @@ def test_chained_layers_whose_input_is_an_earlier_output():
                     assert np.array_equal(bf16_to_np(yd[i][l]), want[i][l]), (rep, i, l)
     finally:
         B.dp_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("M", [64, 300, 2048])
+@pytest.mark.parametrize("feed", ["given", "previous_output", "slice_of_previous_output"])
+def test_plan_layers_beside_each_other(M, feed):
+    """DAQ of a layer runs beside the GEMM before it unless its input is that GEMM's output (whole, or a part of it):
+    ten steps over layers of every weight width give the bits of the layers called one by one."""
+    D = 384
+    bits = [8, 4, 3, 16, 8, 8, 3, 4]
+    dev, Ms = [], []
+    for l, b in enumerate(bits):
+        bias = synth.bias(SEED, l, D)
+        if b == 16:
+            rng = np.random.default_rng(l)
+            wt = torch.from_numpy((rng.standard_normal((D, D)) * 0.05).astype(np.float32)).bfloat16().cuda()
+            bt = to_dev_bf16(bias)
+            dev.append((B.make_weight(wt, bt, bt, D, D, 16), wt, bt))  # (no scales: that pointer is not read)
+        else:
+            w, s_w = synth.weights(SEED, l, D, D, b)
+            layer = DevLayer(w, s_w, bias, b)
+            dev.append((layer.w, layer, None))
+        Ms.append(M if l % 3 else M // 2)
+    x0 = [to_dev_bf16(synth.activations(SEED, l, 0, M, D, 1.0, n_out=4)) for l in range(len(bits))]
+    plan = B.dp_plan_create([d[0] for d in dev], Ms)
+    try:
+        ws = torch.empty(B.dp_plan_workspace(plan), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        outs = []
+        for one_by_one in (True, False):
+            ys = [torch.zeros(M, D, dtype=torch.bfloat16, device="cuda") for _ in bits]
+            xs = list(x0)
+            for l in range(1, len(bits)):
+                if feed == "previous_output":
+                    xs[l] = ys[l - 1]
+                elif feed == "slice_of_previous_output" and Ms[l] < M:
+                    xs[l] = ys[l - 1][M - Ms[l]:]
+            torch.cuda.synchronize()
+            if one_by_one:
+                for l, b in enumerate(bits):
+                    lw = torch.empty(max(256, B.dp_wq_linear_workspace(Ms[l], D, D, b)), dtype=torch.uint8, device="cuda")
+                    B.dp_wq_linear(dev[l][0], xs[l], D, None, Ms[l], ys[l], D, lw, None, status)
+                    torch.cuda.synchronize()
+            else:
+                B.dp_plan_run(plan, list(range(10)), 0, B.ptr_array([t.data_ptr() for t in xs]),
+                              B.ptr_array([t.data_ptr() for t in ys]), ws, status,
+                              flags=B.DP_PLAN_SAME_X | B.DP_PLAN_SAME_Y)
+                torch.cuda.synchronize()
+            outs.append([t.view(torch.int16).cpu() for t in ys])
+        assert int(status.item()) == 0
+        for l, (a, b) in enumerate(zip(*outs)):
+            assert torch.equal(a, b), (l, bits[l])
+    finally:
+        B.dp_plan_destroy(plan)
