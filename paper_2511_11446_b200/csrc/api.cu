@@ -122,8 +122,6 @@ static int forced_bn(uint32_t flags) { return static_cast<int>((flags & DP_FLAG_
 static void choose_tile(uint32_t flags, int64_t M, int32_t N, int32_t K, int32_t bits, bool tiled_a, int* bn,
                         int* cg, int* ws) {
   *ws = 0;
-  // (callers clear tiled_a when the layer's scale / bias pointers lack the alignment that kernel's
-  // vector loads need)
   const bool as_ok = tiled_a && bits == 8 && gemm_as_supported(N, K) &&
                      !(flags & (DP_FLAG_NO_ACT_STATIONARY | DP_FLAG_NO_CTA_PAIR | DP_FLAG_WEIGHT_STATIONARY));
   if (as_ok && (flags & DP_FLAG_ACT_STATIONARY)) {
@@ -200,9 +198,6 @@ static bool use_simt(int64_t M, int32_t N, int32_t K, uint32_t flags) {
   (void)K;
   return M <= kSimtMaxRows;
 }
-
-// (kept for kernels with alignment needs beyond check_weight's; none at present)
-static bool as_pointers_ok(const dp_weight*) { return true; }
 
 // Whether two bf16 ranges share memory (lengths in elements).
 static bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
@@ -398,8 +393,8 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     int st = tiled ? gemm_encode_a_tiled(&g.tmap_a, q, M, w->K) : gemm_encode_a(&g.tmap_a, q, M, w->K, ldq);
     if (st != DP_OK) return st;
   }
-  if (bn == 0) choose_tile(flags, M, w->N, w->K, w->bits, tiled && as_pointers_ok(w), &bn, &cg, &ws);
-  if (ws == 2 && (!tiled || w->bits != 8 || fused || !as_pointers_ok(w)))
+  if (bn == 0) choose_tile(flags, M, w->N, w->K, w->bits, tiled, &bn, &cg, &ws);
+  if (ws == 2 && (!tiled || w->bits != 8 || fused))
     return fail(DP_ERR_INVALID_ARG, "the activation-stationary kernel needs DAQ run by the call, 8-bit weights (or the "
                                     "unpack-first form)");
   // Its weight ring is small (64 KB per CTA): prefetching it while the DAQ launch drains costs that
@@ -691,7 +686,7 @@ static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool al
         if (!eight || gemm_tile_cost(M, w.N, w.K, widths[i], cg) < 1.25 * least) cands.push_back({widths[i], cg, 0, pre});
       }
       if (widths[i] >= 192 && gemm_ws_supported(w.N, w.K) && (!eight || M >= kWsMinRows)) cands.push_back({widths[i], 2, 1, pre});
-      if (allow_as && as_pointers_ok(&w) && gemm_as_supported(w.N, w.K) && eight && M >= kAsMinRows)
+      if (allow_as && gemm_as_supported(w.N, w.K) && eight && M >= kAsMinRows)
         cands.push_back({widths[i], 2, 2, pre});
     }
   // (the default first: a later one has to beat it)
@@ -822,7 +817,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
       if ((lf & DP_FLAG_CTA_PAIR) && L.w.N % 128 && L.w.N % 192) lf &= ~DP_FLAG_CTA_PAIR;
       if ((lf & DP_FLAG_WEIGHT_STATIONARY) && !gemm_ws_supported(L.w.N, L.w.K)) lf &= ~DP_FLAG_WEIGHT_STATIONARY;
       L.pre = want_unpack_first(lf, L.w.bits, true) ? 1 : 0;
-      choose_tile(lf, L.M, L.w.N, L.w.K, L.pre ? 8 : L.w.bits, !fused_daq && as_pointers_ok(&L.w), &L.bn, &L.cg, &L.ws);
+      choose_tile(lf, L.M, L.w.N, L.w.K, L.pre ? 8 : L.w.bits, !fused_daq, &L.bn, &L.cg, &L.ws);
       if (autotune) {
         const TunedShape* hit = nullptr;
         for (const TunedShape& t : tuned)
@@ -954,7 +949,7 @@ extern "C" int dp_plan_set_layer_flags(dp_plan* plan, int32_t layer, uint32_t fl
   if ((flags & DP_FLAG_UNPACK_FIRST) && (flags & DP_FLAG_NO_UNPACK_FIRST))
     return fail(DP_ERR_INVALID_ARG, "UNPACK_FIRST and NO_UNPACK_FIRST are exclusive");
   T.pre = want_unpack_first(flags, T.w.bits, true) ? 1 : 0;
-  choose_tile(flags, T.M, T.w.N, T.w.K, T.pre ? 8 : T.w.bits, plan->daq_sync == nullptr && as_pointers_ok(&T.w), &T.bn,
+  choose_tile(flags, T.M, T.w.N, T.w.K, T.pre ? 8 : T.w.bits, plan->daq_sync == nullptr, &T.bn,
               &T.cg, &T.ws);
   if ((flags & DP_FLAG_ACT_STATIONARY) && T.ws != 2)
     return fail(DP_ERR_SHAPE, "layer %d: the activation-stationary kernel does not take this layer (N=%d K=%d, %d-bit "

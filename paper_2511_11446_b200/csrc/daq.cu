@@ -1,7 +1,7 @@
 // Dynamic activation quantization (Step 3, Eq. "daq"; b = 8, zero-point 0, clip threshold = the
 // token's absolute maximum): bf16 [M][K] -> int8 codes + one fp32 scale per token.
 //
-// One warp owns one token. The row is read once with 16-byte loads and kept in registers; the
+// One warp owns one token, or two or four where a row is long (launch_daq_t). The row is read once with 16-byte loads and kept in registers; the
 // absolute maximum is taken on the bf16 magnitude bits (monotone for finite values, so integer
 // max is exact); the quantizer is one fused multiply-add per element: x * fl(127/a) + 1.5*2^23
 // rounds the exact product once, half to even, and leaves the integer in the low mantissa bits.
