@@ -111,6 +111,7 @@ constexpr uint32_t kLinearFlags =
     DP_FLAG_NO_CTA_PAIR | DP_FLAG_WEIGHT_STATIONARY | DP_FLAG_NO_WEIGHT_STATIONARY | DP_FLAG_UNPACK_FIRST |
     DP_FLAG_NO_UNPACK_FIRST | DP_FLAG_ACT_STATIONARY | DP_FLAG_NO_ACT_STATIONARY;
 constexpr int64_t kAsMinRows = 1024;   // below, its strip fill is never made up for
+constexpr int64_t kSkewMaxRows = 1024;  // see plan_run_step
 constexpr int kTuneReps = 12;
 constexpr int64_t kWsMinRows = 8192;  // from here on a resident weight strip is reused often enough to pay
 static int forced_bn(uint32_t flags) { return static_cast<int>((flags & DP_FLAG_TILE_N_MASK) >> 8) * 64; }
@@ -232,12 +233,15 @@ static int check_weight(const dp_weight* w) {
 // `chained`: the kernel preceding this layer's first launch on the stream is a launch of the same
 // dp_plan_run call, so it cannot be a producer of this layer's weights and they may be prefetched
 // while it drains.
+// `part`: plans launch the DAQ of a layer and its GEMM apart; PART_GEMM_READY: the GEMM, when the kernel before it on the stream
+// is not the last to touch its operands.
+enum { PART_BOTH, PART_DAQ, PART_GEMM, PART_GEMM_READY };
 static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const float* s_a_in, int64_t M,
                       void* y, int64_t ldy, void* workspace, const dp_debug* dbg, int32_t* status,
                       uint32_t flags, cudaStream_t stream, const CUtensorMap* tmap_w, int bn, int cg, int ws,
                       const CUtensorMap* tmap_a_cached, bool chained, int32_t* daq_sync = nullptr,
                       int pre = -1, int daq_rank = 1, int daq_bits = 8, const dp_residual* res = nullptr,
-                      bool ahead = false) {
+                      bool ahead = false, int part = PART_BOTH) {
   const bool pdl = !(flags & DP_FLAG_NO_PDL);
   if (w->bits == 16)  // a layer the plan keeps in 16-bit precision: no DAQ, no scales (checked by the caller)
     return launch_gemm_bf16(x, ldx, w->qweight, static_cast<const uint16_t*>(w->bias), M, w->N, w->K,
@@ -351,7 +355,8 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     int8_t* wq = static_cast<int8_t*>(workspace);
     float* wsa = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + align256(scratch_q_bytes(M, w->K)));
     korder = gemm_korder(w->bits);
-    if (robust) {
+    if (part >= PART_GEMM) {
+    } else if (robust) {
       int st = launch_daq_robust(x, M, w->K, ldx, wq, w->K, wsa, nullptr, daq_rank, daq_bits, true, stream, pdl,
                                  &job);
       if (st != DP_OK) return st;
@@ -360,6 +365,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
                           &job);
       if (st != DP_OK) return st;
     }
+    if (part == PART_DAQ) return DP_OK;
     q = wq;
     s_a = wsa;
     ldq = w->K;
@@ -400,6 +406,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   // Its weight ring is small (64 KB per CTA): prefetching it while the DAQ launch drains costs that
   // launch no bandwidth worth speaking of, whatever M is.
   if (ws == 2 && s_a_in == nullptr && !unpack_first && pdl) g.early_w = 1;
+  if (part == PART_GEMM_READY) g.early_w = g.a_ready = 1;
   g.cg = cg;
   g.ws = ws;
   if (tmap_w != nullptr) {
@@ -641,7 +648,7 @@ struct dp_plan {
   std::vector<PlanLayer> layers;
   uint32_t flags;
   size_t workspace_bytes;
-  size_t half_bytes;  // of the two halves that consecutive layers take in turn
+  size_t part_bytes;  // of the three parts that consecutive layers take in turn
   size_t x_bytes;
   std::vector<TmapACache> a_cache;
   std::vector<std::vector<int>> groups;  // small-M layers of equal shape, run first in every step
@@ -653,8 +660,8 @@ struct dp_plan {
   cudaStream_t copy_stream;
   cudaEvent_t ev_copied[2], ev_consumed[2], ev_entry;
   void need(size_t layer_bytes) {  // room for a layer of this scratch size
-    half_bytes = std::max(half_bytes, align256(layer_bytes));
-    workspace_bytes = std::max(workspace_bytes, 2 * half_bytes);
+    part_bytes = std::max(part_bytes, align256(layer_bytes));
+    workspace_bytes = std::max(workspace_bytes, 3 * part_bytes);
   }
 };
 
@@ -781,7 +788,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   if (!p) return fail(DP_ERR_CUDA, "out of host memory");
   p->flags = flags;
   p->workspace_bytes = 256;
-  p->half_bytes = 0;
+  p->part_bytes = 0;
   p->x_bytes = 0;
   p->copy_stream = nullptr;
   p->daq_sync = nullptr;
@@ -913,7 +920,7 @@ extern "C" int dp_plan_set_daq(dp_plan* plan, int32_t clip_percentile_e3, int32_
   for (int b = 0; b < 3 && n_timesteps > 0; ++b)
     if (act_bits_by_bin[b] < 2 || act_bits_by_bin[b] > 8)
       return fail(DP_ERR_BITS, "dp_plan_set_daq: activation bits %d not in [2, 8]", act_bits_by_bin[b]);
-  size_t need = plan->half_bytes;
+  size_t need = plan->part_bytes;
   for (const PlanLayer& L : plan->layers) {
     if (L.M == 0 || L.w.bits == 16 || L.w.group_size > 0) continue;  // no DAQ / scratch already sized for any rule
     const int rank = clip_rank_of(clip_percentile_e3, L.w.K);
@@ -1013,15 +1020,26 @@ static const CUtensorMap* cached_tmap_a(dp_plan* plan, const void* ws, int64_t M
 // What a call has launched so far.
 struct PlanRun {
   bool chained = false;  // something
-  int half = 0;          // half of the workspace that the next layer takes
-  const void* y = nullptr;  // outputs of the launch before, if that is a tensor-core GEMM: it may still be running when the
-  int64_t y_elems = 0;      // next launch starts, but then nothing before it is (it lets the next one start after its own wait)
+  int slot = 0;          // part of the workspace that the next layer takes
+  const void* y = nullptr;  // outputs of the last launch, if that is a tensor-core GEMM: it may still be running when the
+  int64_t y_elems = 0;      // next launch starts, but then everything before it is done (it lets the next one start after its
+                            // own wait)
+  int pending = -1;         // layer whose DAQ has been launched and whose GEMM has not
+  uint8_t* pending_scratch = nullptr;
+  bool pending_ready = false;  // a tensor-core GEMM has been launched since, so that DAQ is done when the next launch starts
 };
 
-// DAQ (and weight expansion) of a layer runs beside the GEMM of the layer before: it reads only the layer's own input
-// and weights and writes the half of the workspace that that GEMM does not read. Not so where the input overlaps that GEMM's
-// output. Steps of 28 DiT blocks, mixed bits, 256 / 2048 tokens: 915 -> 774 / 1559 -> 1350 us; 1024 tokens with
-// the percentile rule 1385 -> 1244.
+// Tensor-core layers are launched D0 D1 G0 D2 G1 D3 G2 ...: DAQ (and weight expansion) of a layer runs beside the GEMM
+// two layers before it, and a GEMM, whose operands are then complete, starts on each SM as the GEMM before it leaves
+// (only its epilogue waits for that one). A layer's operands are in one of three parts of the workspace: when D(l + 2)
+// starts, G(l) may be running and D(l + 1) waits for its GEMM, while G(l - 1), the last reader of the third part, is done: G(l)
+// lets D(l + 2) start after its own wait, which is for D(l + 1), one CTA of which stays until G(l - 1) has finished.
+// A layer whose input overlaps the outputs of the layer before it is launched after that layer's GEMM, and one that
+// overlaps those of the GEMM that may be running waits for it. Steps of 28 DiT blocks, mixed bits, DAQ and GEMM in turn / DAQ
+// beside the GEMM before, G(l) right after D(l) / this order: 256 tokens 915 / 773 / 670 us; the last two at 1024 tokens 992 / 912,
+// 2048 with cold inputs 1359 / 1366, 4096 1989 / 2028, 8192 3620 / 3690, and 1024 with the percentile rule 1244 / 1290: where a
+// GEMM or the DAQ fills the SMs the codes wait too long and two layers' loads compete. So up to kSkewMaxRows
+// tokens and with the plain rule only; else G(l) follows D(l) at once.
 static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* const* ys, void* workspace,
                          int32_t* status, cudaStream_t stream, PlanRun* run) {
   const int n = static_cast<int>(plan->layers.size());
@@ -1067,25 +1085,12 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     run->chained = true;
     run->y = nullptr;
   }
-  for (int l = 0; l < n; ++l) {
-    const PlanLayer& L = plan->layers[l];
-    if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
-    if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", l);
-    if (!aligned16(xs[l]) || !aligned16(ys[l])) return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", l);
-    uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->half * plan->half_bytes;
-    const bool ahead = run->y != nullptr && plan->daq_sync == nullptr &&
-                       !overlap(xs[l], L.M * L.w.K, run->y, run->y_elems);
-    const CUtensorMap* ta = nullptr;
-    if (!L.simt && L.w.bits != 16 && L.w.group_size == 0) {
-      int st = DP_OK;
-      ta = cached_tmap_a(plan, scratch, L.M, L.w.K, &st);
-      if (st != DP_OK) return st;
-    }
-    // The next tensor-core layer's packed weights and its input start towards L2 while this layer's
-    // GEMM runs. A hint, not a reordering: if that input is still to be written (by this layer, say),
-    // the hint fetches bytes that the write then replaces in L2, and nothing is read before its turn.
+  // A later tensor-core layer's packed weights and its input start towards L2 while a GEMM runs. A hint, not a
+  // reordering: if that input is still to be written (by this layer, say), the hint fetches bytes that the write then
+  // replaces in L2, and nothing is read before its turn.
+  auto hint = [&](int j) {
     gemm_set_next_reads(nullptr, 0, nullptr, 0);
-    for (int j = l + 1; j < n; ++j) {
+    for (; j < n; ++j) {
       const PlanLayer& Nx = plan->layers[j];
       if (Nx.M == 0 || (plan->grouped[j] && !group_splits(j))) continue;
       const size_t wb = static_cast<size_t>(Nx.w.N) * Nx.w.K * Nx.w.bits / 8;
@@ -1095,18 +1100,70 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
       if (!Nx.simt && xs[j] != nullptr) gemm_set_next_reads(Nx.w.qweight, wb, xb <= (32u << 20) ? xs[j] : nullptr, xb);
       break;
     }
-    int st = run_linear(&L.w, xs[l], L.w.K, nullptr, L.M, ys[l], L.w.N, scratch, nullptr, status,
-                        plan->flags, stream, L.simt ? nullptr : &L.tmap_w, L.bn, L.cg, L.ws, ta, run->chained,
-                        L.simt ? nullptr : plan->daq_sync, L.simt ? 0 : L.pre,
-                        robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead);
+  };
+  auto layer = [&](int l, uint8_t* scratch, const CUtensorMap* ta, bool ahead, int part) {
+    const PlanLayer& L = plan->layers[l];
+    const int st = run_linear(&L.w, xs[l], L.w.K, nullptr, L.M, ys[l], L.w.N, scratch, nullptr, status, plan->flags, stream,
+                              L.simt ? nullptr : &L.tmap_w, L.bn, L.cg, L.ws, ta, run->chained,
+                              L.simt ? nullptr : plan->daq_sync, L.simt ? 0 : L.pre,
+                              robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead, part);
     gemm_set_next_reads(nullptr, 0, nullptr, 0);
-    if (st != DP_OK) return st;
     run->chained = true;
-    run->half ^= 1;
-    run->y = !L.simt && L.w.group_size == 0 ? ys[l] : nullptr;
+    return st;
+  };
+  auto flush = [&]() {  // the GEMM that is still to be launched
+    if (run->pending < 0) return static_cast<int>(DP_OK);
+    const int l = run->pending;
+    const PlanLayer& L = plan->layers[l];
+    int st = DP_OK;
+    const CUtensorMap* ta = cached_tmap_a(plan, run->pending_scratch, L.M, L.w.K, &st);
+    if (st != DP_OK) return st;
+    hint(l + 2);
+    st = layer(l, run->pending_scratch, ta, false, run->pending_ready ? PART_GEMM_READY : PART_GEMM);
+    run->pending = -1;
+    run->y = ys[l];
     run->y_elems = L.M * L.w.N;
+    return st;
+  };
+  for (int l = 0; l < n; ++l) {
+    const PlanLayer& L = plan->layers[l];
+    if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
+    if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", l);
+    if (!aligned16(xs[l]) || !aligned16(ys[l])) return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", l);
+    if (L.simt || L.w.bits == 16 || L.w.group_size > 0 || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
+      if (int st = flush()) return st;
+      const CUtensorMap* ta = nullptr;
+      if (!L.simt && L.w.bits != 16 && L.w.group_size == 0) {
+        int st = DP_OK;
+        ta = cached_tmap_a(plan, workspace, L.M, L.w.K, &st);
+        if (st != DP_OK) return st;
+      }
+      hint(l + 1);
+      if (int st = layer(l, static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes, ta, false, PART_BOTH)) return st;
+      run->y = L.w.bits == 16 ? ys[l] : nullptr;
+      run->y_elems = L.M * L.w.N;
+      continue;
+    }
+    const bool skew = L.M <= kSkewMaxRows && !robust;
+    if (run->pending >= 0) {
+      const PlanLayer& P = plan->layers[run->pending];
+      if (!skew || overlap(xs[l], L.M * L.w.K, ys[run->pending], P.M * P.w.N))
+        if (int st = flush()) return st;
+    }
+    uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes;
+    const bool ahead = run->y != nullptr && !overlap(xs[l], L.M * L.w.K, run->y, run->y_elems);
+    if (int st = layer(l, scratch, nullptr, ahead, PART_DAQ)) return st;
+    run->slot = (run->slot + 1) % 3;
+    run->y = nullptr;
+    const bool between = run->pending >= 0;
+    if (int st = flush()) return st;
+    run->pending = l;
+    run->pending_scratch = scratch;
+    run->pending_ready = between;
+    if (!skew)
+      if (int st = flush()) return st;
   }
-  return DP_OK;
+  return flush();
 }
 
 static int check_plan_run(const dp_plan* plan, const int32_t* steps, int32_t n_steps,

@@ -123,6 +123,8 @@ struct GemmProblem {
   int32_t a_tiled;  // the activations behind tmap_a are stored as 128 x 128 tiles (see gemm_encode_a_tiled)
   int32_t early_w;  // the preceding kernel on the stream is this call's own DAQ: weights may be
                     // fetched before it has finished
+  int32_t a_ready = 0;  // (with early_w) nor is it writing the activations or the int8 copy of the weights: only
+                        // the epilogue waits for it
   int32_t* status;
   // In-kernel DAQ (x != nullptr): the GEMM kernel quantizes x into q_out / s_a_out (the buffers
   // behind tmap_a and s_a) itself; sync = zeroed counters, one per 128-token tile plus one.

@@ -102,8 +102,8 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st;
       bool ok = true;
-      bool open = !p.early_w;  // false until griddepcontrol.wait has been executed
-      if (open) pdl_wait();
+      bool open = !p.early_w || p.a_ready;  // false until griddepcontrol.wait has been executed
+      if (!p.early_w) pdl_wait();
       int cur_strip = -1, strips = 0;
       const uint32_t w_full0 = map_to_cta(&w_full[0], 0), a_full0 = map_to_cta(&a_full[0], 0);  // in the leader
       auto load_w = [&](int kb, int w_row) {
@@ -312,6 +312,7 @@ int launch_gemm_as(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   p.sync = nullptr;
   p.sync_tiles = 0;
   p.early_w = (pdl && g.early_w) ? 1 : 0;
+  p.a_ready = p.early_w ? g.a_ready : 0;
   p.status = g.status;
   AsParams ap;
   ap.bns = bns;

@@ -87,7 +87,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (elect_one()) {
       Ring st;
       bool ok = true;
-      if (p.early_w) pdl_wait();
+      if (p.early_w && !p.a_ready) pdl_wait();
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
         mbar_arrive_expect_tx(&full[st.s], A_BYTES);

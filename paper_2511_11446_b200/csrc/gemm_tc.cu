@@ -129,7 +129,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       int ready_tile = -1;  // in-kernel DAQ: last 128-token tile seen complete
       // In a pair both CTAs' bytes are counted on the leader's barrier.
       const uint32_t full0 = CG == 2 ? map_to_cta(&full_a[0], 0) : smem_u32(&full_a[0]);
-      if (p.early_w) pdl_wait();
+      if (p.early_w && !p.a_ready) pdl_wait();
       for (int tile = first_tile; tile < total_tiles && ok; tile += tile_stride) {
         const int m_row = (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM;
         if (p.x != nullptr && (m_row >> 7) != ready_tile) {
@@ -610,6 +610,7 @@ int launch_gemm(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   p.sync = g.sync;
   p.sync_tiles = static_cast<int32_t>((g.M + BM - 1) / BM);
   p.early_w = (pdl && g.early_w) ? 1 : 0;
+  p.a_ready = p.early_w ? g.a_ready : 0;
   p.status = g.status;
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   // (taps, in-kernel DAQ and the test hook belong to the unsplit kernel)

@@ -100,7 +100,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     // ================= TMA producer =================
     if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
       Ring st, pr;
-      bool ok = true, a_open = !p.early_w || p.x != nullptr;
+      bool ok = true, a_open = !p.early_w || p.a_ready || p.x != nullptr;
       int cur_strip = -1, strips = 0, ready_tile = -1;
       const uint32_t full0 = map_to_cta(&full_a[0], 0);
       for (int item = item0; item < item1 && ok; ++item) {
@@ -360,6 +360,7 @@ int launch_gemm_ws(const GemmProblem& g, cudaStream_t stream, bool pdl) {
   p.sync = g.sync;
   p.sync_tiles = static_cast<int32_t>((g.M + BM - 1) / BM);
   p.early_w = (pdl && g.early_w) ? 1 : 0;
+  p.a_ready = p.early_w ? g.a_ready : 0;
   p.status = g.status;
   const int64_t items = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   const int64_t pairs = gemm_max_pairs() > 0 ? gemm_max_pairs() : num_sms() / 2;
