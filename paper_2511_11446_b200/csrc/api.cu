@@ -250,7 +250,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
   const bool robust = s_a_in == nullptr && (daq_rank > 1 || daq_bits < 8);
   if (w->group_size > 0) {
     // Group-wise scales: DAQ into the tiled scratch (packed weights expanded to int8 by the same
-    // launch, which takes their zero-points off: u - z fits a byte up to 4 bits), the per-group code sums
+    // launch, which takes their zero-points off as far as a byte allows), the per-group code sums
     // when 8-bit codes have zero-points, then the folding GEMM.
     const uint8_t* zeros = static_cast<const uint8_t*>(w->zeros);
     uint8_t* ws8 = static_cast<uint8_t*>(workspace);
@@ -270,10 +270,9 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
       job.zeros = zeros;
       job.row_units = w->K / 32;
       job.group_units = w->group_size / 32;
-      zeros = nullptr;
       w8 = dst;
     }
-    int32_t* rowsum = zeros != nullptr ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
+    int32_t* rowsum = zeros != nullptr && w->bits == 8 ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
     int st = robust ? launch_daq_robust(x, M, w->K, ldx, wq, w->K, wsa, nullptr, daq_rank, daq_bits, true, stream, pdl,
                                         &job)
                     : launch_daq(x, M, w->K, ldx, wq, w->K, wsa, nullptr, KORDER_NATURAL, true, stream, pdl,

@@ -278,7 +278,7 @@ __device__ __forceinline__ void expand3(uint32_t s0, uint32_t s1, uint32_t s2, u
   }
 }
 
-// Packed unit -> 8 words of 4 int8 (u - z of the stored codes u, k ascending). z in [0, 2^BITS): the
+// Packed unit -> 8 words of 4 int8 (u - z of the stored codes u, k ascending). z in [0, 128]: the
 // zero-point in use, 2^(BITS-1) for symmetric layers. u + 128 - z stays inside its byte, and flipping the
 // byte's top bit takes the 128 off again.
 template <int BITS>
@@ -308,18 +308,20 @@ __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int blo
   uint32_t w[8];
   if (u < job.units) {
     uint32_t z = 1u << (job.bits - 1);
-    if (job.zeros != nullptr) {  // one zero-point per channel and group (a multiple of 32 codes)
-      const int64_t n = u / job.row_units;
-      z = job.zeros[n * (job.row_units / job.group_units) + (u - n * job.row_units) / job.group_units];
+    // One zero-point per channel and group (a multiple of 32 codes). (Units of a matrix that fits the device count in
+    // 32 bits. The clamp of z stands at its uses: up here it made the packed words wait for z, 1.5 us of a 93 us block.)
+    if (job.zeros != nullptr) {
+      const uint32_t n = static_cast<uint32_t>(u) / job.row_units, at = static_cast<uint32_t>(u) - n * job.row_units;
+      z = job.zeros[static_cast<int64_t>(n) * (job.row_units / job.group_units) + at / job.group_units];
     }
     if (job.bits == 4) {
       const uint4 v = reinterpret_cast<const uint4*>(job.packed)[u];
       const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
-      expand_unit<4>(pk, w, z);
+      expand_unit<4>(pk, w, min(z, 128u));  // (the fold takes off what is above 128)
     } else {
       const uint32_t* p = job.packed + u * 3;
       const uint32_t pk[3] = {p[0], p[1], p[2]};
-      expand_unit<3>(pk, w, z);
+      expand_unit<3>(pk, w, min(z, 128u));
     }
   }
   if (job.early && !job.ahead) pdl_wait();

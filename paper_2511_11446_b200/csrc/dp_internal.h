@@ -18,7 +18,7 @@ enum KOrder {
 int gemm_korder(int32_t bits);
 
 // daq.cu
-// Expansion of a packed weight matrix to int8 [N][K] (codes less their zero-point, k ascending) in global scratch,
+// Expansion of a packed weight matrix to int8 [N][K] (codes less their zero-point, or 128 of it, k ascending) in global scratch,
 // run by extra CTAs of a DAQ launch or on its own: `units` = N * K / 32 units of 32 codes.
 struct UnpackJob {
   const uint32_t* packed = nullptr;
@@ -31,7 +31,7 @@ struct UnpackJob {
   int32_t ahead = 0;        // (with early) nor x, nor reading the destinations: the whole launch runs beside it. One CTA
                             // stays until it has finished, so that whatever waits for this launch waits for both
   const uint8_t* zeros = nullptr;  // group-wise zero-points [N][row_units / group_units], or null (symmetric)
-  int32_t row_units = 0, group_units = 0;
+  uint32_t row_units = 0, group_units = 0;
 };
 int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq,
                float* s_a, int32_t* rowsum, int korder, bool tiled, cudaStream_t stream, bool pdl,
@@ -175,7 +175,7 @@ int gemm_bf16_init_device();
 int gemm_grp_init_device();
 
 // gemm_grp.cu -- layers with group-wise weight scales (and zero-points): folding tensor-core kernel.
-// zeros: 8-bit weights only (for packed ones the expansion has taken the zero-points off already).
+// (for packed weights the expansion has taken the zero-points up to 128 off already)
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
                     int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,
                     int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl);

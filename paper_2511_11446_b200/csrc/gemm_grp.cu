@@ -19,9 +19,13 @@
 // see RowEpilogue): per group two tcgen05.ld, int32 -> fp32 and a packed fma into 32 fp32 partial outputs
 // held in registers, then the buffer goes back to the MMA issuer; after the last group the token scale, bias,
 // bf16 rounding and 16-byte stores.
-// Zero-points of 3- and 4-bit layers are taken off when the packed weights are expanded to int8. For 8-bit
-// codes u - z does not fit a byte: the tensor core multiplies by u - 128 and (128 - z[n,G]) * rowsum_G[m] is
-// added in int32 before the conversion (form ZP, with rowsum from a kernel of its own).
+// Zero-points of 3- and 4-bit layers are taken off when the packed weights are expanded to int8, up to 128 of
+// them: u - 128 is the least an int8 holds. Zero-points are bytes, though no quantizer writes one above 2^bits: a
+// fold warp looks those of its columns over while it waits for its first accumulators, and where one is above 127
+// it takes a fold that adds (128 - z) * rowsum_G[m] of the columns above 128 (ZP_WIDE), with row sums
+// that it takes from the codes itself. For 8-bit
+// codes u - z does not fit a byte at all: the tensor core multiplies by u - 128 and (128 - z[n,G]) * rowsum_G[m] is
+// added in int32 before the conversion (form ZP_8BIT, with rowsum from a kernel of its own).
 // The fold is what bounds this kernel: 1.5 instructions per output and group, the conversion at 64 per
 // clock and SM, 256 clocks per 128 x 128 x g step against 256 of MMA at g = 128. Sixteen warps keep both busy
 // (eight, 64 columns each, left them waiting on each other): block of 4-bit layers with zero-points, g = 128,
@@ -40,11 +44,15 @@ constexpr int kGrpCols = kGrpBN / (kGrpFoldWarps / 4);  // columns of a fold war
 constexpr int kGrpThreads = (kGrpFoldWarp0 + kGrpFoldWarps) * 32;
 constexpr int kGrpScaleWords = 2 * kGrpBufs * kGrpBN + kGrpFoldWarps * kGrpCols;  // scales, zero-point terms, biases
 
+// Zero-points: none; of 8-bit codes; of packed codes; of packed codes, some of them above 127.
+enum { ZP_NONE, ZP_8BIT, ZP_PACKED, ZP_WIDE };
+
 struct GrpParams {
   const float* s_a;       // [M]
   const float* s_w;       // [N][ng]
-  const uint8_t* zeros;   // [N][ng] or null
-  const int32_t* rowsum;  // [M][ng] (zero-points only)
+  const uint8_t* zeros;   // [N][ng] (unless ZP_NONE)
+  const int32_t* rowsum;  // [M][ng] (ZP_8BIT)
+  const int8_t* q;        // the codes behind tmap_a, tiled (ZP_WIDE)
   const uint16_t* bias;
   uint16_t* y;
   int64_t ldy;
@@ -100,24 +108,202 @@ __device__ __forceinline__ void grp_issue(const GrpParams& p, const uint8_t* sA,
   }
 }
 
-template <bool ZP>
+// Shared memory of a CTA.
+struct GrpSmem {
+  uint8_t *a, *b;  // operand stages
+  float* scale;    // [buffer][column] of the group in it
+  int32_t* dz;     // the same, 2^(b-1) - z
+  float* bias;     // per fold warp: its columns'
+  uint64_t *full, *empty, *grp_full, *grp_empty;
+  uint32_t* tmem_slot;
+  volatile int* abort_flag;
+  __device__ __forceinline__ GrpSmem() {
+    extern __shared__ uint8_t smem_raw[];
+    a = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    b = a + kGrpStages * BM * BK;
+    scale = reinterpret_cast<float*>(b + kGrpStages * kGrpBN * BK);
+    dz = reinterpret_cast<int32_t*>(scale + kGrpBufs * kGrpBN);
+    bias = reinterpret_cast<float*>(dz + kGrpBufs * kGrpBN);
+    full = reinterpret_cast<uint64_t*>(scale + kGrpScaleWords);
+    empty = full + kGrpStages;
+    grp_full = empty + kGrpStages;
+    grp_empty = grp_full + kGrpBufs;
+    tmem_slot = reinterpret_cast<uint32_t*>(grp_empty + kGrpBufs);
+    abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  }
+};
+
+// Whether some zero-point of the 32 columns from col0 on of this CTA's tiles is above 127 (a warp together).
+__device__ __forceinline__ bool grp_wide_zeros(const GrpParams& p, int col0, int lane) {
+  const int bytes = kGrpCols * p.ng, total_tiles = p.m_tiles * p.n_tiles;
+  const bool aligned = (reinterpret_cast<uintptr_t>(p.zeros) & 15u) == 0;
+  uint32_t any = 0;
+  int seen = 0;
+  for (int tile = blockIdx.x; tile < total_tiles && seen < p.n_tiles; tile += gridDim.x, ++seen) {
+    const uint8_t* z = p.zeros + static_cast<int64_t>((tile % p.n_tiles) * kGrpBN + col0) * p.ng;
+    if (aligned) {
+      for (int i = lane; i < bytes / 16; i += 32) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(z) + i);
+        any |= v.x | v.y | v.z | v.w;
+      }
+    } else {
+      for (int i = lane; i < bytes; i += 32) any |= __ldg(z + i);
+    }
+  }
+  return __any_sync(0xFFFFFFFFu, (any & 0x80808080u) != 0);
+}
+
+// Code sums of group G of the tokens row0 + 8 * i that are there, by the four lanes of a quad (they share them).
+__device__ __forceinline__ void grp_row_sums(const GrpParams& p, int64_t row0, int G, int lane, const bool (&live)[4],
+                                             int (&rs)[4]) {
+  const int part = p.g >> 2;  // of the group's codes, a multiple of 8
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t m = row0 + 8 * i;
+    int s = 0;
+    for (int k = G * p.g + (lane & 3) * part, end = k + part; live[i] && k < end; k += 8) {
+      const uint2 v = *reinterpret_cast<const uint2*>(p.q + ((m >> 7) * (p.K >> 7) + (k >> 7)) * 16384 + (m & 127) * 128 + (k & 127));
+      s = __dp4a(static_cast<int>(v.x), 0x01010101, __dp4a(static_cast<int>(v.y), 0x01010101, s));
+    }
+    s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+    rs[i] = s + __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+  }
+}
+
+// A fold warp's whole run over this CTA's tiles: quadrant (warp & 3), column quarter (fw >> 2).
+template <int ZP>
+__device__ __forceinline__ void grp_fold(const GrpParams& p) {
+  const GrpSmem sm;
+  const float* s_scale = sm.scale;
+  const int32_t* s_dz = sm.dz;
+  uint64_t *grp_full = sm.grp_full, *grp_empty = sm.grp_empty;
+  volatile int* abort_flag = sm.abort_flag;
+  const uint32_t tmem_base = *sm.tmem_slot;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int total_tiles = p.m_tiles * p.n_tiles;
+  const int fw = warp - kGrpFoldWarp0, qd = warp & 3;
+  const int col0 = (fw >> 2) * kGrpCols;
+  const int tc = (lane & 3) * 8;  // this lane's channels of the warp's 32 (see RowEpilogue)
+  float* wb = sm.bias + fw * kGrpCols;
+  bool ok = true;
+  uint32_t gcount = 0;
+  for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    const int n0 = (tile % p.n_tiles) * kGrpBN + col0;
+    const int64_t row0 = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + (lane >> 2);
+    bool live[4];
+    float sa[4];
+    int rs[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      live[i] = row0 + 8 * i < p.M;
+      sa[i] = live[i] ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
+      rs[i] = (ZP == ZP_8BIT && live[i]) ? __ldg(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
+    }
+    __syncwarp();
+    wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
+    uint64_t t[4][4];  // fp32 partial outputs: token row0 + 8 * i, channels tc + 2j, tc + 2j + 1
+#pragma unroll
+    for (int i = 0; i < 16; ++i) t[i >> 2][i & 3] = 0;
+    // A group is folded in two halves of 16 tokens, each read while the other is computed, the first
+    // half of the next group under the second of this one.
+    const uint32_t t_row = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + col0;
+    auto wait_group = [&](uint32_t g) {
+      ok = mbar_wait(&grp_full[g % kGrpBufs], (g / kGrpBufs) & 1u, abort_flag);
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      tc_fence_after();
+    };
+    float sc[8];
+    int dz[8];
+    auto fold = [&](const uint32_t (&a)[16], int i0, const int* rs_g) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          int a0 = static_cast<int>(a[4 * j + 2 * k]), a1 = static_cast<int>(a[4 * j + 2 * k + 1]);
+          if constexpr (ZP != ZP_NONE) {
+            a0 += dz[2 * j] * rs_g[i0 + k];
+            a1 += dz[2 * j + 1] * rs_g[i0 + k];
+          }
+          t[i0 + k][j] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)),
+                                   f32x2_pack(sc[2 * j], sc[2 * j + 1]), t[i0 + k][j]);
+        }
+    };
+    uint32_t lo[16], hi[16];
+    wait_group(gcount);
+    if (!ok) break;
+    tmem_ld_16x256b_x4(t_row + (gcount % kGrpBufs) * kGrpBN, lo);
+    for (int G = 0; G < p.ng; ++G, ++gcount) {
+      const uint32_t buf = gcount % kGrpBufs;
+      const float4* s4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0 + tc);
+      *reinterpret_cast<float4*>(sc) = s4[0];
+      *reinterpret_cast<float4*>(sc + 4) = s4[1];
+      int rs_g[4];
+      if constexpr (ZP == ZP_8BIT) {
+        const int4* d4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0 + tc);
+        *reinterpret_cast<int4*>(dz) = d4[0];
+        *reinterpret_cast<int4*>(dz + 4) = d4[1];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          rs_g[i] = rs[i];
+          if (live[i] && G + 1 < p.ng) rs[i] = __ldg(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
+        }
+      }
+      if constexpr (ZP == ZP_WIDE) {
+        grp_row_sums(p, row0, G, lane, live, rs_g);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int z = __ldg(p.zeros + static_cast<int64_t>(n0 + tc + j) * p.ng + G);
+          dz[j] = z > 128 ? 128 - z : 0;
+        }
+      }
+      tmem_ld_wait();
+      tmem_ld_16x256b_x4(t_row + (16u << 16) + buf * kGrpBN, hi);
+      fold(lo, 0, rs_g);
+      tmem_ld_wait();
+      tc_fence_before();  // accumulators and scales are in registers: the buffer may take another group
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&grp_empty[buf]);
+      if (G + 1 < p.ng) {
+        wait_group(gcount + 1);
+        if (!ok) break;
+        tmem_ld_16x256b_x4(t_row + ((gcount + 1) % kGrpBufs) * kGrpBN, lo);
+      }
+      fold(hi, 2, rs_g);
+    }
+    if (!ok) break;
+    float bb[8];
+    *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(wb + tc);
+    *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(wb + tc + 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float y0, y1;
+        f32x2_unpack(f32x2_fma(t[i][j], f32x2_pack(sa[i], sa[i]), f32x2_pack(bb[2 * j], bb[2 * j + 1])), y0, y1);
+        const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
+        w[j] = *reinterpret_cast<const uint32_t*>(&v);
+      }
+      if (live[i]) st_global_v4(p.y + (row0 + 8 * i) * p.ldy + n0 + tc, w);
+    }
+  }
+}
+// (A function of its own: inlined, it cost the usual fold registers. Block of 4-bit layers with zero-points, g = 128,
+// M = 2048: 92.7 us without this form, 96.4 with it inlined, 93.0 this way.)
+__device__ __noinline__ void grp_fold_wide(const GrpParams& p) { grp_fold<ZP_WIDE>(p); }
+
+template <int ZP>
 __global__ void __launch_bounds__(kGrpThreads, 1)
 gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
-                const GrpParams p) {
+                const __grid_constant__ GrpParams p) {
   constexpr int NS = kGrpStages, A_BYTES = BM * BK, B_BYTES = kGrpBN * BK;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = smem;
-  uint8_t* sB = sA + NS * A_BYTES;
-  float* s_scale = reinterpret_cast<float*>(sB + NS * B_BYTES);               // [buffer][column] of the group in it
-  int32_t* s_dz = reinterpret_cast<int32_t*>(s_scale + kGrpBufs * kGrpBN);    // the same, 2^(b-1) - z
-  float* s_bias = reinterpret_cast<float*>(s_dz + kGrpBufs * kGrpBN);         // per fold warp: its columns'
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_scale + kGrpScaleWords);
-  uint64_t* empty = full + NS;
-  uint64_t* grp_full = empty + NS;
-  uint64_t* grp_empty = grp_full + kGrpBufs;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(grp_empty + kGrpBufs);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const GrpSmem sm;
+  uint8_t *sA = sm.a, *sB = sm.b;
+  float* s_scale = sm.scale;
+  int32_t* s_dz = sm.dz;
+  uint64_t *full = sm.full, *empty = sm.empty, *grp_full = sm.grp_full, *grp_empty = sm.grp_empty;
+  uint32_t* tmem_slot = sm.tmem_slot;
+  volatile int* abort_flag = sm.abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int KB = p.K / BK;
@@ -208,7 +394,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             const int64_t at = (n0 + 32 * c) * p.ng + G0 + i;
             if (G0 + i < p.ng) {
               nx[i][c] = __ldg(p.s_w + at);
-              if constexpr (ZP) nz[i][c] = __ldg(p.zeros + at);
+              if constexpr (ZP == ZP_8BIT) nz[i][c] = __ldg(p.zeros + at);
             }
           }
       };
@@ -221,7 +407,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             sc[i][c] = nx[i][c];
-            if constexpr (ZP) dz[i][c] = p.half - nz[i][c];
+            if constexpr (ZP == ZP_8BIT) dz[i][c] = p.half - nz[i][c];
           }
         fetch(G0 + AHEAD);
 #pragma unroll
@@ -234,7 +420,7 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             s_scale[buf * kGrpBN + c0 + 32 * c] = sc[i][c];
-            if constexpr (ZP) s_dz[buf * kGrpBN + c0 + 32 * c] = dz[i][c];
+            if constexpr (ZP == ZP_8BIT) s_dz[buf * kGrpBN + c0 + 32 * c] = dz[i][c];
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&grp_full[buf]);
@@ -243,104 +429,12 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
     }
   } else {
-    // ================= fold + epilogue: quadrant (warp & 3), column quarter (fw >> 2) =================
-    const int fw = warp - kGrpFoldWarp0, qd = warp & 3;
-    const int col0 = (fw >> 2) * kGrpCols;
-    const int tc = (lane & 3) * 8;  // this lane's channels of the warp's 32 (see RowEpilogue)
-    float* wb = s_bias + fw * kGrpCols;
-    bool ok = true;
-    uint32_t gcount = 0;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int n0 = (tile % p.n_tiles) * kGrpBN + col0;
-      const int64_t row0 = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + (lane >> 2);
-      bool live[4];
-      float sa[4];
-      int rs[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        live[i] = row0 + 8 * i < p.M;
-        sa[i] = live[i] ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
-        rs[i] = (ZP && live[i]) ? __ldg(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
-      }
-      __syncwarp();
-      wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
-      uint64_t t[4][4];  // fp32 partial outputs: token row0 + 8 * i, channels tc + 2j, tc + 2j + 1
-#pragma unroll
-      for (int i = 0; i < 16; ++i) t[i >> 2][i & 3] = 0;
-      // A group is folded in two halves of 16 tokens, each read while the other is computed, the first
-      // half of the next group under the second of this one.
-      const uint32_t t_row = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + col0;
-      auto wait_group = [&](uint32_t g) {
-        ok = mbar_wait(&grp_full[g % kGrpBufs], (g / kGrpBufs) & 1u, abort_flag);
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        tc_fence_after();
-      };
-      float sc[8];
-      int dz[8];
-      auto fold = [&](const uint32_t (&a)[16], int i0, const int* rs_g) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            int a0 = static_cast<int>(a[4 * j + 2 * k]), a1 = static_cast<int>(a[4 * j + 2 * k + 1]);
-            if constexpr (ZP) {
-              a0 += dz[2 * j] * rs_g[i0 + k];
-              a1 += dz[2 * j + 1] * rs_g[i0 + k];
-            }
-            t[i0 + k][j] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)),
-                                     f32x2_pack(sc[2 * j], sc[2 * j + 1]), t[i0 + k][j]);
-          }
-      };
-      uint32_t lo[16], hi[16];
-      wait_group(gcount);
-      if (!ok) break;
-      tmem_ld_16x256b_x4(t_row + (gcount % kGrpBufs) * kGrpBN, lo);
-      for (int G = 0; G < p.ng; ++G, ++gcount) {
-        const uint32_t buf = gcount % kGrpBufs;
-        const float4* s4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0 + tc);
-        *reinterpret_cast<float4*>(sc) = s4[0];
-        *reinterpret_cast<float4*>(sc + 4) = s4[1];
-        int rs_g[4];
-        if constexpr (ZP) {
-          const int4* d4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0 + tc);
-          *reinterpret_cast<int4*>(dz) = d4[0];
-          *reinterpret_cast<int4*>(dz + 4) = d4[1];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            rs_g[i] = rs[i];
-            if (live[i] && G + 1 < p.ng) rs[i] = __ldg(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
-          }
-        }
-        tmem_ld_wait();
-        tmem_ld_16x256b_x4(t_row + (16u << 16) + buf * kGrpBN, hi);
-        fold(lo, 0, rs_g);
-        tmem_ld_wait();
-        tc_fence_before();  // accumulators and scales are in registers: the buffer may take another group
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&grp_empty[buf]);
-        if (G + 1 < p.ng) {
-          wait_group(gcount + 1);
-          if (!ok) break;
-          tmem_ld_16x256b_x4(t_row + ((gcount + 1) % kGrpBufs) * kGrpBN, lo);
-        }
-        fold(hi, 2, rs_g);
-      }
-      if (!ok) break;
-      float bb[8];
-      *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(wb + tc);
-      *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(wb + tc + 4);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float y0, y1;
-          f32x2_unpack(f32x2_fma(t[i][j], f32x2_pack(sa[i], sa[i]), f32x2_pack(bb[2 * j], bb[2 * j + 1])), y0, y1);
-          const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
-          w[j] = *reinterpret_cast<const uint32_t*>(&v);
-        }
-        if (live[i]) st_global_v4(p.y + (row0 + 8 * i) * p.ldy + n0 + tc, w);
-      }
+    // ================= fold + epilogue =================
+    if constexpr (ZP == ZP_PACKED) {
+      if (grp_wide_zeros(p, ((warp - kGrpFoldWarp0) >> 2) * kGrpCols, lane)) grp_fold_wide(p);
+      else grp_fold<ZP_NONE>(p);
+    } else {
+      grp_fold<ZP>(p);
     }
   }
 
@@ -390,15 +484,14 @@ constexpr size_t grp_smem_bytes() {
 }
 
 int gemm_grp_init_device() {
-  DP_CUDA_OK(cudaFuncSetAttribute(gemm_grp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(grp_smem_bytes())));
-  DP_CUDA_OK(cudaFuncSetAttribute(gemm_grp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(grp_smem_bytes())));
+  for (auto kernel : {gemm_grp_kernel<ZP_NONE>, gemm_grp_kernel<ZP_8BIT>, gemm_grp_kernel<ZP_PACKED>})
+    DP_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(grp_smem_bytes())));
   return DP_OK;
 }
 
-// q / s_a: the quantized activations (tiled scratch when a_tiled); w8: int8 [N][K] (codes less their
-// zero-point; with `zeros`, which 8-bit layers pass, u - 2^(bits-1)); rowsum: scratch int32 [M][K/g], used (and filled here) only with zero-points.
+// q / s_a: the quantized activations (tiled scratch when a_tiled, as packed layers with zero-points need it); w8:
+// int8 [N][K], u - 2^(bits-1) of 8-bit codes and of layers without zero-points, else u - min(z, 128); rowsum: scratch
+// int32 [M][K/g], used (and filled here) only for 8-bit codes with zero-points.
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
                     int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,
                     int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl) {
@@ -406,7 +499,9 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   if (N % kGrpBN || g <= 0 || g % 32 || K % g)
     return fail(DP_ERR_SHAPE, "group-wise layer: need N %% 128 == 0, g %% 32 == 0, K %% g == 0 (N=%d K=%d g=%d)", N, K, g);
   const int ng = K / g;
-  if (zeros != nullptr) {
+  const int form = zeros == nullptr ? ZP_NONE : bits == 8 ? ZP_8BIT : ZP_PACKED;
+  if (form == ZP_PACKED && !a_tiled) return fail(DP_ERR_INVALID_ARG, "packed group-wise layer: the codes are not tiled");
+  if (form == ZP_8BIT) {
     if (ng > kRowsumMaxGroups) return fail(DP_ERR_SHAPE, "group-wise zero-points: more than %d groups per row", kRowsumMaxGroups);
     const cudaError_t e = launch(group_rowsum_kernel, dim3(static_cast<unsigned>((M + kRowsumWarps - 1) / kRowsumWarps)),
                                  dim3(kRowsumWarps * 32), 0, stream, pdl, q, M, static_cast<int>(K), ldq,
@@ -423,6 +518,7 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   p.s_w = s_w;
   p.zeros = zeros;
   p.rowsum = rowsum;
+  p.q = q;
   p.bias = bias;
   p.y = y;
   p.ldy = ldy;
@@ -438,7 +534,9 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   p.status = status;
   const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
   const int sms = num_sms() > 0 ? num_sms() : 148;
-  const cudaError_t e = launch(zeros != nullptr ? gemm_grp_kernel<true> : gemm_grp_kernel<false>, dim3(static_cast<unsigned>(tiles < sms ? tiles : sms)), dim3(kGrpThreads),
+  const auto kernel = form == ZP_NONE ? gemm_grp_kernel<ZP_NONE> : form == ZP_8BIT ? gemm_grp_kernel<ZP_8BIT>
+                                                                                  : gemm_grp_kernel<ZP_PACKED>;
+  const cudaError_t e = launch(kernel, dim3(static_cast<unsigned>(tiles < sms ? tiles : sms)), dim3(kGrpThreads),
                                grp_smem_bytes(), stream, pdl, ta, tw, p);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "group-wise GEMM launch failed: %s", cudaGetErrorString(e));
   return DP_OK;

@@ -110,6 +110,27 @@ def test_plan_mixes_grouped_per_channel_and_16_bit_layers():
         B.dp_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("bits,g,K", [(4, 32, 1152), (4, 128, 256), (3, 192, 1152), (3, 256, 256)])
+@pytest.mark.parametrize("offset", [0, 1], ids=["aligned", "odd_address"])
+def test_zero_points_of_any_byte_value(bits, g, K, offset):
+    """Zero-points are bytes: u - z of a packed layer need not fit an int8. Values around 2^bits, 128 and 255, in some of
+    the column tiles and groups only, more tiles than SMs, and zero-points that start at an odd address."""
+    M, N = 1301, 1920
+    L = GroupedLayer(N, K, bits, g, True)
+    rng = np.random.default_rng(bits * g)
+    z = rng.choice(np.array([0, (1 << bits) - 1, 1 << bits, 127, 128, 129, 200, 255], np.uint8), size=L.z.shape)
+    L.z[128:256] = z[128:256]                       # a whole tile
+    L.z[700, K // g - 1] = 255                      # one group of one channel
+    L.z[1900:] = 128
+    d = torch.zeros(L.z.size + 1, dtype=torch.uint8, device="cuda")
+    L.d_z = d[offset:offset + L.z.size]
+    L.d_z.copy_(torch.from_numpy(L.z).ravel())
+    L.dw = B.make_weight(L.d_w, L.d_s, L.d_b, N, K, bits, g, L.d_z)
+    x = synth.activations(SEED, 3, 0, M, K, 1.0, n_out=3)
+    got, ref = _run(L, x), L.ref(x)
+    assert np.array_equal(got, ref), int((got != ref).sum())
+
+
 def test_grouped_argument_errors():
     L = GroupedLayer(128, 256, 4, 64, False)
     bad = B.make_weight(L.d_w, L.d_s, None, 128, 256, 4, 48)          # g % 32 != 0
