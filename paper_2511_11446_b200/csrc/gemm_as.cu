@@ -216,7 +216,7 @@ gemm_as_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         const int buf = g & 1;
         ok = epi.tile(p, slice * slice_w + sub * ap.bns + col0, ncols,
                       strip * (2 * BM) + static_cast<int>(rank) * BM, tmem_base, buf * (TCOLS / 2) + col0,
-                      &acc_full[buf], (g >> 1) & 1u, buf, abort_flag);
+                      &acc_full[buf], (g >> 1) & 1u, buf, g + 2 < (unit1 - unit0) * ap.nsub, abort_flag);
       }
     }
   }

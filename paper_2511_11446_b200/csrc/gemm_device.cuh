@@ -264,11 +264,14 @@ struct RowEpilogue {
   // Output columns col .. col + ncols - 1 (col and ncols multiples of 32, ncols at most 128), this
   // CTA's tokens cta_row0 .. +127; their accumulators start at tensor-memory column t_col (buffer
   // `buf`, published on acc_full with phase aph). False if the wait was aborted.
+  // reused: another tile will be accumulated in the buffer. Only then is it handed back: the arrival may be a
+  // write into the other CTA of a pair, and one that no tile waits for could land after that CTA has exited, on a
+  // barrier of the next CTA there.
   // RES: the kernel takes the residual (and gate) of GemmParams into the output; without it those
   // members are ignored.
   template <bool RES = false>
   __device__ __forceinline__ bool tile(const GemmParams& p, int col, int ncols, int cta_row0, uint32_t tmem_base,
-                                       uint32_t t_col, uint64_t* acc_full, uint32_t aph, int buf,
+                                       uint32_t t_col, uint64_t* acc_full, uint32_t aph, int buf, bool reused,
                                        volatile int* abort_flag) {
     // this lane's tokens: row0 + 8 * i, i < 4; its channels of a round: col + 32 * round + tc .. + 7
     const int64_t row0 = static_cast<int64_t>(cta_row0) + qd * 32 + (lane >> 2);
@@ -403,7 +406,7 @@ struct RowEpilogue {
       } else {  // this warp's last accumulators are in registers: hand the buffer back
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(buf ? acc_empty_addr1 : acc_empty_addr0);
+        if (lane == 0 && reused) mbar_arrive_cluster(buf ? acc_empty_addr1 : acc_empty_addr0);
       }
       emit(hi, c, 2, rr, gg);
     }

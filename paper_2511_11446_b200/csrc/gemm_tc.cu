@@ -294,7 +294,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const int buf = tcount & 1;
       ok = epi.template tile<RES>(p, (tile % p.n_tiles) * BN + col0, NCOLS,
                     (tile / p.n_tiles) * (BM * CG) + static_cast<int>(rank) * BM, tmem_base,
-                    buf * (TCOLS / 2) + col0, &acc_full[buf], (tcount >> 1) & 1, buf, abort_flag);
+                    buf * (TCOLS / 2) + col0, &acc_full[buf], (tcount >> 1) & 1, buf,
+                    tile + 2 * tile_stride < total_tiles, abort_flag);
     }
   } else {
     // ================= unpack (3/4-bit weights) =================

@@ -236,7 +236,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     for (int item = item0; item < item1 && ok; ++item, ++tcount) {
       const int buf = tcount & 1;
       ok = epi.tile(p, strip_of(item) * BN + col0, NCOLS, mtile_of(item) * (BM * CG) + static_cast<int>(rank) * BM,
-                    tmem_base, buf * (TCOLS / 2) + col0, &acc_full[buf], (tcount >> 1) & 1, buf, abort_flag);
+                    tmem_base, buf * (TCOLS / 2) + col0, &acc_full[buf], (tcount >> 1) & 1, buf, item + 2 < item1, abort_flag);
     }
   } else {
     // ================= weight expansion (3/4-bit): once per strip =================

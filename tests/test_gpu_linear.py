@@ -328,6 +328,28 @@ def test_default_dispatch_and_argument_errors():
     B.dp_wq_linear(L.w, xt, 1152, None, 0, y, 128, ws)   # M = 0: no-op
 
 
+@pytest.mark.parametrize("flags", [B.DP_FLAG_CTA_PAIR | B.DP_FLAG_TILE_N(128), B.DP_FLAG_CTA_PAIR | B.DP_FLAG_TILE_N(192),
+                                   B.DP_FLAG_ACT_STATIONARY | B.DP_FLAG_TILE_N(64), B.DP_FLAG_WEIGHT_STATIONARY],
+                         ids=["pair128", "pair192", "act_stationary", "weight_stationary"])
+@pytest.mark.parametrize("K", [128, 384])
+def test_pair_kernels_in_quick_succession(flags, K):
+    """CTA pairs of a few k-blocks and one or two tiles, one launch taking the SMs that the one before it leaves: no
+    arrival on a barrier of a CTA that has exited may reach its successor's."""
+    M, N, calls = 1300, 768, 200
+    x, w, s_w, b = _case(M, K, N, 8)
+    L = DevLayer(w, s_w, b, 8)
+    xd = torch.from_numpy(x.view(np.int16).copy()).cuda().view(torch.bfloat16)
+    ys = torch.zeros((calls, M, N), dtype=torch.bfloat16, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(B.dp_wq_linear_workspace(M, N, K, 8, flags), dtype=torch.uint8, device="cuda")
+    for i in range(calls):
+        B.dp_wq_linear(L.w, xd, K, None, M, ys[i], N, ws, None, status, flags | B.DP_FLAG_FORCE_MMA)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(ys.view(torch.int16), ys[:1].view(torch.int16).expand(calls, M, N))
+    assert np.array_equal(ys[0].view(torch.int16).cpu().numpy().view(np.uint16), oracle.wq_linear(x, oracle.pack(w, 8), s_w, b, 8))
+
+
 @pytest.mark.parametrize("bits", [8, 3])
 @pytest.mark.parametrize("bn", [0, 64])
 @pytest.mark.parametrize("M,K,N", [(33, 4608, 1152), (128, 2304, 128), (129, 4608, 256), (300, 4608, 1152), (520, 4608, 1152),
