@@ -241,7 +241,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
                       uint32_t flags, cudaStream_t stream, const CUtensorMap* tmap_w, int bn, int cg, int ws,
                       const CUtensorMap* tmap_a_cached, bool chained, int32_t* daq_sync = nullptr,
                       int pre = -1, int daq_rank = 1, int daq_bits = 8, const dp_residual* res = nullptr,
-                      bool ahead = false, int part = PART_BOTH) {
+                      bool ahead = false, int part = PART_BOTH, bool in_plan = false) {
   const bool pdl = !(flags & DP_FLAG_NO_PDL);
   if (w->bits == 16)  // a layer the plan keeps in 16-bit precision: no DAQ, no scales (checked by the caller)
     return launch_gemm_bf16(x, ldx, w->qweight, static_cast<const uint16_t*>(w->bias), M, w->N, w->K,
@@ -314,6 +314,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     a.dbg_acc = dbg ? dbg->acc : nullptr;
     a.dbg_ldacc = dbg ? dbg->ldacc : 0;
     a.early_w = chained ? 1 : 0;
+    a.hold = in_plan && !chained;
     a.status = status;
     return launch_simt_linear(a, stream, pdl);
   }
@@ -1060,6 +1061,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     ga.K = G.w.K;
     ga.n_layers = static_cast<int32_t>(grp.size());
     ga.early_w = run->chained ? 1 : 0;
+    ga.hold = !run->chained;
     ga.status = status;
     ga.daq_rank = robust ? clip_rank_of(plan->daq_p_e3, G.w.K) : 1;
     ga.daq_bits = act_bits;
@@ -1105,7 +1107,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     const int st = run_linear(&L.w, xs[l], L.w.K, nullptr, L.M, ys[l], L.w.N, scratch, nullptr, status, plan->flags, stream,
                               L.simt ? nullptr : &L.tmap_w, L.bn, L.cg, L.ws, ta, run->chained,
                               L.simt ? nullptr : plan->daq_sync, L.simt ? 0 : L.pre,
-                              robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead, part);
+                              robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead, part, true);
     gemm_set_next_reads(nullptr, 0, nullptr, 0);
     run->chained = true;
     return st;

@@ -64,6 +64,7 @@ struct SimtArgs {
   int32_t* dbg_acc;
   int64_t dbg_ldacc;
   int32_t early_w;  // weights may be fetched before the preceding kernel on the stream has finished
+  int32_t hold;     // first launch of a plan run: dependents start only once what precedes it has finished
   int32_t* status;  // device word raised to DP_ERR_TIMEOUT when a bounded wait expires (may be null)
 };
 int launch_simt_linear(const SimtArgs& a, cudaStream_t stream, bool pdl);
@@ -80,7 +81,7 @@ struct SimtGroupArgs {
   } layer[kSimtGroupMax];
   int64_t M;
   int32_t N, K, n_layers;
-  int32_t early_w;
+  int32_t early_w, hold;  // as in SimtArgs
   // Scratch for the group's int8 tokens [n_layers][M][K] and scales [n_layers][M]: when given, one
   // small kernel quantizes all tokens of the group first and the main kernel's CTAs only fetch the
   // codes; when null every CTA quantizes its tokens itself.

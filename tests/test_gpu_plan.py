@@ -442,3 +442,83 @@ def test_plan_layers_beside_each_other(M, feed):
             assert torch.equal(a, b), (l, bits[l])
     finally:
         B.dp_plan_destroy(plan)
+
+
+LATE_COPY = r"""
+extern "C" __global__ void late_copy(unsigned int* dst, const unsigned int* src, int n, long long cycles) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const long long t0 = clock64();
+  while (clock64() - t0 < cycles) {}
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+"""
+
+
+@pytest.mark.parametrize("clip", [100000, 99900])
+@pytest.mark.parametrize("grouped", [True, False], ids=["grouped_small_m", "one_by_one"])
+@pytest.mark.parametrize("first", ["small", "packed", "group_wise", "sixteen", "eight"])
+def test_constants_written_by_a_kernel_that_starts_its_dependents_early(first, grouped, clip):
+    """Whatever a plan launches first, no layer reads its constants (weights, scales, zero-points, biases) before
+    the kernel in front of the call has written them, although that kernel lets the plan's first launch start at once."""
+    K, N, M = 256, 256, 200
+    kinds = ["small", "packed", "group_wise", "sixteen", "eight", "small", "group_wise"]
+    kinds = kinds[kinds.index(first):] + kinds[:kinds.index(first)]
+    rng = np.random.default_rng(len(first))
+    parts, size = [], 0  # per layer: byte offsets of weights, scales, zero-points, bias
+
+    def place(a):
+        nonlocal size
+        b = np.ascontiguousarray(a).view(np.uint8).ravel()
+        at, size = size, size + (b.size + 255) // 256 * 256
+        parts.append((at, b))
+        return at
+
+    spec = []
+    for l, kind in enumerate(kinds):
+        bits = {"small": 4, "packed": 3, "group_wise": 4, "sixteen": 16, "eight": 8}[kind]
+        g = 64 if kind == "group_wise" else 0
+        if bits == 16:
+            wt = (rng.standard_normal((N, K)) * 0.05).astype(np.float32).view(np.uint32) >> 16
+            w_at, s_at = place(wt.astype(np.uint16)), 0
+        else:
+            w, s_w = synth.weights(SEED, l, N, K, bits)
+            w_at = place(B.dp_pack_weights_host(w, bits))
+            s_at = place(rng.random((N, K // g)).astype(np.float32) * 1e-2 if g else s_w)
+        z_at = place(rng.integers(0, 16, (N, K // g)).astype(np.uint8)) if g else None
+        spec.append((bits, g, w_at, s_at, z_at, place(synth.bias(SEED, l, N))))
+    real = np.zeros(size, np.uint8)
+    for at, b in parts:
+        real[at:at + b.size] = b
+    real = torch.from_numpy(real).cuda()
+    live = real.clone()
+    base = live.data_ptr()
+    ws_ = [B.dp_weight(N, K, bits, g, base + w, base + s, base + b, None if z is None else base + z)
+           for bits, g, w, s, z, b in spec]
+    Ms = [8 if kind == "small" else M for kind in kinds]
+    plan = B.dp_plan_create(ws_, Ms, B.DP_FLAG_GROUP_SMALL_M if grouped else 0)
+    try:
+        B.dp_plan_set_daq(plan, clip, 0)
+        ws = torch.empty(B.dp_plan_workspace(plan), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        xs = [to_dev_bf16(synth.activations(SEED, l, 0, m, K, 1.0, n_out=2)) for l, m in enumerate(Ms)]
+        ys = [torch.zeros((m, N), dtype=torch.bfloat16, device="cuda") for m in Ms]
+        xp, yp = B.ptr_array([t.data_ptr() for t in xs]), B.ptr_array([t.data_ptr() for t in ys])
+        late = torch.cuda._compile_kernel(LATE_COPY, "late_copy")
+        want = None
+        for cycles in (0, 400000, 400000):
+            live.fill_(0xA7)
+            for t in ys:
+                t.zero_()
+            torch.cuda.synchronize()
+            late((8, 1, 1), (256, 1, 1), (live.view(torch.int32), real.view(torch.int32), size // 4, cycles))
+            if want is None:  # once with everything written before the call
+                torch.cuda.synchronize()
+            B.dp_plan_run(plan, [0], 0, xp, yp, ws, status)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0
+            got = [t.view(torch.int16).clone() for t in ys]
+            want = got if want is None else want
+            for l, (a, b) in enumerate(zip(got, want)):
+                assert torch.equal(a, b), (l, kinds[l])
+    finally:
+        B.dp_plan_destroy(plan)
