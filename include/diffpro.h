@@ -68,7 +68,7 @@ typedef void* dp_stream;
  * channels with a scale and a zero-point each): group_size = g > 0 (g % 32 == 0, K % g == 0, bits in
  * {3, 4, 8}, N % 128 == 0) makes s_w fp32 [N][K/g], one scale per output channel and group of g
  * consecutive k, and `zeros` uint8 [N][K/g] or NULL the zero-points in code units (any byte value; NULL =
- * 2^(bits-1), the symmetric code): the weight is s_w[n][k/g] * (u[n][k] - zeros[n][k/g]). The layer is then
+ * 2^(bits-1), the symmetric code; K/g <= 160 with zero-points): the weight is s_w[n][k/g] * (u[n][k] - zeros[n][k/g]). The layer is then
  *     acc_G = sum_{k in group G} q[m,k] * (u[n,k] - z[n,G])            (exact int32)
  *     t = 0;  for G = 0 .. K/g - 1:  t = fma((float)acc_G, s_w[n][G], t)   (fp32, in this order)
  *     y = bf16_rne(fma(t, s_a[m], bias[n]))

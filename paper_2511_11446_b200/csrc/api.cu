@@ -253,6 +253,8 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     // launch, which takes their zero-points off as far as a byte allows), the per-group code sums
     // when 8-bit codes have zero-points, then the folding GEMM.
     const uint8_t* zeros = static_cast<const uint8_t*>(w->zeros);
+    if (zeros != nullptr && w->K / w->group_size > kGrpZeroMaxGroups)
+      return fail(DP_ERR_SHAPE, "group-wise zero-points: more than %d groups per row", kGrpZeroMaxGroups);
     uint8_t* ws8 = static_cast<uint8_t*>(workspace);
     int8_t* wq = static_cast<int8_t*>(workspace);
     float* wsa = reinterpret_cast<float*>(ws8 + align256(scratch_q_bytes(M, w->K)));

@@ -176,6 +176,7 @@ int gemm_bf16_init_device();
 int gemm_grp_init_device();
 
 // gemm_grp.cu -- layers with group-wise weight scales (and zero-points): folding tensor-core kernel.
+constexpr int kGrpZeroMaxGroups = 160;  // per row, of a layer with zero-points (K <= 5120 at g = 32)
 // (for packed weights the expansion has taken the zero-points up to 128 off already)
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
                     int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,

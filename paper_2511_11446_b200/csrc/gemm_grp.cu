@@ -451,11 +451,11 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
 // fold), from the tiled scratch the DAQ launch wrote ([row tile][k block][128][128]) or a row-major q.
 // One warp per token: a lane sums 16 consecutive codes per load (a group is a multiple of 32 codes,
 // so the 16 belong to one group) and adds the partial sum to the group's counter in shared memory.
-constexpr int kRowsumWarps = 8, kRowsumMaxGroups = 160;  // K <= 5120 at g = 32
+constexpr int kRowsumWarps = 8;
 __global__ void __launch_bounds__(kRowsumWarps * 32)
 group_rowsum_kernel(const int8_t* __restrict__ q, int64_t M, int K, int64_t ldq, int tiled, int g, int ng,
                     int32_t* __restrict__ rowsum) {
-  __shared__ int sums[kRowsumWarps][kRowsumMaxGroups];
+  __shared__ int sums[kRowsumWarps][kGrpZeroMaxGroups];
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t m = static_cast<int64_t>(blockIdx.x) * kRowsumWarps + warp;
@@ -502,7 +502,6 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   const int form = zeros == nullptr ? ZP_NONE : bits == 8 ? ZP_8BIT : ZP_PACKED;
   if (form == ZP_PACKED && !a_tiled) return fail(DP_ERR_INVALID_ARG, "packed group-wise layer: the codes are not tiled");
   if (form == ZP_8BIT) {
-    if (ng > kRowsumMaxGroups) return fail(DP_ERR_SHAPE, "group-wise zero-points: more than %d groups per row", kRowsumMaxGroups);
     const cudaError_t e = launch(group_rowsum_kernel, dim3(static_cast<unsigned>((M + kRowsumWarps - 1) / kRowsumWarps)),
                                  dim3(kRowsumWarps * 32), 0, stream, pdl, q, M, static_cast<int>(K), ldq,
                                  a_tiled ? 1 : 0, static_cast<int>(g), ng, rowsum);

@@ -41,11 +41,15 @@ class GroupedLayer:
 
 
 def _run(L, x):
+    return _run_dev(L, to_dev_bf16(x))
+
+
+def _run_dev(L, x):
     M = x.shape[0]
     y = torch.full((M, L.N), float("nan"), dtype=torch.bfloat16, device="cuda")
     ws = torch.empty(B.dp_wq_linear_workspace_grouped(M, L.dw), dtype=torch.uint8, device="cuda")
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
-    B.dp_wq_linear(L.dw, to_dev_bf16(x), L.K, None, M, y, L.N, ws, None, st, 0)
+    B.dp_wq_linear(L.dw, x, L.K, None, M, y, L.N, ws, None, st, 0)
     torch.cuda.synchronize()
     assert int(st.item()) == 0
     return bf16_to_np(y)
@@ -143,6 +147,12 @@ def test_grouped_argument_errors():
     with pytest.raises(B.DiffproError) as e:                          # workspace too small
         B.dp_wq_linear(L.dw, x, 256, None, 8, y, 128, ws[:256])
     assert e.value.status == B.DP_ERR_WORKSPACE
+    for bits in (3, 4, 8):                                            # more than 160 groups of zero-points to a row
+        Lw = GroupedLayer(128, 5248, bits, 32, True)
+        xw = torch.zeros((8, 5248), dtype=torch.bfloat16, device="cuda")
+        with pytest.raises(B.DiffproError) as e:
+            _run_dev(Lw, xw)
+        assert e.value.status == B.DP_ERR_SHAPE
     zl = B.make_weight(L.d_w, L.d_s, None, 128, 256, 4, 0, L.d_s)     # zero-points without groups
     with pytest.raises(B.DiffproError) as e:
         B.dp_wq_linear(zl, x, 256, None, 8, y, 128, ws)
