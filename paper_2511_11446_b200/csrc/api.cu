@@ -229,6 +229,12 @@ static int check_weight(const dp_weight* w) {
   return DP_OK;
 }
 
+static int check_zero_groups(const dp_weight& w) {
+  if (w.group_size > 0 && w.zeros != nullptr && w.K / w.group_size > kGrpZeroMaxGroups)
+    return fail(DP_ERR_SHAPE, "group-wise zero-points: more than %d groups per row", kGrpZeroMaxGroups);
+  return DP_OK;
+}
+
 // One layer, all checks done. tmap_w may be a pre-encoded descriptor (plan) or nullptr.
 // `chained`: the kernel preceding this layer's first launch on the stream is a launch of the same
 // dp_plan_run call, so it cannot be a producer of this layer's weights and they may be prefetched
@@ -253,8 +259,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     // launch, which takes their zero-points off as far as a byte allows), the per-group code sums
     // when 8-bit codes have zero-points, then the folding GEMM.
     const uint8_t* zeros = static_cast<const uint8_t*>(w->zeros);
-    if (zeros != nullptr && w->K / w->group_size > kGrpZeroMaxGroups)
-      return fail(DP_ERR_SHAPE, "group-wise zero-points: more than %d groups per row", kGrpZeroMaxGroups);
+    if (int zst = check_zero_groups(*w)) return zst;
     uint8_t* ws8 = static_cast<uint8_t*>(workspace);
     int8_t* wq = static_cast<int8_t*>(workspace);
     float* wsa = reinterpret_cast<float*>(ws8 + align256(scratch_q_bytes(M, w->K)));
@@ -1078,8 +1083,6 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     for (size_t i = 0; i < grp.size(); ++i) {
       const int l = grp[i];
       const PlanLayer& L = plan->layers[l];
-      if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", l);
-      if (!aligned16(xs[l]) || !aligned16(ys[l])) return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", l);
       ga.layer[i] = {xs[l], static_cast<uint16_t*>(ys[l]), L.w.qweight, L.w.s_w,
                      static_cast<const uint16_t*>(L.w.bias), L.w.bits};
     }
@@ -1131,8 +1134,6 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
   for (int l = 0; l < n; ++l) {
     const PlanLayer& L = plan->layers[l];
     if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
-    if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", l);
-    if (!aligned16(xs[l]) || !aligned16(ys[l])) return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", l);
     if (L.simt || L.w.bits == 16 || L.w.group_size > 0 || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
       if (int st = flush()) return st;
       const CUtensorMap* ta = nullptr;
@@ -1181,6 +1182,19 @@ static int check_plan_run(const dp_plan* plan, const int32_t* steps, int32_t n_s
   return DP_OK;
 }
 
+// The layers' pointers of one step (xs: host memory when the plan stages its inputs, of any alignment then).
+static int check_plan_step(const dp_plan* plan, const void* const* xs, void* const* ys, bool x_on_host) {
+  for (size_t l = 0; l < plan->layers.size(); ++l) {
+    const PlanLayer& L = plan->layers[l];
+    if (L.M == 0) continue;
+    if (!xs[l] || !ys[l]) return fail(DP_ERR_INVALID_ARG, "layer %d: NULL x or y", static_cast<int>(l));
+    if ((!x_on_host && !aligned16(xs[l])) || !aligned16(ys[l]))
+      return fail(DP_ERR_ALIGN, "layer %d: x/y misaligned", static_cast<int>(l));
+    if (int st = check_zero_groups(L.w)) return st;
+  }
+  return DP_OK;
+}
+
 extern "C" int dp_plan_run(const dp_plan* plan_c, const int32_t* steps, int32_t n_steps,
                            int32_t start_index, const void* const* x_ptrs, void* const* y_ptrs,
                            void* workspace, size_t workspace_bytes, int32_t* device_status,
@@ -1190,8 +1204,15 @@ extern "C" int dp_plan_run(const dp_plan* plan_c, const int32_t* steps, int32_t 
   if (st != DP_OK) return st;
   dp_plan* plan = const_cast<dp_plan*>(plan_c);
   const int64_t n = static_cast<int64_t>(plan->layers.size());
+  const int32_t visited = n_steps - start_index;
+  for (int32_t i = 0; i < visited; ++i) {  // before anything is launched
+    if (i > 0 && (flags & DP_PLAN_SAME_X) && (flags & DP_PLAN_SAME_Y)) break;
+    st = check_plan_step(plan, x_ptrs + ((flags & DP_PLAN_SAME_X) ? 0 : i * n), y_ptrs + ((flags & DP_PLAN_SAME_Y) ? 0 : i * n),
+                         false);
+    if (st != DP_OK) return st;
+  }
   PlanRun run;
-  for (int32_t i = n_steps - 1 - start_index; i >= 0; --i) {  // reverse(K*)
+  for (int32_t i = visited - 1; i >= 0; --i) {  // reverse(K*)
     const void* const* xs = x_ptrs + ((flags & DP_PLAN_SAME_X) ? 0 : i * n);
     void* const* ys = y_ptrs + ((flags & DP_PLAN_SAME_Y) ? 0 : i * n);
     st = plan_run_step(plan, steps[i], xs, ys, workspace, device_status, static_cast<cudaStream_t>(stream), &run);
@@ -1215,6 +1236,10 @@ extern "C" int dp_plan_run_host(const dp_plan* plan_c, const int32_t* steps, int
     return fail(DP_ERR_WORKSPACE, "x_stage needs %zu bytes, 256-byte aligned", 2 * plan->x_bytes);
   if (d2h_layer >= n || (d2h_layer >= 0 && !y_host))
     return fail(DP_ERR_INVALID_ARG, "bad d2h_layer / y_host");
+  for (int32_t i = 0; i < ((flags & DP_PLAN_SAME_X) ? std::min(n_steps, 1) : n_steps); ++i) {
+    st = check_plan_step(plan, x_host + i * n, y_dev, true);
+    if (st != DP_OK) return st;
+  }
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   std::vector<const void*> xs(n);
   // The copy stream starts behind everything already enqueued on `stream`: an earlier call's last
@@ -1231,7 +1256,6 @@ extern "C" int dp_plan_run_host(const dp_plan* plan_c, const int32_t* steps, int
       const PlanLayer& L = plan->layers[l];
       xs[l] = stage + L.x_offset;
       if (L.M == 0) continue;
-      if (!src[l]) return fail(DP_ERR_INVALID_ARG, "layer %lld: NULL host input", (long long)l);
       DP_CUDA_OK(cudaMemcpyAsync(stage + L.x_offset, src[l], static_cast<size_t>(L.M) * L.w.K * 2,
                                  cudaMemcpyHostToDevice, plan->copy_stream));
     }

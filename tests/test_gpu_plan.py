@@ -303,6 +303,41 @@ def test_plan_errors():
         B.dp_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("host", [False, True], ids=["device_inputs", "host_inputs"])
+@pytest.mark.parametrize("fault", ["null_y", "odd_y", "null_x"])
+def test_nothing_runs_when_a_pointer_of_any_step_is_wrong(host, fault):
+    """Argument errors are found before the first launch, wherever in the schedule the bad pointer stands: no output of
+    the call is written (dp_plan_run launches a layer's GEMM behind the quantization of the next)."""
+    K, Ms, n_steps = 256, [200, 300, 8, 200], 2
+    dev = []
+    for l in range(len(Ms)):
+        w, s_w = synth.weights(SEED, l, 256, K, (8, 4, 4, 3)[l])
+        dev.append(DevLayer(w, s_w, None, (8, 4, 4, 3)[l]))
+    plan = B.dp_plan_create([d.w for d in dev], Ms, B.DP_FLAG_GROUP_SMALL_M)
+    try:
+        n = len(Ms)
+        ws = torch.empty(B.dp_plan_workspace(plan), dtype=torch.uint8, device="cuda")
+        x = torch.zeros((n_steps, n, 300, K), dtype=torch.bfloat16, device="cpu" if host else "cuda")
+        y = torch.full((n_steps, n, 300, 256), 7.0, dtype=torch.bfloat16, device="cuda")
+        xp = [x[i, l].data_ptr() for i in range(n_steps) for l in range(n)]
+        yp = [y[i, l].data_ptr() for i in range(1 if host else n_steps) for l in range(n)]
+        if fault == "null_x":
+            xp[n - 1] = None        # of the step visited last
+        else:
+            yp[n - 1] = None if fault == "null_y" else yp[n - 1] + 2
+        with pytest.raises(B.DiffproError) as e:
+            if host:
+                stage = torch.empty(2 * B.dp_plan_x_bytes(plan), dtype=torch.uint8, device="cuda")
+                B.dp_plan_run_host(plan, [0, 1], B.ptr_array(xp), stage, B.ptr_array(yp), -1, None, ws)
+            else:
+                B.dp_plan_run(plan, [0, 1], 0, B.ptr_array(xp), B.ptr_array(yp), ws)
+        assert e.value.status == (B.DP_ERR_ALIGN if fault == "odd_y" else B.DP_ERR_INVALID_ARG)
+        torch.cuda.synchronize()
+        assert bool((y == 7.0).all())
+    finally:
+        B.dp_plan_destroy(plan)
+
+
 def test_phase_a_on_measured_latencies_matches_oracle_and_runs():
     """Algorithm 2 end to end on a small stack: c_lat(l, b) measured with the library's kernels, Phase A
     (library) equal to the oracle's on the same table, and the resulting bit plan and kept steps run by
