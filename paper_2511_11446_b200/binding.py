@@ -151,7 +151,7 @@ def _calls():
             raise RuntimeError("the call module is missing: build it with `python -m paper_2511_11446_b200.build`") from e
         addr = lambda f: C.cast(f, C.c_void_p).value
         m.bind(addr(L.dp_wq_linear), addr(L.dp_wq_linear_residual), addr(L.dp_daq_quantize), addr(L.dp_ln_modulate_daq),
-               torch.cuda.current_device, torch._C._cuda_getCurrentRawStream)
+               torch.cuda.current_device, torch._C._cuda_getCurrentRawStream, dp_weight, dp_debug, C.ArgumentError)
         _call = m
     return _call
 
@@ -195,8 +195,7 @@ def dp_daq_quantize_robust(x, M, K, ldx, q, ldq, s_a, rank, act_bits=8, rowsum=N
 
 def dp_wq_linear(w: dp_weight, x, ldx, s_a_in, M, y, ldy, workspace, dbg: dp_debug | None = None,
                  device_status=None, flags=0, stream=None):
-    _check((_call or _calls()).wq_linear(C.addressof(w), x, ldx, s_a_in, M, y, ldy, workspace,
-                                         0 if dbg is None else C.addressof(dbg), device_status, flags, stream),
+    _check((_call or _calls()).wq_linear(w, x, ldx, s_a_in, M, y, ldy, workspace, dbg, device_status, flags, stream),
            "dp_wq_linear")
 
 
@@ -214,7 +213,7 @@ def dp_wq_linear_residual(w: dp_weight, x, ldx, M, residual, ldr, gate, rows_per
                           device_status=None, flags=0, stream=None):
     """dp_wq_linear on bf16 activations with y = bf16(gate * lin + residual) (gate None: lin + residual)
     in the epilogue; residual may be y."""
-    _check((_call or _calls()).wq_linear_residual(C.addressof(w), x, ldx, M, residual, ldr, gate, rows_per_gate, y, ldy,
+    _check((_call or _calls()).wq_linear_residual(w, x, ldx, M, residual, ldr, gate, rows_per_gate, y, ldy,
                                                   workspace, ws_bytes, device_status, flags, stream),
            "dp_wq_linear_residual")
 

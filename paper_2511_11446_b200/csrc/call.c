@@ -2,7 +2,7 @@
  * arguments costs 1.5 us before the library sees it and the Python around it (pointers, sizes, the current
  * stream) another 1.5, next to 2.3 us for a launch: a one-launch call took 5.9 us of host time, 4.3 this way (the
  * adaLN layer for one token 6.0 -> 5.2 us a call, proj at 256 tokens 8.0 -> 6.7).
- * The functions' addresses and torch's stream lookup are handed in once by the binding (bind). */
+ * The functions' addresses, torch's stream lookup and the structures' types are handed in once by the binding (bind). */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -17,6 +17,7 @@ static int (*f_daq)(const void*, int64_t, int64_t, int64_t, int8_t*, int64_t, fl
 static int (*f_ln)(const void*, int64_t, int64_t, int64_t, const void*, const void*, int64_t, float, int8_t*, int64_t,
                    float*, dp_stream);
 static PyObject *g_get_device, *g_get_stream; /* torch.cuda.current_device, torch._C._cuda_getCurrentRawStream */
+static PyObject *g_weight, *g_debug, *g_arg_error; /* the ctypes structures dp_weight and dp_debug, ctypes.ArgumentError */
 static PyObject *s_data_ptr, *s_nbytes, *s_cuda_stream;
 
 /* The converters leave a Python error behind; callers look once, before the call, with PyErr_Occurred. */
@@ -53,6 +54,19 @@ static dp_stream stream_of(PyObject* s) { /* a torch stream, or None: the curren
 }
 static int64_t as_i64(PyObject* o) { return PyErr_Occurred() ? 0 : PyLong_AsLongLong(o); }
 static void* as_addr(PyObject* o) { return PyErr_Occurred() ? NULL : PyLong_AsVoidPtr(o); }
+/* The memory of a ctypes structure, which has to be of that type: another one's would be read past its end. */
+static void* as_struct(PyObject* o, PyObject* type) {
+  Py_buffer b;
+  if (PyErr_Occurred()) return NULL;
+  if (!PyObject_TypeCheck(o, (PyTypeObject*)type)) {
+    PyErr_Format(g_arg_error, "expected %s instance instead of %s", ((PyTypeObject*)type)->tp_name, Py_TYPE(o)->tp_name);
+    return NULL;
+  }
+  if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE)) return NULL;
+  void* p = b.buf;
+  PyBuffer_Release(&b); /* (the caller's reference keeps it) */
+  return p;
+}
 static uint32_t as_flags(PyObject* o) { return PyErr_Occurred() ? 0 : (uint32_t)PyLong_AsUnsignedLongMask(o); }
 
 static int args_ok(Py_ssize_t n, Py_ssize_t want) {
@@ -61,11 +75,11 @@ static int args_ok(Py_ssize_t n, Py_ssize_t want) {
   return 0;
 }
 
-/* (weight address, x, ldx, s_a_in, M, y, ldy, workspace, debug address or 0, device_status, flags, stream) */
+/* (weight, x, ldx, s_a_in, M, y, ldy, workspace, debug or None, device_status, flags, stream) */
 static PyObject* wq_linear(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   (void)self;
   if (!args_ok(n, 12)) return NULL;
-  const dp_weight* w = as_addr(a[0]);
+  const dp_weight* w = as_struct(a[0], g_weight);
   const void* x = tensor_ptr(a[1]);
   const int64_t ldx = as_i64(a[2]);
   const float* sa = tensor_ptr(a[3]);
@@ -74,7 +88,7 @@ static PyObject* wq_linear(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   const int64_t ldy = as_i64(a[6]);
   void* ws = tensor_ptr(a[7]);
   const size_t wsb = tensor_bytes(a[7]);
-  const dp_debug* dbg = as_addr(a[8]);
+  const dp_debug* dbg = a[8] == Py_None ? NULL : as_struct(a[8], g_debug);
   int32_t* status = tensor_ptr(a[9]);
   const uint32_t flags = as_flags(a[10]);
   const dp_stream s = stream_of(a[11]);
@@ -86,12 +100,12 @@ static PyObject* wq_linear(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   return PyLong_FromLong(st);
 }
 
-/* (weight address, x, ldx, M, residual, ldr, gate, rows_per_gate, y, ldy, workspace, ws_bytes, device_status, flags,
+/* (weight, x, ldx, M, residual, ldr, gate, rows_per_gate, y, ldy, workspace, ws_bytes, device_status, flags,
  * stream) */
 static PyObject* wq_linear_residual(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   (void)self;
   if (!args_ok(n, 15)) return NULL;
-  const dp_weight* w = as_addr(a[0]);
+  const dp_weight* w = as_struct(a[0], g_weight);
   const void* x = tensor_ptr(a[1]);
   const int64_t ldx = as_i64(a[2]), M = as_i64(a[3]);
   dp_residual r;
@@ -154,11 +168,12 @@ static PyObject* ln_modulate_daq(PyObject* self, PyObject* const* a, Py_ssize_t 
   return PyLong_FromLong(st);
 }
 
-/* (addresses of dp_wq_linear, dp_wq_linear_residual, dp_daq_quantize, dp_ln_modulate_daq, device getter, stream getter) */
+/* (addresses of dp_wq_linear, dp_wq_linear_residual, dp_daq_quantize, dp_ln_modulate_daq, device getter, stream getter,
+ * dp_weight, dp_debug, ctypes.ArgumentError) */
 static PyObject* bind(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   (void)self;
-  if (n != 6) {
-    PyErr_SetString(PyExc_TypeError, "bind takes four addresses and two callables");
+  if (n != 9 || !PyType_Check(a[6]) || !PyType_Check(a[7])) {
+    PyErr_SetString(PyExc_TypeError, "bind takes four addresses, two callables and three types");
     return NULL;
   }
   void* p[4];
@@ -168,12 +183,11 @@ static PyObject* bind(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   *(void**)&f_residual = p[1];
   *(void**)&f_daq = p[2];
   *(void**)&f_ln = p[3];
-  Py_INCREF(a[4]);
-  Py_XDECREF(g_get_device);
-  g_get_device = a[4];
-  Py_INCREF(a[5]);
-  Py_XDECREF(g_get_stream);
-  g_get_stream = a[5];
+  PyObject** keep[5] = {&g_get_device, &g_get_stream, &g_weight, &g_debug, &g_arg_error};
+  for (int i = 0; i < 5; ++i) {
+    Py_INCREF(a[4 + i]);
+    Py_XSETREF(*keep[i], a[4 + i]);
+  }
   Py_RETURN_NONE;
 }
 

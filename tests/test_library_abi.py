@@ -24,6 +24,21 @@ def test_exports_match_header():
     assert L.dp_status_string(B.DP_ERR_TIMEOUT).decode() == "DP_ERR_TIMEOUT"
 
 
+def test_per_layer_calls_take_their_own_structures_only():
+    """The call module reads a structure's memory: anything but a dp_weight (and a dp_debug or None) is refused before that,
+    as ctypes refuses it for the other calls."""
+    import ctypes
+    w = B.dp_weight(128, 128, 8, 0)
+    for bad in (B.dp_debug(), ctypes.pointer(w), ctypes.byref(w), 0, None):
+        with pytest.raises(ctypes.ArgumentError):
+            B.dp_wq_linear(bad, None, 128, None, 0, None, 128, None)
+        with pytest.raises(ctypes.ArgumentError):
+            B.dp_wq_linear_residual(bad, None, 128, 0, None, 128, None, 1, None, 128, None, 0)
+    for bad in (w, 0):
+        with pytest.raises(ctypes.ArgumentError):
+            B.dp_wq_linear(w, None, 128, None, 0, None, 128, None, bad)
+
+
 def test_probe_library_exports_its_header():
     """The measurement probes live in a library of their own, outside the product ABI."""
     from paper_2511_11446_b200 import probe
