@@ -25,7 +25,8 @@ SOURCES = ["api.cu", "daq.cu", "simt.cu", "gemm_tc.cu", "gemm_ws.cu", "gemm_as.c
 SYNTH_SOURCES = ["synth_cuda.cu"]
 PROBE_LIB = os.path.join(HERE, "libdpprobe.so")
 PROBE_SOURCES = ["peak.cu"]
-CALL_LIB = os.path.join(HERE, "_call.so")
+# Named for this interpreter: another version builds (and imports) its own.
+CALL_LIB = os.path.join(HERE, "_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 CALL_SOURCE = os.path.join(CSRC, "call.c")
 CC = os.environ.get("CC", "gcc")
 

@@ -39,6 +39,12 @@ def test_per_layer_calls_take_their_own_structures_only():
             B.dp_wq_linear(w, None, 128, None, 0, None, 128, None, bad)
 
 
+def test_call_module_is_this_interpreters():
+    """The call module is C against this interpreter's headers, so its file name carries the interpreter's tag."""
+    import sysconfig
+    assert B._calls().__file__.endswith("_call" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
 def test_probe_library_exports_its_header():
     """The measurement probes live in a library of their own, outside the product ABI."""
     from paper_2511_11446_b200 import probe
