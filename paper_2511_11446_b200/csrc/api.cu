@@ -1008,8 +1008,8 @@ extern "C" void dp_plan_destroy(dp_plan* plan) {
   delete plan;
 }
 
-// The int8 activations of every tensor-path layer live at the start of the workspace, so their TMA
-// descriptor depends only on (workspace, M, K): encoded once and reused across layers and steps.
+// The int8 activations of every tensor-path layer live at the start of its part of the workspace, so their TMA
+// descriptor depends only on (part, M, K): encoded once and reused across layers and steps.
 static const CUtensorMap* cached_tmap_a(dp_plan* plan, const void* ws, int64_t M, int64_t K, int* st) {
   for (const TmapACache& c : plan->a_cache)
     if (c.ptr == ws && c.M == M && c.K == K) return &c.map;
@@ -1136,14 +1136,15 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
     if (L.simt || L.w.bits == 16 || L.w.group_size > 0 || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
       if (int st = flush()) return st;
+      uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes;
       const CUtensorMap* ta = nullptr;
       if (!L.simt && L.w.bits != 16 && L.w.group_size == 0) {
         int st = DP_OK;
-        ta = cached_tmap_a(plan, workspace, L.M, L.w.K, &st);
+        ta = cached_tmap_a(plan, scratch, L.M, L.w.K, &st);
         if (st != DP_OK) return st;
       }
       hint(l + 1);
-      if (int st = layer(l, static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes, ta, false, PART_BOTH)) return st;
+      if (int st = layer(l, scratch, ta, false, PART_BOTH)) return st;
       run->y = L.w.bits == 16 ? ys[l] : nullptr;
       run->y_elems = L.M * L.w.N;
       continue;
