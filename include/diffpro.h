@@ -321,6 +321,10 @@ int dp_wq_linear_static(const dp_weight* w, const void* x_bf16, int64_t ldx, int
 typedef struct dp_plan dp_plan;
 int dp_plan_create(const dp_weight* layers, int32_t n_layers, const int64_t* M_per_layer,
                    uint32_t flags, dp_plan** out);
+/* Bytes of device scratch a run of the plan needs (256-byte aligned). Consecutive layers use the scratch in turn, in as
+ * many parts of the largest layer's dp_wq_linear_workspace as the launch order overlaps: three where a per-channel 3-, 4- or
+ * 8-bit layer has 33 to 1024 rows, two where such layers all have more, one with DP_FLAG_NO_PDL, DP_FLAG_FUSED_DAQ or
+ * without such layers; grouped small-M layers under a DAQ policy may need more. */
 size_t dp_plan_workspace(const dp_plan* plan);
 /* Which kernel the plan runs layer `layer` with (for reports and for timing that kernel alone):
  * *tile_n = tile width in output channels, *cta_group = 1 or 2 CTAs per row tile,

@@ -655,7 +655,8 @@ struct dp_plan {
   std::vector<PlanLayer> layers;
   uint32_t flags;
   size_t workspace_bytes;
-  size_t part_bytes;  // of the three parts that consecutive layers take in turn
+  size_t part_bytes;  // of the parts that consecutive layers take in turn
+  int parts;          // see plan_parts
   size_t x_bytes;
   std::vector<TmapACache> a_cache;
   std::vector<std::vector<int>> groups;  // small-M layers of equal shape, run first in every step
@@ -668,9 +669,23 @@ struct dp_plan {
   cudaEvent_t ev_copied[2], ev_consumed[2], ev_entry;
   void need(size_t layer_bytes) {  // room for a layer of this scratch size
     part_bytes = std::max(part_bytes, align256(layer_bytes));
-    workspace_bytes = std::max(workspace_bytes, 3 * part_bytes);
+    workspace_bytes = std::max(workspace_bytes, parts * part_bytes);
   }
 };
+
+// Whether a plan launches the DAQ of this layer apart from its GEMM.
+static bool runs_in_two(const PlanLayer& L) {
+  return L.M > 0 && !L.simt && L.w.bits != 16 && L.w.group_size == 0;
+}
+// Parts of the workspace that the launch order of plan_run_step keeps in use: three where DAQ runs two layers ahead, two
+// where it runs beside the GEMM before, one where every layer runs whole.
+static int plan_parts(const dp_plan& p, bool fused_daq) {
+  if (fused_daq || (p.flags & DP_FLAG_NO_PDL)) return 1;
+  int parts = 1;
+  for (const PlanLayer& L : p.layers)
+    if (runs_in_two(L)) parts = std::max(parts, L.M <= kSkewMaxRows ? 3 : 2);
+  return parts;
+}
 
 // Times every kernel variant that can run this layer shape (the whole layer: DAQ + GEMM, as the
 // plan will launch it) and returns the fastest. Plan creation only.
@@ -796,6 +811,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   p->flags = flags;
   p->workspace_bytes = 256;
   p->part_bytes = 0;
+  p->parts = 1;
   p->x_bytes = 0;
   p->copy_stream = nullptr;
   p->daq_sync = nullptr;
@@ -868,6 +884,8 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
     p->x_bytes += align256(static_cast<size_t>(L.M) * L.w.K * 2);
     p->layers.push_back(L);
   }
+  p->parts = plan_parts(*p, fused_daq);
+  p->need(0);
   p->grouped.assign(p->layers.size(), 0);
   if (group_small) {
     for (size_t l = 0; l < p->layers.size(); ++l) {
@@ -1038,7 +1056,7 @@ struct PlanRun {
 
 // Tensor-core layers are launched D0 D1 G0 D2 G1 D3 G2 ...: DAQ (and weight expansion) of a layer runs beside the GEMM
 // two layers before it, and a GEMM, whose operands are then complete, starts on each SM as the GEMM before it leaves
-// (only its epilogue waits for that one). A layer's operands are in one of three parts of the workspace: when D(l + 2)
+// (only its epilogue waits for that one). A layer's operands are in one of three parts (plan_parts) of the workspace: when D(l + 2)
 // starts, G(l) may be running and D(l + 1) waits for its GEMM, while G(l - 1), the last reader of the third part, is done: G(l)
 // lets D(l + 2) start after its own wait, which is for D(l + 1), one CTA of which stays until G(l - 1) has finished.
 // A layer whose input overlaps the outputs of the layer before it is launched after that layer's GEMM, and one that
@@ -1046,7 +1064,8 @@ struct PlanRun {
 // beside the GEMM before, G(l) right after D(l) / this order: 256 tokens 915 / 773 / 670 us; the last two at 1024 tokens 992 / 912,
 // 2048 with cold inputs 1359 / 1366, 4096 1989 / 2028, 8192 3620 / 3690, and 1024 with the percentile rule 1244 / 1290: where a
 // GEMM or the DAQ fills the SMs the codes wait too long and two layers' loads compete. So up to kSkewMaxRows
-// tokens and with the plain rule only; else G(l) follows D(l) at once.
+// tokens and with the plain rule only; else G(l) follows D(l) at once, and two parts are enough: D(l + 1) starts when G(l)
+// has waited for D(l), hence for G(l - 1).
 static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* const* ys, void* workspace,
                          int32_t* status, cudaStream_t stream, PlanRun* run) {
   const int n = static_cast<int>(plan->layers.size());
@@ -1134,7 +1153,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
   for (int l = 0; l < n; ++l) {
     const PlanLayer& L = plan->layers[l];
     if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
-    if (L.simt || L.w.bits == 16 || L.w.group_size > 0 || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
+    if (!runs_in_two(L) || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
       if (int st = flush()) return st;
       uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes;
       const CUtensorMap* ta = nullptr;
@@ -1158,7 +1177,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes;
     const bool ahead = run->y != nullptr && !overlap(xs[l], L.M * L.w.K, run->y, run->y_elems);
     if (int st = layer(l, scratch, nullptr, ahead, PART_DAQ)) return st;
-    run->slot = (run->slot + 1) % 3;
+    run->slot = (run->slot + 1) % plan->parts;
     run->y = nullptr;
     const bool between = run->pending >= 0;
     if (int st = flush()) return st;

@@ -338,6 +338,19 @@ def test_nothing_runs_when_a_pointer_of_any_step_is_wrong(host, fault):
         B.dp_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("Ms,flags,parts", [([2048, 1100], 0, 2), ([2048, 1024], 0, 3), ([300], 0, 3),
+                                            ([300, 2048], B.DP_FLAG_NO_PDL, 1), ([300, 2048], B.DP_FLAG_FUSED_DAQ, 1)])
+def test_workspace_has_the_parts_that_the_launch_order_uses(Ms, flags, parts):
+    K, N = 256, 256
+    w, s_w = synth.weights(SEED, 0, N, K, 8)
+    d = DevLayer(w, s_w, None, 8)
+    plan = B.dp_plan_create([d.w] * len(Ms), Ms, flags)
+    try:
+        assert B.dp_plan_workspace(plan) == parts * max(B.dp_wq_linear_workspace(M, N, K, 8) for M in Ms)
+    finally:
+        B.dp_plan_destroy(plan)
+
+
 def test_phase_a_on_measured_latencies_matches_oracle_and_runs():
     """Algorithm 2 end to end on a small stack: c_lat(l, b) measured with the library's kernels, Phase A
     (library) equal to the oracle's on the same table, and the resulting bit plan and kept steps run by
