@@ -119,11 +119,11 @@ static int forced_bn(uint32_t flags) { return static_cast<int>((flags & DP_FLAG_
 // Tile width and CTA-group size of the tensor-core kernel for this problem, honouring the tuning
 // flags (validated by check_tile_flags).
 // `bits` is the width the GEMM kernel sees (8 in the unpack-first form); `tiled_a`: the activations
-// are the library's own tiled scratch (DAQ run by the call).
-static void choose_tile(uint32_t flags, int64_t M, int32_t N, int32_t K, int32_t bits, bool tiled_a, int* bn,
+// are the library's own tiled scratch (DAQ run by the call). `fused_daq`: the kernel quantizes them itself.
+static void choose_tile(uint32_t flags, int64_t M, int32_t N, int32_t K, int32_t bits, bool tiled_a, bool fused_daq, int* bn,
                         int* cg, int* ws) {
   *ws = 0;
-  const bool as_ok = tiled_a && bits == 8 && gemm_as_supported(N, K) &&
+  const bool as_ok = tiled_a && !fused_daq && bits == 8 && gemm_as_supported(N, K) &&
                      !(flags & (DP_FLAG_NO_ACT_STATIONARY | DP_FLAG_NO_CTA_PAIR | DP_FLAG_WEIGHT_STATIONARY));
   if (as_ok && (flags & DP_FLAG_ACT_STATIONARY)) {
     int nsub = 1;
@@ -151,7 +151,7 @@ static void choose_tile(uint32_t flags, int64_t M, int32_t N, int32_t K, int32_t
   if (flags & DP_FLAG_CTA_PAIR) allow = 0x4;
   if (flags & DP_FLAG_NO_CTA_PAIR) allow = 0x2;
   int splits = 1;  // decided again by the launch, from the same numbers
-  gemm_pick_tile(M, N, K, bits, allow, 0, bn, cg, &splits);
+  gemm_pick_tile(M, N, K, bits, fused_daq ? allow | 0x10 : allow, 0, bn, cg, &splits);
   const int fb = forced_bn(flags);
   if (fb != 0 && N % fb == 0) {
     *bn = fb;
@@ -406,7 +406,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
     int st = tiled ? gemm_encode_a_tiled(&g.tmap_a, q, M, w->K) : gemm_encode_a(&g.tmap_a, q, M, w->K, ldq);
     if (st != DP_OK) return st;
   }
-  if (bn == 0) choose_tile(flags, M, w->N, w->K, w->bits, tiled, &bn, &cg, &ws);
+  if (bn == 0) choose_tile(flags, M, w->N, w->K, w->bits, tiled, fused, &bn, &cg, &ws);
   if (ws == 2 && (!tiled || w->bits != 8 || fused))
     return fail(DP_ERR_INVALID_ARG, "the activation-stationary kernel needs DAQ run by the call, 8-bit weights (or the "
                                     "unpack-first form)");
@@ -694,7 +694,7 @@ struct TunedShape {
   int32_t N, K, bits;
   int bn, cg, ws, pre;
 };
-static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool allow_as, int* bn_out, int* cg_out,
+static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool fused_daq, int* bn_out, int* cg_out,
                           int* ws_out, int* pre_out) {
   struct Cand {
     int bn, cg, ws, pre;
@@ -702,20 +702,21 @@ static int autotune_shape(const dp_weight& w, int64_t M, uint32_t flags, bool al
   std::vector<Cand> cands;
   const int widths[4] = {64, 128, 192, 256};
   // Packed layers are tried in the unpack-first form (faster at every measured size) unless the flags say otherwise.
-  const bool pre = w.bits < 8 && !(flags & (DP_FLAG_NO_UNPACK_FIRST | DP_FLAG_FUSED_DAQ));
+  const bool pre = want_unpack_first(flags, w.bits, true);
+  const bool fused = fused_daq && !pre;  // (the candidates are timed with DAQ in a kernel of its own all the same)
   const bool eight = w.bits == 8 || pre;  // the kernel sees 8-bit weights: the time model applies
   double least = 1e30;
   for (int i = 0; i < 4; ++i)
     for (int cg = 1; cg <= 2; ++cg)
-      if (w.N % widths[i] == 0) least = std::min(least, gemm_tile_cost(M, w.N, w.K, widths[i], cg));
+      if (w.N % widths[i] == 0) least = std::min(least, gemm_tile_cost(M, w.N, w.K, widths[i], cg, !fused));
   for (int i = 0; i < 4; ++i)
     if (w.N % widths[i] == 0) {
       for (int cg = 1; cg <= 2; ++cg) {
         if (cg == 2 && widths[i] < 128) continue;
-        if (!eight || gemm_tile_cost(M, w.N, w.K, widths[i], cg) < 1.25 * least) cands.push_back({widths[i], cg, 0, pre});
+        if (!eight || gemm_tile_cost(M, w.N, w.K, widths[i], cg, !fused) < 1.25 * least) cands.push_back({widths[i], cg, 0, pre});
       }
       if (widths[i] >= 192 && gemm_ws_supported(w.N, w.K) && (!eight || M >= kWsMinRows)) cands.push_back({widths[i], 2, 1, pre});
-      if (allow_as && gemm_as_supported(w.N, w.K) && eight && M >= kAsMinRows)
+      if (!fused_daq && gemm_as_supported(w.N, w.K) && eight && M >= kAsMinRows)
         cands.push_back({widths[i], 2, 2, pre});
     }
   // (the default first: a later one has to beat it)
@@ -843,18 +844,18 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
     if (!L.simt && L.M > 0 && L.w.bits != 16 && L.w.group_size == 0) {
       uint32_t lf = flags;  // a pair request that this layer's N cannot honour falls back to the default
       // DAQ inside the GEMM kernel and a DAQ launch that also expands the weights exclude each other
-      if ((lf & DP_FLAG_FUSED_DAQ) && !(lf & DP_FLAG_UNPACK_FIRST)) lf |= DP_FLAG_NO_UNPACK_FIRST;
+      if (fused_daq && !(lf & DP_FLAG_UNPACK_FIRST)) lf |= DP_FLAG_NO_UNPACK_FIRST;
       if ((lf & DP_FLAG_CTA_PAIR) && L.w.N % 128 && L.w.N % 192) lf &= ~DP_FLAG_CTA_PAIR;
       if ((lf & DP_FLAG_WEIGHT_STATIONARY) && !gemm_ws_supported(L.w.N, L.w.K)) lf &= ~DP_FLAG_WEIGHT_STATIONARY;
       L.pre = want_unpack_first(lf, L.w.bits, true) ? 1 : 0;
-      choose_tile(lf, L.M, L.w.N, L.w.K, L.pre ? 8 : L.w.bits, !fused_daq, &L.bn, &L.cg, &L.ws);
+      choose_tile(lf, L.M, L.w.N, L.w.K, L.pre ? 8 : L.w.bits, !fused_daq, fused_daq && !L.pre, &L.bn, &L.cg, &L.ws);
       if (autotune) {
         const TunedShape* hit = nullptr;
         for (const TunedShape& t : tuned)
           if (t.M == L.M && t.N == L.w.N && t.K == L.w.K && t.bits == L.w.bits) hit = &t;
         if (hit == nullptr) {
           TunedShape t = {L.M, L.w.N, L.w.K, L.w.bits, L.bn, L.cg, L.ws, L.pre};
-          st = autotune_shape(L.w, L.M, flags, !fused_daq, &t.bn, &t.cg, &t.ws, &t.pre);
+          st = autotune_shape(L.w, L.M, lf, fused_daq, &t.bn, &t.cg, &t.ws, &t.pre);
           if (st != DP_OK) {
             delete p;
             return st;
@@ -980,9 +981,9 @@ extern "C" int dp_plan_set_layer_flags(dp_plan* plan, int32_t layer, uint32_t fl
   PlanLayer T = L;
   if ((flags & DP_FLAG_UNPACK_FIRST) && (flags & DP_FLAG_NO_UNPACK_FIRST))
     return fail(DP_ERR_INVALID_ARG, "UNPACK_FIRST and NO_UNPACK_FIRST are exclusive");
-  T.pre = want_unpack_first(flags, T.w.bits, true) ? 1 : 0;
-  choose_tile(flags, T.M, T.w.N, T.w.K, T.pre ? 8 : T.w.bits, plan->daq_sync == nullptr, &T.bn,
-              &T.cg, &T.ws);
+  const bool fused_daq = plan->daq_sync != nullptr;
+  T.pre = want_unpack_first(fused_daq && !(flags & DP_FLAG_UNPACK_FIRST) ? flags | DP_FLAG_NO_UNPACK_FIRST : flags, T.w.bits, true);
+  choose_tile(flags, T.M, T.w.N, T.w.K, T.pre ? 8 : T.w.bits, !fused_daq, fused_daq && !T.pre, &T.bn, &T.cg, &T.ws);
   if ((flags & DP_FLAG_ACT_STATIONARY) && T.ws != 2)
     return fail(DP_ERR_SHAPE, "layer %d: the activation-stationary kernel does not take this layer (N=%d K=%d, %d-bit "
                               "weights without the unpack-first form, or DAQ fused into the GEMM)",

@@ -135,12 +135,13 @@ struct GemmProblem {
   float* s_a_out;
   int32_t* sync;
 };
-// allow: bit 1 = single-CTA tiles permitted, bit 2 = CTA-pair tiles permitted, bit 3 = no 192-wide ones
+// allow: bit 1 = single-CTA tiles permitted, bit 2 = CTA-pair tiles permitted, bit 3 = no 192-wide ones, bit 4 = no
+// tile shared along K (a kernel that quantizes its own activations)
 // forced_bn: 0, or the width to take; *splits_out: CTAs that share a tile along K (1: not split).
 void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allow, int forced_bn, int* bn_out, int* cg_out,
                     int* splits_out);
 // The model's estimate (us) for one width and CTA count of an 8-bit layer's GEMM.
-double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg);
+double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg, bool may_split);
 int gemm_max_pairs();
 // gemm_split.cu -- split-K form of the single-CTA streaming kernel and of the 16-bit kernel (64-wide tiles).
 constexpr int kMaxSplits = 4;

@@ -485,14 +485,15 @@ struct TileForm {
 constexpr TileForm kTileForms[] = {{256, 2, 2.39, 0.211, 1.16}, {192, 2, 1.91, 0.179, 1.03}, {128, 2, 1.47, 0.139, 0.89},
                                    {256, 1, 1.71, 0.313, 1.52}, {192, 1, 1.45, 0.235, 1.21}, {128, 1, 1.14, 0.182, 0.98},
                                    {64, 1, 0.86, 0.152, 0.76}};
-double tile_cost(const TileForm& f, const GemmLimits& lim, int64_t M, int32_t N, int32_t K, int32_t bits, int* splits) {
+double tile_cost(const TileForm& f, const GemmLimits& lim, int64_t M, int32_t N, int32_t K, int32_t bits, bool may_split,
+                 int* splits) {
   const int64_t slots = f.cg == 2 ? lim.pairs : lim.sms;
   const int64_t tiles = ((M + BM * f.cg - 1) / (BM * f.cg)) * (N / f.bn);
   const double waves = static_cast<double>((tiles + slots - 1) / slots);
   *splits = 1;
   if (bits < 8) return waves * (f.bn + 24.0) * (f.cg == 2 ? 0.98 : 1.0);
   double cost = f.fixed + waves * fmax(f.per_kb * (K / BK), f.min_tile);
-  if (f.bn == 64) {
+  if (f.bn == 64 && may_split) {
     double saved = 0.0;
     *splits = gemm_split_factor(lim, tiles, K / BK, bits == 16 ? 0.8 * f.per_kb : f.per_kb, &saved);
     cost -= saved;
@@ -501,10 +502,10 @@ double tile_cost(const TileForm& f, const GemmLimits& lim, int64_t M, int32_t N,
 }
 }  // namespace
 
-double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg) {
+double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg, bool may_split) {
   int splits;
   for (const TileForm& f : kTileForms)
-    if (f.bn == bn && f.cg == cg) return tile_cost(f, gemm_limits(), M, N, K, 8, &splits);
+    if (f.bn == bn && f.cg == cg) return tile_cost(f, gemm_limits(), M, N, K, 8, may_split, &splits);
   return 1e30;
 }
 
@@ -517,7 +518,7 @@ void gemm_pick_tile(int64_t M, int32_t N, int32_t K, int32_t bits, uint32_t allo
   for (const TileForm& f : kTileForms) {
     if (N % f.bn || !(allow & (1u << f.cg)) || (f.bn == 192 && (allow & 0x8)) || (forced_bn != 0 && f.bn != forced_bn)) continue;
     int splits;
-    const double cost = tile_cost(f, lim, M, N, K, bits, &splits);
+    const double cost = tile_cost(f, lim, M, N, K, bits, !(allow & 0x10), &splits);
     if (cost < best_cost) {
       best_cost = cost;
       *bn_out = f.bn;

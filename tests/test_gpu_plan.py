@@ -351,6 +351,41 @@ def test_workspace_has_the_parts_that_the_launch_order_uses(Ms, flags, parts):
         B.dp_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("autotune", [0, B.DP_FLAG_AUTOTUNE], ids=["model", "autotuned"])
+@pytest.mark.parametrize("M", [40, 300, 8200])
+def test_in_kernel_quantization_covers_packed_layers(M, autotune):
+    """DP_FLAG_FUSED_DAQ: packed layers too quantize in the GEMM kernel (which then expands their weights itself, so not in
+    the unpack-first form, unless that is asked for), with the bits of the layers called one by one."""
+    K, N, bits = 384, 384, (4, 8, 3)
+    dev = [DevLayer(*synth.weights(SEED, l, N, K, b), synth.bias(SEED, l, N), b) for l, b in enumerate(bits)]
+    plan = B.dp_plan_create([d.w for d in dev], [M] * 3, B.DP_FLAG_FUSED_DAQ | autotune)
+    first = B.dp_plan_create([d.w for d in dev], [M] * 3, B.DP_FLAG_FUSED_DAQ | B.DP_FLAG_UNPACK_FIRST | autotune)
+    try:
+        assert [B.dp_plan_layer_variant(plan, l)["unpack_first"] for l in range(3)] == [0, 0, 0]
+        assert [B.dp_plan_layer_variant(first, l)["unpack_first"] for l in range(3)] == [1, 0, 1]
+        xs = [to_dev_bf16(synth.activations(SEED, l, 0, M, K, 1.0, n_out=3)) for l in range(3)]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        want = []
+        for d, x in zip(dev, xs):
+            y = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+            ws = torch.empty(B.dp_wq_linear_workspace(M, N, K, d.bits), dtype=torch.uint8, device="cuda")
+            B.dp_wq_linear(d.w, x, K, None, M, y, N, ws, None, status)
+            torch.cuda.synchronize()
+            want.append(y.view(torch.int16))
+        for p in (plan, first):
+            ys = [torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in bits]
+            ws = torch.empty(B.dp_plan_workspace(p), dtype=torch.uint8, device="cuda")
+            B.dp_plan_run(p, [0, 1, 2], 0, B.ptr_array([t.data_ptr() for t in xs]), B.ptr_array([t.data_ptr() for t in ys]),
+                          ws, status, flags=B.DP_PLAN_SAME_X | B.DP_PLAN_SAME_Y)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0
+            for a, b in zip(ys, want):
+                assert torch.equal(a.view(torch.int16), b)
+    finally:
+        B.dp_plan_destroy(plan)
+        B.dp_plan_destroy(first)
+
+
 def test_phase_a_on_measured_latencies_matches_oracle_and_runs():
     """Algorithm 2 end to end on a small stack: c_lat(l, b) measured with the library's kernels, Phase A
     (library) equal to the oracle's on the same table, and the resulting bit plan and kept steps run by
