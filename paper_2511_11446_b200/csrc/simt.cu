@@ -29,12 +29,13 @@
 // 5.0 -> 3.1 at 3, 6.0 -> 3.0 at 8 (weights alone 0.5 to 1.2 at the copy rate); 16 tokens 8.5 -> 3.8, 32 tokens 9.0 -> 5.2.
 // Of that, with 4 bits and one token: the loads of a token all at once 4.7 -> 3.7 (load_token), blocks dealt out
 // to all SMs before a second warp of one takes any 3.7 -> 2.8; with 8 bits, one copy to a stage instead of 24
-// short ones 4.0 -> 3.0. Short code matters as well: a CTA runs it once, from a cold instruction cache (the
-// contraction as a loop of three units instead of nine written out: K = 128 2.5 -> 2.3 us).
+// short ones 4.0 -> 3.0. Short code matters as well: a CTA runs it once, from a cold instruction cache (see
+// simt_linear_kernel).
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 
 #include "daq_device.cuh"
 
@@ -361,11 +362,12 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
 // instruction's k index of a register is immaterial here: lane (g, t) supplies, for step s of its
 // unit, words 2s and 2s + 1 of the unit as the (k-low, k-high) registers of BOTH operands, so every
 // k meets its partner exactly once.
-template <int BITS>
+// KJ: K / 128 as a constant of the code, or 0 (then it is read from the arguments).
+template <int BITS, int KJ>
 __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block_x, const int block_y,
                                               const int grid_x) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const int K = a.K, qpitch = K + 16;
+  const int K = KJ > 0 ? 128 * KJ : a.K, qpitch = K + 16;
   int8_t* sq = reinterpret_cast<int8_t*>(smem);                             // [kMmaRows][qpitch]
   float* ssa = reinterpret_cast<float*>(smem + kMmaRows * qpitch);          // [kMmaRows]
   volatile int* abort_flag = reinterpret_cast<volatile int*>(ssa + kMmaRows);
@@ -561,9 +563,9 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
     };
     if (two) {
       contract(std::true_type{});
-    } else if (kj == kMmaUnits) {  // K = 1152, up to 8 tokens: written out, 2.90 -> 2.74 us
+    } else if constexpr (KJ > 0) {  // up to 8 tokens: written out
 #pragma unroll
-      for (int jj = 0; jj < kMmaUnits; ++jj) unit_step(srow, qrow + jj * 128, 4 * jj + t, std::false_type{});
+      for (int jj = 0; jj < KJ; ++jj) unit_step(srow, qrow + jj * 128, 4 * jj + t, std::false_type{});
     } else {
       contract(std::false_type{});
     }
@@ -584,10 +586,14 @@ __device__ __forceinline__ void simt_mma_body(const SimtArgs& a, const int block
   if (threadIdx.x == 0 && *abort_flag && a.status != nullptr) atomicExch(a.status, DP_ERR_TIMEOUT);
 }
 
-template <int BITS, bool MMA>
-__global__ void __launch_bounds__(kSimtWarps * 32, MMA ? kMmaCtasPerSm : 0)
+// KJ = K / 128 of the matrix-instruction form, 0: the other form, any K. A kernel for each row length of the first (nine):
+// with K a constant the contraction of up to 8 tokens is written out and nothing else is in the code that a launch
+// brings in cold. N = 6 K, 8 tokens, K = 384 / 768 / 1024 / 1152 against one kernel with a loop of three units: 4-bit 2.40 /
+// 2.51 / 2.86 / 2.97 -> 2.39 / 2.49 / 2.79 / 2.91 us, 8-bit 2.32 / 2.56 / 3.09 / 3.56 -> 2.31 / 2.46 / 2.88 / 3.38.
+template <int BITS, int KJ>
+__global__ void __launch_bounds__(kSimtWarps * 32, KJ > 0 ? kMmaCtasPerSm : 0)
 simt_linear_kernel(SimtArgs a) {
-  if constexpr (MMA) simt_mma_body<BITS>(a, blockIdx.x, blockIdx.y, gridDim.x);
+  if constexpr (KJ > 0) simt_mma_body<BITS, KJ>(a, blockIdx.x, blockIdx.y, gridDim.x);
   else simt_linear_body<BITS>(a, blockIdx.x, blockIdx.y);
 }
 
@@ -662,9 +668,9 @@ simt_group_kernel(SimtGroupArgs g) {
   a.hold = g.hold;
   a.status = g.status;
   if constexpr (MMA) {
-    if (L.bits == 8) simt_mma_body<8>(a, block_x, blockIdx.y, grid_x);
-    else if (L.bits == 4) simt_mma_body<4>(a, block_x, blockIdx.y, grid_x);
-    else simt_mma_body<3>(a, block_x, blockIdx.y, grid_x);
+    if (L.bits == 8) simt_mma_body<8, 0>(a, block_x, blockIdx.y, grid_x);
+    else if (L.bits == 4) simt_mma_body<4, 0>(a, block_x, blockIdx.y, grid_x);
+    else simt_mma_body<3, 0>(a, block_x, blockIdx.y, grid_x);
   } else {
     if (L.bits == 8) simt_linear_body<8>(a, blockIdx.x, blockIdx.y);
     else if (L.bits == 4) simt_linear_body<4>(a, blockIdx.x, blockIdx.y);
@@ -696,18 +702,26 @@ static_assert(kMmaRows == 2 * kMmaWarps && kMmaMaxK <= 256 * kTokVec, "a warp ho
 
 size_t simt_max_k() { return 16384; }
 
+using SimtKernel = void (*)(SimtArgs);
+template <int BITS, int... KJ>
+static SimtKernel simt_kernel(int kj, std::integer_sequence<int, KJ...>) {
+  static constexpr SimtKernel kernels[] = {simt_linear_kernel<BITS, KJ>...};
+  return kernels[kj];
+}
+// The kernel of a bit width, kj = K / 128 of the matrix-instruction form or 0.
+static SimtKernel simt_kernel(int bits, int kj) {
+  constexpr std::make_integer_sequence<int, kMmaUnits + 1> all;
+  return bits == 8 ? simt_kernel<8>(kj, all) : bits == 4 ? simt_kernel<4>(kj, all) : simt_kernel<3>(kj, all);
+}
+
 // Once per device: the shared-memory limits of the kernels (a launch that set its own, and asked for the
 // occupancy, spent 0.24 us of host time on it: 3.72 -> 3.48 us a call).
 int simt_init_device() {
   const int mma = static_cast<int>(simt_smem_bytes(kMmaMaxK)), dp4a = 227 * 1024;
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<3, true>, attr, mma));
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<4, true>, attr, mma));
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<8, true>, attr, mma));
+  for (int bits : {3, 4, 8})
+    for (int kj = 0; kj <= kMmaUnits; ++kj) DP_CUDA_OK(cudaFuncSetAttribute(simt_kernel(bits, kj), attr, kj > 0 ? mma : dp4a));
   DP_CUDA_OK(cudaFuncSetAttribute(simt_group_kernel<true>, attr, mma));
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<3, false>, attr, dp4a));
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<4, false>, attr, dp4a));
-  DP_CUDA_OK(cudaFuncSetAttribute(simt_linear_kernel<8, false>, attr, dp4a));
   DP_CUDA_OK(cudaFuncSetAttribute(simt_group_kernel<false>, attr, dp4a));
   return DP_OK;
 }
@@ -776,11 +790,7 @@ int launch_simt_linear(const SimtArgs& a, cudaStream_t stream, bool pdl) {
   const int64_t m_groups = (a.M + rows - 1) / rows;
   dim3 grid((a.N + kSimtChPerCta - 1) / kSimtChPerCta, static_cast<unsigned>(m_groups));
   const dim3 block(kSimtWarps * 32);
-  void (*kern)(SimtArgs);
-  if (mma) kern = a.bits == 8 ? simt_linear_kernel<8, true> : a.bits == 4 ? simt_linear_kernel<4, true>
-                                                                          : simt_linear_kernel<3, true>;
-  else kern = a.bits == 8 ? simt_linear_kernel<8, false> : a.bits == 4 ? simt_linear_kernel<4, false>
-                                                                       : simt_linear_kernel<3, false>;
+  const SimtKernel kern = simt_kernel(a.bits, mma ? a.K / 128 : 0);
   if (mma) grid.x = mma_grid_x(a.N, m_groups);
   SimtArgs args = a;
   args.rows = rows;

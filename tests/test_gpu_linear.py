@@ -66,6 +66,16 @@ def test_simt_token_lengths(bits, codes, M, K):
     _check(run_linear(L, x, flags=B.DP_FLAG_FORCE_SIMT, prequant=pre), x, w, s_w, b, bits)
 
 
+@pytest.mark.parametrize("bits", [3, 4, 8])
+@pytest.mark.parametrize("K", range(128, 1281, 128))
+def test_simt_every_row_length(bits, K):
+    """Each row length of the matrix-instruction form has a kernel of its own, longer rows one for all: one token, and 19
+    (two groups of 8 and a part of one)."""
+    for M in (1, 19):
+        x, w, s_w, b = _case(M, K, 48, bits, full_range=True)
+        _check(run_linear(DevLayer(w, s_w, b, bits), x, flags=B.DP_FLAG_FORCE_SIMT), x, w, s_w, b, bits)
+
+
 @pytest.mark.parametrize("bits", [8, 4, 3])
 @pytest.mark.parametrize("M,K,N", [(128, 128, 64), (128, 256, 128), (256, 1152, 1152),
                                    (300, 1152, 384), (1000, 4608, 1152), (77, 384, 192),
