@@ -85,27 +85,7 @@ struct QRow {
   }
 };
 
-// One token by one warp, any K (multiple of 8): two passes over the row, the second served by
-// L1/L2. Writes the codes through `qr` and returns the scale (valid in every lane).
-template <bool EO>
-__device__ __forceinline__ float daq_row_2pass(const uint16_t* __restrict__ x_row, int K, const QRow& qr, int lane) {
-  const int nvec = K >> 3;
-  const uint4* xr = reinterpret_cast<const uint4*>(x_row);
-  uint32_t m = 0;
-#pragma unroll 5
-  for (int idx = lane; idx < nvec; idx += 32) {
-    const uint4 v = xr[idx];
-    m = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(m, v.x), v.y), v.z), v.w);
-  }
-  m = warp_max_u32(max(m & 0xFFFFu, m >> 16));
-  float sc, inv;
-  token_scale(m, sc, inv);
-#pragma unroll 5
-  for (int idx = lane; idx < nvec; idx += 32) qr.store(idx, quant_vec<EO>(xr[idx], inv));
-  return sc;
-}
-
-// Two tokens by one warp at once (the loads of both are in flight together, which matters when the
+// Two tokens by one warp at once, any K (multiple of 8), in two passes over the rows, the second served by L1/L2 (the loads of both are in flight together, which matters when the
 // warp has several tokens to do and each costs a full memory round trip). has_b == false: only A.
 template <bool EO>
 __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ xa, const uint16_t* __restrict__ xb,

@@ -82,9 +82,9 @@ struct SimtGroupArgs {
   int64_t M;
   int32_t N, K, n_layers;
   int32_t early_w, hold;  // as in SimtArgs
-  // Scratch for the group's int8 tokens [n_layers][M][K] and scales [n_layers][M]: when given, one
-  // small kernel quantizes all tokens of the group first and the main kernel's CTAs only fetch the
-  // codes; when null every CTA quantizes its tokens itself.
+  // Scratch for the group's int8 tokens [n_layers][M][K] and scales [n_layers][M]: when given (a DAQ rule other
+  // than the plain one), one small kernel quantizes all tokens of the group first and the main kernel's CTAs only
+  // fetch the codes; when null every CTA quantizes its tokens itself.
   int8_t* q_scratch;
   float* sa_scratch;
   int32_t* status;  // as SimtArgs::status
@@ -98,9 +98,6 @@ int launch_simt_group(const SimtGroupArgs& g, cudaStream_t stream, bool pdl);
 size_t simt_max_k();
 
 // gemm_tc.cu — tcgen05 kind::i8 GEMM with in-smem weight unpack and fused dequant epilogue.
-struct GemmTile {  // kernel variant
-  int bn;          // tile width in output channels: 64, 128, 192 or 256
-};
 struct GemmProblem {
   CUtensorMap tmap_a;  // int8 activations [M][K]
   CUtensorMap tmap_w;  // packed weights, byte view [N][K*bits/8]

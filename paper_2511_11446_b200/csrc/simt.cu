@@ -600,21 +600,8 @@ simt_linear_kernel(SimtArgs a) {
 // Several layers of one shape (M, K, N) in one launch: blockIdx.z picks the layer. Used for the
 // adaLN modulation linears of a timestep, which are mutually independent and, one at a time, far
 // too small (3..8 MB of weights) to fill the GPU for longer than a launch takes.
-// DAQ of every token of a group (one warp per token; grid = (ceil(M / 8), layers)).
-__global__ void __launch_bounds__(kSimtWarps * 32)
-daq_group_kernel(SimtGroupArgs g) {
-  simt_begin(0, g.hold);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kSimtWarps + warp;
-  if (row >= g.M) return;
-  const int layer = blockIdx.y;
-  const uint16_t* x = static_cast<const uint16_t*>(g.layer[layer].x) + row * g.K;
-  const QRow qr(g.q_scratch + static_cast<int64_t>(layer) * g.M * g.K, row, g.K, 0);
-  const float sc = daq_row_2pass<false>(x, g.K, qr, lane);
-  if (lane == 0) g.sa_scratch[static_cast<int64_t>(layer) * g.M + row] = sc;
-}
-
-// The same under a DAQ policy (percentile clip, a-bit codes): rows of up to 1280 elements in registers.
+// DAQ of every token of a group under a policy (percentile clip, a-bit codes; one warp per token, grid = (ceil(M / 8),
+// layers)): rows of up to 1280 elements in registers.
 __global__ void __launch_bounds__(kSimtWarps * 32)
 daq_group_robust_kernel(SimtGroupArgs g) {
   simt_begin(0, g.hold);
@@ -645,7 +632,7 @@ simt_group_kernel(SimtGroupArgs g) {
   a.x = L.x;
   a.ldx = g.K;
   a.s_a_in = nullptr;
-  if (g.q_scratch != nullptr) {  // tokens already quantized by daq_group_kernel
+  if (g.q_scratch != nullptr) {  // tokens already quantized by daq_group_robust_kernel
     a.x = g.q_scratch + static_cast<int64_t>(layer) * g.M * g.K;
     a.s_a_in = g.sa_scratch + static_cast<int64_t>(layer) * g.M;
   }
@@ -735,10 +722,8 @@ int launch_simt_group(const SimtGroupArgs& g, cudaStream_t stream, bool pdl) {
   if (g.M == 0 || g.n_layers == 0) return DP_OK;
   if (g.q_scratch != nullptr) {
     const dim3 dgrid(static_cast<unsigned>((g.M + kSimtWarps - 1) / kSimtWarps), static_cast<unsigned>(g.n_layers));
-    const bool robust = g.daq_rank > 1 || g.daq_bits < 8;
-    if (robust && g.K > 1280) return fail(DP_ERR_SHAPE, "grouped DAQ policy: K=%d above 1280", g.K);
-    cudaError_t e = robust ? launch(daq_group_robust_kernel, dgrid, dim3(kSimtWarps * 32), 0, stream, pdl, g)
-                           : launch(daq_group_kernel, dgrid, dim3(kSimtWarps * 32), 0, stream, pdl, g);
+    if (g.K > 1280) return fail(DP_ERR_SHAPE, "grouped DAQ policy: K=%d above 1280", g.K);
+    const cudaError_t e = launch(daq_group_robust_kernel, dgrid, dim3(kSimtWarps * 32), 0, stream, pdl, g);
     if (e != cudaSuccess) return fail(DP_ERR_CUDA, "grouped DAQ launch failed: %s", cudaGetErrorString(e));
   }
   const size_t smem = simt_smem_bytes(g.K);
