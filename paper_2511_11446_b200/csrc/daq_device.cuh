@@ -85,8 +85,9 @@ struct QRow {
   }
 };
 
-// Two tokens by one warp at once, any K (multiple of 8), in two passes over the rows, the second served by L1/L2 (the loads of both are in flight together, which matters when the
-// warp has several tokens to do and each costs a full memory round trip). has_b == false: only A.
+// Two tokens by one warp at once, any K (multiple of 8): two passes over the rows, the second served by L1/L2 (the
+// loads of both are in flight together, which matters when the warp has several tokens to do and each costs a full
+// memory round trip). has_b == false: only A.
 template <bool EO>
 __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ xa, const uint16_t* __restrict__ xb,
                                                    bool has_b, int K, const QRow& qa, const QRow& qb, int lane,

@@ -605,3 +605,77 @@ def test_constants_written_by_a_kernel_that_starts_its_dependents_early(first, g
                 assert torch.equal(a, b), (l, kinds[l])
     finally:
         B.dp_plan_destroy(plan)
+
+def _order_stack(M, mixed):
+    """Layers of every kind, (weight, rows, what holds its memory): per-channel 3, 4 and 8 bits, group-wise with and without
+    zero-points, 16-bit, small-M. mixed: row counts on both sides of the one up to which plans run two layers ahead."""
+    D = 384
+    kinds = [8, 4, "g4", 3, 16, 8, "s4", 8, 3, "s8", "g8", 4, 8, 16, 4]
+    out = []
+    for l, kind in enumerate(kinds):
+        bias = synth.bias(SEED, l, D)
+        bits = kind if isinstance(kind, int) else int(kind[1:])
+        rng = np.random.default_rng(l)
+        if kind == 16:
+            wt = torch.from_numpy((rng.standard_normal((D, D)) * 0.05).astype(np.float32)).bfloat16().cuda()
+            keep = (wt, to_dev_bf16(bias))
+            w = B.make_weight(wt, keep[1], keep[1], D, D, 16)
+        else:
+            w8, s_w = synth.weights(SEED, l, D, D, bits)
+            layer = DevLayer(w8, s_w, bias, bits)
+            keep, w = (layer,), layer.w
+            if kind in ("g4", "g8"):
+                s = torch.from_numpy((rng.random((D, D // 64)) * 4e-3 + 1e-4).astype(np.float32)).cuda()
+                z = torch.from_numpy(rng.integers(0, 16, (D, D // 64)).astype(np.uint8)).cuda() if kind == "g4" else None
+                keep = (layer, s, z)
+                w = B.make_weight(layer.qweight, s, layer.bias, D, D, bits, 64, z)
+        rows = 8 if kind in ("s4", "s8") else (M if l % 2 else 300) if mixed else (M if l % 3 else M // 2)
+        out.append((w, rows, keep))
+    return D, out
+
+
+@pytest.mark.parametrize("grouped", [0, B.DP_FLAG_GROUP_SMALL_M], ids=["one_by_one", "grouped_small_m"])
+@pytest.mark.parametrize("clip", [100000, 99900])
+@pytest.mark.parametrize("M,mixed", [(64, False), (300, False), (2048, False), (1500, True)])
+@pytest.mark.parametrize("feed", ["two_back", "ping_pong", "one_output", "run_after_run"])
+def test_plan_launch_orders(feed, M, mixed, clip, grouped):
+    """Quantization runs up to two layers ahead of or beside the GEMMs before it: whatever the layers read and write, the
+    results are those of a plan that runs one kernel at a time. Inputs from two layers back, two buffers written and
+    read in turn, one output buffer for all, and a run on what the run before it (not waited for) has written."""
+    D, stack = _order_stack(M, mixed)
+    Ms = [m for _, m, _ in stack]
+    n, top = len(stack), max(Ms)
+    x0 = [to_dev_bf16(synth.activations(SEED, l, 0, m, D, 1.0, n_out=4)) for l, m in enumerate(Ms)]
+    small = [m <= 32 for m in Ms]
+    got = []
+    for flags in (B.DP_FLAG_NO_PDL | grouped, grouped):
+        plan = B.dp_plan_create([w for w, _, _ in stack], Ms, flags)
+        try:
+            B.dp_plan_set_daq(plan, clip, 0)
+            ws = torch.full((B.dp_plan_workspace(plan),), 0x5A, dtype=torch.uint8, device="cuda")
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            buf = torch.zeros((2 * n, top, D), dtype=torch.bfloat16, device="cuda")
+            xs, ys = list(x0), [buf[l] for l in range(n)]
+            if feed == "two_back":
+                xs = [x0[l] if small[l] or l < 2 or small[l - 2] else ys[l - 2] for l in range(n)]
+            elif feed == "ping_pong":
+                order = {l: i for i, l in enumerate(l for l in range(n) if not small[l])}
+                ys = [buf[2 + l] if small[l] else buf[order[l] % 2] for l in range(n)]
+                xs = [x0[l] if small[l] or l == 0 else buf[(order[l] + 1) % 2] for l in range(n)]
+            elif feed == "one_output":
+                ys = [buf[2 + l] if small[l] else buf[0] for l in range(n)]
+            runs = [(xs, ys)]
+            if feed == "run_after_run":
+                runs.append(([x0[l] if small[l] else ys[n - 1 - l if not small[n - 1 - l] else 0] for l in range(n)],
+                             [buf[n + l] for l in range(n)]))
+            torch.cuda.synchronize()
+            for a, b in runs:
+                B.dp_plan_run(plan, [0, 1], 0, B.ptr_array([t.data_ptr() for t in a]), B.ptr_array([t.data_ptr() for t in b]),
+                              ws, status, flags=B.DP_PLAN_SAME_X | B.DP_PLAN_SAME_Y)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0 and bool(torch.isfinite(buf).all())
+            got.append(buf.view(torch.int16))
+        finally:
+            B.dp_plan_destroy(plan)
+    assert int((got[0] != 0).sum()) > 0
+    assert torch.equal(got[0], got[1])
