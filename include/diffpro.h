@@ -120,9 +120,10 @@ typedef struct dp_debug {
 #define DP_FLAG_NO_ACT_STATIONARY 0x400000u
 
 /* dp_plan_create only: choose each layer's tensor-core kernel variant (tile width, single CTA /
- * CTA pair / weight-stationary) by timing the candidates on the device during plan creation
- * (allocates scratch, launches and synchronises; a few milliseconds per distinct layer shape)
- * instead of by the built-in cost model. */
+ * CTA pair / weight-stationary / activation-stationary) by timing, on the device during plan creation, the
+ * candidates that the built-in cost model does not put more than a quarter behind its best one, each as a
+ * replayed graph of twelve layers (allocates scratch, launches and synchronises; five to ten milliseconds per
+ * distinct layer shape) instead of by the cost model alone. */
 #define DP_FLAG_AUTOTUNE 0x10000u
 /* dp_plan_create only: the caller states that, within one timestep, the inputs of the plan's
  * small-M layers (M <= 32: in a DiT the adaLN modulation linears, which consume only the
@@ -135,7 +136,8 @@ typedef struct dp_debug {
  * the tokens, publish finished 128-token tiles on counters the plan owns, and start the tiles
  * whose tokens are ready. One launch per layer instead of two; results are identical. Off by
  * default: on B200 the two-kernel form is faster, because its small DAQ kernel is already resident
- * (programmatic dependent launch) while the previous GEMM drains. */
+ * (programmatic dependent launch) while the previous GEMM drains. Packed layers then expand their weights inside
+ * the GEMM; with DP_FLAG_UNPACK_FIRST they keep a quantization launch of their own instead. */
 #define DP_FLAG_FUSED_DAQ 0x40000u
 
 /* dp_wq_linear and dp_plan_create, packed bit-widths (3, 4) on the tensor-core path: where the
@@ -148,8 +150,8 @@ typedef struct dp_debug {
  * itself; with quantized activations (s_a given) the default is the in-GEMM form, which needs no
  * workspace. The copy lives only for the call, the weights stay packed in memory, results are
  * identical. Adds N*K bytes to the workspace (dp_wq_linear_workspace counts them unless
- * NO_UNPACK_FIRST is given). With DP_FLAG_AUTOTUNE the plan times both forms per layer shape.
- * Giving both flags is an error. */
+ * NO_UNPACK_FIRST is given). DP_FLAG_AUTOTUNE times the kernel variants of the form that the flags (or the
+ * default) say. Giving both flags is an error. */
 #define DP_FLAG_UNPACK_FIRST 0x80000u
 #define DP_FLAG_NO_UNPACK_FIRST 0x100000u
 
@@ -225,7 +227,9 @@ size_t dp_wq_linear_workspace_grouped(int64_t M, const dp_weight* w);
  * next call on that stream. A layer with w->group_size > 0 needs dp_wq_linear_workspace_grouped bytes,
  * takes bf16 activations only (s_a_in NULL) and has no taps. For w->bits == 16 (pass-through layer) x is bf16, s_a_in and dbg must be
  * NULL, no workspace is used, and the output is bf16_rne(fp32 sum + bias) with the sum accumulated in
- * fp32 on the tensor cores (order unspecified: compare with a tolerance, not bit for bit).
+ * fp32 on the tensor cores. The order is unspecified and may depend on M (few tokens: several CTAs sum parts of
+ * K), so that a token's result in a small batch and in a large one may differ in the last bit: compare with a
+ * tolerance, not bit for bit. (Every quantized layer gives a token the same bits in any batch.)
  */
 int dp_wq_linear(const dp_weight* w, const void* x, int64_t ldx, const float* s_a_in, int64_t M,
                  void* y_bf16, int64_t ldy, void* workspace, size_t workspace_bytes,
@@ -371,12 +375,15 @@ void dp_plan_destroy(dp_plan* plan);
  * y is bf16 [M_l][N_l] contiguous. `steps` holds the timestep labels (host array; only its order
  * and length matter to the linears). Visits i = n_steps-1-start_index, ..., 0, so a caller can
  * resume an interrupted schedule by passing the number of steps already done as start_index.
- * x_ptrs / y_ptrs are HOST arrays of device pointers. Enqueues only; capturable in a CUDA graph.
- * While a layer's GEMM runs, its kernel issues L2 prefetch hints for the next layer's packed weights
- * and (up to 32 MB) for the next layer's input buffer. These are hints on memory the call is going to
- * read anyway: no layer is computed before its turn, and an input that an earlier layer of the same
- * step still writes (x of one layer aliasing y of another) is read only after that write, as the
- * stream order says.
+ * x_ptrs / y_ptrs are HOST arrays of device pointers, checked for every layer and step before anything
+ * is enqueued. Enqueues only; capturable in a CUDA graph.
+ * Results are those of running the layers in this order. The quantization (and weight expansion) of a
+ * layer may run beside the GEMMs of the one or two layers before it: it reads only its own x and constants.
+ * Where a layer's x overlaps an earlier layer's y (a linear fed by another; the call compares the ranges
+ * M_l * K_l and M_l * N_l elements long) it waits for the GEMM that writes it. Weights, scales,
+ * zero-points and biases of all layers are constants of the call: no y may overlap them. While a layer's
+ * GEMM runs, its kernel issues L2 prefetch hints for a later layer's packed weights and (up to 32 MB) its
+ * input buffer: hints on memory the call is going to read anyway, whatever is still to be written there.
  */
 int dp_plan_run(const dp_plan* plan, const int32_t* steps, int32_t n_steps, int32_t start_index,
                 const void* const* x_ptrs, void* const* y_ptrs, void* workspace,

@@ -198,9 +198,9 @@ int launch_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t ldx, con
   if (M == 0) return DP_OK;
   LnArgs a{static_cast<const uint16_t*>(x), M, ldx, static_cast<int>(K), static_cast<const uint16_t*>(shift),
            static_cast<const uint16_t*>(scale), rows_per_sample, eps, q, ldq, s_a};
-  // As many warps to a row as leave a lane at most five vectors, one more thing than in plain quantization
-  // speaking for few: every warp of a row repeats the statistics' division and root in double. K = 1152, M = 64 /
-  // 2056 / 32768: one warp 2.4 / 4.5 / 38 us, two 2.3 / 4.4 / 46, four 2.0 / 5.4 / 62.
+  // The fewest warps to a row that leave a lane at most five vectors (three for rows that two or four can hold that
+  // way), because every warp of a row repeats the statistics' division and root in double. K = 1152, M = 64 / 2056 /
+  // 32768: one warp 2.4 / 4.5 / 38 us, two 2.3 / 4.4 / 46, four 2.0 / 5.4 / 62. Up to 512 rows leave SMs idle: four.
   const cudaError_t e = M <= 512 && K <= 2048 ? launch_ln_v<4, 2>(a, stream, pdl)
                         : K <= 256 * 5        ? launch_ln_v<1, 5>(a, stream, pdl)
                         : K <= 512 * 3        ? launch_ln_v<2, 3>(a, stream, pdl)
