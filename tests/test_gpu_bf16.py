@@ -53,9 +53,11 @@ def _check(got, x, w, b):
 
 @pytest.mark.parametrize("M,K,N", [(128, 128, 64), (200, 384, 192), (77, 1152, 384), (300, 256, 512),
                                    (1000, 4608, 1152), (16, 1152, 6912), (2048, 1152, 1152),
-                                   (130, 4608, 1152), (520, 2304, 128)])
+                                   (130, 4608, 1152), (520, 2304, 128), (256, 4608, 1280), (512, 4608, 1152),
+                                   (5000, 384, 1536)])
 def test_passthrough_layer_matches_double_precision_linear(M, K, N):
-    """Every tile width (64, 128, 256), ragged and small M, short and long K, more tiles than SMs."""
+    """Every tile width (64, 128, and 256 with the last shape), ragged and small M, short and long K, more tiles than SMs,
+    tiles shared along K by two, three and four CTAs."""
     x = synth.activations(SEED, N % 7, 0, M, K, 1.0, n_out=max(1, K // 100))
     w = _weights_bf16(1, N, K)
     b = synth.bias(SEED, 1, N) if N != 192 else None

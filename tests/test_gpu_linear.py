@@ -363,10 +363,11 @@ def test_pair_kernels_in_quick_succession(flags, K):
 @pytest.mark.parametrize("bits", [8, 3])
 @pytest.mark.parametrize("bn", [0, 64])
 @pytest.mark.parametrize("M,K,N", [(33, 4608, 1152), (128, 2304, 128), (129, 4608, 256), (300, 4608, 1152), (520, 4608, 1152),
-                                   (40, 3200, 64)])
+                                   (40, 3200, 64), (300, 9216, 1152), (200, 4608, 1280)])
 def test_mma_split_k(bits, bn, M, K, N):
-    """Layers with fewer tiles than SMs and many k-blocks (25 and 36: uneven shares too) run split along K
-    when no taps are asked for; ragged token counts, one and several tiles."""
+    """Layers with fewer tiles than SMs and many k-blocks (25, 36 and 72: uneven shares too) run split along K
+    when no taps are asked for, by two CTAs (K = 9216), three (N = 1280) or four; ragged token counts, one and several
+    tiles; and shapes on the other side of the rule's lines (K = 2304, 54 and 90 tiles), which do not."""
     if bn and N % bn:
         pytest.skip("width does not divide N")
     x, w, s_w, b = _case(M, K, N, bits)
