@@ -277,6 +277,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
       job.zeros = zeros;
       job.row_units = w->K / 32;
       job.group_units = w->group_size / 32;
+      job.wide = ws8 + off;
       w8 = dst;
     }
     int32_t* rowsum = zeros != nullptr && w->bits == 8 ? reinterpret_cast<int32_t*>(ws8 + off) : nullptr;
@@ -285,7 +286,7 @@ static int run_linear(const dp_weight* w, const void* x, int64_t ldx, const floa
                     : launch_daq(x, M, w->K, ldx, wq, w->K, wsa, nullptr, KORDER_NATURAL, true, stream, pdl,
                                  &job);
     if (st != DP_OK) return st;
-    return launch_gemm_grp(wq, w->K, true, wsa, w8, w->bits, w->group_size, w->s_w, zeros,
+    return launch_gemm_grp(wq, w->K, true, wsa, w8, w->bits, w->group_size, w->s_w, zeros, job.wide,
                            static_cast<const uint16_t*>(w->bias), rowsum, M, w->N, w->K, static_cast<uint16_t*>(y), ldy,
                            status, stream, pdl);
   }
@@ -521,7 +522,11 @@ extern "C" size_t dp_wq_linear_workspace_grouped(int64_t M, const dp_weight* w) 
   if (!w || M <= 0 || w->K <= 0 || w->group_size <= 0) return 256;
   size_t need = align256(scratch_q_bytes(M, w->K)) + align256(sizeof(float) * static_cast<size_t>(M));
   if (w->bits < 8) need += align256(static_cast<size_t>(w->N) * w->K);
-  if (w->zeros != nullptr) need += align256(sizeof(int32_t) * static_cast<size_t>(M) * (w->K / w->group_size));
+  // per-group code sums of 8-bit layers; packed ones, which had them too, keep the expansion's notes there (more bytes
+  // only for a handful of tokens)
+  if (w->zeros != nullptr)
+    need += std::max(align256(sizeof(int32_t) * static_cast<size_t>(M) * (w->K / w->group_size)),
+                     w->bits < 8 ? align256(unpack_notes(static_cast<int64_t>(w->N) * w->K / 32)) : 0);
   return need;
 }
 

@@ -286,9 +286,8 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&pk)[BITS], uint32_t
 __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int block) {
   const int64_t u = static_cast<int64_t>(block) * blockDim.x + threadIdx.x;
   if (!job.early) pdl_wait();
-  uint32_t w[8];
+  uint32_t w[8], z = 1u << (job.bits - 1);
   if (u < job.units) {
-    uint32_t z = 1u << (job.bits - 1);
     // One zero-point per channel and group (a multiple of 32 codes). (Units of a matrix that fits the device count in
     // 32 bits. The clamp of z stands at its uses: up here it made the packed words wait for z, 1.5 us of a 93 us block.)
     if (job.zeros != nullptr) {
@@ -308,6 +307,10 @@ __device__ __forceinline__ void unpack_units(const UnpackJob& job, const int blo
   if (job.early && !job.ahead) pdl_wait();
   if (u < job.units)
     st_global_v8(reinterpret_cast<uint4*>(job.out) + u * 2, w);  // 32 bytes, read next by the GEMM through L2
+  if (job.zeros != nullptr) {  // (uniform; whole CTAs come here; behind the stores, which must not wait for it)
+    const bool wide = __syncthreads_or(z > 127) != 0;
+    if (threadIdx.x % 128 == 0 && u < job.units) job.wide[u / 128] = wide;
+  }
 }
 
 }  // namespace dp

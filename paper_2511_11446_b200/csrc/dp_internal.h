@@ -32,7 +32,12 @@ struct UnpackJob {
                             // stays until it has finished, so that whatever waits for this launch waits for both
   const uint8_t* zeros = nullptr;  // group-wise zero-points [N][row_units / group_units], or null (symmetric)
   uint32_t row_units = 0, group_units = 0;
+  // With zeros: a byte for every 128 units, nonzero where a zero-point above 127 was among them (128 of it are taken
+  // off; the fold that reads `out` has to know).
+  uint8_t* wide = nullptr;
 };
+// Notes of a matrix of `units` units (a multiple of 512: N and K are multiples of 128).
+inline int64_t unpack_notes(int64_t units) { return units / 128; }
 int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq,
                float* s_a, int32_t* rowsum, int korder, bool tiled, cudaStream_t stream, bool pdl,
                const UnpackJob* unpack = nullptr);
@@ -177,8 +182,8 @@ int gemm_grp_init_device();
 constexpr int kGrpZeroMaxGroups = 160;  // per row, of a layer with zero-points (K <= 5120 at g = 32)
 // (for packed weights the expansion has taken the zero-points up to 128 off already)
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
-                    int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,
-                    int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl);
+                    int32_t g, const float* s_w, const uint8_t* zeros, const uint8_t* wide, const uint16_t* bias,
+                    int32_t* rowsum, int64_t M, int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl);
 
 // gemm_bf16.cu -- pass-through linear of 16-bit layers (bf16 x bf16 -> fp32 -> bf16, tcgen05 kind::f16).
 int launch_gemm_bf16(const void* x, int64_t ldx, const void* w, const uint16_t* bias, int64_t M, int32_t N, int32_t K,

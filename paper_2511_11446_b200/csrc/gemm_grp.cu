@@ -20,10 +20,11 @@
 // held in registers, then the buffer goes back to the MMA issuer; after the last group the token scale, bias,
 // bf16 rounding and 16-byte stores.
 // Zero-points of 3- and 4-bit layers are taken off when the packed weights are expanded to int8, up to 128 of
-// them: u - 128 is the least an int8 holds. Zero-points are bytes, though no quantizer writes one above 2^bits: a
-// fold warp looks those of its columns over while it waits for its first accumulators, and where one is above 127
-// it takes a fold that adds (128 - z) * rowsum_G[m] of the columns above 128 (ZP_WIDE), with row sums
-// that it takes from the codes itself. For 8-bit
+// them: u - 128 is the least an int8 holds. Zero-points are bytes, though no quantizer writes one above 2^bits: the
+// expansion notes where it met one above 127, the fold warps read the notes while they wait for their first
+// accumulators, and if there is one they leave the accumulators alone and sum the codes themselves, (128 - z) *
+// rowsum_G[m] included (grp_fold_wide: exact, several times slower, and short of registers on purpose, so that the
+// usual fold keeps its own: as a second copy of the fold it cost layers with zero-points up to 7 %). For 8-bit
 // codes u - z does not fit a byte at all: the tensor core multiplies by u - 128 and (128 - z[n,G]) * rowsum_G[m] is
 // added in int32 before the conversion (form ZP_8BIT, with rowsum from a kernel of its own).
 // The fold is what bounds this kernel: 1.5 instructions per output and group, the conversion at 64 per
@@ -44,15 +45,17 @@ constexpr int kGrpCols = kGrpBN / (kGrpFoldWarps / 4);  // columns of a fold war
 constexpr int kGrpThreads = (kGrpFoldWarp0 + kGrpFoldWarps) * 32;
 constexpr int kGrpScaleWords = 2 * kGrpBufs * kGrpBN + kGrpFoldWarps * kGrpCols;  // scales, zero-point terms, biases
 
-// Zero-points: none; of 8-bit codes; of packed codes; of packed codes, some of them above 127.
-enum { ZP_NONE, ZP_8BIT, ZP_PACKED, ZP_WIDE };
+// Zero-points: none; of 8-bit codes; of packed codes.
+enum { ZP_NONE, ZP_8BIT, ZP_PACKED };
 
 struct GrpParams {
   const float* s_a;       // [M]
   const float* s_w;       // [N][ng]
   const uint8_t* zeros;   // [N][ng] (unless ZP_NONE)
   const int32_t* rowsum;  // [M][ng] (ZP_8BIT)
-  const int8_t* q;        // the codes behind tmap_a, tiled (ZP_WIDE)
+  const int8_t *q, *w8;   // ZP_PACKED: what tmap_a (tiled) and tmap_w read,
+  const uint32_t* wide;   // and the expansion's notes, n_wide words: nonzero for a zero-point above 127
+  int32_t n_wide;
   const uint16_t* bias;
   uint16_t* y;
   int64_t ldy;
@@ -133,41 +136,17 @@ struct GrpSmem {
   }
 };
 
-// Whether some zero-point of the 32 columns from col0 on of this CTA's tiles is above 127 (a warp together).
-__device__ __forceinline__ bool grp_wide_zeros(const GrpParams& p, int col0, int lane) {
-  const int bytes = kGrpCols * p.ng, total_tiles = p.m_tiles * p.n_tiles;
-  const bool aligned = (reinterpret_cast<uintptr_t>(p.zeros) & 15u) == 0;
+// Whether the expansion met a zero-point above 127 (a warp together).
+__device__ __forceinline__ bool grp_wide_zeros(const GrpParams& p, int lane) {
   uint32_t any = 0;
-  int seen = 0;
-  for (int tile = blockIdx.x; tile < total_tiles && seen < p.n_tiles; tile += gridDim.x, ++seen) {
-    const uint8_t* z = p.zeros + static_cast<int64_t>((tile % p.n_tiles) * kGrpBN + col0) * p.ng;
-    if (aligned) {
-      for (int i = lane; i < bytes / 16; i += 32) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(z) + i);
-        any |= v.x | v.y | v.z | v.w;
-      }
-    } else {
-      for (int i = lane; i < bytes; i += 32) any |= __ldg(z + i);
-    }
-  }
-  return __any_sync(0xFFFFFFFFu, (any & 0x80808080u) != 0);
-}
-
-// Code sums of group G of the tokens row0 + 8 * i that are there, by the four lanes of a quad (they share them).
-__device__ __forceinline__ void grp_row_sums(const GrpParams& p, int64_t row0, int G, int lane, const bool (&live)[4],
-                                             int (&rs)[4]) {
-  const int part = p.g >> 2;  // of the group's codes, a multiple of 8
+  for (int i = lane; i < p.n_wide; i += 32 * 8) {  // eight loads in flight, predicated: a loop's remainder goes one by one
+    uint32_t v[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t m = row0 + 8 * i;
-    int s = 0;
-    for (int k = G * p.g + (lane & 3) * part, end = k + part; live[i] && k < end; k += 8) {
-      const uint2 v = *reinterpret_cast<const uint2*>(p.q + ((m >> 7) * (p.K >> 7) + (k >> 7)) * 16384 + (m & 127) * 128 + (k & 127));
-      s = __dp4a(static_cast<int>(v.x), 0x01010101, __dp4a(static_cast<int>(v.y), 0x01010101, s));
-    }
-    s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
-    rs[i] = s + __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+    for (int j = 0; j < 8; ++j) v[j] = i + 32 * j < p.n_wide ? __ldg(p.wide + i + 32 * j) : 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) any |= v[j];
   }
+  return __any_sync(0xFFFFFFFFu, any != 0);
 }
 
 // A fold warp's whole run over this CTA's tiles: quadrant (warp & 3), column quarter (fw >> 2).
@@ -220,7 +199,7 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           int a0 = static_cast<int>(a[4 * j + 2 * k]), a1 = static_cast<int>(a[4 * j + 2 * k + 1]);
-          if constexpr (ZP != ZP_NONE) {
+          if constexpr (ZP == ZP_8BIT) {
             a0 += dz[2 * j] * rs_g[i0 + k];
             a1 += dz[2 * j + 1] * rs_g[i0 + k];
           }
@@ -246,14 +225,6 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
         for (int i = 0; i < 4; ++i) {
           rs_g[i] = rs[i];
           if (live[i] && G + 1 < p.ng) rs[i] = __ldg(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
-        }
-      }
-      if constexpr (ZP == ZP_WIDE) {
-        grp_row_sums(p, row0, G, lane, live, rs_g);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int z = __ldg(p.zeros + static_cast<int64_t>(n0 + tc + j) * p.ng + G);
-          dz[j] = z > 128 ? 128 - z : 0;
         }
       }
       tmem_ld_wait();
@@ -288,9 +259,61 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
     }
   }
 }
-// (A function of its own: inlined, it cost the usual fold registers. Block of 4-bit layers with zero-points, g = 128,
-// M = 2048: 92.7 us without this form, 96.4 with it inlined, 93.0 this way.)
-__device__ __noinline__ void grp_fold_wide(const GrpParams& p) { grp_fold<ZP_WIDE>(p); }
+// The same without the accumulators: a lane takes one token, eight channels at a time.
+__device__ __forceinline__ void grp_fold_wide(const GrpParams& p) {
+  const GrpSmem sm;
+  const int fw = (threadIdx.x >> 5) - kGrpFoldWarp0, qd = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+  uint32_t gcount = 0;
+  for (int tile = blockIdx.x; tile < p.m_tiles * p.n_tiles; tile += gridDim.x) {
+#pragma unroll 1
+    for (int G = 0; G < p.ng; ++G, ++gcount) {  // hand the buffers back as they come
+      const bool ok = mbar_wait(&sm.grp_full[gcount % kGrpBufs], (gcount / kGrpBufs) & 1u, sm.abort_flag);
+      if (!__all_sync(0xFFFFFFFFu, ok)) return;
+      if (lane == 0) mbar_arrive(&sm.grp_empty[gcount % kGrpBufs]);
+    }
+    const int64_t m = static_cast<int64_t>(tile / p.n_tiles) * BM + qd * 32 + lane;
+    if (m >= p.M) continue;
+    const int8_t* q = p.q + (m >> 7) * (p.K >> 7) * 16384 + (m & 127) * 128;
+#pragma unroll 1
+    for (int c = 0; c < kGrpCols; c += 8) {
+      const int n0 = (tile % p.n_tiles) * kGrpBN + (fw >> 2) * kGrpCols + c;
+      float t[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+      for (int G = 0; G < p.ng; ++G) {
+        int acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rs = 0;
+#pragma unroll 1
+        for (int k = G * p.g; k < (G + 1) * p.g; k += 16) {
+          const int4 a = *reinterpret_cast<const int4*>(q + (k >> 7) * 16384 + (k & 127));
+          rs = __dp4a(a.x, 0x01010101, __dp4a(a.y, 0x01010101, __dp4a(a.z, 0x01010101, __dp4a(a.w, 0x01010101, rs))));
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int4 b = *reinterpret_cast<const int4*>(p.w8 + static_cast<int64_t>(n0 + j) * p.K + k);
+            acc[j] = __dp4a(a.x, b.x, __dp4a(a.y, b.y, __dp4a(a.z, b.z, __dp4a(a.w, b.w, acc[j]))));
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int64_t at = static_cast<int64_t>(n0 + j) * p.ng + G;
+          const int z = p.zeros[at];
+          if (z > 128) acc[j] += (128 - z) * rs;
+          t[j] = __fmaf_rn(__int2float_rn(acc[j]), p.s_w[at], t[j]);
+        }
+      }
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float y[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          y[e] = __fmaf_rn(t[2 * j + e], p.s_a[m], p.bias != nullptr
+                                                       ? __uint_as_float(static_cast<uint32_t>(p.bias[n0 + 2 * j + e]) << 16) : 0.0f);
+        const __nv_bfloat162 v = __floats2bfloat162_rn(y[0], y[1]);
+        w[j] = *reinterpret_cast<const uint32_t*>(&v);
+      }
+      st_global_v4(p.y + m * p.ldy + n0, w);
+    }
+  }
+}
 
 template <int ZP>
 __global__ void __launch_bounds__(kGrpThreads, 1)
@@ -430,12 +453,8 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     }
   } else {
     // ================= fold + epilogue =================
-    if constexpr (ZP == ZP_PACKED) {
-      if (grp_wide_zeros(p, ((warp - kGrpFoldWarp0) >> 2) * kGrpCols, lane)) grp_fold_wide(p);
-      else grp_fold<ZP_NONE>(p);
-    } else {
-      grp_fold<ZP>(p);
-    }
+    if (ZP == ZP_PACKED && grp_wide_zeros(p, lane)) grp_fold_wide(p);
+    else grp_fold<ZP == ZP_8BIT ? ZP_8BIT : ZP_NONE>(p);
   }
 
   tc_fence_before();
@@ -491,10 +510,11 @@ int gemm_grp_init_device() {
 
 // q / s_a: the quantized activations (tiled scratch when a_tiled, as packed layers with zero-points need it); w8:
 // int8 [N][K], u - 2^(bits-1) of 8-bit codes and of layers without zero-points, else u - min(z, 128); rowsum: scratch
-// int32 [M][K/g], used (and filled here) only for 8-bit codes with zero-points.
+// int32 [M][K/g], used (and filled here) only for 8-bit codes with zero-points. wide: the expansion's notes (packed
+// layers with zero-points).
 int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a, const int8_t* w8, int32_t bits,
-                    int32_t g, const float* s_w, const uint8_t* zeros, const uint16_t* bias, int32_t* rowsum, int64_t M,
-                    int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl) {
+                    int32_t g, const float* s_w, const uint8_t* zeros, const uint8_t* wide, const uint16_t* bias,
+                    int32_t* rowsum, int64_t M, int32_t N, int32_t K, uint16_t* y, int64_t ldy, int32_t* status, cudaStream_t stream, bool pdl) {
   if (M == 0) return DP_OK;
   if (N % kGrpBN || g <= 0 || g % 32 || K % g)
     return fail(DP_ERR_SHAPE, "group-wise layer: need N %% 128 == 0, g %% 32 == 0, K %% g == 0 (N=%d K=%d g=%d)", N, K, g);
@@ -518,6 +538,9 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   p.zeros = zeros;
   p.rowsum = rowsum;
   p.q = q;
+  p.w8 = w8;
+  p.wide = reinterpret_cast<const uint32_t*>(wide);
+  p.n_wide = static_cast<int32_t>(unpack_notes(static_cast<int64_t>(N) * K / 32) / 4);
   p.bias = bias;
   p.y = y;
   p.ldy = ldy;

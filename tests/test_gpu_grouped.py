@@ -116,10 +116,11 @@ def test_plan_mixes_grouped_per_channel_and_16_bit_layers():
 
 @pytest.mark.parametrize("bits,g,K", [(4, 32, 1152), (4, 128, 256), (3, 192, 1152), (3, 256, 256)])
 @pytest.mark.parametrize("offset", [0, 1], ids=["aligned", "odd_address"])
-def test_zero_points_of_any_byte_value(bits, g, K, offset):
+@pytest.mark.parametrize("M", [5, 1301])
+def test_zero_points_of_any_byte_value(M, bits, g, K, offset):
     """Zero-points are bytes: u - z of a packed layer need not fit an int8. Values around 2^bits, 128 and 255, in some of
     the column tiles and groups only, more tiles than SMs, and zero-points that start at an odd address."""
-    M, N = 1301, 1920
+    N = 1920
     L = GroupedLayer(N, K, bits, g, True)
     rng = np.random.default_rng(bits * g)
     z = rng.choice(np.array([0, (1 << bits) - 1, 1 << bits, 127, 128, 129, 200, 255], np.uint8), size=L.z.shape)
@@ -133,6 +134,9 @@ def test_zero_points_of_any_byte_value(bits, g, K, offset):
     x = synth.activations(SEED, 3, 0, M, K, 1.0, n_out=3)
     got, ref = _run(L, x), L.ref(x)
     assert np.array_equal(got, ref), int((got != ref).sum())
+    L.d_z[:] = 3                                    # the same layer with small ones: nothing is left of the call before
+    L.z[:] = 3
+    assert np.array_equal(_run(L, x), L.ref(x))
 
 
 def test_grouped_argument_errors():
