@@ -305,13 +305,20 @@ struct RowEpilogue {
     const bool has_res = RES && p.res != nullptr;
     const bool has_gate = has_res && p.gate != nullptr;
     const uint16_t* rrow = has_res ? p.res + row0 * p.ldr + col + tc : nullptr;
+    // The gate rows of the four tokens, once per tile (a 64-bit division each).
+    const uint16_t* grow[4] = {nullptr, nullptr, nullptr, nullptr};
+    if constexpr (RES) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (has_gate && i < live) grow[i] = p.gate + ((row0 + 8 * i) / p.rows_per_gate) * p.N + col + tc;
+    }
     uint4 rn[4], gn[4];
     auto fetch_res = [&](int c) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         rn[i] = gn[i] = make_uint4(0, 0, 0, 0);
         if (has_res && i < live) rn[i] = ld_global_v4(rrow + 8 * i * p.ldr + c * CW);
-        if (has_gate && i < live) gn[i] = ld_global_v4(p.gate + ((row0 + 8 * i) / p.rows_per_gate) * p.N + col + tc + c * CW);
+        if (has_gate && i < live) gn[i] = ld_global_v4(grow[i] + c * CW);
       }
     };
     if constexpr (RES) {
