@@ -20,7 +20,7 @@
 // conversions (16 per clock and SM; building the doubles with integer operations was slower), two additions
 // per element, a division and a root per token. M = 2048, K = 1152 / 2304 / 4608: 4.6 / 9.0 / 15.1 us with one
 // warp, a single chain of additions and the modulation read after the statistics, 4.4 / 7.0 / 11.5 this way;
-// M = 32768, K = 1152: 42 -> 38 us against 19 for DAQ alone.
+// M = 32768, K = 1152: 33 us against 18 for DAQ alone (the modulation read at its use there, see the launch).
 #include "daq_device.cuh"
 
 namespace dp {
@@ -58,8 +58,8 @@ __device__ __forceinline__ uint64_t ln_pair(uint32_t w, uint32_t sw, uint32_t hw
   return h;
 }
 
-// RW warps share a row, MAXV = 16-byte vectors held per lane.
-template <int RW, int MAXV, bool MOD>
+// RW warps share a row, MAXV = 16-byte vectors held per lane. LATE: the modulation is read where it is used.
+template <int RW, int MAXV, bool MOD, bool LATE>
 __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArgs a) {
   constexpr int kRows = kLnThreads / 32 / RW, TPR = 32 * RW;
   __shared__ double part1[kLnThreads / 32], part2[kLnThreads / 32];
@@ -79,14 +79,14 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArg
     shr = reinterpret_cast<const uint4*>(a.shift + sample * a.K);
     scr = reinterpret_cast<const uint4*>(a.scale + sample * a.K);
   }
-  uint4 v[MAXV], sh[MAXV], sc[MAXV];  // the modulation's vectors fly beside the row's
+  uint4 v[MAXV], sh[MAXV], sc[MAXV];  // (unless LATE the modulation's vectors fly beside the row's)
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
     const int idx = lane + TPR * i;
     v[i] = sh[i] = sc[i] = make_uint4(0, 0, 0, 0);
     if (idx < nvec) {
       ld_nc_u32x4(xr + idx, v[i]);
-      if constexpr (MOD) {
+      if constexpr (MOD && !LATE) {
         sh[i] = __ldg(shr + idx);
         sc[i] = __ldg(scr + idx);
       }
@@ -141,6 +141,10 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArg
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
     if (lane + TPR * i >= nvec) continue;
+    if constexpr (MOD && LATE) {
+      sh[i] = __ldg(shr + lane + TPR * i);
+      sc[i] = __ldg(scr + lane + TPR * i);
+    }
     h[i][0] = ln_pair<MOD>(v[i].x, sc[i].x, sh[i].x, nmean2, rstd2, one2);
     h[i][1] = ln_pair<MOD>(v[i].y, sc[i].y, sh[i].y, nmean2, rstd2, one2);
     h[i][2] = ln_pair<MOD>(v[i].z, sc[i].z, sh[i].z, nmean2, rstd2, one2);
@@ -184,12 +188,12 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArg
   if (lane == 0) a.s_a[row] = sa;
 }
 
-template <int RW, int MAXV>
+template <int RW, int MAXV, bool LATE = false>
 static cudaError_t launch_ln_v(const LnArgs& a, cudaStream_t stream, bool pdl) {
   constexpr int kRows = kLnThreads / 32 / RW;
   const dim3 grid(static_cast<unsigned>((a.M + kRows - 1) / kRows));
-  if (a.shift != nullptr) return launch(ln_modulate_daq_kernel<RW, MAXV, true>, grid, dim3(kLnThreads), 0, stream, pdl, a);
-  return launch(ln_modulate_daq_kernel<RW, MAXV, false>, grid, dim3(kLnThreads), 0, stream, pdl, a);
+  if (a.shift != nullptr) return launch(ln_modulate_daq_kernel<RW, MAXV, true, LATE>, grid, dim3(kLnThreads), 0, stream, pdl, a);
+  return launch(ln_modulate_daq_kernel<RW, MAXV, false, LATE>, grid, dim3(kLnThreads), 0, stream, pdl, a);
 }
 
 int launch_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t ldx, const void* shift, const void* scale,
@@ -201,7 +205,14 @@ int launch_ln_modulate_daq(const void* x, int64_t M, int64_t K, int64_t ldx, con
   // The fewest warps to a row that leave a lane at most five vectors (three for rows that two or four can hold that
   // way), because every warp of a row repeats the statistics' division and root in double. K = 1152, M = 64 / 2056 /
   // 32768: one warp 2.4 / 4.5 / 38 us, two 2.3 / 4.4 / 46, four 2.0 / 5.4 / 62. Up to 512 rows leave SMs idle: four.
+  // From 4096 rows on there are warps enough to cover the modulation's way through L2, and what counts is how many fit an
+  // SM: it is read where it is used (94 registers otherwise), into as many vectors as the row has. M = 32768, K = 384 /
+  // 768 / 1152: read ahead into five vectors 27 / 31 / 37.9 us, this way 18.6 / 23.6 / 33.3 (M = 2048: 2.9 / 3.4 / 4.4 read ahead).
   const cudaError_t e = M <= 512 && K <= 2048 ? launch_ln_v<4, 2>(a, stream, pdl)
+                        : M >= 4096 && K <= 256 * 2 ? launch_ln_v<1, 2, true>(a, stream, pdl)
+                        : M >= 4096 && K <= 256 * 3 ? launch_ln_v<1, 3, true>(a, stream, pdl)
+                        : M >= 4096 && K <= 256 * 4 ? launch_ln_v<1, 4, true>(a, stream, pdl)
+                        : M >= 4096 && K <= 256 * 5 ? launch_ln_v<1, 5, true>(a, stream, pdl)
                         : K <= 256 * 5        ? launch_ln_v<1, 5>(a, stream, pdl)
                         : K <= 512 * 3        ? launch_ln_v<2, 3>(a, stream, pdl)
                         : K <= 1024 * 3       ? launch_ln_v<4, 3>(a, stream, pdl)

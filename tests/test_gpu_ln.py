@@ -37,7 +37,10 @@ def _run(x, shift, scale, rps, ldq=None):
 
 @pytest.mark.parametrize("M,K,rps", [(2048, 1152, 256), (300, 1152, 77), (9, 64, 4), (1000, 4608, 256), (37, 1280, 1),
                                      (3, 2048, 2), (5, 2064, 2), (515, 1296, 64), (514, 1536, 64),
-                                     (513, 1552, 64), (6, 3088, 3)])
+                                     (513, 1552, 64), (6, 3088, 3),
+                                     # (the pitch of the codes is K here, a multiple of 16)
+                                     (4096, 512, 300), (4095, 528, 64), (4099, 528, 64), (4097, 784, 500), (4101, 1040, 7),
+                                     (4098, 1280, 4098), (4100, 1296, 64)])
 @pytest.mark.parametrize("mod", [True, False])
 def test_codes_and_scales_match_the_oracle(M, K, rps, mod):
     x, shift, scale = _inputs(M, K, K % 97 + M % 13, rps)
