@@ -197,8 +197,12 @@ static cudaError_t launch_daq_t(const uint16_t* xp, int64_t M, int k, int64_t ld
   // ~90 registers) left one CTA beside a running GEMM and a long serial chain per warp. Whole 8-bit layer,
   // K = 4608, N = 1152, M = 256 / 2048 / 32768: one warp 12.1 / 18.8 / 182.5 us, two 12.3 / 17.6 / 182.5,
   // four 12.1 / 17.4 / 181.7. Shorter rows want one: K = 1152 whole layer (N = 1152), M = 2048 / 32768: one
-  // 8.8 / 56.8 us, two 9.2 / 58.1, four 8.8 / 70.3 (their warps spend longer starting than working).
+  // 8.8 / 56.8 us, two 9.2 / 58.1, four 8.8 / 70.3 (their warps spend longer starting than working). So do rows of up to
+  // 2048 where there are many: DAQ alone, K = 1536, M = 333 / 2048 / 9000: one warp 1.72 / 3.18 / 7.9 us, two 1.66 / 3.58 /
+  // 8.7; K = 2048: one 1.88 / 3.66 / 9.98, two 1.72 / 4.10 / 10.1.
   if (k <= 256 * 5) return DP_ROWS(1, 5);
+  if (k <= 256 * 6 && M > 512) return DP_ROWS(1, 6);
+  if (k <= 256 * 8 && M > 512) return DP_ROWS(1, 8);
   if (k <= 512 * 5) return DP_ROWS(2, 5);
   if (k <= 1024 * 5) return DP_ROWS(4, 5);
 #undef DP_ROWS

@@ -37,7 +37,8 @@ def test_daq_matches_oracle(M, K):
 
 
 @pytest.mark.parametrize("rowsum", [True, False])
-@pytest.mark.parametrize("M,K", [(1, 1280), (6, 1288), (3, 2560), (5, 2568), (2, 4616), (3, 5120), (2, 5128)])
+@pytest.mark.parametrize("M,K", [(1, 1280), (6, 1288), (3, 2560), (5, 2568), (2, 4616), (3, 5120), (2, 5128),
+                                 (512, 1288), (513, 1288), (515, 1536), (514, 1544), (517, 2048), (513, 2056)])
 def test_daq_rows_shared_by_warps(M, K, rowsum):
     """Row lengths on both sides of every change in the number of warps that share a row."""
     x = synth.activations(synth.BASE_SEED, 4, 2, M, K, 1.0, n_out=max(1, K // 100))
