@@ -50,7 +50,7 @@ daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
     const int idx = lane + TPR * i;
-    if (idx < nvec) ld_nc_u32x4(xr + idx, v[i]);
+    if (idx < nvec) ld_stream_u32x4(xr + idx, v[i]);
     else v[i] = make_uint4(0, 0, 0, 0);
   }
   uint32_t m = 0;
@@ -120,7 +120,7 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
   uint32_t m = 0;
   for (int idx = lane; idx < nvec; idx += 32) {
-    uint4 v = xr[idx];
+    const uint4 v = ld_global_v4(xr + idx);
     m = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(m, v.x), v.y), v.z), v.w);
   }
   m = warp_max_u32(max(m & 0xFFFFu, m >> 16));
@@ -129,7 +129,7 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
   const QRow qr(q, row, ldq, tiled_kb);
   int sum = 0;
   for (int idx = lane; idx < nvec; idx += 32) {
-    uint2 o = quant_vec<EO>(xr[idx], inv);
+    uint2 o = quant_vec<EO>(ld_global_v4(xr + idx), inv);
     qr.store(idx, o);
     sum = __dp4a(static_cast<int>(o.x), 0x01010101, sum);
     sum = __dp4a(static_cast<int>(o.y), 0x01010101, sum);

@@ -8,11 +8,14 @@
 
 namespace dp {
 
-__device__ __forceinline__ uint32_t ld_nc_u32x4(const uint4* p, uint4& v) {
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+// Input of a kernel that starts ahead of its predecessor: an ordinary load, not the read-only path. Loads of the latter kind
+// may be moved ahead of griddepcontrol.wait (read-only means for the whole kernel): a restructured quantization
+// kernel read its input before the GEMM that wrote it had finished.
+__device__ __forceinline__ void ld_stream_u32x4(const uint4* p, uint4& v) {
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return 0;
+               : "l"(p)
+               : "memory");
 }
 
 __device__ __forceinline__ uint32_t absmax_bits2(uint32_t m, uint32_t w) {
@@ -158,7 +161,7 @@ __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
     const int idx = lane + 32 * i;
-    if (idx < nvec) ld_nc_u32x4(xr + idx, v[i]);
+    if (idx < nvec) ld_stream_u32x4(xr + idx, v[i]);
     else v[i] = make_uint4(0, 0, 0, 0);
   }
   // threshold: magnitude bits (bf16 pattern, sign cleared) of the clip_rank-th largest element

@@ -369,6 +369,18 @@ __device__ __forceinline__ uint4 ld_global_v4(const void* p) {
   return v;
 }
 
+// A word that an earlier kernel on the stream has written, read behind griddepcontrol.wait (see ld_stream_u32x4).
+__device__ __forceinline__ float ld_global_f32(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int ld_global_s32(const int32_t* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // 32-byte global store (sm_100): `p` 32-byte aligned. Output rows are written once and not read back
 // by the kernel, so they bypass L1 allocation (measured: 2-8 % shorter layers at M = 2048, 3 % at
 // M = 32768 for the widest outputs; an L2 evict-first policy on top changed nothing).

@@ -280,7 +280,7 @@ struct RowEpilogue {
     float sa[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)  // from an earlier kernel: fetched while waiting
-      sa[i] = (p.x == nullptr && i < live) ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
+      sa[i] = (p.x == nullptr && i < live) ? ld_global_f32(p.s_a + row0 + 8 * i) : 0.0f;
     if (col != staged_col) {
       float sv[4], bv[4];
 #pragma unroll

@@ -175,8 +175,8 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       live[i] = row0 + 8 * i < p.M;
-      sa[i] = live[i] ? __ldg(p.s_a + row0 + 8 * i) : 0.0f;
-      rs[i] = (ZP == ZP_8BIT && live[i]) ? __ldg(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
+      sa[i] = live[i] ? ld_global_f32(p.s_a + row0 + 8 * i) : 0.0f;
+      rs[i] = (ZP == ZP_8BIT && live[i]) ? ld_global_s32(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
     }
     __syncwarp();
     wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
@@ -224,7 +224,7 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           rs_g[i] = rs[i];
-          if (live[i] && G + 1 < p.ng) rs[i] = __ldg(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
+          if (live[i] && G + 1 < p.ng) rs[i] = ld_global_s32(p.rowsum + (row0 + 8 * i) * p.ng + G + 1);
         }
       }
       tmem_ld_wait();
@@ -485,7 +485,7 @@ group_rowsum_kernel(const int8_t* __restrict__ q, int64_t M, int K, int64_t ldq,
   for (int k = lane * 16; k < K; k += 32 * 16) {
     const int8_t* src = tiled ? q + ((m >> 7) * (K >> 7) + (k >> 7)) * 16384 + (m & 127) * 128 + (k & 127)
                               : q + m * ldq + k;
-    const uint4 v = *reinterpret_cast<const uint4*>(src);
+    const uint4 v = ld_global_v4(src);
     int s = __dp4a(static_cast<int>(v.x), 0x01010101, 0);
     s = __dp4a(static_cast<int>(v.y), 0x01010101, s);
     s = __dp4a(static_cast<int>(v.z), 0x01010101, s);

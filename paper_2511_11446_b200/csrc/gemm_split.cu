@@ -146,7 +146,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (p.early_w) pdl_wait();  // s_a is written by the preceding kernel
     pdl_launch_dependents();  // as in gemm_tc.cu
     if constexpr (!F16) {
-      if (et >= 128) s_sa[et - 128] = m_row + et - 128 < p.M ? __ldg(p.s_a + m_row + et - 128) : 0.0f;
+      if (et >= 128) s_sa[et - 128] = m_row + et - 128 < p.M ? ld_global_f32(p.s_a + m_row + et - 128) : 0.0f;
     }
     bool ok = mbar_wait(acc_full, 0u, abort_flag);
     ok = __all_sync(0xFFFFFFFFu, ok);

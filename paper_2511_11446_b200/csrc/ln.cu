@@ -85,10 +85,10 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArg
     const int idx = lane + TPR * i;
     v[i] = sh[i] = sc[i] = make_uint4(0, 0, 0, 0);
     if (idx < nvec) {
-      ld_nc_u32x4(xr + idx, v[i]);
+      ld_stream_u32x4(xr + idx, v[i]);
       if constexpr (MOD && !LATE) {
-        sh[i] = __ldg(shr + idx);
-        sc[i] = __ldg(scr + idx);
+        sh[i] = ld_global_v4(shr + idx);
+        sc[i] = ld_global_v4(scr + idx);
       }
     }
   }
@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(kLnThreads) ln_modulate_daq_kernel(const LnArg
   for (int i = 0; i < MAXV; ++i) {
     if (lane + TPR * i >= nvec) continue;
     if constexpr (MOD && LATE) {
-      sh[i] = __ldg(shr + lane + TPR * i);
-      sc[i] = __ldg(scr + lane + TPR * i);
+      sh[i] = ld_global_v4(shr + lane + TPR * i);
+      sc[i] = ld_global_v4(scr + lane + TPR * i);
     }
     h[i][0] = ln_pair<MOD>(v[i].x, sc[i].x, sh[i].x, nmean2, rstd2, one2);
     h[i][1] = ln_pair<MOD>(v[i].y, sc[i].y, sh[i].y, nmean2, rstd2, one2);
