@@ -325,12 +325,16 @@ int dp_wq_linear_static(const dp_weight* w, const void* x_bf16, int64_t ldx, int
 typedef struct dp_plan dp_plan;
 int dp_plan_create(const dp_weight* layers, int32_t n_layers, const int64_t* M_per_layer,
                    uint32_t flags, dp_plan** out);
-/* Bytes of device scratch a run of the plan needs (256-byte aligned). Consecutive layers use the scratch in turn, in as
+/* Bytes of device scratch a run of the plan needs (256-byte aligned). Three or more tensor-core layers in a row (per-channel or
+ * 16-bit ones, in a plan that names no kernel variant) are launched together, up to 16 layers and up to 64 MB of scratch
+ * to a unit: where there are such units, two parts of the largest one's scratch (codes, scales, weights expanded to int8),
+ * at most 128 MB. At least, for layers launched one by one: consecutive layers use the scratch in turn, in as
  * many parts of the largest layer's dp_wq_linear_workspace as the launch order overlaps: three where a per-channel 3-, 4- or
  * 8-bit layer has 33 to 1024 rows, two where such layers all have more, one with DP_FLAG_NO_PDL, DP_FLAG_FUSED_DAQ or
- * without such layers; grouped small-M layers under a DAQ policy may need more. */
+ * without such layers; grouped small-M layers under a DAQ policy may need more. What a plan needs is the larger. */
 size_t dp_plan_workspace(const dp_plan* plan);
-/* Which kernel the plan runs layer `layer` with (for reports and for timing that kernel alone):
+/* Which kernel the plan runs layer `layer` with where it is launched on its own (for reports and for timing that kernel alone;
+ * layers launched together share a kernel of their own, see dp_plan_run):
  * *tile_n = tile width in output channels, *cta_group = 1 or 2 CTAs per row tile,
  * *weight_stationary = 0, 1 (weight-stationary kernel) or 2 (activation-stationary kernel; *tile_n is
  * then its sub-block width), *small_m = 1 when the CUDA-core small-M kernel is used (the other three
@@ -342,7 +346,7 @@ int dp_plan_layer_variant(const dp_plan* plan, int32_t layer, int32_t* tile_n, i
 int dp_plan_layer_unpack_first(const dp_plan* plan, int32_t layer, int32_t* unpack_first);
 /* Replaces the kernel variant of layer `layer` by the one `flags` names (the tuning flags of
  * dp_wq_linear: DP_FLAG_TILE_N, [NO_]CTA_PAIR, [NO_]WEIGHT_STATIONARY, [NO_]ACT_STATIONARY, UNPACK_FIRST; anything left
- * open is chosen as dp_wq_linear would): lets a deployment keep the outcome of one
+ * open is chosen as dp_wq_linear would), with which it is then launched on its own: lets a deployment keep the outcome of one
  * DP_FLAG_AUTOTUNE run and apply it to later plans. Host only; may raise dp_plan_workspace, so ask
  * again afterwards. Small-M layers and unknown bits are refused (DP_ERR_INVALID_ARG), tile widths
  * that do not fit the layer with DP_ERR_SHAPE; the plan is unchanged on error. Not to be called
@@ -379,6 +383,9 @@ void dp_plan_destroy(dp_plan* plan);
  * is enqueued. Enqueues only; capturable in a CUDA graph.
  * Results are those of running the layers in this order. The quantization (and weight expansion) of a
  * layer may run beside the GEMMs of the one or two layers before it: it reads only its own x and constants.
+ * Up to 16 consecutive tensor-core layers are one launch that prepares their operands and one for all their GEMMs (see
+ * dp_plan_workspace), in steps in which no x of theirs overlaps the y of an earlier one of them, no y another's, and
+ * no 16-bit layer's x a later one's y; in other steps they are launched one by one.
  * Where a layer's x overlaps an earlier layer's y (a linear fed by another; the call compares the ranges
  * M_l * K_l and M_l * N_l elements long) it waits for the GEMM that writes it. Weights, scales,
  * zero-points and biases of all layers are constants of the call: no y may overlap them. While a layer's

@@ -648,6 +648,7 @@ struct PlanLayer {
   bool simt;
   int bn, cg, ws;
   int pre;  // weights expanded to int8 scratch first, 8-bit kernel on the copy
+  bool fixed = false;  // dp_plan_set_layer_flags has named its variant
   CUtensorMap tmap_w;
   size_t x_offset;  // byte offset of this layer's input inside one staged step (host-input path)
 };
@@ -655,6 +656,21 @@ struct TmapACache {
   const void* ptr;
   int64_t M, K;
   CUtensorMap map;
+};
+// Consecutive layers whose quantization (with the expansion of their weights) is one launch and whose GEMMs are another,
+// in a step whose pointers let them run in any order (group_independent).
+struct PlanGroup {
+  std::vector<int> layers;
+  GemmPlanSchedule sched;
+  struct Place {
+    size_t q, s_a, w8;  // offsets in the group's part of the workspace: codes, scales, expanded weights
+  };
+  std::vector<Place> place;
+  // The tensor maps of the members, by place in the launch, for the address that a part of the workspace had last.
+  struct Maps {
+    const uint8_t* base = nullptr;
+    CUtensorMap a[kPlanGroupMax], w[kPlanGroupMax];
+  } maps[2];
 };
 struct dp_plan {
   std::vector<PlanLayer> layers;
@@ -666,6 +682,10 @@ struct dp_plan {
   std::vector<TmapACache> a_cache;
   std::vector<std::vector<int>> groups;  // small-M layers of equal shape, run first in every step
   std::vector<char> grouped;             // per layer: member of a group
+  std::vector<PlanGroup> units;          // tensor-core layers launched together
+  std::vector<int> unit_of;              // per layer: its unit, or -1
+  size_t unit_bytes;                     // of the two parts that units take in turn
+  std::mutex maps_lock;                  // of the units' tensor maps
   int32_t* daq_sync;                     // device counters of the in-kernel DAQ (nullptr: DAQ in its own kernel)
   // DAQ policy (dp_plan_set_daq): clip percentile in 1/1000 %, 100000 = the maximum; activation bits
   // of the three time bins of [0, daq_timesteps)
@@ -675,6 +695,7 @@ struct dp_plan {
   void need(size_t layer_bytes) {  // room for a layer of this scratch size
     part_bytes = std::max(part_bytes, align256(layer_bytes));
     workspace_bytes = std::max(workspace_bytes, parts * part_bytes);
+    workspace_bytes = std::max(workspace_bytes, 2 * unit_bytes);
   }
 };
 
@@ -690,6 +711,64 @@ static int plan_parts(const dp_plan& p, bool fused_daq) {
   for (const PlanLayer& L : p.layers)
     if (runs_in_two(L)) parts = std::max(parts, L.M <= kSkewMaxRows ? 3 : 2);
   return parts;
+}
+
+// Layers are launched together (gemm_plan.cu) where three or more that follow each other can be: per-channel or 16-bit layers
+// whose variant nobody has named. A unit takes layers until its part of the workspace would be larger than kUnitBytes.
+constexpr size_t kUnitBytes = 64u << 20;
+constexpr size_t kUnitMinLayers = 3;
+static bool unit_takes(const dp_plan& p, const PlanLayer& L) {
+  constexpr uint32_t kNeutral = DP_FLAG_FORCE_MMA | DP_FLAG_NO_PDL | DP_FLAG_UNPACK_FIRST;
+  if ((p.flags & ~kNeutral) || p.daq_sync != nullptr || L.simt || L.fixed || L.M <= 0 || L.w.group_size > 0) return false;
+  return (L.w.N % 128 == 0 || L.w.N % 192 == 0) && (L.w.bits == 16 || L.w.K <= kPlanMaxK);
+}
+static size_t unit_layer_bytes(const PlanLayer& L, PlanGroup::Place* at, size_t off) {
+  if (L.w.bits == 16) return 0;
+  const size_t q = align256(scratch_q_bytes(L.M, L.w.K)), sa = align256(sizeof(float) * static_cast<size_t>(L.M));
+  if (at) *at = {off, off + q, off + q + sa};
+  return q + sa + (L.w.bits < 8 ? align256(static_cast<size_t>(L.w.N) * L.w.K) : 0);
+}
+static void plan_build_units(dp_plan* p) {
+  p->units.clear();
+  p->unit_of.assign(p->layers.size(), -1);
+  p->unit_bytes = 0;
+  std::vector<int> run;
+  size_t bytes = 0;
+  auto close = [&]() {
+    PlanGroup u;
+    u.layers = run;
+    run.clear();
+    size_t off = 0;
+    if (u.layers.size() >= kUnitMinLayers) {
+      GemmPlanShape shape[kPlanGroupMax];
+      for (size_t i = 0; i < u.layers.size(); ++i) {
+        const PlanLayer& L = p->layers[u.layers[i]];
+        shape[i] = {L.M, L.w.N, L.w.K * (L.w.bits == 16 ? 2 : 1) / 128};
+        PlanGroup::Place at = {0, 0, 0};
+        off += unit_layer_bytes(L, &at, off);
+        u.place.push_back(at);
+      }
+      if (gemm_plan_schedule(shape, static_cast<int>(u.layers.size()), &u.sched)) {
+        for (int l : u.layers) p->unit_of[l] = static_cast<int>(p->units.size());
+        p->unit_bytes = std::max(p->unit_bytes, align256(off));
+        p->units.push_back(std::move(u));
+      }
+    }
+    bytes = 0;
+  };
+  for (size_t l = 0; l < p->layers.size(); ++l) {
+    const PlanLayer& L = p->layers[l];
+    // (a grouped small-M layer runs before everything else, but for long rows under a policy: see plan_run_step)
+    if (L.M == 0 || (p->grouped[l] && L.w.K <= 1280)) continue;
+    const bool takes = unit_takes(*p, L) && unit_layer_bytes(L, nullptr, 0) <= kUnitBytes;
+    const size_t add = takes ? unit_layer_bytes(L, nullptr, 0) : 0;
+    if (!run.empty() && (!takes || bytes + add > kUnitBytes || run.size() == static_cast<size_t>(kPlanGroupMax))) close();
+    if (!takes) continue;
+    run.push_back(static_cast<int>(l));
+    bytes += add;
+  }
+  close();
+  p->need(0);
 }
 
 // Times every kernel variant that can run this layer shape (the whole layer: DAQ + GEMM, as the
@@ -821,6 +900,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   p->x_bytes = 0;
   p->copy_stream = nullptr;
   p->daq_sync = nullptr;
+  p->unit_bytes = 0;
   p->daq_p_e3 = 100000;
   p->daq_timesteps = 0;
   p->daq_bits[0] = p->daq_bits[1] = p->daq_bits[2] = 8;
@@ -936,6 +1016,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
     dp_plan_destroy(p);
     return fail(DP_ERR_CUDA, "plan stream/event creation: %s", cudaGetErrorString(e));
   }
+  plan_build_units(p);
   *out = p;
   return DP_OK;
 }
@@ -995,6 +1076,8 @@ extern "C" int dp_plan_set_layer_flags(dp_plan* plan, int32_t layer, uint32_t fl
                 layer, L.w.N, L.w.K, L.w.bits);
   if (int st = gemm_encode_w(&T.tmap_w, T.w.qweight, T.w.N, T.w.K, T.w.bits, T.bn, T.cg)) return st;
   L = T;
+  L.fixed = true;
+  plan_build_units(plan);
   const size_t ws = dp_wq_linear_workspace(L.M, L.w.N, L.w.K, L.w.bits,
                                            L.pre ? DP_FLAG_UNPACK_FIRST : DP_FLAG_NO_UNPACK_FIRST);
   plan->need(ws);
@@ -1057,8 +1140,128 @@ struct PlanRun {
                             // own wait)
   int pending = -1;         // layer whose DAQ has been launched and whose GEMM has not
   uint8_t* pending_scratch = nullptr;
+  int unit = -1;               // the last launch is this unit's GEMM kernel, with the outputs unit_ys; the next takes the other part
+  void* const* unit_ys = nullptr;
+  int unit_slot = 0;
   bool pending_ready = false;  // a tensor-core GEMM has been launched since, so that DAQ is done when the next launch starts
 };
+
+// Whether a step's pointers let a unit's layers run in any order and beside each other: no x overlaps the y of an earlier
+// member, no y another's, and no 16-bit layer's x (read by the GEMM itself) a later one.
+static bool unit_independent(const dp_plan& p, const PlanGroup& u, const void* const* xs, void* const* ys) {
+  for (size_t j = 0; j < u.layers.size(); ++j) {
+    const int b = u.layers[j];
+    const PlanLayer& B = p.layers[b];
+    for (size_t i = 0; i < j; ++i) {
+      const int a = u.layers[i];
+      const PlanLayer& A = p.layers[a];
+      if (overlap(xs[b], B.M * B.w.K, ys[a], A.M * A.w.N) || overlap(ys[b], B.M * B.w.N, ys[a], A.M * A.w.N)) return false;
+      if (A.w.bits == 16 && overlap(xs[a], A.M * A.w.K, ys[b], B.M * B.w.N)) return false;
+    }
+  }
+  return true;
+}
+
+// Tensor maps of a unit in the part of the workspace at `base`.
+static int unit_maps(dp_plan* plan, PlanGroup* u, uint8_t* base, int slot, CUtensorMap* a, CUtensorMap* w) {
+  std::lock_guard<std::mutex> lock(plan->maps_lock);
+  PlanGroup::Maps& m = u->maps[slot];
+  if (m.base != base) {
+    m.base = nullptr;
+    for (int o = 0; o < u->sched.n; ++o) {
+      const PlanLayer& L = plan->layers[u->layers[u->sched.order[o]]];
+      const PlanGroup::Place& at = u->place[u->sched.order[o]];
+      int st = DP_OK;
+      if (L.w.bits == 16) {
+        st = gemm_encode_w_rows(&m.w[o], L.w.qweight, static_cast<uint64_t>(L.w.K) * 2, L.w.N, 128, u->sched.bn[o] / 2, true);
+      } else {
+        st = gemm_encode_a_tiled(&m.a[o], reinterpret_cast<int8_t*>(base + at.q), L.M, L.w.K);
+        if (st == DP_OK)
+          st = gemm_encode_w(&m.w[o], L.w.bits == 8 ? L.w.qweight : base + at.w8, L.w.N, L.w.K, 8, u->sched.bn[o], 2);
+      }
+      if (st != DP_OK) return st;
+    }
+    m.base = base;
+  }
+  memcpy(a, m.a, sizeof(CUtensorMap) * u->sched.n);
+  memcpy(w, m.w, sizeof(CUtensorMap) * u->sched.n);
+  return DP_OK;
+}
+
+// A unit's two launches. The first runs beside the GEMM kernel of the unit before, if that was the last launch and this
+// unit reads none of its outputs; then the part of the workspace it writes is free, for the unit before that has finished (a
+// GEMM kernel lets its successor start after its own wait).
+static int run_unit(dp_plan* plan, int unit, const void* const* xs, void* const* ys, void* workspace, bool robust, int act_bits,
+                    int32_t* status, cudaStream_t stream, PlanRun* run) {
+  PlanGroup& u = plan->units[unit];
+  const bool pdl = !(plan->flags & DP_FLAG_NO_PDL);
+  bool ahead = pdl && run->unit >= 0;
+  if (ahead)
+    for (int a : plan->units[run->unit].layers)
+      for (int b : u.layers)
+        if (overlap(xs[b], plan->layers[b].M * plan->layers[b].w.K, run->unit_ys[a], plan->layers[a].M * plan->layers[a].w.N))
+          ahead = false;
+  const int slot = run->unit_slot;
+  uint8_t* base = static_cast<uint8_t*>(workspace) + slot * plan->unit_bytes;
+  GemmPlanParams g;
+  int st = unit_maps(plan, &u, base, slot, g.tmap_a, g.tmap_w);
+  if (st != DP_OK) return st;
+  PlanPrepParams pp;
+  pp.n_seg = 0;
+  pp.early = run->chained && pdl;
+  pp.ahead = ahead;
+  pp.qmax = static_cast<float>((1 << (act_bits - 1)) - 1);
+  for (int o = 0; o < u.sched.n; ++o) {
+    const int i = u.sched.order[o], l = u.layers[i];
+    const PlanLayer& L = plan->layers[l];
+    const PlanGroup::Place& at = u.place[i];
+    GemmPlanLayer& G = g.layer[o];
+    G.f16 = L.w.bits == 16;
+    G.s_a = reinterpret_cast<const float*>(base + at.s_a);
+    G.s_w = L.w.s_w;
+    G.bias = static_cast<const uint16_t*>(L.w.bias);
+    G.y = static_cast<uint16_t*>(ys[l]);
+    G.M = L.M;
+    G.N = L.w.N;
+    G.kb = L.w.K * (G.f16 ? 2 : 1) / 128;
+    G.bn = u.sched.bn[o];
+    G.n_tiles = L.w.N / G.bn;
+    auto seg = [&](PlanPrepSeg::Kind kind, const void* src, void* dst, int64_t count, int arg) {
+      PlanPrepSeg& s = pp.seg[pp.n_seg++];
+      s.src = src;
+      s.dst = static_cast<int8_t*>(dst);
+      s.s_a = reinterpret_cast<float*>(base + at.s_a);
+      s.count = count;
+      s.kind = static_cast<int16_t>(kind);
+      s.arg = static_cast<int16_t>(arg);
+      s.rank = robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1;
+    };
+    const int64_t codes = static_cast<int64_t>(L.w.N) * L.w.K;
+    if (G.f16) {
+      st = gemm_encode_bytes_2d(&g.tmap_a[o], xs[l], static_cast<uint64_t>(L.w.K) * 2, static_cast<uint64_t>(L.M),
+                                static_cast<uint64_t>(L.w.K) * 2, 128, 128);
+      if (st != DP_OK) return st;
+    } else {
+      seg(PlanPrepSeg::ROWS, xs[l], base + at.q, L.M, L.w.K / 8);
+    }
+    if (L.w.bits < 8) seg(PlanPrepSeg::EXPAND, L.w.qweight, base + at.w8, codes / 32, L.w.bits);
+    else seg(PlanPrepSeg::FETCH, L.w.qweight, nullptr, codes * L.w.bits / 8, 0);
+  }
+  st = launch_plan_prep(pp, robust, stream, pdl);
+  if (st != DP_OK) return st;
+  memcpy(g.runs, u.sched.runs, sizeof(g.runs));
+  g.n_layers = u.sched.n;
+  g.pairs = u.sched.pairs;
+  g.status = status;
+  st = launch_gemm_plan(g, stream, pdl);
+  if (st != DP_OK) return st;
+  run->chained = true;
+  run->y = nullptr;
+  run->unit = unit;
+  run->unit_ys = ys;
+  run->unit_slot = slot ^ 1;
+  return DP_OK;
+}
 
 // Tensor-core layers are launched D0 D1 G0 D2 G1 D3 G2 ...: DAQ (and weight expansion) of a layer runs beside the GEMM
 // two layers before it, and a GEMM, whose operands are then complete, starts on each SM as the GEMM before it leaves
@@ -1115,6 +1318,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     if (st != DP_OK) return st;
     run->chained = true;
     run->y = nullptr;
+    run->unit = -1;
   }
   // A later tensor-core layer's packed weights and its input start towards L2 while a GEMM runs. A hint, not a
   // reordering: if that input is still to be written (by this layer, say), the hint fetches bytes that the write then
@@ -1140,6 +1344,7 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
                               robust ? clip_rank_of(plan->daq_p_e3, L.w.K) : 1, act_bits, nullptr, ahead, part, true);
     gemm_set_next_reads(nullptr, 0, nullptr, 0);
     run->chained = true;
+    run->unit = -1;
     return st;
   };
   auto flush = [&]() {  // the GEMM that is still to be launched
@@ -1156,9 +1361,20 @@ static int plan_run_step(dp_plan* plan, int32_t t, const void* const* xs, void* 
     run->y_elems = L.M * L.w.N;
     return st;
   };
+  bool together = false;  // the unit that l belongs to is launched as one
   for (int l = 0; l < n; ++l) {
     const PlanLayer& L = plan->layers[l];
     if (L.M == 0 || (plan->grouped[l] && !group_splits(l))) continue;
+    if (const int u = plan->unit_of[l]; u >= 0) {
+      const PlanGroup& U = plan->units[u];
+      if (l == U.layers.front()) together = unit_independent(*plan, U, xs, ys);
+      if (together) {
+        if (l != U.layers.front()) continue;
+        if (int st = flush()) return st;
+        if (int st = run_unit(plan, u, xs, ys, workspace, robust, act_bits, status, stream, run)) return st;
+        continue;
+      }
+    }
     if (!runs_in_two(L) || plan->daq_sync != nullptr || (plan->flags & DP_FLAG_NO_PDL)) {
       if (int st = flush()) return st;
       uint8_t* scratch = static_cast<uint8_t*>(workspace) + run->slot * plan->part_bytes;

@@ -6,6 +6,8 @@
 // max is exact); the quantizer is one fused multiply-add per element: x * fl(127/a) + 1.5*2^23
 // rounds the exact product once, half to even, and leaves the integer in the low mantissa bits.
 // HBM-bound: 2 bytes read + 1 byte written per element.
+#include <limits.h>
+
 #include "daq_device.cuh"
 
 namespace dp {
@@ -25,24 +27,16 @@ __device__ __forceinline__ void daq_end(const UnpackJob& job) {
   if (job.ahead && blockIdx.x == 0) pdl_wait();
 }
 
-// RW warps share a row: MAXV = 16-byte vectors held per lane (a row of up to 256 * RW * MAXV elements in
-// registers). SUM: also the row's code sum.
+// CTA `block` of a launch over rows: RW warps share a row, MAXV = 16-byte vectors held per lane (a row of up to 256 * RW *
+// MAXV elements in registers). SUM: also the row's code sum. part: a word per warp of the CTA.
 template <int RW, int MAXV, bool EO, bool SUM>
-__global__ void __launch_bounds__(kDaqThreads)
-daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
-                int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
-                int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
+__device__ __forceinline__ void daq_rows(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
+                                         int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
+                                         int32_t* __restrict__ rowsum, int tiled_kb, int block, uint32_t* part) {
   constexpr int kRows = kDaqThreads / 32 / RW;  // rows of a CTA
   constexpr int TPR = 32 * RW;
-  __shared__ uint32_t part[kDaqThreads / 32];
-  daq_begin(job);
-  if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
-    unpack_units(job, blockIdx.x - job.first_block);
-    return;
-  }
-  if (!job.ahead) pdl_wait();
   const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;  // row of the CTA, position in the row
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + rw;
+  const int64_t row = static_cast<int64_t>(block) * kRows + rw;
   const bool live = row < M;
   const int nvec = live ? K >> 3 : 0;
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
@@ -98,6 +92,21 @@ daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
     }
     if (lane == 0 && live) rowsum[row] = sum;
   }
+}
+
+template <int RW, int MAXV, bool EO, bool SUM>
+__global__ void __launch_bounds__(kDaqThreads)
+daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
+                int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
+                int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
+  __shared__ uint32_t part[kDaqThreads / 32];
+  daq_begin(job);
+  if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
+    unpack_units(job, blockIdx.x - job.first_block);
+    return;
+  }
+  if (!job.ahead) pdl_wait();
+  daq_rows<RW, MAXV, EO, SUM>(x, M, K, ldx, q, ldq, s_a, rowsum, tiled_kb, blockIdx.x, part);
   daq_end(job);
 }
 
@@ -173,6 +182,87 @@ __global__ void __launch_bounds__(kDaqWarps * 32)
 unpack_kernel(const UnpackJob job) {
   daq_begin(job);
   unpack_units(job, blockIdx.x);
+}
+
+// ---- the preparation of a plan's group of layers (gemm_plan.cu), in one launch ------------------------
+// A CTA works on one segment: rows of a layer to quantize, codes to expand, weights to send into L2. It runs beside the
+// GEMM kernel of the group before, which leaves room for a few CTAs of this size on an SM, so a CTA is small (128 threads,
+// register rows of five vectors a lane, longer rows by two or four warps) and keeps enough loads in flight: four units of
+// 32 codes a thread.
+constexpr int kExpandUnits = 4, kFetchBytes = 32768, kFetchThreads = 4;
+
+template <int BITS>
+__device__ __forceinline__ void prep_expand(const PlanPrepSeg& s, int block, bool wait) {
+  const int64_t u0 = static_cast<int64_t>(block) * (kDaqThreads * kExpandUnits) + threadIdx.x;
+  uint32_t pk[kExpandUnits][BITS];
+#pragma unroll
+  for (int i = 0; i < kExpandUnits; ++i) {
+    const int64_t u = u0 + i * kDaqThreads;
+    if (u >= s.count) continue;
+    if constexpr (BITS == 4) {
+      uint4 v;
+      ld_stream_u32x4(static_cast<const uint4*>(s.src) + u, v);
+      pk[i][0] = v.x, pk[i][1] = v.y, pk[i][2] = v.z, pk[i][3] = v.w;
+    } else {
+      const uint32_t* w = static_cast<const uint32_t*>(s.src) + u * 3;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) pk[i][j] = __ldg(w + j);
+    }
+  }
+  if (wait) pdl_wait();
+#pragma unroll
+  for (int i = 0; i < kExpandUnits; ++i) {
+    const int64_t u = u0 + i * kDaqThreads;
+    if (u >= s.count) continue;
+    uint32_t w[8];
+    expand_unit<BITS>(pk[i], w, 1u << (BITS - 1));
+    st_global_v8(reinterpret_cast<uint4*>(s.dst) + u * 2, w);
+  }
+}
+
+template <bool ROBUST>
+__global__ void __launch_bounds__(kDaqThreads, ROBUST ? 4 : 12)
+plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
+  __shared__ uint32_t part[kDaqThreads / 32];
+  if (!p.early) pdl_wait();
+  pdl_launch_dependents();
+  // (a search over the segments one by one was a chain of constant-cache misses: 3 us of a CTA's 5)
+  int i = 0;
+#pragma unroll
+  for (int step = kPlanPrepSegs / 2; step > 0; step >>= 1)
+    if (static_cast<int>(blockIdx.x) >= p.first_block[i + step]) i += step;
+  const PlanPrepSeg& s = p.seg[i];
+  const int block = blockIdx.x - p.first_block[i];
+  if (s.kind == PlanPrepSeg::EXPAND) {
+    if (s.arg == 4) prep_expand<4>(s, block, !p.ahead);
+    else prep_expand<3>(s, block, !p.ahead);
+  } else if (s.kind == PlanPrepSeg::FETCH) {
+    const int64_t at = (static_cast<int64_t>(block) * kFetchThreads + threadIdx.x) * kFetchBytes;
+    if (threadIdx.x < kFetchThreads && at < s.count)
+      bulk_prefetch_l2(static_cast<const uint8_t*>(s.src) + at,
+                       static_cast<uint32_t>(s.count - at < kFetchBytes ? s.count - at : kFetchBytes));
+  } else {
+    if (!p.ahead) pdl_wait();
+    const uint16_t* x = static_cast<const uint16_t*>(s.src);
+    const int K = s.arg * 8, kb = K >> 7;
+    if constexpr (ROBUST) {
+      const int64_t row = static_cast<int64_t>(block) * (kDaqThreads / 32) + (threadIdx.x >> 5);
+      if (row < s.count) {
+        const int lane = threadIdx.x & 31;
+        const QRow qr(s.dst, row, K, kb);
+        float sc;
+        int sum;
+        if (K <= 256 * 5) robust_row<5>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
+        else robust_row<18>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
+        if (lane == 0) s.s_a[row] = sc;
+      }
+    } else {
+      if (K <= 256 * 5) daq_rows<1, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
+      else if (K <= 512 * 5) daq_rows<2, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
+      else daq_rows<4, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
+    }
+  }
+  if (p.ahead && blockIdx.x == 0) pdl_wait();  // as daq_end
 }
 
 static unsigned unpack_blocks(const UnpackJob& job, int threads) {
@@ -254,6 +344,28 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
     e = launch(daq_rows_robust_kernel<18>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank,
                qmax, tiled_kb, job);
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "robust DAQ launch failed: %s", cudaGetErrorString(e));
+  return DP_OK;
+}
+
+int launch_plan_prep(PlanPrepParams& p, bool robust, cudaStream_t stream, bool pdl) {
+  int64_t at = 0;
+  for (int i = 0; i < p.n_seg; ++i) {
+    PlanPrepSeg& s = p.seg[i];
+    p.first_block[i] = static_cast<int32_t>(at);
+    int64_t per = kDaqThreads * kExpandUnits;
+    if (s.kind == PlanPrepSeg::FETCH) {
+      per = static_cast<int64_t>(kFetchBytes) * kFetchThreads;
+    } else if (s.kind == PlanPrepSeg::ROWS) {
+      const int K = s.arg * 8;
+      per = kDaqThreads / 32 / (robust || K <= 256 * 5 ? 1 : K <= 512 * 5 ? 2 : 4);
+    }
+    at += (s.count + per - 1) / per;
+  }
+  for (int i = p.n_seg; i < kPlanPrepSegs; ++i) p.first_block[i] = INT_MAX;
+  const dim3 grid(static_cast<unsigned>(at)), block(kDaqThreads);
+  const cudaError_t e = robust ? launch(plan_prep_kernel<true>, grid, block, 0, stream, pdl, p)
+                               : launch(plan_prep_kernel<false>, grid, block, 0, stream, pdl, p);
+  if (e != cudaSuccess) return fail(DP_ERR_CUDA, "plan preparation launch failed: %s", cudaGetErrorString(e));
   return DP_OK;
 }
 

@@ -165,6 +165,66 @@ void gemm_debug_skip_stage_load(int32_t kb);  // see dp_debug_skip_stage_load
 // device ranges of the caller's, or nullptr.
 void gemm_set_next_reads(const void* w, size_t w_bytes, const void* x, size_t x_bytes);
 
+// gemm_plan.cu -- the GEMMs of several layers of a plan in one launch.
+constexpr int kPlanGroupMax = 16, kPlanMaxPairs = 80;
+struct GemmPlanLayer {  // of a layer, copied into shared memory by each CTA
+  const float* s_a;
+  const float* s_w;
+  const uint16_t* bias;
+  uint16_t* y;  // [M][N]
+  int64_t M;
+  int32_t N, kb;  // kb: 128-byte k-blocks
+  int32_t bn, n_tiles;
+  int32_t f16, pad;
+};
+struct GemmPlanRuns {  // of a pair: tiles [begin[l], end[l]) of layer l
+  uint16_t begin[kPlanGroupMax], end[kPlanGroupMax];
+};
+struct GemmPlanParams {
+  CUtensorMap tmap_a[kPlanGroupMax];  // int8 codes as 128 x 128 tiles, or (f16) bf16 [M][K]
+  CUtensorMap tmap_w[kPlanGroupMax];  // int8 or bf16 weights, boxes of bn / 2 rows x 128 bytes
+  GemmPlanRuns runs[kPlanMaxPairs];
+  GemmPlanLayer layer[kPlanGroupMax];
+  int32_t n_layers, pairs;
+  int32_t* status;
+};
+struct GemmPlanShape {
+  int64_t M;
+  int32_t N, kb;
+};
+struct GemmPlanSchedule {  // by place in the launch: which layer, its tile width, its tiles' runs
+  int n, pairs;
+  int order[kPlanGroupMax], bn[kPlanGroupMax];
+  GemmPlanRuns runs[kPlanMaxPairs];
+};
+bool gemm_plan_schedule(const GemmPlanShape* shape, int n, GemmPlanSchedule* out);
+int launch_gemm_plan(const GemmPlanParams& p, cudaStream_t stream, bool pdl);
+int gemm_plan_init_device();
+double gemm_pair_tile_us(int bn, int kb);  // expected time of a pair's tile
+
+// daq.cu -- what those GEMMs read, prepared in one launch: activations quantized, packed weights expanded, weights that
+// are read as they are sent on their way into L2.
+struct PlanPrepSeg {
+  enum Kind { ROWS, EXPAND, FETCH };
+  const void* src;      // bf16 [M][K]; packed codes; weights
+  int8_t* dst;          // codes as 128 x 128 tiles; int8 [N][K]
+  float* s_a;
+  int64_t count;        // rows; units of 32 codes; bytes
+  int16_t kind, arg;    // arg: K / 8; bits
+  int32_t rank;         // ROWS under a clip policy: rank of the threshold from the top
+};
+constexpr int kPlanPrepSegs = 2 * kPlanGroupMax;
+struct PlanPrepParams {
+  int32_t first_block[kPlanPrepSegs];  // filled by the launch (INT_MAX beyond the last segment)
+  PlanPrepSeg seg[kPlanPrepSegs];
+  int32_t n_seg;
+  int32_t early;  // the preceding kernel on the stream is of the same call: it does not write packed weights
+  int32_t ahead;  // (with early) nor x, nor does it read what this launch writes: see UnpackJob::ahead
+  float qmax;
+};
+int launch_plan_prep(PlanPrepParams& p, bool robust, cudaStream_t stream, bool pdl);
+constexpr int kPlanMaxK = 4608;  // rows that every form of the preparation holds in registers
+
 // gemm_ws.cu -- weight-stationary CTA-pair kernel (K <= 1152, N a multiple of 192 or 256).
 bool gemm_ws_supported(int32_t N, int32_t K);
 int gemm_ws_pick_bn(int32_t N);

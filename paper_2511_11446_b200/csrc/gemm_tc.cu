@@ -411,6 +411,8 @@ int gemm_init_device(int dev, int* num_sms_out, int* max_pairs_out, int* max_clu
   if (st != DP_OK) return st;
   st = gemm_grp_init_device();
   if (st != DP_OK) return st;
+  st = gemm_plan_init_device();
+  if (st != DP_OK) return st;
   *num_sms_out = sms;
   *max_pairs_out = pairs;
   return DP_OK;
@@ -506,6 +508,12 @@ double gemm_tile_cost(int64_t M, int32_t N, int32_t K, int bn, int cg, bool may_
   int splits;
   for (const TileForm& f : kTileForms)
     if (f.bn == bn && f.cg == cg) return tile_cost(f, gemm_limits(), M, N, K, 8, may_split, &splits);
+  return 1e30;
+}
+
+double gemm_pair_tile_us(int bn, int kb) {
+  for (const TileForm& f : kTileForms)
+    if (f.bn == bn && f.cg == 2) return fmax(f.per_kb * kb, f.min_tile);
   return 1e30;
 }
 
