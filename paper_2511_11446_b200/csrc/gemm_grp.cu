@@ -9,16 +9,16 @@
 //       y = bf16_rne(fma(t, s_a[m], bias[n]))
 //
 // One persistent CTA per SM walks 128 x 128 output tiles. Warp 0: TMA producer (int8 activation and
-// weight tiles, 128 bytes of K per stage). Warp 1: MMA issuer: tcgen05.mma kind::i8 in steps of 32
+// weight tiles, 128 bytes of K per stage). Warps 1 and 2: MMA issuers, which take groups in turn: tcgen05.mma kind::i8 in steps of 32
 // bytes of K; the steps of one group accumulate in one of FOUR 128-column tensor-memory buffers, the
 // next group starts in the next buffer (group boundaries need not fall on stage boundaries: g = 192
-// or 288 span one and a half or two and a quarter stages). Warps 2 and 3 bring each group's 128 scales
-// into the buffer's slot in shared memory, eight groups ahead in registers (they lie ng apart in memory, a
-// trip to L2 each; fetched by the folding warps one group ahead they set the pace). Warps 4-19: fold and
-// epilogue, 32 tokens and 32 columns per warp, read as accumulator fragments (four tokens and eight channels to a lane,
-// see RowEpilogue): per group two tcgen05.ld, int32 -> fp32 and a packed fma into 32 fp32 partial outputs
-// held in registers, then the buffer goes back to the MMA issuer; after the last group the token scale, bias,
-// bf16 rounding and 16-byte stores.
+// or 288 span one and a half or two and a quarter stages). Warp 3 brings each group's 128 scales
+// into the buffer's slot in shared memory, four groups ahead in registers (they lie ng apart in memory, a
+// trip to L2 each; fetched by the folding warps one group ahead they set the pace). Warps 4-11: fold and
+// epilogue, 32 tokens and 64 columns per warp in two blocks of 32, read as accumulator fragments (four tokens and eight
+// channels of a block to a lane, see RowEpilogue): per block two tcgen05.ld, int32 -> fp32 and fma into 64 fp32 partial
+// outputs held in registers, one block read while the other is folded; then the buffer goes back to the issuers; after the
+// last group the token scale, bias, bf16 rounding and 16-byte stores.
 // Zero-points of 3- and 4-bit layers are taken off when the packed weights are expanded to int8, up to 128 of
 // them: u - 128 is the least an int8 holds. Zero-points are bytes, though no quantizer writes one above 2^bits: the
 // expansion notes where it met one above 127, the fold warps read the notes while they wait for their first
@@ -27,11 +27,16 @@
 // usual fold keeps its own: as a second copy of the fold it cost layers with zero-points up to 7 %). For 8-bit
 // codes u - z does not fit a byte at all: the tensor core multiplies by u - 128 and (128 - z[n,G]) * rowsum_G[m] is
 // added in int32 before the conversion (form ZP_8BIT, with rowsum from a kernel of its own).
-// The fold is what bounds this kernel: 1.5 instructions per output and group, the conversion at 64 per
-// clock and SM, 256 clocks per 128 x 128 x g step against 256 of MMA at g = 128. Sixteen warps keep both busy
-// (eight, 64 columns each, left them waiting on each other): block of 4-bit layers with zero-points, g = 128,
-// M = 2048: 173 -> 110 us; with fragments and a straight-line issuer 92. Counters (K = 1152, N = 3456, g = 128, M = 8192,
-// 62.6 us): issue slots 68 %, ALU pipe 62 %, DRAM 4 %.
+// The fold is what bounds this kernel: the waits of a fold warp for the tensor core are a tenth of its time. 32 values a
+// lane and warp, conversion and fma, take a scheduler 104 clocks in a loop of nothing else (packed fma 113, fma without
+// the conversion 69), so a 128 x 128 group costs 420 clocks, with the loop around it 680 (g = 128, M = 64), against 560
+// for a k-block of the plain kernel with this tile when all SMs load. Eight warps of 64 columns do with fewer instructions a value than sixteen
+// of 32 and leave each 168 registers; packed fma needs its operands moved into pairs. K = 1152, N = 3456, M = 2048,
+// sixteen warps, packed, one issuer -> this: 4 bits with zero-points, g = 128 19.2 -> 18.8 us, g = 32 45.6 -> 44.2; 8 bits,
+// g = 64 27.5 -> 27.0, with zero-points, g = 128, 33.5 -> 29.8; K = 4608, N = 1152, M = 64, 3 bits, g = 32 54.0 -> 51.4, 8 bits with
+// zero-points, g = 64, 64.0 -> 55.0; but M = 2048, 4 bits, g = 128 23.1 -> 23.3. Block of 4-bit layers with zero-points, g = 128, M =
+// 2048: 90.6 -> 90.2. (Tried: accumulators that start at the word of the float 1.5 * 2^23, so that an addition in
+// place of the conversion makes the float: the tensor-memory stores cost more, g = 32 44 -> 58 us.)
 #include "gemm_device.cuh"
 
 namespace dp {
@@ -39,8 +44,8 @@ namespace dp {
 constexpr int kGrpBN = 128;
 constexpr int kGrpBufs = 4;
 constexpr int kGrpStages = 6;
-constexpr int kGrpFoldWarp0 = 4, kGrpFoldWarps = 16;  // (warp & 3) is the tensor-memory quadrant
-constexpr int kGrpLoadWarps = 2;                         // warps 2 and 3
+constexpr int kGrpFoldWarp0 = 4, kGrpFoldWarps = 8;  // (warp & 3) is the tensor-memory quadrant
+constexpr int kGrpIssuers = 2, kGrpScaleWarp = 3;  // warps 1 and 2 issue MMAs
 constexpr int kGrpCols = kGrpBN / (kGrpFoldWarps / 4);  // columns of a fold warp
 constexpr int kGrpThreads = (kGrpFoldWarp0 + kGrpFoldWarps) * 32;
 constexpr int kGrpScaleWords = 2 * kGrpBufs * kGrpBN + kGrpFoldWarps * kGrpCols;  // scales, zero-point terms, biases
@@ -65,21 +70,21 @@ struct GrpParams {
   int32_t* status;
 };
 
-// The MMA issuer's whole run over this CTA's tiles (one thread).
+// An MMA issuer's whole run over this CTA's tiles (one thread). The issuers take groups in turn.
 template <int U>
 __device__ __forceinline__ void grp_issue(const GrpParams& p, const uint8_t* sA, const uint8_t* sB, uint64_t* full,
                                           uint64_t* empty, uint64_t* grp_full, uint64_t* grp_empty, uint32_t tmem_base,
-                                          volatile int* abort_flag) {
+                                          int issuer, volatile int* abort_flag) {
   constexpr uint32_t idesc = idesc_i8(BM, kGrpBN);
   constexpr int NS = kGrpStages;
   const uint64_t adesc0 = smem_desc_sw128(smem_u32(sA)), bdesc0 = smem_desc_sw128(smem_u32(sB));
   const int KB = p.K / BK, total_tiles = p.m_tiles * p.n_tiles;
   const int rpg = (p.g >> 5) / U;  // runs per group
   Ring st, gb;                     // operand stage; group buffer
-  // both polled ahead: the next stage, the next group's buffer
-  bool full_next = mbar_test_wait(&full[0], 0u), room_next = true;
+  bool mine = issuer == 0;         // this issuer takes the current group
+  int pos = 0;                     // run inside the current group
+  bool full_next = mbar_test_wait(&full[0], 0u);  // polled ahead
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-    int pos = 0;  // run inside the current group
     for (int kb = 0; kb < KB; ++kb) {
       if (!full_next && !mbar_spin_wait(&full[st.s], st.ph, abort_flag)) return;
       tc_fence_after();
@@ -88,24 +93,29 @@ __device__ __forceinline__ void grp_issue(const GrpParams& p, const uint8_t* sA,
       full_next = mbar_test_wait(&full[nx.s], nx.ph);
       const uint64_t adesc = adesc0 + static_cast<uint64_t>(st.s * ((BM * BK) >> 4));
       const uint64_t bdesc = bdesc0 + static_cast<uint64_t>(st.s * ((kGrpBN * BK) >> 4));
+      bool used = false;
 #pragma unroll
       for (int u = 0; u < BK / 32 / U; ++u) {
-        if (pos == 0) {  // a new group: its buffer must have been folded
-          if (!room_next && !mbar_spin_wait(&grp_empty[gb.s], gb.ph ^ 1u, abort_flag)) return;
-          tc_fence_after();
-        }
-        const uint32_t d_tmem = tmem_base + gb.s * kGrpBN;
+        if (mine) {
+          if (pos == 0) {  // a new group: its buffer must have been folded
+            if (!mbar_spin_wait(&grp_empty[gb.s], gb.ph ^ 1u, abort_flag)) return;
+            tc_fence_after();
+          }
+          const uint32_t d_tmem = tmem_base + gb.s * kGrpBN;
 #pragma unroll
-        for (int j = 0; j < U; ++j)
-          mma_i8_ss(d_tmem, adesc + 2 * (u * U + j), bdesc + 2 * (u * U + j), idesc, (pos | j) != 0 ? 1u : 0u);
+          for (int j = 0; j < U; ++j)
+            mma_i8_ss(d_tmem, adesc + 2 * (u * U + j), bdesc + 2 * (u * U + j), idesc, (pos | j) != 0 ? 1u : 0u);
+          used = true;
+        }
         if (++pos == rpg) {
-          mma_commit(&grp_full[gb.s]);
+          if (mine) mma_commit(&grp_full[gb.s]);
           pos = 0;
+          mine = !mine;
           gb.next(kGrpBufs);
-          room_next = mbar_test_wait(&grp_empty[gb.s], gb.ph ^ 1u);
         }
       }
-      mma_commit(&empty[st.s]);
+      if (used) mma_commit(&empty[st.s]);
+      else mbar_arrive(&empty[st.s]);  // (the other issuer's alone)
       st = nx;
     }
   }
@@ -149,7 +159,8 @@ __device__ __forceinline__ bool grp_wide_zeros(const GrpParams& p, int lane) {
   return __any_sync(0xFFFFFFFFu, any != 0);
 }
 
-// A fold warp's whole run over this CTA's tiles: quadrant (warp & 3), column quarter (fw >> 2).
+// A fold warp's whole run over this CTA's tiles: quadrant (warp & 3), column half (fw >> 2). A lane folds four tokens and
+// eight channels of each of the warp's two 32-column blocks.
 template <int ZP>
 __device__ __forceinline__ void grp_fold(const GrpParams& p) {
   const GrpSmem sm;
@@ -162,7 +173,7 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
   const int total_tiles = p.m_tiles * p.n_tiles;
   const int fw = warp - kGrpFoldWarp0, qd = warp & 3;
   const int col0 = (fw >> 2) * kGrpCols;
-  const int tc = (lane & 3) * 8;  // this lane's channels of the warp's 32 (see RowEpilogue)
+  const int tc = (lane & 3) * 8;  // this lane's channels of a block of 32 (see RowEpilogue)
   float* wb = sm.bias + fw * kGrpCols;
   bool ok = true;
   uint32_t gcount = 0;
@@ -179,48 +190,56 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
       rs[i] = (ZP == ZP_8BIT && live[i]) ? ld_global_s32(p.rowsum + (row0 + 8 * i) * p.ng) : 0;
     }
     __syncwarp();
-    wb[lane] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + lane)) << 16) : 0.0f;
-    uint64_t t[4][4];  // fp32 partial outputs: token row0 + 8 * i, channels tc + 2j, tc + 2j + 1
 #pragma unroll
-    for (int i = 0; i < 16; ++i) t[i >> 2][i & 3] = 0;
-    // A group is folded in two halves of 16 tokens, each read while the other is computed, the first
-    // half of the next group under the second of this one.
+    for (int c = lane; c < kGrpCols; c += 32)
+      wb[c] = p.bias != nullptr ? __uint_as_float(static_cast<uint32_t>(__ldg(p.bias + n0 + c)) << 16) : 0.0f;
+    float t[2][4][8];  // fp32 partial outputs: block, token row0 + 8 * i, channel tc + j
+#pragma unroll
+    for (int i = 0; i < 64; ++i) t[i >> 5][(i >> 3) & 3][i & 7] = 0.0f;
     const uint32_t t_row = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) + col0;
     auto wait_group = [&](uint32_t g) {
       ok = mbar_wait(&grp_full[g % kGrpBufs], (g / kGrpBufs) & 1u, abort_flag);
       ok = __all_sync(0xFFFFFFFFu, ok);
       tc_fence_after();
     };
-    float sc[8];
-    int dz[8];
-    auto fold = [&](const uint32_t (&a)[16], int i0, const int* rs_g) {
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int a0 = static_cast<int>(a[4 * j + 2 * k]), a1 = static_cast<int>(a[4 * j + 2 * k + 1]);
-          if constexpr (ZP == ZP_8BIT) {
-            a0 += dz[2 * j] * rs_g[i0 + k];
-            a1 += dz[2 * j + 1] * rs_g[i0 + k];
-          }
-          t[i0 + k][j] = f32x2_fma(f32x2_pack(__int2float_rn(a0), __int2float_rn(a1)),
-                                   f32x2_pack(sc[2 * j], sc[2 * j + 1]), t[i0 + k][j]);
-        }
+    auto load = [&](uint32_t (&lo)[16], uint32_t (&hi)[16], uint32_t at) {
+      tmem_ld_16x256b_x4(at, lo);
+      tmem_ld_16x256b_x4(at + (16u << 16), hi);
     };
-    uint32_t lo[16], hi[16];
-    wait_group(gcount);
-    if (!ok) break;
-    tmem_ld_16x256b_x4(t_row + (gcount % kGrpBufs) * kGrpBN, lo);
-    for (int G = 0; G < p.ng; ++G, ++gcount) {
-      const uint32_t buf = gcount % kGrpBufs;
-      const float4* s4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0 + tc);
+    auto fold = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], int b, uint32_t buf, const int* rs_g) {
+      float sc[8];
+      int dz[8];
+      const float4* s4 = reinterpret_cast<const float4*>(s_scale + buf * kGrpBN + col0 + 32 * b + tc);
       *reinterpret_cast<float4*>(sc) = s4[0];
       *reinterpret_cast<float4*>(sc + 4) = s4[1];
-      int rs_g[4];
       if constexpr (ZP == ZP_8BIT) {
-        const int4* d4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0 + tc);
+        const int4* d4 = reinterpret_cast<const int4*>(s_dz + buf * kGrpBN + col0 + 32 * b + tc);
         *reinterpret_cast<int4*>(dz) = d4[0];
         *reinterpret_cast<int4*>(dz + 4) = d4[1];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t(&a)[16] = i < 2 ? lo : hi;
+          int a0 = static_cast<int>(a[4 * j + 2 * (i & 1)]), a1 = static_cast<int>(a[4 * j + 2 * (i & 1) + 1]);
+          if constexpr (ZP == ZP_8BIT) {
+            a0 += dz[2 * j] * rs_g[i];
+            a1 += dz[2 * j + 1] * rs_g[i];
+          }
+          t[b][i][2 * j] = __fmaf_rn(__int2float_rn(a0), sc[2 * j], t[b][i][2 * j]);
+          t[b][i][2 * j + 1] = __fmaf_rn(__int2float_rn(a1), sc[2 * j + 1], t[b][i][2 * j + 1]);
+        }
+    };
+    // One block is folded while the next is read, the first of the next group under the second of this one.
+    uint32_t lo0[16], hi0[16], lo1[16], hi1[16];
+    wait_group(gcount);
+    if (!ok) break;
+    load(lo0, hi0, t_row + (gcount % kGrpBufs) * kGrpBN);
+    for (int G = 0; G < p.ng; ++G, ++gcount) {
+      const uint32_t buf = gcount % kGrpBufs;
+      int rs_g[4];
+      if constexpr (ZP == ZP_8BIT) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           rs_g[i] = rs[i];
@@ -228,34 +247,38 @@ __device__ __forceinline__ void grp_fold(const GrpParams& p) {
         }
       }
       tmem_ld_wait();
-      tmem_ld_16x256b_x4(t_row + (16u << 16) + buf * kGrpBN, hi);
-      fold(lo, 0, rs_g);
+      load(lo1, hi1, t_row + buf * kGrpBN + 32);
+      fold(lo0, hi0, 0, buf, rs_g);
       tmem_ld_wait();
-      tc_fence_before();  // accumulators and scales are in registers: the buffer may take another group
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&grp_empty[buf]);
+      tc_fence_before();
       if (G + 1 < p.ng) {
         wait_group(gcount + 1);
         if (!ok) break;
-        tmem_ld_16x256b_x4(t_row + ((gcount + 1) % kGrpBufs) * kGrpBN, lo);
+        load(lo0, hi0, t_row + ((gcount + 1) % kGrpBufs) * kGrpBN);
       }
-      fold(hi, 2, rs_g);
+      fold(lo1, hi1, 1, buf, rs_g);
+      __syncwarp();  // accumulators and scales have been read: the buffer may take another group
+      if (lane == 0) mbar_arrive(&grp_empty[buf]);
     }
     if (!ok) break;
-    float bb[8];
-    *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(wb + tc);
-    *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(wb + tc + 4);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      uint32_t w[4];
+    for (int b = 0; b < 2; ++b) {
+      float bb[8];
+      *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(wb + 32 * b + tc);
+      *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(wb + 32 * b + tc + 4);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float y0, y1;
-        f32x2_unpack(f32x2_fma(t[i][j], f32x2_pack(sa[i], sa[i]), f32x2_pack(bb[2 * j], bb[2 * j + 1])), y0, y1);
-        const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
-        w[j] = *reinterpret_cast<const uint32_t*>(&v);
+      for (int i = 0; i < 4; ++i) {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float y0, y1;
+          y0 = __fmaf_rn(t[b][i][2 * j], sa[i], bb[2 * j]);
+          y1 = __fmaf_rn(t[b][i][2 * j + 1], sa[i], bb[2 * j + 1]);
+          const __nv_bfloat162 v = __floats2bfloat162_rn(y0, y1);
+          w[j] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+        if (live[i]) st_global_v4(p.y + (row0 + 8 * i) * p.ldy + n0 + 32 * b + tc, w);
       }
-      if (live[i]) st_global_v4(p.y + (row0 + 8 * i) * p.ldy + n0 + tc, w);
     }
   }
 }
@@ -336,10 +359,10 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
+      mbar_init(&empty[i], kGrpIssuers);
     }
     for (int i = 0; i < kGrpBufs; ++i) {
-      mbar_init(&grp_full[i], 1 + kGrpLoadWarps);  // the group's MMAs, its scales
+      mbar_init(&grp_full[i], 2);  // the group's MMAs, its scales
       mbar_init(&grp_empty[i], kGrpFoldWarps);
     }
     *abort_flag = 0;
@@ -364,45 +387,34 @@ gemm_grp_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       Ring st;
       bool ok = true, free_next = mbar_test_wait(&empty[0], 1u);
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int n_blk = tile % p.n_tiles, m_row = (tile / p.n_tiles) * BM;
-        for (int kb = 0; kb < KB; ++kb) {
+        const int w_row = (tile % p.n_tiles) * kGrpBN, m_row = (tile / p.n_tiles) * BM;
+        int c0 = 0, c1 = p.a_tiled ? (m_row >> 7) * KB * BM : m_row;
+        const int c0_step = p.a_tiled ? 0 : BK, c1_step = p.a_tiled ? BM : 0;
+        for (int kb = 0; kb < KB; ++kb, c0 += c0_step, c1 += c1_step) {
           if (!free_next && !(ok = mbar_spin_wait(&empty[st.s], st.ph ^ 1u, abort_flag))) break;
           Ring nx = st;
           nx.next(NS);
           free_next = mbar_test_wait(&empty[nx.s], nx.ph ^ 1u);  // one k-block ahead
           mbar_arrive_expect_tx(&full[st.s], A_BYTES + B_BYTES);
-          int c0, c1;
-          if (p.a_tiled) {
-            c0 = 0;
-            c1 = ((m_row >> 7) * KB + kb) * BM;
-          } else {
-            c0 = kb * BK;
-            c1 = m_row;
-          }
           tma_load_2d(sA + st.s * A_BYTES, &tmap_a, c0, c1, &full[st.s]);
-          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, n_blk * kGrpBN, &full[st.s]);
+          tma_load_w(sB + st.s * B_BYTES, &tmap_w, kb * BK, w_row, &full[st.s]);
           st = nx;
         }
       }
-      if (!ok) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) {
-        }
-      }
+      if (!ok) producer_drain();
     }
-  } else if (warp == 1) {
-    if (elect_one()) {  // see gemm_tc.cu: uniform registers for the single-thread roles
-      // Steps are issued in straight-line runs of U, the largest power of two up to a stage's four that
-      // divides a group: group bookkeeping between single steps kept the issuing thread busy for 570-930
-      // cycles per k-block (a run of four takes ~100), which was the pace of the whole kernel.
-      if (spg % 4 == 0) grp_issue<4>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
-      else if (spg % 2 == 0) grp_issue<2>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
-      else grp_issue<1>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, abort_flag);
+  } else if (warp < kGrpScaleWarp) {
+    if (elect_one()) {
+      // Steps are issued in straight-line runs of U, the largest power of two up to a stage's four that divides a group.
+      const int issuer = warp - 1;
+      if (spg % 4 == 0) grp_issue<4>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, issuer, abort_flag);
+      else if (spg % 2 == 0) grp_issue<2>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, issuer, abort_flag);
+      else grp_issue<1>(p, sA, sB, full, empty, grp_full, grp_empty, tmem_base, issuer, abort_flag);
     }
-  } else if (warp < kGrpFoldWarp0) {
-    // ================= scales of each group: this warp's columns lane, lane + 32 =================
-    constexpr int AHEAD = 8, C = kGrpBN / 32 / kGrpLoadWarps;
-    const int c0 = (warp - 2) * 32 * C + lane;
+  } else if (warp == kGrpScaleWarp) {
+    // ================= scales of each group, columns lane + 32 c =================
+    constexpr int AHEAD = 4, C = kGrpBN / 32;
+    const int c0 = lane;
     bool ok = true;
     uint32_t gcount = 0;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
