@@ -252,7 +252,8 @@ def layer_alg_bytes(stack, l):
 
 def gemm_roofline(stack, peaks, mma_peak):
     """The dominant kernel family (the tcgen05 GEMMs) timed without the rest of the path: the 112
-    GEMM launches of one timestep, each with the kernel variant the plan chose for its layer, on
+    GEMMs of one timestep, one launch each, with the kernel variant the plan chose for its layer on its own (a
+    run of the plan launches those of several layers together), on
     pre-quantized activations (so no DAQ launch in between), captured in one CUDA graph and timed
     with CUDA events on the replay stream. One timestep's operands (0.4 GB of int8 activations,
     0.4 GB of weights, 1.1 GB of outputs) exceed L2, so every launch streams from HBM. A layer the
@@ -313,7 +314,7 @@ def gemm_roofline(stack, peaks, mma_peak):
     traffic = None
     if LAYER_DRAM_BYTES is not None:
         traffic = sum(LAYER_DRAM_BYTES[(stack.table[l][0].split(".")[1], stack.bits[l])] for l in idx) / len(idx)
-    return {"kernel": "gemm_i8_kernel (tcgen05 kind::i8), the 112 launches of one timestep",
+    return {"kernel": "gemm_i8_kernel (tcgen05 kind::i8), the 112 GEMMs of one timestep, one launch each",
             "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TOPS", "frac": achieved / peak,
             "peak_note": f"max of {peaks['source']} bf16 burst x2 = {bf16x2:.0f} (nominal int8:bf16 ratio; the file has "
                          f"no int8 row) and the kind::i8 instruction ceiling measured in this run = "
