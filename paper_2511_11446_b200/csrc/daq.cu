@@ -151,28 +151,39 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
   daq_end(job);
 }
 
-// ---- DAQ with a percentile clip and a-bit codes: robust_row in daq_device.cuh, one warp per token ----
-template <int MAXV>
-__global__ void __launch_bounds__(kDaqWarps * 32, MAXV <= 5 ? 3 : 2)  // register caps that keep 2-3 CTAs per SM
+// ---- DAQ with a percentile clip and a-bit codes: robust_row in daq_device.cuh ------------------------
+// RW warps to a token, MAXV vectors a lane (see launch_daq_robust).
+constexpr int kRobustWarpK = 256 * 6;  // rows that one warp takes in a plan's preparation
+template <int RW, int MAXV>
+__global__ void __launch_bounds__(kDaqThreads, MAXV <= 6 ? 10 : 6)
 daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx, int8_t* __restrict__ q,
                        int64_t ldq, float* __restrict__ s_a, int32_t* __restrict__ rowsum, int clip_rank,
                        float qmax, int tiled_kb, const UnpackJob job) {
+  __shared__ uint2 meet[2 * RW];
   daq_begin(job);
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kDaqWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
   if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
     unpack_units(job, blockIdx.x - job.first_block);
     return;
   }
   if (!job.ahead) pdl_wait();
+  const int64_t row = static_cast<int64_t>(blockIdx.x) * (kDaqThreads / 32 / RW) + threadIdx.x / (32 * RW);
+  const int lane = threadIdx.x % (32 * RW);
   if (row >= M) return;
   const QRow qr(q, row, ldq, tiled_kb);
   float sc;
   int sum;
-  robust_row<MAXV>(x + row * ldx, K, lane, clip_rank, qmax, qr, sc, sum);
+  robust_row<RW, MAXV>(x + row * ldx, K, lane, clip_rank, qmax, qr, sc, sum, meet);
   if (lane == 0) s_a[row] = sc;
   if (rowsum != nullptr) {
     sum = warp_sum_i32(sum);
+    if constexpr (RW > 1) {
+      __syncthreads();  // all have read the last maxima
+      if ((lane & 31) == 0) meet[lane >> 5].x = static_cast<uint32_t>(sum);
+      __syncthreads();
+      sum = 0;
+#pragma unroll
+      for (int w = 0; w < RW; ++w) sum += static_cast<int>(meet[w].x);
+    }
     if (lane == 0) rowsum[row] = sum;
   }
   daq_end(job);
@@ -187,7 +198,9 @@ unpack_kernel(const UnpackJob job) {
 // ---- the preparation of a plan's group of layers (gemm_plan.cu), in one launch ------------------------
 // A CTA works on one segment: rows of a layer to quantize, codes to expand, weights to send into L2. It runs beside the
 // GEMM kernel of the group before, which leaves room for a few CTAs of this size on an SM, so a CTA is small (128 threads,
-// register rows of five vectors a lane, longer rows by two or four warps) and keeps enough loads in flight: four units of
+// register rows of five vectors a lane, longer rows by two or four warps) (with the percentile rule 48 registers;
+// one warp to every row, 18 vectors a lane and 128 registers left room for one CTA, expansion included: 28 blocks, 1024 tokens, 16-bit
+// layers 769 -> 745 us a step) and keeps enough loads in flight: four units of
 // 32 codes a thread.
 constexpr int kExpandUnits = 4, kFetchBytes = 32768, kFetchThreads = 4;
 
@@ -221,9 +234,10 @@ __device__ __forceinline__ void prep_expand(const PlanPrepSeg& s, int block, boo
 }
 
 template <bool ROBUST>
-__global__ void __launch_bounds__(kDaqThreads, ROBUST ? 4 : 12)
+__global__ void __launch_bounds__(kDaqThreads, ROBUST ? 10 : 12)
 plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
   __shared__ uint32_t part[kDaqThreads / 32];
+  __shared__ uint2 meet[2 * kDaqThreads / 32];
   if (!p.early) pdl_wait();
   pdl_launch_dependents();
   // (a search over the segments one by one was a chain of constant-cache misses: 3 us of a CTA's 5)
@@ -246,14 +260,15 @@ plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
     const uint16_t* x = static_cast<const uint16_t*>(s.src);
     const int K = s.arg * 8, kb = K >> 7;
     if constexpr (ROBUST) {
-      const int64_t row = static_cast<int64_t>(block) * (kDaqThreads / 32) + (threadIdx.x >> 5);
+      const bool one = K <= kRobustWarpK;  // one warp to a row
+      const int64_t row = one ? static_cast<int64_t>(block) * (kDaqThreads / 32) + (threadIdx.x >> 5) : block;
       if (row < s.count) {
-        const int lane = threadIdx.x & 31;
+        const int lane = one ? threadIdx.x & 31 : threadIdx.x;
         const QRow qr(s.dst, row, K, kb);
         float sc;
         int sum;
-        if (K <= 256 * 5) robust_row<5>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
-        else robust_row<18>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
+        if (one) robust_row<1, 6>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
+        else robust_row<kDaqThreads / 32, 5>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum, meet);
         if (lane == 0) s.s_a[row] = sc;
       }
     } else {
@@ -320,6 +335,15 @@ int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int6
   return DP_OK;
 }
 
+template <int RW, int MAXV, typename... A>
+static cudaError_t launch_robust_rows(int64_t M, UnpackJob job, cudaStream_t stream, bool pdl, A... a) {
+  constexpr int kRows = kDaqThreads / 32 / RW;
+  const unsigned daq_blocks = static_cast<unsigned>((M + kRows - 1) / kRows);
+  job.first_block = static_cast<int32_t>(daq_blocks);
+  const dim3 grid(daq_blocks + unpack_blocks(job, kDaqThreads));
+  return launch(daq_rows_robust_kernel<RW, MAXV>, grid, dim3(kDaqThreads), 0, stream, pdl, a..., job);
+}
+
 int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq, float* s_a,
                       int32_t* rowsum, int clip_rank, int act_bits, bool tiled, cudaStream_t stream, bool pdl,
                       const UnpackJob* unpack) {
@@ -330,19 +354,19 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
   const float qmax = static_cast<float>((1 << (act_bits - 1)) - 1);
   UnpackJob job;
   if (unpack != nullptr) job = *unpack;
-  const unsigned daq_blocks = static_cast<unsigned>((M + kDaqWarps - 1) / kDaqWarps);
-  job.first_block = static_cast<int32_t>(daq_blocks);
-  const dim3 grid(daq_blocks + unpack_blocks(job, kDaqWarps * 32)), block(kDaqWarps * 32);
-  cudaError_t e;
-  if (k <= 256 * 5)
-    e = launch(daq_rows_robust_kernel<5>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank,
-               qmax, tiled_kb, job);
-  else if (k <= 256 * 9)
-    e = launch(daq_rows_robust_kernel<9>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank,
-               qmax, tiled_kb, job);
-  else
-    e = launch(daq_rows_robust_kernel<18>, grid, block, 0, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank,
-               qmax, tiled_kb, job);
+#define DP_ROWS(RW, MAXV) \
+  launch_robust_rows<RW, MAXV>(M, job, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank, qmax, tiled_kb)
+  // Four warps to a row of more than 2304 elements, and to one of more than 1280 where there are few. One warp, 18 vectors a lane
+  // (five peeling rounds, two CTAs of 256 threads on an SM) -> this: K = 4608, p = 99.9, M = 100 / 1024 / 8192 / 32768 6.4 / 7.8 /
+  // 32.0 / 108 us -> 2.8 / 7.3 / 28.0 / 100 (threshold of rank 47, p = 99: 23.8 / 25.9 / 101 / 359 -> 9.6 / 22.3 / 98 / 369);
+  // K = 3072 5.4 / 5.8 / 25.9 / 89 -> 2.4 / 5.2 / 22.7 / 81. Shorter rows, many of them, spend longer on the exchanges than on
+  // the row: K = 2304, one warp and nine vectors in CTAs of 256 / four warps / one warp and nine vectors in CTAs of 128:
+  // M = 100 3.3 / 2.2 / -, 1024 3.5 / 4.4 / 3.2, 32768 54 / 68 / 39; K = 1536 (nine, -, six) 2.4 / 1.9 / -, 2.5 / 3.5 / 2.4, 38 / 56 / 26.
+  const cudaError_t e = k <= 256 * 5               ? DP_ROWS(1, 5)
+                        : k > 256 * 9 || M <= 512 ? DP_ROWS(kDaqThreads / 32, 5)
+                        : k <= 256 * 6            ? DP_ROWS(1, 6)
+                                                  : DP_ROWS(1, 9);
+#undef DP_ROWS
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "robust DAQ launch failed: %s", cudaGetErrorString(e));
   return DP_OK;
 }
@@ -357,7 +381,7 @@ int launch_plan_prep(PlanPrepParams& p, bool robust, cudaStream_t stream, bool p
       per = static_cast<int64_t>(kFetchBytes) * kFetchThreads;
     } else if (s.kind == PlanPrepSeg::ROWS) {
       const int K = s.arg * 8;
-      per = kDaqThreads / 32 / (robust || K <= 256 * 5 ? 1 : K <= 512 * 5 ? 2 : 4);
+      per = kDaqThreads / 32 / (robust ? (K <= kRobustWarpK ? 1 : kDaqThreads / 32) : K <= 256 * 5 ? 1 : K <= 512 * 5 ? 2 : 4);
     }
     at += (s.count + per - 1) / per;
   }

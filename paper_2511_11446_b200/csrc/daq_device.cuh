@@ -125,12 +125,14 @@ __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ 
 // ---- DAQ with a percentile clip and a-bit codes -------------------------------------------------------
 // Eq. "daq" with tau = Percentile(|v|, p) below the maximum (nearest-rank reading: the clip_rank-th
 // largest magnitude of the token, repeats counted) and alpha = tau / qmax, qmax = 2^(a-1) - 1 for the
-// activation bits a of the step's time bin (Step 6). One warp per token, row in registers as above.
+// activation bits a of the step's time bin (Step 6). One warp per token, or four (rows of more than 1280
+// elements), row in registers as above.
 // The threshold is found by peeling maxima: each round takes the largest magnitude below the
 // previous one together with its multiplicity until clip_rank values are covered (for p = 99.9: 2
 // rounds at K = 1152, 5 at K = 4608). A lane keeps the maximum of each of its 8-element vectors, so
 // a round is a max over those few numbers plus a rescan of only the vectors that held the peeled
-// value. Values beyond tau are clipped to it before the multiplication and so land on +-qmax.
+// value; the same round finds the next maximum, so that warps which share a row meet once a round.
+// Values beyond tau are clipped to it before the multiplication and so land on +-qmax.
 // Packed helpers on words of two 15-bit magnitudes (bit 15 of each half clear):
 // number of halves equal to the value replicated in t2
 __device__ __forceinline__ int count_eq2(uint32_t e, uint32_t t2) {
@@ -150,31 +152,28 @@ __device__ __forceinline__ uint32_t quant_pair_clipped(uint32_t w, uint32_t tau2
   return quant_pair((w & 0x80008000u) | __vminu2(w & 0x7FFF7FFFu, tau2), inv);
 }
 
-// One token by one warp: x[K] bf16 (16-byte aligned) -> codes through `qr`, scale in `sc`, the lane's
-// partial code sum in `sum`. K <= 256 * MAXV.
-template <int MAXV>
+// One token by RW warps, the whole CTA where RW > 1: x[K] bf16 (16-byte aligned) -> codes through `qr`, scale in `sc`,
+// the lane's partial code sum in `sum`. K <= 256 * RW * MAXV. lane: position among the row's threads. meet (RW > 1):
+// 2 * RW pairs of words in shared memory.
+template <int RW, int MAXV>
 __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K, int lane, int clip_rank, float qmax,
-                                           const QRow& qr, float& sc, int& sum) {
+                                           const QRow& qr, float& sc, int& sum, uint2* meet = nullptr) {
+  constexpr int TPR = 32 * RW;
   const int nvec = K >> 3;
   const uint4* xr = reinterpret_cast<const uint4*>(x);
   uint4 v[MAXV];
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
+    const int idx = lane + TPR * i;
     if (idx < nvec) ld_stream_u32x4(xr + idx, v[i]);
     else v[i] = make_uint4(0, 0, 0, 0);
   }
-  // threshold: magnitude bits (bf16 pattern, sign cleared) of the clip_rank-th largest element
-  uint32_t gmax[MAXV];  // per vector: its largest magnitude not yet peeled (padding vectors: 0)
-#pragma unroll
-  for (int i = 0; i < MAXV; ++i)
-    gmax[i] = fold_max2(absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(0u, v[i].x), v[i].y), v[i].z), v[i].w));
-  uint32_t tau_bits = 0;
-  int remaining = clip_rank;
+  // Threshold: magnitude bits (bf16 pattern, sign cleared) of the clip_rank-th largest element.
+  uint32_t tau_bits;
   if (clip_rank == 2) {
     // The second largest magnitude (p = 99.9 at K = 1152) without peeling: a running (largest, second)
     // pair per packed half, three packed operations per two elements, then merged across the halves
-    // and the warp; (a1, a2) + (b1, b2) = (max(a1, b1), max(min(a1, b1), max(a2, b2))) keeps repeats.
+    // and the warps; (a1, a2) + (b1, b2) = (max(a1, b1), max(min(a1, b1), max(a2, b2))) keeps repeats.
     uint32_t m1 = 0, m2 = 0;
 #pragma unroll
     for (int i = 0; i < MAXV; ++i) {
@@ -187,40 +186,73 @@ __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K
     }
     uint32_t t1 = max(m1 & 0xFFFFu, m1 >> 16);
     uint32_t t2 = max(min(m1 & 0xFFFFu, m1 >> 16), max(m2 & 0xFFFFu, m2 >> 16));
+    auto merge = [&](uint32_t u1, uint32_t u2) {
+      t2 = max(min(t1, u1), max(t2, u2));
+      t1 = max(t1, u1);
+    };
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const uint32_t u1 = __shfl_xor_sync(0xFFFFFFFFu, t1, o), u2 = __shfl_xor_sync(0xFFFFFFFFu, t2, o);
-      t2 = max(min(t1, u1), max(t2, u2));
-      t1 = max(t1, u1);
+      merge(u1, u2);
+    }
+    if constexpr (RW > 1) {
+      if ((lane & 31) == 0) meet[lane >> 5] = make_uint2(t1, t2);
+      __syncthreads();
+      t1 = t2 = 0;
+#pragma unroll
+      for (int w = 0; w < RW; ++w) merge(meet[w].x, meet[w].y);
     }
     tau_bits = t2;
-  }
-  for (int round = 0; round < (clip_rank == 2 ? 0 : clip_rank); ++round) {
+  } else {
+    uint32_t gmax[MAXV];  // per vector: its largest magnitude not yet peeled (padding vectors: 0)
     uint32_t mx = 0;
 #pragma unroll
-    for (int i = 0; i < MAXV; ++i) mx = max(mx, gmax[i]);
-    const uint32_t wmx = __reduce_max_sync(0xFFFFFFFFu, mx);
-    tau_bits = wmx;
-    if (wmx == 0) break;  // all that is left are zeros
-    const uint32_t t2 = wmx | (wmx << 16);
-    int cnt = 0;
-#pragma unroll
     for (int i = 0; i < MAXV; ++i) {
-      if (gmax[i] == wmx) {  // this vector holds the value: count it and find the vector's next maximum
-        const uint32_t w[4] = {v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu, v[i].z & 0x7FFF7FFFu,
-                               v[i].w & 0x7FFF7FFFu};
-        uint32_t m2 = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          cnt += count_eq2(w[j], t2);
-          m2 = __vmaxu2(m2, keep_below2(w[j], t2));
-        }
-        gmax[i] = fold_max2(m2);
-      }
+      gmax[i] = fold_max2(absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(0u, v[i].x), v[i].y), v[i].z), v[i].w));
+      mx = max(mx, gmax[i]);
     }
-    const int wcnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if (wcnt >= remaining) break;
-    remaining -= wcnt;
+    int cnt = 0, slot = 0;
+    // The row's largest mx and its cnt in all. Slots in turn: a warp may still read the one of the round before.
+    auto row_reduce = [&]() {
+      mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+      cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+      if constexpr (RW > 1) {
+        if ((lane & 31) == 0) meet[slot * RW + (lane >> 5)] = make_uint2(mx, static_cast<uint32_t>(cnt));
+        __syncthreads();
+        mx = 0, cnt = 0;
+#pragma unroll
+        for (int w = 0; w < RW; ++w) {
+          mx = max(mx, meet[slot * RW + w].x);
+          cnt += static_cast<int>(meet[slot * RW + w].y);
+        }
+        slot ^= 1;
+      }
+    };
+    row_reduce();
+    tau_bits = mx;
+    for (int remaining = clip_rank; remaining > 1 && tau_bits != 0;) {  // (0: all that is left are zeros)
+      const uint32_t t2 = tau_bits | (tau_bits << 16);
+      mx = 0, cnt = 0;
+#pragma unroll
+      for (int i = 0; i < MAXV; ++i) {
+        if (gmax[i] == tau_bits) {  // this vector holds the value: count it and find the vector's next maximum
+          const uint32_t w[4] = {v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu, v[i].z & 0x7FFF7FFFu,
+                                 v[i].w & 0x7FFF7FFFu};
+          uint32_t m2 = 0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            cnt += count_eq2(w[j], t2);
+            m2 = __vmaxu2(m2, keep_below2(w[j], t2));
+          }
+          gmax[i] = fold_max2(m2);
+        }
+        mx = max(mx, gmax[i]);
+      }
+      row_reduce();
+      if (cnt >= remaining) break;
+      remaining -= cnt;
+      tau_bits = mx;
+    }
   }
   const float tau = __uint_as_float(tau_bits << 16);
   float inv = 0.0f;
@@ -233,7 +265,7 @@ __device__ __forceinline__ void robust_row(const uint16_t* __restrict__ x, int K
   sum = 0;
 #pragma unroll
   for (int i = 0; i < MAXV; ++i) {
-    const int idx = lane + 32 * i;
+    const int idx = lane + TPR * i;
     if (idx < nvec) {
       const uint32_t p0 = quant_pair_clipped(v[i].x, tau2, inv), p1 = quant_pair_clipped(v[i].y, tau2, inv);
       const uint32_t p2 = quant_pair_clipped(v[i].z, tau2, inv), p3 = quant_pair_clipped(v[i].w, tau2, inv);

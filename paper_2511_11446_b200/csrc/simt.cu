@@ -613,7 +613,7 @@ daq_group_robust_kernel(SimtGroupArgs g) {
   const QRow qr(g.q_scratch + static_cast<int64_t>(layer) * g.M * g.K, row, g.K, 0);
   float sc;
   int sum;
-  robust_row<5>(x, g.K, lane, g.daq_rank, static_cast<float>((1 << (g.daq_bits - 1)) - 1), qr, sc, sum);
+  robust_row<1, 5>(x, g.K, lane, g.daq_rank, static_cast<float>((1 << (g.daq_bits - 1)) - 1), qr, sc, sum);
   if (lane == 0) g.sa_scratch[static_cast<int64_t>(layer) * g.M + row] = sc;
 }
 

@@ -72,6 +72,22 @@ def test_repeats_sparse_rows_and_pitches():
         _same(_run(x, rank, bits, ldx=K + 8, ldq=K + 32), x, rank, bits)
 
 
+@pytest.mark.parametrize("M,K", [(9, 1280), (9, 1288), (512, 1536), (513, 1536), (513, 1544), (513, 2304), (9, 2312), (9, 4608)])
+def test_equal_magnitudes_across_the_warps_of_a_row(M, K):
+    """Ranks that end inside, at and behind a run of equal magnitudes spread over the whole row, on both sides of the row
+    lengths and counts at which one warp, with six or nine vectors a lane, or four warps take a row."""
+    x = synth.activations(synth.BASE_SEED, 8, 5, M, K, 1.0, n_out=9)
+    at = np.linspace(0, K - 1, 7).astype(int)
+    x[0, at] = 0x4300                                  # seven of the largest
+    x[1, at] = 0xC300
+    x[1, at[3]] = 0x4380                               # one above them
+    x[2, :] = 0
+    x[2, at[:4]] = 0x3F80                              # fewer non-zero values than the rank
+    x[3, :] = 0xBF80                                   # all equal
+    for rank, bits in ((1, 7), (2, 8), (3, 8), (7, 8), (8, 6), (9, 8), (64, 8)):
+        _same(_run(x, rank, bits), x, rank, bits)
+
+
 def test_pipeline_with_the_linear_matches_the_oracle_composition():
     """Robust DAQ's codes and scales fed to dp_wq_linear as quantized activations (tensor-core and
     small-M kernels): int32 sums and outputs as the oracle composes them."""
