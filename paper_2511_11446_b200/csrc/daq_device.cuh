@@ -125,8 +125,8 @@ __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ 
 // ---- DAQ with a percentile clip and a-bit codes -------------------------------------------------------
 // Eq. "daq" with tau = Percentile(|v|, p) below the maximum (nearest-rank reading: the clip_rank-th
 // largest magnitude of the token, repeats counted) and alpha = tau / qmax, qmax = 2^(a-1) - 1 for the
-// activation bits a of the step's time bin (Step 6). One warp per token, or four (rows of more than 1280
-// elements), row in registers as above.
+// activation bits a of the step's time bin (Step 6). One warp per token, or four (see
+// launch_daq_robust), row in registers as above.
 // The threshold is found by peeling maxima: each round takes the largest magnitude below the
 // previous one together with its multiplicity until clip_rank values are covered (for p = 99.9: 2
 // rounds at K = 1152, 5 at K = 4608). A lane keeps the maximum of each of its 8-element vectors, so
