@@ -277,7 +277,9 @@ plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
       else daq_rows<4, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
     }
   }
-  if (p.ahead && blockIdx.x == 0) pdl_wait();  // as daq_end
+  // One CTA of every launch stays until everything before it has finished. Rows and expansion wait by themselves unless `ahead`,
+  // but a unit of 16-bit layers has neither, and the GEMM kernel behind this one waits for this one only.
+  if (p.early && blockIdx.x == 0) pdl_wait();
 }
 
 static unsigned unpack_blocks(const UnpackJob& job, int threads) {

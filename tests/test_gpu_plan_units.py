@@ -83,3 +83,99 @@ def test_layers_launched_together_match_the_oracle(name, clip, act_bits):
                 assert torch.equal(ys[i][l].view(torch.int16), ys[0][l].view(torch.int16)), (i, l, stack[l])
     finally:
         B.dp_plan_destroy(plan)
+
+
+def _layer(l, K, N, bits, group=0):
+    """(weight, what holds its memory) of a layer of 3, 4, 8 or 16 bits, group-wise with `group`."""
+    bias = synth.bias(SEED, l, N)
+    if bits == 16:
+        wt = torch.from_numpy((np.random.default_rng(l).standard_normal((N, K)) * 0.05).astype(np.float32)).bfloat16().cuda()
+        keep = (wt, to_dev_bf16(bias))
+        return B.make_weight(wt, keep[1], keep[1], N, K, 16), keep  # (no scales: that pointer is not read)
+    w, s_w = synth.weights(SEED, l, N, K, bits)
+    keep = DevLayer(w, s_w, bias, bits)
+    if not group:
+        return keep.w, keep
+    s = torch.from_numpy((np.random.default_rng(l).random((N, K // group)) * 4e-3 + 1e-4).astype(np.float32)).cuda()
+    return B.make_weight(keep.qweight, s, keep.bias, N, K, bits, group), (keep, s)
+
+
+# name: (M, K, N, bits, group) a layer, and which layer's output each one reads (None: an input of its own). What feeds a unit
+# takes long, the layers that read it little.
+def _fed(bits):
+    b = lambda l: bits[l % len(bits)]
+    behind = [(300, 1152, 384, b(l), 0) for l in range(3)]
+    return {
+        "behind_group_wise": ([(6000, 1152, 1152, 4, 32)] + behind, [None, 0, 0, 0]),
+        "behind_one_by_one": ([(6000, 1152, 1152 + 64, 8, 0)] + behind, [None, 0, 0, 0]),
+        "behind_small_m": ([(8, 1152, 6912, 8, 0)] * 4 + [(144, 384, 256, b(l), 0) for l in range(3)],
+                           [None] * 4 + [3, 3, 3]),
+        "unit_behind_unit": ([(2000, 384, 384, b(l), 0) for l in range(48)],
+                             [None] * 16 + [15 - l for l in range(16)] + [15 + (5 * l) % 16 for l in range(16)]),
+        # the first unit's outputs feed the third, beside which they could only run if the second did not wait
+        "unit_two_back": ([(2000, 384, 384, b(l), 0) for l in range(48)], [None] * 32 + [l for l in range(16)]),
+    }
+
+
+@pytest.mark.parametrize("bits,clip", [((16,), 100000), ((8,), 100000), ((3, 4), 99900), ((16, 4, 8), 100000)],
+                         ids=["sixteen", "eight", "packed_percentile", "mixed"])
+@pytest.mark.parametrize("feed", list(_fed((8,))))
+def test_units_wait_for_what_feeds_them(feed, bits, clip):
+    """Layers launched together that read outputs of the launch before them, whatever that is, over two steps: the bits of
+    a plan that runs one kernel at a time."""
+    stack, src = _fed(bits)[feed]
+    layers = [_layer(l, K, N, b, g) for l, (_, K, N, b, g) in enumerate(stack)]
+    x0 = [to_dev_bf16(synth.activations(SEED, l, 0, M, K, 1.0, n_out=3)) for l, (M, K, *_) in enumerate(stack)]
+    got = []
+    for flags in (B.DP_FLAG_NO_PDL, 0):
+        plan = B.dp_plan_create([w for w, _ in layers], [s[0] for s in stack], flags | B.DP_FLAG_GROUP_SMALL_M)
+        try:
+            B.dp_plan_set_daq(plan, clip, 0)
+            ws = torch.full((B.dp_plan_workspace(plan),), 0x5A, dtype=torch.uint8, device="cuda")
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            ys = [torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for M, _, N, *_ in stack]
+            # (the end of the output, whose tiles are the last to be written)
+            xp = B.ptr_array([x0[l].data_ptr() if s is None else ys[s].view(-1)[-x0[l].numel():].data_ptr()
+                              for l, s in enumerate(src)])
+            for _ in range(3):
+                for t in ys:
+                    t.zero_()
+                B.dp_plan_run(plan, [0, 1], 0, xp, B.ptr_array([t.data_ptr() for t in ys]), ws, status,
+                              flags=B.DP_PLAN_SAME_X | B.DP_PLAN_SAME_Y)
+                torch.cuda.synchronize()
+                assert int(status.item()) == 0
+                got.append([t.view(torch.int16).clone() for t in ys])
+        finally:
+            B.dp_plan_destroy(plan)
+    for run in got[1:]:
+        for l, (a, b) in enumerate(zip(got[0], run)):
+            assert torch.equal(a, b), (l, stack[l])
+
+
+@pytest.mark.parametrize("bits", [(16,), (8, 3)], ids=["sixteen", "quantized"])
+@pytest.mark.parametrize("small", [True, False], ids=["small_m_between", "units_only"])
+def test_steps_that_write_one_set_of_outputs(bits, small):
+    """Three steps with inputs of their own and one set of outputs, with and without the grouped small-M launch in front of
+    each step's unit: what stays is the last visited step's."""
+    stack = [(2048, 768, 768, bits[l % len(bits)], 0) for l in range(4)] + ([(8, 768, 4608, 4, 0)] * 3 if small else [])
+    layers = [_layer(l, K, N, b, g) for l, (_, K, N, b, g) in enumerate(stack)]
+    xs = [[to_dev_bf16(synth.activations(SEED, l, t, M, K, 1.0, n_out=3)) for l, (M, K, *_) in enumerate(stack)] for t in range(3)]
+    got = []
+    for flags in (B.DP_FLAG_NO_PDL, 0):
+        plan = B.dp_plan_create([w for w, _ in layers], [s[0] for s in stack], flags | B.DP_FLAG_GROUP_SMALL_M)
+        try:
+            ws = torch.full((B.dp_plan_workspace(plan),), 0x5A, dtype=torch.uint8, device="cuda")
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            for _ in range(3):
+                ys = [torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for M, _, N, *_ in stack]
+                torch.cuda.synchronize()
+                B.dp_plan_run(plan, [0, 1, 2], 0, B.ptr_array([t.data_ptr() for x in xs for t in x]),
+                              B.ptr_array([t.data_ptr() for t in ys]), ws, status, flags=B.DP_PLAN_SAME_Y)
+                torch.cuda.synchronize()
+                assert int(status.item()) == 0
+                got.append([t.view(torch.int16) for t in ys])
+        finally:
+            B.dp_plan_destroy(plan)
+    for run in got[1:]:
+        for l, (a, b) in enumerate(zip(got[0], run)):
+            assert torch.equal(a, b), (l, stack[l])
