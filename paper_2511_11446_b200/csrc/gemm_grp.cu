@@ -59,7 +59,7 @@ struct GrpParams {
   const uint8_t* zeros;   // [N][ng] (unless ZP_NONE)
   const int32_t* rowsum;  // [M][ng] (ZP_8BIT)
   const int8_t *q, *w8;   // ZP_PACKED: what tmap_a (tiled) and tmap_w read,
-  const uint32_t* wide;   // and the expansion's notes, n_wide words: nonzero for a zero-point above 127
+  const int32_t* wide;    // and the expansion's notes, n_wide words: nonzero for a zero-point above 127
   int32_t n_wide;
   const uint16_t* bias;
   uint16_t* y;
@@ -148,11 +148,11 @@ struct GrpSmem {
 
 // Whether the expansion met a zero-point above 127 (a warp together).
 __device__ __forceinline__ bool grp_wide_zeros(const GrpParams& p, int lane) {
-  uint32_t any = 0;
+  int any = 0;
   for (int i = lane; i < p.n_wide; i += 32 * 8) {  // eight loads in flight, predicated: a loop's remainder goes one by one
-    uint32_t v[8];
+    int v[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = i + 32 * j < p.n_wide ? __ldg(p.wide + i + 32 * j) : 0u;
+    for (int j = 0; j < 8; ++j) v[j] = i + 32 * j < p.n_wide ? ld_global_s32(p.wide + i + 32 * j) : 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) any |= v[j];
   }
@@ -551,7 +551,7 @@ int launch_gemm_grp(const int8_t* q, int64_t ldq, bool a_tiled, const float* s_a
   p.rowsum = rowsum;
   p.q = q;
   p.w8 = w8;
-  p.wide = reinterpret_cast<const uint32_t*>(wide);
+  p.wide = reinterpret_cast<const int32_t*>(wide);
   p.n_wide = static_cast<int32_t>(unpack_notes(static_cast<int64_t>(N) * K / 32) / 4);
   p.bias = bias;
   p.y = y;

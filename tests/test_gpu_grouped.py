@@ -139,6 +139,27 @@ def test_zero_points_of_any_byte_value(M, bits, g, K, offset):
     assert np.array_equal(_run(L, x), L.ref(x))
 
 
+def test_small_and_large_zero_points_in_turn_on_one_workspace():
+    """Calls that follow each other without waiting, on one workspace: each takes its own layer's notes on zero-points above
+    127, not those that the call before left at the same place."""
+    M, N, K, g = 40, 1920, 1152, 128
+    layers = [GroupedLayer(N, K, 4, g, True) for _ in range(2)]
+    layers[1].d_z[:] = 200
+    layers[1].z[:] = 200
+    x = synth.activations(SEED, 4, 0, M, K, 1.0, n_out=3)
+    xd, refs = to_dev_bf16(x), [L.ref(x) for L in layers]
+    ys = [torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(8)]
+    ws = torch.empty(B.dp_wq_linear_workspace_grouped(M, layers[0].dw), dtype=torch.uint8, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for i, y in enumerate(ys):
+        B.dp_wq_linear(layers[i % 2].dw, xd, K, None, M, y, N, ws, None, st, 0)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    for i, y in enumerate(ys):
+        assert np.array_equal(bf16_to_np(y), refs[i % 2]), i
+
+
 def test_grouped_argument_errors():
     L = GroupedLayer(128, 256, 4, 64, False)
     bad = B.make_weight(L.d_w, L.d_s, None, 128, 256, 4, 48)          # g % 32 != 0
