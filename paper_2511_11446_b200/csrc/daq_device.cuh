@@ -90,18 +90,19 @@ struct QRow {
 
 // Two tokens by one warp at once, any K (multiple of 8): two passes over the rows, the second served by L1/L2 (the
 // loads of both are in flight together, which matters when the warp has several tokens to do and each costs a full
-// memory round trip). has_b == false: only A.
+// memory round trip). has_b == false: only A. (Ordinary loads, as above: the caller has waited for what wrote the rows.)
 template <bool EO>
 __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ xa, const uint16_t* __restrict__ xb,
                                                    bool has_b, int K, const QRow& qa, const QRow& qb, int lane,
                                                    float& sc_a, float& sc_b) {
+  constexpr int kBatch = 5;
   const int nvec = K >> 3;
   const uint4* ra = reinterpret_cast<const uint4*>(xa);
   const uint4* rb = reinterpret_cast<const uint4*>(has_b ? xb : xa);
   uint32_t ma = 0, mb = 0;
 #pragma unroll 5
   for (int idx = lane; idx < nvec; idx += 32) {
-    const uint4 va = ra[idx], vb = rb[idx];
+    const uint4 va = ld_global_v4(ra + idx), vb = ld_global_v4(rb + idx);
     ma = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(ma, va.x), va.y), va.z), va.w);
     mb = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(mb, vb.x), vb.y), vb.z), vb.w);
   }
@@ -115,10 +116,22 @@ __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ 
   float inv_a, inv_b;
   token_scale(ma, sc_a, inv_a);
   token_scale(mb, sc_b, inv_b);
-#pragma unroll 5
-  for (int idx = lane; idx < nvec; idx += 32) {
-    qa.store(idx, quant_vec<EO>(ra[idx], inv_a));
-    if (has_b) qb.store(idx, quant_vec<EO>(rb[idx], inv_b));
+  // Batches of loads first: one does not move ahead of a store (K = 1152, N = 3456, 8 bits, M = 300 / 8192: a layer takes 11.8 /
+  // 59.2 us with a load and a store in turn, 10.6 / 49.5 this way).
+  for (int base = lane; base < nvec; base += 32 * kBatch) {
+    uint4 va[kBatch], vb[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j)
+      if (base + 32 * j < nvec) {
+        va[j] = ld_global_v4(ra + base + 32 * j);
+        vb[j] = ld_global_v4(rb + base + 32 * j);
+      }
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j)
+      if (base + 32 * j < nvec) {
+        qa.store(base + 32 * j, quant_vec<EO>(va[j], inv_a));
+        if (has_b) qb.store(base + 32 * j, quant_vec<EO>(vb[j], inv_b));
+      }
   }
 }
 

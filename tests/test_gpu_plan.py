@@ -386,6 +386,33 @@ def test_in_kernel_quantization_covers_packed_layers(M, autotune):
         B.dp_plan_destroy(first)
 
 
+@pytest.mark.parametrize("M", [300, 8200])
+@pytest.mark.parametrize("K", [256, 1408, 2816])
+def test_in_kernel_quantization_of_an_earlier_output(K, M):
+    """DP_FLAG_FUSED_DAQ with layers that read the output of the layer before, rows on both sides of one batch of loads (1280
+    elements) and of two: the bits of a plan that runs one kernel at a time."""
+    dims, bits = (K, 384, K, 384), (4, 8, 3)
+    dev = [DevLayer(*synth.weights(SEED, l, dims[l + 1], dims[l], b), synth.bias(SEED, l, dims[l + 1]), b)
+           for l, b in enumerate(bits)]
+    x0 = to_dev_bf16(synth.activations(SEED, 0, 0, M, K, 1.0, n_out=3))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    got = []
+    for flags in (B.DP_FLAG_NO_PDL, B.DP_FLAG_FUSED_DAQ):
+        plan = B.dp_plan_create([d.w for d in dev], [M] * 3, flags)
+        try:
+            ys = [torch.zeros((M, n), dtype=torch.bfloat16, device="cuda") for n in dims[1:]]
+            ws = torch.empty(B.dp_plan_workspace(plan), dtype=torch.uint8, device="cuda")
+            B.dp_plan_run(plan, [0, 1], 0, B.ptr_array([t.data_ptr() for t in [x0] + ys[:-1]]),
+                          B.ptr_array([t.data_ptr() for t in ys]), ws, status, flags=B.DP_PLAN_SAME_X | B.DP_PLAN_SAME_Y)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0
+            got.append([t.view(torch.int16) for t in ys])
+        finally:
+            B.dp_plan_destroy(plan)
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+
+
 def test_phase_a_on_measured_latencies_matches_oracle_and_runs():
     """Algorithm 2 end to end on a small stack: c_lat(l, b) measured with the library's kernels, Phase A
     (library) equal to the oracle's on the same table, and the resulting bit plan and kept steps run by
