@@ -90,12 +90,14 @@ struct QRow {
 
 // Two tokens by one warp at once, any K (multiple of 8): two passes over the rows, the second served by L1/L2 (the
 // loads of both are in flight together, which matters when the warp has several tokens to do and each costs a full
-// memory round trip). has_b == false: only A. (Ordinary loads, as above: the caller has waited for what wrote the rows.)
+// memory round trip). has_b == false: only A. Ordinary loads, as above: the caller has waited for what wrote the rows. (Loads in
+// batches ahead of the stores, 40 registers more for them, make these layers 10-20 % faster but every other 8-bit layer slower,
+// whose kernels are the same: 118 -> 128 registers a thread leave quantization less room beside a GEMM, M = 2048, K = 1152: 8.9 ->
+// 9.2 us.)
 template <bool EO>
 __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ xa, const uint16_t* __restrict__ xb,
                                                    bool has_b, int K, const QRow& qa, const QRow& qb, int lane,
                                                    float& sc_a, float& sc_b) {
-  constexpr int kBatch = 5;
   const int nvec = K >> 3;
   const uint4* ra = reinterpret_cast<const uint4*>(xa);
   const uint4* rb = reinterpret_cast<const uint4*>(has_b ? xb : xa);
@@ -116,22 +118,10 @@ __device__ __forceinline__ void daq_two_rows_2pass(const uint16_t* __restrict__ 
   float inv_a, inv_b;
   token_scale(ma, sc_a, inv_a);
   token_scale(mb, sc_b, inv_b);
-  // Batches of loads first: one does not move ahead of a store (K = 1152, N = 3456, 8 bits, M = 300 / 8192: a layer takes 11.8 /
-  // 59.2 us with a load and a store in turn, 10.6 / 49.5 this way).
-  for (int base = lane; base < nvec; base += 32 * kBatch) {
-    uint4 va[kBatch], vb[kBatch];
-#pragma unroll
-    for (int j = 0; j < kBatch; ++j)
-      if (base + 32 * j < nvec) {
-        va[j] = ld_global_v4(ra + base + 32 * j);
-        vb[j] = ld_global_v4(rb + base + 32 * j);
-      }
-#pragma unroll
-    for (int j = 0; j < kBatch; ++j)
-      if (base + 32 * j < nvec) {
-        qa.store(base + 32 * j, quant_vec<EO>(va[j], inv_a));
-        if (has_b) qb.store(base + 32 * j, quant_vec<EO>(vb[j], inv_b));
-      }
+#pragma unroll 5
+  for (int idx = lane; idx < nvec; idx += 32) {
+    qa.store(idx, quant_vec<EO>(ld_global_v4(ra + idx), inv_a));
+    if (has_b) qb.store(idx, quant_vec<EO>(ld_global_v4(rb + idx), inv_b));
   }
 }
 
