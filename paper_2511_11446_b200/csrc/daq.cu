@@ -27,16 +27,24 @@ __device__ __forceinline__ void daq_end(const UnpackJob& job) {
   if (job.ahead && blockIdx.x == 0) pdl_wait();
 }
 
-// CTA `block` of a launch over rows: RW warps share a row, MAXV = 16-byte vectors held per lane (a row of up to 256 * RW *
-// MAXV elements in registers). SUM: also the row's code sum. part: a word per warp of the CTA.
+// RW warps share a row: MAXV = 16-byte vectors held per lane (a row of up to 256 * RW * MAXV elements in
+// registers). SUM: also the row's code sum.
 template <int RW, int MAXV, bool EO, bool SUM>
-__device__ __forceinline__ void daq_rows(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
-                                         int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
-                                         int32_t* __restrict__ rowsum, int tiled_kb, int block, uint32_t* part) {
+__global__ void __launch_bounds__(kDaqThreads)
+daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
+                int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
+                int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
   constexpr int kRows = kDaqThreads / 32 / RW;  // rows of a CTA
   constexpr int TPR = 32 * RW;
+  __shared__ uint32_t part[kDaqThreads / 32];
+  daq_begin(job);
+  if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
+    unpack_units(job, blockIdx.x - job.first_block);
+    return;
+  }
+  if (!job.ahead) pdl_wait();
   const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;  // row of the CTA, position in the row
-  const int64_t row = static_cast<int64_t>(block) * kRows + rw;
+  const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + rw;
   const bool live = row < M;
   const int nvec = live ? K >> 3 : 0;
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * ldx);
@@ -92,21 +100,6 @@ __device__ __forceinline__ void daq_rows(const uint16_t* __restrict__ x, int64_t
     }
     if (lane == 0 && live) rowsum[row] = sum;
   }
-}
-
-template <int RW, int MAXV, bool EO, bool SUM>
-__global__ void __launch_bounds__(kDaqThreads)
-daq_rows_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx,
-                int8_t* __restrict__ q, int64_t ldq, float* __restrict__ s_a,
-                int32_t* __restrict__ rowsum, int tiled_kb, const UnpackJob job) {
-  __shared__ uint32_t part[kDaqThreads / 32];
-  daq_begin(job);
-  if (static_cast<int>(blockIdx.x) >= job.first_block) {  // the launch's weight-expansion CTAs
-    unpack_units(job, blockIdx.x - job.first_block);
-    return;
-  }
-  if (!job.ahead) pdl_wait();
-  daq_rows<RW, MAXV, EO, SUM>(x, M, K, ldx, q, ldq, s_a, rowsum, tiled_kb, blockIdx.x, part);
   daq_end(job);
 }
 
@@ -195,13 +188,12 @@ unpack_kernel(const UnpackJob job) {
   unpack_units(job, blockIdx.x);
 }
 
-// ---- the preparation of a plan's group of layers (gemm_plan.cu), in one launch ------------------------
+// ---- the preparation of a plan's unit of layers (gemm_plan.cu), in one launch -------------------------
 // A CTA works on one segment: rows of a layer to quantize, codes to expand, weights to send into L2. It runs beside the
-// GEMM kernel of the group before, which leaves room for a few CTAs of this size on an SM, so a CTA is small (128 threads,
-// register rows of five vectors a lane, longer rows by two or four warps) (with the percentile rule 48 registers;
-// one warp to every row, 18 vectors a lane and 128 registers left room for one CTA, expansion included: 28 blocks, 1024 tokens, 16-bit
-// layers 769 -> 745 us a step) and keeps enough loads in flight: four units of
-// 32 codes a thread.
+// GEMM kernel of the unit before, which leaves room for a few small CTAs on an SM. So a CTA has 128 threads, holds rows as five
+// vectors a lane (longer rows by two or four warps), and keeps four units of 32 codes a thread in flight. With the
+// percentile rule a thread takes 48 registers, five CTAs beside a GEMM CTA; with one warp to every row, 18 vectors a lane and 128
+// registers there was room for one, and a step of 28 blocks, 1024 tokens, 16-bit layers took 769 us instead of 745.
 constexpr int kExpandUnits = 4, kFetchBytes = 32768, kFetchThreads = 4;
 
 template <int BITS>
@@ -233,6 +225,46 @@ __device__ __forceinline__ void prep_expand(const PlanPrepSeg& s, int block, boo
   }
 }
 
+// CTA `block` over the rows of a segment, RW warps to a row, `part` a word per warp: daq_rows_kernel without its options. (One
+// function for both costs that kernel registers, 40 -> 42 with four warps to a row, and with them two CTAs of an SM:
+// K = 3072, M = 2048 / 8192 4.6 / 13.2 -> 5.0 / 14.1 us.)
+template <int RW>
+__device__ __forceinline__ void prep_rows(const PlanPrepSeg& s, int block, uint32_t* part) {
+  constexpr int TPR = 32 * RW, MAXV = 5;
+  const int K = s.arg * 8;
+  const int rw = threadIdx.x / TPR, lane = threadIdx.x % TPR;
+  const int64_t row = static_cast<int64_t>(block) * (kDaqThreads / TPR) + rw;
+  const int nvec = row < s.count ? K >> 3 : 0;
+  const uint4* xr = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(s.src) + row * K);
+  uint4 v[MAXV];
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) {
+    const int idx = lane + TPR * i;
+    if (idx < nvec) ld_stream_u32x4(xr + idx, v[i]);
+    else v[i] = make_uint4(0, 0, 0, 0);
+  }
+  uint32_t m = 0;
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) m = absmax_bits2(absmax_bits2(absmax_bits2(absmax_bits2(m, v[i].x), v[i].y), v[i].z), v[i].w);
+  m = warp_max_u32(max(m & 0xFFFFu, m >> 16));
+  if constexpr (RW > 1) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < RW; ++w) m = max(m, part[rw * RW + w]);
+  }
+  if (nvec == 0) return;
+  float sc, inv;
+  token_scale(m, sc, inv);
+  const QRow qr(s.dst, row, K, K >> 7);
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) {
+    const int idx = lane + TPR * i;
+    if (idx < nvec) qr.store(idx, quant_vec<false>(v[i], inv));
+  }
+  if (lane == 0) s.s_a[row] = sc;
+}
+
 template <bool ROBUST>
 __global__ void __launch_bounds__(kDaqThreads, ROBUST ? 10 : 12)
 plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
@@ -257,24 +289,24 @@ plan_prep_kernel(const __grid_constant__ PlanPrepParams p) {
                        static_cast<uint32_t>(s.count - at < kFetchBytes ? s.count - at : kFetchBytes));
   } else {
     if (!p.ahead) pdl_wait();
-    const uint16_t* x = static_cast<const uint16_t*>(s.src);
-    const int K = s.arg * 8, kb = K >> 7;
+    const int K = s.arg * 8;
     if constexpr (ROBUST) {
       const bool one = K <= kRobustWarpK;  // one warp to a row
       const int64_t row = one ? static_cast<int64_t>(block) * (kDaqThreads / 32) + (threadIdx.x >> 5) : block;
       if (row < s.count) {
+        const uint16_t* x = static_cast<const uint16_t*>(s.src) + row * K;
         const int lane = one ? threadIdx.x & 31 : threadIdx.x;
-        const QRow qr(s.dst, row, K, kb);
+        const QRow qr(s.dst, row, K, K >> 7);
         float sc;
         int sum;
-        if (one) robust_row<1, 6>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum);
-        else robust_row<kDaqThreads / 32, 5>(x + row * K, K, lane, s.rank, p.qmax, qr, sc, sum, meet);
+        if (one) robust_row<1, 6>(x, K, lane, s.rank, p.qmax, qr, sc, sum);
+        else robust_row<kDaqThreads / 32, 5>(x, K, lane, s.rank, p.qmax, qr, sc, sum, meet);
         if (lane == 0) s.s_a[row] = sc;
       }
     } else {
-      if (K <= 256 * 5) daq_rows<1, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
-      else if (K <= 512 * 5) daq_rows<2, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
-      else daq_rows<4, 5, false, false>(x, s.count, K, K, s.dst, K, s.s_a, nullptr, kb, block, part);
+      if (K <= 256 * 5) prep_rows<1>(s, block, part);
+      else if (K <= 512 * 5) prep_rows<2>(s, block, part);
+      else prep_rows<4>(s, block, part);
     }
   }
   // One CTA of every launch stays until everything before it has finished. Rows and expansion wait by themselves unless `ahead`,
