@@ -344,6 +344,9 @@ int dp_plan_layer_variant(const dp_plan* plan, int32_t layer, int32_t* tile_n, i
 /* *unpack_first = 1 when the plan runs layer `layer` in the DP_FLAG_UNPACK_FIRST form (the
  * variant dp_plan_layer_variant reports is then the 8-bit kernel's). No counterpart in the paper. */
 int dp_plan_layer_unpack_first(const dp_plan* plan, int32_t layer, int32_t* unpack_first);
+/* *unit = the unit that layer `layer` is launched with, units counted from 0 (two launches for all of its layers, in steps
+ * whose pointers allow it: see dp_plan_run), or -1 where the layer is launched on its own. No counterpart in the paper. */
+int dp_plan_layer_unit(const dp_plan* plan, int32_t layer, int32_t* unit);
 /* Replaces the kernel variant of layer `layer` by the one `flags` names (the tuning flags of
  * dp_wq_linear: DP_FLAG_TILE_N, [NO_]CTA_PAIR, [NO_]WEIGHT_STATIONARY, [NO_]ACT_STATIONARY, UNPACK_FIRST; anything left
  * open is chosen as dp_wq_linear would), with which it is then launched on its own: lets a deployment keep the outcome of one

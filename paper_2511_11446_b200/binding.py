@@ -35,7 +35,7 @@ def DP_FLAG_TILE_N(bn: int) -> int:
 DP_STATIC_SCRATCH_BYTES = 10 << 20
 
 EXPORTS = ["dp_daq_quantize", "dp_daq_quantize_robust", "dp_wq_linear_workspace", "dp_wq_linear_workspace_grouped", "dp_wq_linear", "dp_wq_linear_static", "dp_wq_linear_residual", "dp_ln_modulate_daq", "dp_plan_create",
-           "dp_plan_workspace", "dp_plan_layer_variant", "dp_plan_layer_unpack_first", "dp_plan_set_layer_flags", "dp_plan_set_daq", "dp_plan_destroy", "dp_plan_run", "dp_plan_x_bytes",
+           "dp_plan_workspace", "dp_plan_layer_variant", "dp_plan_layer_unpack_first", "dp_plan_layer_unit", "dp_plan_set_layer_flags", "dp_plan_set_daq", "dp_plan_destroy", "dp_plan_run", "dp_plan_x_bytes",
            "dp_plan_run_host", "dp_plan_phase_a", "dp_layer_latency_us", "dp_pack_weights_host", "dp_clip_rank", "dp_debug_skip_stage_load",
            "dp_status_string",
            "dp_last_error", "dp_version"]
@@ -83,6 +83,7 @@ def lib():
         L.dp_plan_workspace.argtypes = [C.c_void_p]
         L.dp_plan_layer_variant.argtypes = [C.c_void_p, C.c_int32] + [C.POINTER(C.c_int32)] * 4
         L.dp_plan_layer_unpack_first.argtypes = [C.c_void_p, C.c_int32, C.POINTER(C.c_int32)]
+        L.dp_plan_layer_unit.argtypes = [C.c_void_p, C.c_int32, C.POINTER(C.c_int32)]
         L.dp_plan_set_layer_flags.argtypes = [C.c_void_p, C.c_int32, C.c_uint32]
         L.dp_plan_set_daq.argtypes = [C.c_void_p, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
         L.dp_plan_x_bytes.restype = C.c_size_t
@@ -245,6 +246,13 @@ def dp_plan_layer_variant(plan, layer: int) -> dict:
     _check(lib().dp_plan_layer_unpack_first(plan, layer, C.byref(u)), "dp_plan_layer_unpack_first")
     return dict(tile_n=v[0].value, cta_group=v[1].value, weight_stationary=v[2].value, small_m=v[3].value,
                 unpack_first=u.value)
+
+
+def dp_plan_layer_unit(plan, layer: int) -> int:
+    """The unit that a layer of a plan is launched with, or -1 where it is launched on its own."""
+    u = C.c_int32(0)
+    _check(lib().dp_plan_layer_unit(plan, layer, C.byref(u)), "dp_plan_layer_unit")
+    return u.value
 
 
 def dp_plan_set_layer_flags(plan, layer: int, flags: int):

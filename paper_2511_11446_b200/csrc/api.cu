@@ -1090,6 +1090,12 @@ extern "C" int dp_plan_layer_unpack_first(const dp_plan* plan, int32_t layer, in
   *unpack_first = (!L.simt && L.pre) ? 1 : 0;
   return DP_OK;
 }
+extern "C" int dp_plan_layer_unit(const dp_plan* plan, int32_t layer, int32_t* unit) {
+  if (!plan || layer < 0 || layer >= static_cast<int32_t>(plan->layers.size()) || !unit)
+    return fail(DP_ERR_INVALID_ARG, "dp_plan_layer_unit: bad plan, layer index or NULL output");
+  *unit = plan->unit_of[layer];
+  return DP_OK;
+}
 extern "C" int dp_plan_layer_variant(const dp_plan* plan, int32_t layer, int32_t* tile_n, int32_t* cta_group,
                                      int32_t* weight_stationary, int32_t* small_m) {
   if (!plan || layer < 0 || layer >= static_cast<int32_t>(plan->layers.size()))

@@ -47,7 +47,7 @@ class DitStack:
         entries: small-M layers); given, the plan applies them instead of timing variants itself."""
         if variants is not None:
             flags &= ~B.DP_FLAG_AUTOTUNE
-        self.seed, self.T, self.flags, self.named = seed, T, flags, variants is not None
+        self.seed, self.T, self.flags = seed, T, flags
         self.table = synth.dit_layers(batch, tokens, blocks)
         self.bits = synth.bit_plan(seed, len(self.table), bit_choices)
         self.kept = synth.kept_timesteps(seed, T, keep, 0.2)
@@ -96,32 +96,20 @@ class DitStack:
         return tot
 
     def launches_per_timestep(self):
-        """Kernel launches of this library per timestep: two (preparation, GEMMs) per unit of up to 16
-        token linears and 64 MB of int8 codes, scales and expanded weights, DAQ + GEMM for each one outside a unit
-        (fewer than three in a row, or a named variant); the small-M (adaLN) linears of a step share, per 32 of
-        them, one grouped launch that also quantizes their tokens when the plan groups them (under a percentile /
-        a-bit DAQ policy a second, small quantization launch goes in front of it)."""
-        small = sum(1 for M in self.Ms if M <= 32)
-        grouped = bool(self.flags & B.DP_FLAG_GROUP_SMALL_M)
-        neutral = B.DP_FLAG_AUTOTUNE | B.DP_FLAG_GROUP_SMALL_M | B.DP_FLAG_FORCE_MMA | B.DP_FLAG_NO_PDL | B.DP_FLAG_UNPACK_FIRST
-        total, layers, nbytes = (-(-small // 32) if grouped else small), 0, 0
-
-        def close():
-            return 2 if layers >= 3 else 2 * layers
-
-        for L, (_, M, K, N) in zip(self.layers, self.table):
-            if M <= 32:
-                if not grouped:  # stands between its neighbours
-                    total, layers, nbytes = total + close(), 0, 0
-                continue
-            if self.named or self.flags & ~neutral:
-                total += 2
-                continue
-            need = -(-M // 128) * 128 * K + -(-4 * M // 256) * 256 + (N * K if L.w.bits < 8 else 0)
-            if layers == 16 or (layers and nbytes + need > 64 << 20):
-                total, layers, nbytes = total + close(), 0, 0
-            layers, nbytes = layers + 1, nbytes + need
-        return total + close()
+        """Kernel launches of this library per timestep: two (preparation, GEMMs) per unit of token linears, DAQ + GEMM for
+        each one outside a unit (one launch where it is kept in 16 bits or quantizes in its GEMM); the small-M (adaLN) linears of a
+        step share, per 32 of them, one grouped launch that also quantizes their tokens when the plan groups them (under a
+        percentile / a-bit DAQ policy a second, small quantization launch goes in front of it)."""
+        small, total, units = 0, 0, set()
+        for l, bits in enumerate(self.bits):
+            unit = B.dp_plan_layer_unit(self.plan, l)
+            if unit >= 0:
+                units.add(unit)
+            elif B.dp_plan_layer_variant(self.plan, l)["small_m"]:
+                small += 1
+            else:
+                total += 1 if bits == 16 or self.flags & B.DP_FLAG_FUSED_DAQ else 2
+        return total + 2 * len(units) + (-(-small // 32) if self.flags & B.DP_FLAG_GROUP_SMALL_M else small)
 
     # ---- execution ----
     def ptrs(self, n_steps=None):

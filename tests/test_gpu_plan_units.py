@@ -179,3 +179,25 @@ def test_steps_that_write_one_set_of_outputs(bits, small):
     for run in got[1:]:
         for l, (a, b) in enumerate(zip(got[0], run)):
             assert torch.equal(a, b), (l, stack[l])
+
+
+@pytest.mark.parametrize("flags", [B.DP_FLAG_GROUP_SMALL_M, 0, B.DP_FLAG_GROUP_SMALL_M | B.DP_FLAG_CTA_PAIR,
+                                   B.DP_FLAG_GROUP_SMALL_M | B.DP_FLAG_FUSED_DAQ],
+                         ids=["units", "small_m_between", "named_variant", "daq_in_gemm"])
+@pytest.mark.parametrize("bit_choices", [(3, 4, 8), (4, 16), (16,)])
+def test_launch_count_is_that_of_a_captured_step(bit_choices, flags):
+    from cuda.bindings import runtime
+    from paper_2511_11446_b200.workloads import DitStack
+    stack = DitStack(seed=SEED, batch=2, tokens=128, blocks=5, T=2, keep=1, bit_choices=bit_choices, flags=flags)
+    try:
+        stack.run(1)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph):
+            stack.run(1)
+        err, _, n = runtime.cudaGraphGetNodes(runtime.cudaGraph_t(graph.raw_cuda_graph()))
+        assert err == runtime.cudaError_t.cudaSuccess
+        assert n == stack.launches_per_timestep()
+        assert int(stack.status.item()) == 0
+    finally:
+        stack.close()
