@@ -327,8 +327,9 @@ int dp_plan_create(const dp_weight* layers, int32_t n_layers, const int64_t* M_p
                    uint32_t flags, dp_plan** out);
 /* Bytes of device scratch a run of the plan needs (256-byte aligned). Three or more tensor-core layers in a row (per-channel or
  * 16-bit ones, in a plan that names no kernel variant) are launched together, up to 16 layers and up to 64 MB of scratch
- * to a unit: where there are such units, two parts of the largest one's scratch (codes, scales, weights expanded to int8),
- * at most 128 MB. At least, for layers launched one by one: consecutive layers use the scratch in turn, in as
+ * to a unit, unless layers are so large that a row of them would change between units and single layers all the time
+ * (dp_plan_layer_unit says which go together): where there are such units, two parts of the largest one's scratch (codes,
+ * scales, weights expanded to int8), at most 128 MB. At least, for layers launched one by one: consecutive layers use the scratch in turn, in as
  * many parts of the largest layer's dp_wq_linear_workspace as the launch order overlaps: three where a per-channel 3-, 4- or
  * 8-bit layer has 33 to 1024 rows, two where such layers all have more, one with DP_FLAG_NO_PDL, DP_FLAG_FUSED_DAQ or
  * without such layers; grouped small-M layers under a DAQ policy may need more. What a plan needs is the larger. */

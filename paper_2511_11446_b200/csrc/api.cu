@@ -658,12 +658,12 @@ struct TmapACache {
   CUtensorMap map;
 };
 // Consecutive layers whose quantization (with the expansion of their weights) is one launch and whose GEMMs are another,
-// in a step whose pointers let them run in any order (group_independent).
+// in a step whose pointers let them run in any order (unit_independent).
 struct PlanGroup {
   std::vector<int> layers;
   GemmPlanSchedule sched;
   struct Place {
-    size_t q, s_a, w8;  // offsets in the group's part of the workspace: codes, scales, expanded weights
+    size_t q, s_a, w8;  // offsets in the unit's part of the workspace: codes, scales, expanded weights
   };
   std::vector<Place> place;
   // The tensor maps of the members, by place in the launch, for the address that a part of the workspace had last.
@@ -717,6 +717,7 @@ static int plan_parts(const dp_plan& p, bool fused_daq) {
 // whose variant nobody has named. A unit takes layers until its part of the workspace would be larger than kUnitBytes.
 constexpr size_t kUnitBytes = 64u << 20;
 constexpr size_t kUnitMinLayers = 3;
+constexpr size_t kUnitLayersPerBreak = 4;
 static bool unit_takes(const dp_plan& p, const PlanLayer& L) {
   constexpr uint32_t kNeutral = DP_FLAG_FORCE_MMA | DP_FLAG_NO_PDL | DP_FLAG_UNPACK_FIRST;
   if ((p.flags & ~kNeutral) || p.daq_sync != nullptr || L.simt || L.fixed || L.M <= 0 || L.w.group_size > 0) return false;
@@ -728,43 +729,60 @@ static size_t unit_layer_bytes(const PlanLayer& L, PlanGroup::Place* at, size_t 
   if (at) *at = {off, off + q, off + q + sa};
   return q + sa + (L.w.bits < 8 ? align256(static_cast<size_t>(L.w.N) * L.w.K) : 0);
 }
+static void plan_add_unit(dp_plan* p, const std::vector<int>& layers) {
+  PlanGroup u;
+  u.layers = layers;
+  size_t off = 0;
+  GemmPlanShape shape[kPlanGroupMax];
+  for (size_t i = 0; i < layers.size(); ++i) {
+    const PlanLayer& L = p->layers[layers[i]];
+    shape[i] = {L.M, L.w.N, L.w.K * (L.w.bits == 16 ? 2 : 1) / 128};
+    PlanGroup::Place at = {0, 0, 0};
+    off += unit_layer_bytes(L, &at, off);
+    u.place.push_back(at);
+  }
+  if (!gemm_plan_schedule(shape, static_cast<int>(layers.size()), &u.sched)) return;
+  for (int l : layers) p->unit_of[l] = static_cast<int>(p->units.size());
+  p->unit_bytes = std::max(p->unit_bytes, align256(off));
+  p->units.push_back(std::move(u));
+}
 static void plan_build_units(dp_plan* p) {
   p->units.clear();
   p->unit_of.assign(p->layers.size(), -1);
   p->unit_bytes = 0;
-  std::vector<int> run;
+  std::vector<std::vector<int>> cut;  // a row of layers that units take, cut where a unit is full
   size_t bytes = 0;
   auto close = [&]() {
-    PlanGroup u;
-    u.layers = run;
-    run.clear();
-    size_t off = 0;
-    if (u.layers.size() >= kUnitMinLayers) {
-      GemmPlanShape shape[kPlanGroupMax];
-      for (size_t i = 0; i < u.layers.size(); ++i) {
-        const PlanLayer& L = p->layers[u.layers[i]];
-        shape[i] = {L.M, L.w.N, L.w.K * (L.w.bits == 16 ? 2 : 1) / 128};
-        PlanGroup::Place at = {0, 0, 0};
-        off += unit_layer_bytes(L, &at, off);
-        u.place.push_back(at);
-      }
-      if (gemm_plan_schedule(shape, static_cast<int>(u.layers.size()), &u.sched)) {
-        for (int l : u.layers) p->unit_of[l] = static_cast<int>(p->units.size());
-        p->unit_bytes = std::max(p->unit_bytes, align256(off));
-        p->units.push_back(std::move(u));
-      }
+    // What is left in pieces of one or two goes layer by layer, and each change between the two forms costs the overlap of
+    // quantization and GEMM on both sides. Where layers are so large that a piece is left between every two units, that is
+    // more than a unit of three saves: four blocks of mixed bits, width 1152, 10000 / 16384 tokens, layer by layer 648 / 1010 us,
+    // with such units 659 / 1081, width 768, 16384 573 / 586, 1024, 12000 621 / 636, but width 1024, 8192 and 768, 12000 (units of
+    // three and four without a piece between them) 436 / 402 and 418 / 398. One block, width 1024, 12000 tokens (three layers and
+    // one) 156 / 160.
+    size_t together = 0, breaks = 0;
+    for (size_t i = 0; i < cut.size(); ++i) {
+      if (cut[i].size() >= kUnitMinLayers) together += cut[i].size();
+      else if (i == 0 || cut[i - 1].size() >= kUnitMinLayers) ++breaks;
     }
-    bytes = 0;
+    if (together >= kUnitLayersPerBreak * breaks)
+      for (const std::vector<int>& u : cut)
+        if (u.size() >= kUnitMinLayers) plan_add_unit(p, u);
+    cut.clear();
   };
   for (size_t l = 0; l < p->layers.size(); ++l) {
     const PlanLayer& L = p->layers[l];
     // (a grouped small-M layer runs before everything else, but for long rows under a policy: see plan_run_step)
     if (L.M == 0 || (p->grouped[l] && L.w.K <= 1280)) continue;
-    const bool takes = unit_takes(*p, L) && unit_layer_bytes(L, nullptr, 0) <= kUnitBytes;
-    const size_t add = takes ? unit_layer_bytes(L, nullptr, 0) : 0;
-    if (!run.empty() && (!takes || bytes + add > kUnitBytes || run.size() == static_cast<size_t>(kPlanGroupMax))) close();
-    if (!takes) continue;
-    run.push_back(static_cast<int>(l));
+    if (!unit_takes(*p, L)) {
+      close();
+      continue;
+    }
+    const size_t add = unit_layer_bytes(L, nullptr, 0);
+    if (cut.empty() || bytes + add > kUnitBytes || cut.back().size() == static_cast<size_t>(kPlanGroupMax)) {
+      cut.emplace_back();
+      bytes = 0;
+    }
+    cut.back().push_back(static_cast<int>(l));
     bytes += add;
   }
   close();

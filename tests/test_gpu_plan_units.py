@@ -201,3 +201,20 @@ def test_launch_count_is_that_of_a_captured_step(bit_choices, flags):
         assert int(stack.status.item()) == 0
     finally:
         stack.close()
+
+
+@pytest.mark.parametrize("sizes,units", [
+    ("aaa", [0, 0, 0]), ("aaaa", [-1] * 4), ("aaaaa", [-1] * 5), ("aaaaaa", [0] * 3 + [1] * 3),
+    ("aaaaaaa", [0] * 3 + [1] * 3 + [-1]), ("aaac", [-1] * 4), ("aaacaaa", [0] * 3 + [-1] + [1] * 3),
+    ("aaacaaac", [-1] * 8), ("cccc" + "aaa" + "bb", [-1] * 9), ("c" + "s" * 17, [-1] + [0] * 16 + [-1]), ("sssgaaa", [0] * 3 + [-1] + [1] * 3)])
+def test_which_layers_are_launched_together(sizes, units):
+    """Three layers of size a fill a unit, two of size b, none of size c; g is a group-wise layer. Layers go together where at
+    least four times as many are in units of three or more as there are pieces left between or behind them."""
+    K, N = {"s": 128, "a": 128, "b": 256, "c": 640, "g": 128}, 128
+    rows = {"s": 300, "a": 130048, "b": 100000, "c": 130048, "g": 300}
+    layers = [_layer(l, K[s], N, 8, 64 if s == "g" else 0) for l, s in enumerate(sizes)]
+    plan = B.dp_plan_create([w for w, _ in layers], [rows[s] for s in sizes])
+    try:
+        assert [B.dp_plan_layer_unit(plan, l) for l in range(len(sizes))] == units
+    finally:
+        B.dp_plan_destroy(plan)
