@@ -685,7 +685,8 @@ struct dp_plan {
   std::vector<PlanGroup> units;          // tensor-core layers launched together
   std::vector<int> unit_of;              // per layer: its unit, or -1
   size_t unit_bytes;                     // of the two parts that units take in turn
-  std::mutex maps_lock;                  // of the units' tensor maps
+  std::atomic<bool> units_stale;         // a layer has left the units since they were made
+  std::mutex units_lock;                 // of the units' making and of their tensor maps
   int32_t* daq_sync;                     // device counters of the in-kernel DAQ (nullptr: DAQ in its own kernel)
   // DAQ policy (dp_plan_set_daq): clip percentile in 1/1000 %, 100000 = the maximum; activation bits
   // of the three time bins of [0, daq_timesteps)
@@ -787,6 +788,16 @@ static void plan_build_units(dp_plan* p) {
   }
   close();
   p->need(0);
+}
+// The units are made again when they are next asked for, not with every layer that leaves them (dp_plan_set_layer_flags for
+// 112 layers of 2048 tokens: 82 ms so).
+static void plan_refresh_units(const dp_plan* plan) {
+  if (!plan->units_stale.load(std::memory_order_acquire)) return;
+  dp_plan* p = const_cast<dp_plan*>(plan);
+  std::lock_guard<std::mutex> lock(p->units_lock);
+  if (!p->units_stale.load(std::memory_order_relaxed)) return;
+  plan_build_units(p);
+  p->units_stale.store(false, std::memory_order_release);
 }
 
 // Times every kernel variant that can run this layer shape (the whole layer: DAQ + GEMM, as the
@@ -919,6 +930,7 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   p->copy_stream = nullptr;
   p->daq_sync = nullptr;
   p->unit_bytes = 0;
+  p->units_stale = false;
   p->daq_p_e3 = 100000;
   p->daq_timesteps = 0;
   p->daq_bits[0] = p->daq_bits[1] = p->daq_bits[2] = 8;
@@ -1039,7 +1051,11 @@ extern "C" int dp_plan_create(const dp_weight* layers, int32_t n_layers, const i
   return DP_OK;
 }
 
-extern "C" size_t dp_plan_workspace(const dp_plan* plan) { return plan ? plan->workspace_bytes : 0; }
+extern "C" size_t dp_plan_workspace(const dp_plan* plan) {
+  if (!plan) return 0;
+  plan_refresh_units(plan);
+  return plan->workspace_bytes;
+}
 extern "C" int dp_plan_set_daq(dp_plan* plan, int32_t clip_percentile_e3, int32_t n_timesteps,
                                const int32_t* act_bits_by_bin) {
   if (!plan) return fail(DP_ERR_INVALID_ARG, "dp_plan_set_daq: plan is NULL");
@@ -1093,9 +1109,9 @@ extern "C" int dp_plan_set_layer_flags(dp_plan* plan, int32_t layer, uint32_t fl
                               "weights without the unpack-first form, or DAQ fused into the GEMM)",
                 layer, L.w.N, L.w.K, L.w.bits);
   if (int st = gemm_encode_w(&T.tmap_w, T.w.qweight, T.w.N, T.w.K, T.w.bits, T.bn, T.cg)) return st;
+  if (!L.fixed) plan->units_stale.store(true, std::memory_order_release);
   L = T;
   L.fixed = true;
-  plan_build_units(plan);
   const size_t ws = dp_wq_linear_workspace(L.M, L.w.N, L.w.K, L.w.bits,
                                            L.pre ? DP_FLAG_UNPACK_FIRST : DP_FLAG_NO_UNPACK_FIRST);
   plan->need(ws);
@@ -1111,6 +1127,7 @@ extern "C" int dp_plan_layer_unpack_first(const dp_plan* plan, int32_t layer, in
 extern "C" int dp_plan_layer_unit(const dp_plan* plan, int32_t layer, int32_t* unit) {
   if (!plan || layer < 0 || layer >= static_cast<int32_t>(plan->layers.size()) || !unit)
     return fail(DP_ERR_INVALID_ARG, "dp_plan_layer_unit: bad plan, layer index or NULL output");
+  plan_refresh_units(plan);
   *unit = plan->unit_of[layer];
   return DP_OK;
 }
@@ -1188,7 +1205,7 @@ static bool unit_independent(const dp_plan& p, const PlanGroup& u, const void* c
 
 // Tensor maps of a unit in the part of the workspace at `base`.
 static int unit_maps(dp_plan* plan, PlanGroup* u, uint8_t* base, int slot, CUtensorMap* a, CUtensorMap* w) {
-  std::lock_guard<std::mutex> lock(plan->maps_lock);
+  std::lock_guard<std::mutex> lock(plan->units_lock);
   PlanGroup::Maps& m = u->maps[slot];
   if (m.base != base) {
     m.base = nullptr;
@@ -1443,6 +1460,7 @@ static int check_plan_run(const dp_plan* plan, const int32_t* steps, int32_t n_s
   if (n_steps < 0 || start_index < 0 || start_index > n_steps || (n_steps > 0 && !steps))
     return fail(DP_ERR_INVALID_ARG, "bad steps/n_steps/start_index");
   if (flags & ~(DP_PLAN_SAME_X | DP_PLAN_SAME_Y)) return fail(DP_ERR_INVALID_ARG, "unknown plan-run flags");
+  plan_refresh_units(plan);
   if (!workspace || workspace_bytes < plan->workspace_bytes || (reinterpret_cast<uintptr_t>(workspace) & 255u))
     return fail(DP_ERR_WORKSPACE, "plan workspace needs %zu bytes, 256-byte aligned", plan->workspace_bytes);
   return DP_OK;

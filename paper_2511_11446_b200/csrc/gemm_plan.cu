@@ -21,8 +21,7 @@
 // Roles as in gemm_tc.cu: warps 0 and 10 bring in activations and weights, warp 1 of the pair's leader issues the MMAs,
 // warps 2-9 convert and store.
 #include <algorithm>
-#include <functional>
-#include <queue>
+#include <iterator>
 #include <utility>
 #include <vector>
 
@@ -323,24 +322,31 @@ bool gemm_plan_schedule(const GemmPlanShape* shape, int n, GemmPlanSchedule* out
       order[l] = l;
     }
     std::stable_sort(order, order + n, [&](int a, int b) { return us[a] > us[b]; });
+    // Pairs by their load so far, least first. All tiles of a layer take as long, so the pairs that have taken one are in
+    // order too, behind each other: the least of all is the first of one queue or of the other.
     using Load = std::pair<double, int>;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> least;
-    for (int i = 0; i < pairs_max; ++i) least.push({0.0, i});
+    std::vector<Load> loads, taken;
+    for (int i = 0; i < pairs_max; ++i) loads.push_back({0.0, i});
     std::vector<int> count(static_cast<size_t>(n) * kPlanMaxPairs, 0);
     double end = 0.0;
     int used = 0;
     for (int o = 0; o < n; ++o) {
       const GemmPlanShape& s = shape[order[o]];
       const int64_t tiles = (s.M + 2 * BM - 1) / (2 * BM) * (s.N / bn[order[o]]);
+      taken.clear();
+      size_t first = 0, first_taken = 0;
       for (int64_t t = 0; t < tiles; ++t) {
-        Load top = least.top();
-        least.pop();
-        top.first += us[order[o]];
-        end = std::max(end, top.first);
-        used = std::max(used, top.second + 1);
-        ++count[o * kPlanMaxPairs + top.second];
-        least.push(top);
+        const bool again = first == loads.size() || (first_taken < taken.size() && taken[first_taken] < loads[first]);
+        Load least = again ? taken[first_taken++] : loads[first++];
+        least.first += us[order[o]];
+        end = std::max(end, least.first);
+        used = std::max(used, least.second + 1);
+        ++count[o * kPlanMaxPairs + least.second];
+        taken.push_back(least);
       }
+      std::vector<Load> next;
+      std::merge(loads.begin() + first, loads.end(), taken.begin() + first_taken, taken.end(), std::back_inserter(next));
+      loads.swap(next);
     }
     if (end >= best) continue;
     best = end;

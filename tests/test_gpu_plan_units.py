@@ -218,3 +218,38 @@ def test_which_layers_are_launched_together(sizes, units):
         assert [B.dp_plan_layer_unit(plan, l) for l in range(len(sizes))] == units
     finally:
         B.dp_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("Ms,K,named,before,after", [
+    ([130048] * 4, 128, [3], [-1] * 4, [0] * 3 + [-1]),             # the piece behind a unit is what kept it from being one
+    ([300] * 6, 128, [2], [0] * 6, [-1] * 3 + [0] * 3),
+    ([300] * 6, 128, [4, 1, 2], [0] * 6, [-1] * 6)])
+def test_units_after_variants_have_been_named(Ms, K, named, before, after):
+    """Layers whose variant is named leave their unit, whatever is asked of the plan first: its units, its workspace, a run."""
+    layers = [_layer(l, K, 128, 8) for l in range(len(Ms))]
+    x = torch.ones((max(Ms), K), dtype=torch.bfloat16, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for ask in ("units", "workspace", "run"):
+        plan = B.dp_plan_create([w for w, _ in layers], Ms)
+        try:
+            units = lambda: [B.dp_plan_layer_unit(plan, l) for l in range(len(Ms))]
+            assert units() == before
+            room = B.dp_plan_workspace(plan)
+            for l in named:
+                B.dp_plan_set_layer_flags(plan, l, B.DP_FLAG_TILE_N(128))
+            if ask == "workspace":
+                assert B.dp_plan_workspace(plan) >= room
+            elif ask == "run":
+                fresh = B.dp_plan_create([w for w, _ in layers], Ms, B.DP_FLAG_NO_PDL)
+                ys = []
+                for p in (fresh, plan):
+                    ys.append([torch.zeros((M, 128), dtype=torch.bfloat16, device="cuda") for M in Ms])
+                    ws = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+                    B.dp_plan_run(p, [0], 0, B.ptr_array([x.data_ptr()] * len(Ms)), B.ptr_array([t.data_ptr() for t in ys[-1]]),
+                                  ws, status)
+                torch.cuda.synchronize()
+                B.dp_plan_destroy(fresh)
+                assert int(status.item()) == 0 and all(torch.equal(a, b) for a, b in zip(*ys))
+            assert units() == after
+        finally:
+            B.dp_plan_destroy(plan)
