@@ -351,7 +351,8 @@ int dp_plan_layer_unit(const dp_plan* plan, int32_t layer, int32_t* unit);
 /* Replaces the kernel variant of layer `layer` by the one `flags` names (the tuning flags of
  * dp_wq_linear: DP_FLAG_TILE_N, [NO_]CTA_PAIR, [NO_]WEIGHT_STATIONARY, [NO_]ACT_STATIONARY, UNPACK_FIRST; anything left
  * open is chosen as dp_wq_linear would), with which it is then launched on its own: lets a deployment keep the outcome of one
- * DP_FLAG_AUTOTUNE run and apply it to later plans. Host only; may raise dp_plan_workspace, so ask
+ * DP_FLAG_AUTOTUNE run and apply it to later plans. Not for layers that dp_plan_layer_unit finds in a unit, unless they are
+ * to leave it: layers launched together take half the time or less where they are small. Host only; may raise dp_plan_workspace, so ask
  * again afterwards. Small-M layers and unknown bits are refused (DP_ERR_INVALID_ARG), tile widths
  * that do not fit the layer with DP_ERR_SHAPE; the plan is unchanged on error. Not to be called
  * while a dp_plan_run of the plan is being issued. No counterpart in the paper. */

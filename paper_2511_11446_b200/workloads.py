@@ -43,8 +43,8 @@ class DitStack:
     def __init__(self, seed=synth.BASE_SEED + 4, batch=8, tokens=256, blocks=synth.BLOCKS, T=50, keep=25,
                  bit_choices=(3, 4, 8), resident_steps=None,
                  flags=B.DP_FLAG_AUTOTUNE | B.DP_FLAG_GROUP_SMALL_M, variants=None):
-        """variants: per-layer tuning flags from an earlier autotuned stack's layer_variants() (None
-        entries: small-M layers); given, the plan applies them instead of timing variants itself."""
+        """variants: per-layer tuning flags from an earlier autotuned stack's layer_variants() (None entries: layers
+        without a variant of their own); given, the plan applies them instead of timing variants itself."""
         if variants is not None:
             flags &= ~B.DP_FLAG_AUTOTUNE
         self.seed, self.T, self.flags = seed, T, flags
@@ -77,12 +77,13 @@ class DitStack:
                                  rows=rows)
 
     def layer_variants(self):
-        """Per layer: the tuning flags naming the kernel variant the plan runs (None: small-M kernel)."""
+        """Per layer: the tuning flags naming the kernel variant the plan runs, None where there is none of the layer's
+        own: small-M and 16-bit layers, and layers launched together (one whose variant is named leaves its unit)."""
         out = []
         for l in range(len(self.table)):
             v = B.dp_plan_layer_variant(self.plan, l)
-            out.append(None if v["small_m"] else
-                       B.variant_flags(v) & ~(B.DP_FLAG_FORCE_MMA | B.DP_FLAG_FORCE_SIMT))
+            own = not v["small_m"] and self.bits[l] != 16 and B.dp_plan_layer_unit(self.plan, l) < 0
+            out.append(B.variant_flags(v) & ~(B.DP_FLAG_FORCE_MMA | B.DP_FLAG_FORCE_SIMT) if own else None)
         return out
 
     # ---- accounting ----

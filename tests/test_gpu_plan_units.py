@@ -253,3 +253,18 @@ def test_units_after_variants_have_been_named(Ms, K, named, before, after):
             assert units() == after
         finally:
             B.dp_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("blocks,bit_choices", [(2, (3, 4, 8)), (2, (4, 8, 16)), (1, (4,))])
+def test_saved_variants_leave_the_units_as_they_are(blocks, bit_choices):
+    from paper_2511_11446_b200.workloads import DitStack
+    args = dict(seed=SEED, batch=2, tokens=128, blocks=blocks, T=2, keep=1, bit_choices=bit_choices)
+    first = DitStack(flags=B.DP_FLAG_AUTOTUNE | B.DP_FLAG_GROUP_SMALL_M, **args)
+    again = DitStack(variants=first.layer_variants(), **args)
+    try:
+        units = [[B.dp_plan_layer_unit(s.plan, l) for l in range(len(s.table))] for s in (first, again)]
+        assert units[0] == units[1] and max(units[0]) >= 0
+        assert again.launches_per_timestep() == first.launches_per_timestep()
+    finally:
+        first.close()
+        again.close()
