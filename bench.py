@@ -34,6 +34,9 @@ LAYER_DRAM_BYTES = {("qkv", 8): 22843183, ("qkv", 4): 18999936, ("qkv", 3): 1909
                     ("proj", 8): 10176524, ("proj", 4): 9465519, ("proj", 3): 9522281,
                     ("fc1", 8): 28825742, ("fc1", 4): 24417254, ("fc1", 3): 23730637,
                     ("fc2", 8): 28603063, ("fc2", 4): 22994528, ("fc2", 3): 22215648}
+# The same bytes over the algorithmic ones for token layers launched together, from the capture summarised in
+# profiles/plan_units_ncu.txt.
+UNIT_DRAM_RATIO = 1.49
 
 
 def measured_peaks():
@@ -218,9 +221,10 @@ def run_ours(args):
     if rank == 0 and args.timed_only:
         print(json.dumps(out))
     elif rank == 0:
-        # ---- roofline of the dominant kernel (tcgen05 GEMM), timed alone with CUDA events ----
+        # ---- rooflines: the launches of the timed region; the tcgen05 GEMMs of single layers, timed alone with CUDA events ----
         mma_peak = measure_mma_peak()
-        out["roofline"] = gemm_roofline(stack, peaks, mma_peak)
+        out["roofline_layer_gemms"] = gemm_roofline(stack, peaks, mma_peak)
+        out["roofline"] = run_roofline(stack, out["roofline_layer_gemms"], value / world)
         # ideal time of a timestep: per layer max(ops / int8 peak, bytes / HBM); the int8 peak is the
         # larger of sustained bf16 x2 (the step is seconds of back-to-back work) and the measured
         # instruction ceiling
@@ -250,10 +254,22 @@ def layer_alg_bytes(stack, l):
     return 2 * M * K + stack.layers[l].packed_bytes() + 6 * N + 2 * M * N
 
 
+def run_roofline(stack, gemms, achieved):
+    """The launches that the timed region consists of (preparation and GEMMs of layers launched together, grouped adaLN), at
+    the rate of the timed region itself: all of its time counts, the operations are those of all linears."""
+    return {"kernel": "gemm_plan_kernel (tcgen05 kind::i8) with plan_prep_kernel and simt_group_kernel beside it: the launches "
+                      "of the timed region",
+            "bound": "tensor", "achieved": achieved, "peak": gemms["peak"], "unit": "TOPS", "frac": achieved / gemms["peak"],
+            "peak_note": gemms["peak_note"], "frac_of_nominal": achieved / NOMINAL_INT8_TOPS,
+            "launches": stack.launches_per_timestep(), "traffic": UNIT_DRAM_RATIO * gemms["algorithmic_bytes_per_layer"],
+            "traffic_note": "DRAM bytes of a token layer (its share of both launches, reads + writes), mean; algorithmic bytes beside it",
+            "algorithmic_bytes_per_layer": gemms["algorithmic_bytes_per_layer"]}
+
+
 def gemm_roofline(stack, peaks, mma_peak):
-    """The dominant kernel family (the tcgen05 GEMMs) timed without the rest of the path: the 112
+    """The tcgen05 GEMMs of single layers, timed without the rest of the path: the 112
     GEMMs of one timestep, one launch each, with the kernel variant the plan chose for its layer on its own (a
-    run of the plan launches those of several layers together), on
+    run of the plan launches those of several layers together with a kernel of their own), on
     pre-quantized activations (so no DAQ launch in between), captured in one CUDA graph and timed
     with CUDA events on the replay stream. One timestep's operands (0.4 GB of int8 activations,
     0.4 GB of weights, 1.1 GB of outputs) exceed L2, so every launch streams from HBM. A layer the

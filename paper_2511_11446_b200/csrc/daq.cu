@@ -227,7 +227,8 @@ __device__ __forceinline__ void prep_expand(const PlanPrepSeg& s, int block, boo
 
 // CTA `block` over the rows of a segment, RW warps to a row, `part` a word per warp: daq_rows_kernel without its options. (One
 // function for both costs that kernel registers, 40 -> 42 with four warps to a row, and with them two CTAs of an SM:
-// K = 3072, M = 2048 / 8192 4.6 / 13.2 -> 5.0 / 14.1 us.)
+// K = 3072, M = 2048 / 8192 4.6 / 13.2 -> 5.0 / 14.1 us. Where ten CTAs an SM hold all rows and twelve leave SMs with fewer, that was
+// the better: K = 3072 / 4608, M = 1285 3.5 / 4.5 -> 3.4 / 4.35, but M = 1600 3.6 / 4.8 -> 4.1 / 4.75.)
 template <int RW>
 __device__ __forceinline__ void prep_rows(const PlanPrepSeg& s, int block, uint32_t* part) {
   constexpr int TPR = 32 * RW, MAXV = 5;

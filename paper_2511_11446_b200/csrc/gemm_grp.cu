@@ -30,13 +30,15 @@
 // The fold is what bounds this kernel: the waits of a fold warp for the tensor core are a tenth of its time. 32 values a
 // lane and warp, conversion and fma, take a scheduler 104 clocks in a loop of nothing else (packed fma 113, fma without
 // the conversion 69), so a 128 x 128 group costs 420 clocks, with the loop around it 680 (g = 128, M = 64), against 560
-// for a k-block of the plain kernel with this tile when all SMs load. Eight warps of 64 columns do with fewer instructions a value than sixteen
-// of 32 and leave each 168 registers; packed fma needs its operands moved into pairs. K = 1152, N = 3456, M = 2048,
-// sixteen warps, packed, one issuer -> this: 4 bits with zero-points, g = 128 19.2 -> 18.8 us, g = 32 45.6 -> 44.2; 8 bits,
-// g = 64 27.5 -> 27.0, with zero-points, g = 128, 33.5 -> 29.8; K = 4608, N = 1152, M = 64, 3 bits, g = 32 54.0 -> 51.4, 8 bits with
-// zero-points, g = 64, 64.0 -> 55.0; but M = 2048, 4 bits, g = 128 23.1 -> 23.3. Block of 4-bit layers with zero-points, g = 128, M =
-// 2048: 90.6 -> 90.2. (Tried: accumulators that start at the word of the float 1.5 * 2^23, so that an addition in
-// place of the conversion makes the float: the tensor-memory stores cost more, g = 32 44 -> 58 us.)
+// for a k-block of the plain kernel with this tile when all SMs load. Counters (K = 1152, N = 3456, g = 128, 4 bits with zero-points,
+// M = 8192): issue slots 60 %, ALU pipe 52 %, FMA pipe 22 %, tensor pipe 30 %, DRAM 4 %. Eight warps of 64 columns take
+// fewer instructions a value than sixteen of 32 and leave each 168 registers; packed fma needs its operands moved into pairs.
+// K = 1152, N = 3456, M = 2048, sixteen warps, packed, one issuer -> this: 4 bits with zero-points, g = 128 19.2 -> 18.8 us, g = 32
+// 45.6 -> 44.2; 8 bits, g = 64 27.5 -> 27.0, with zero-points, g = 128, 33.5 -> 29.8; K = 4608, N = 1152, M = 64, 3 bits, g = 32
+// 54.0 -> 51.4, 8 bits with zero-points, g = 64, 64.0 -> 55.0; but K = 4608, N = 1152, M = 2048, 4 bits, g = 128 23.1 -> 23.3. Block of
+// 4-bit layers with zero-points, g = 128, M = 2048: 91.0 -> 89.9. (Tried: accumulators that start at the word of the float
+// 1.5 * 2^23, so that an addition in place of the conversion makes the float: the tensor-memory stores cost more, g = 32
+// 44 -> 58 us.)
 #include "gemm_device.cuh"
 
 namespace dp {

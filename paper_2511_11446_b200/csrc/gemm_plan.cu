@@ -7,15 +7,20 @@
 // the operand ring and the two accumulator buffers running on across layers; the runs are levelled by the host with the
 // tiles' expected times, long contractions first (gemm_plan_schedule).
 //
-// Operands are int8 (the group's packed weights have been expanded and its activations quantized by launch_plan_prep,
+// Operands are int8 (the unit's packed weights have been expanded and its activations quantized by launch_plan_prep,
 // kind::i8) or, for layers kept in 16 bits, the caller's bf16 matrices (kind::f16); a k-block is 128 bytes of either.
 // A CTA is held to 96 registers a thread: that leaves an SM room for six CTAs of the next unit's preparation (40 registers, 128
 // threads), which runs beside this kernel; with 130 and 56 it had room for two and ran after it (28 blocks, mixed
 // bits, 2048 tokens: 1050 -> 985 us a step; 1024 tokens with 16-bit layers and the percentile rule 752 -> 700).
-// A step of 28 blocks, a launch or two a layer -> two a unit of up to 64 MB of operands: 256 tokens 663 -> 255 us, 1024 (policy,
-// 16-bit layers) 1269 -> 670, 2048 1271 -> 945; 12 blocks of width 384, 64 tokens, 220 -> 46. Units of 24 / 50 / 70 MB:
-// 256 tokens 294 / 264 / 254, 2048 1043 / 963 / 941, 4096 (12 blocks) 870 / 773 / 771. What bounds it: at 2048 tokens
-// the MMAs (24 of 34 us a block with the preparation left out), at 256 the preparation.
+// A step of 28 blocks of width 1152, a launch or two a layer -> two a unit of up to 64 MB of operands, the first pass on new inputs /
+// passes one behind the other over the same: 256 tokens 715 -> 308 / 659 -> 267 us, 2048 1330 -> 951 / 1363 -> 1086, 1024 (policy, 16-bit
+// layers) 1329 -> 648 / 1268 -> 708. Units of 24 / 48 / 64 / 72 MB, two sets of inputs in turn: 256 tokens 287 / 256 / 246 / 246, 2048
+// 1100 / 991 / 986 / 998, 1024 663 / 654 / 637 / 637, 4096 (12 blocks) 918 / 827 / 789 / 805. One block on its own (one unit, nothing
+// beside its preparation): 256 tokens 32.9 -> 19.9, 4096 77.7 -> 70.4. 16-bit layers take no scratch, so units of any token count:
+// four blocks of them, 32768 tokens, 4150 -> 3900.
+// What bounds it, by counters of the two kernels launched alone: at 2048 tokens the MMAs (tensor pipe busy 74 % of this kernel's time,
+// 54 us to the preparation's 23), at 256 bringing operands in (43 %, 23 us to 17). Through DRAM go 1.5 times the
+// bytes that the method must move: of the codes and expanded weights a part leaves L2 before it is read.
 // Starting a unit's GEMMs on a count of finished preparation CTAs, ahead of the end of the unit before, was
 // tried and left out: it once hung, and why was not found.
 // Roles as in gemm_tc.cu: warps 0 and 10 bring in activations and weights, warp 1 of the pair's leader issues the MMAs,

@@ -1,8 +1,9 @@
 """Phase A of Algorithm 2 fed by this library's own measured latencies.
 
 `latency_table` times every distinct (layer shape, bit option) of a stack with dp_layer_latency_us
-(the whole quantized linear as dp_wq_linear runs it: the c_lat(l, b) input of the algorithm, which the
-paper measures with its own integer kernels); `joint_plan` assembles the algorithm's inputs (per-layer
+(the whole quantized linear as dp_wq_linear runs it, on its own: the c_lat(l, b) input of the algorithm, which the
+paper measures with its own integer kernels; layers that a plan launches together take less, half of it or less at a few
+hundred tokens, so C_lat is an upper bound there too); `joint_plan` assembles the algorithm's inputs (per-layer
 options with measured latency and packed-weight bytes, sensitivities, per-step drift and cost, budgets)
 and calls dp_plan_phase_a. Sensitivities and drifts come from the caller: the paper derives them from
 its checkpoints and calibration data, which this repository does not have. Bookkeeping only: the
