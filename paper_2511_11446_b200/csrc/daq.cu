@@ -145,10 +145,10 @@ daq_rows_2pass_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t 
 }
 
 // ---- DAQ with a percentile clip and a-bit codes: robust_row in daq_device.cuh ------------------------
-// RW warps to a token, MAXV vectors a lane (see launch_daq_robust).
+// RW warps to a token, MAXV vectors a lane, registers for CTAS resident CTAs (see launch_daq_robust).
 constexpr int kRobustWarpK = 256 * 6;  // rows that one warp takes in a plan's preparation
-template <int RW, int MAXV>
-__global__ void __launch_bounds__(kDaqThreads, MAXV <= 6 ? 10 : 6)
+template <int RW, int MAXV, int CTAS>
+__global__ void __launch_bounds__(kDaqThreads, CTAS)
 daq_rows_robust_kernel(const uint16_t* __restrict__ x, int64_t M, int K, int64_t ldx, int8_t* __restrict__ q,
                        int64_t ldq, float* __restrict__ s_a, int32_t* __restrict__ rowsum, int clip_rank,
                        float qmax, int tiled_kb, const UnpackJob job) {
@@ -370,13 +370,13 @@ int launch_daq(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int6
   return DP_OK;
 }
 
-template <int RW, int MAXV, typename... A>
+template <int RW, int MAXV, int CTAS, typename... A>
 static cudaError_t launch_robust_rows(int64_t M, UnpackJob job, cudaStream_t stream, bool pdl, A... a) {
   constexpr int kRows = kDaqThreads / 32 / RW;
   const unsigned daq_blocks = static_cast<unsigned>((M + kRows - 1) / kRows);
   job.first_block = static_cast<int32_t>(daq_blocks);
   const dim3 grid(daq_blocks + unpack_blocks(job, kDaqThreads));
-  return launch(daq_rows_robust_kernel<RW, MAXV>, grid, dim3(kDaqThreads), 0, stream, pdl, a..., job);
+  return launch(daq_rows_robust_kernel<RW, MAXV, CTAS>, grid, dim3(kDaqThreads), 0, stream, pdl, a..., job);
 }
 
 int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* q, int64_t ldq, float* s_a,
@@ -389,18 +389,24 @@ int launch_daq_robust(const void* x, int64_t M, int64_t K, int64_t ldx, int8_t* 
   const float qmax = static_cast<float>((1 << (act_bits - 1)) - 1);
   UnpackJob job;
   if (unpack != nullptr) job = *unpack;
-#define DP_ROWS(RW, MAXV) \
-  launch_robust_rows<RW, MAXV>(M, job, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank, qmax, tiled_kb)
+#define DP_ROWS(RW, MAXV, CTAS) \
+  launch_robust_rows<RW, MAXV, CTAS>(M, job, stream, pdl, xp, M, k, ldx, q, ldq, s_a, rowsum, clip_rank, qmax, tiled_kb)
   // Four warps to a row of more than 2304 elements, and to one of more than 1280 where there are few. One warp, 18 vectors a lane
   // (five peeling rounds, two CTAs of 256 threads on an SM) -> this: K = 4608, p = 99.9, M = 100 / 1024 / 8192 / 32768 6.4 / 7.8 /
   // 32.0 / 108 us -> 2.8 / 7.3 / 28.0 / 100 (threshold of rank 47, p = 99: 23.8 / 25.9 / 101 / 359 -> 9.6 / 22.3 / 98 / 369);
   // K = 3072 5.4 / 5.8 / 25.9 / 89 -> 2.4 / 5.2 / 22.7 / 81. Shorter rows, many of them, spend longer on the exchanges than on
   // the row: K = 2304, one warp and nine vectors in CTAs of 256 / four warps / one warp and nine vectors in CTAs of 128:
   // M = 100 3.3 / 2.2 / -, 1024 3.5 / 4.4 / 3.2, 32768 54 / 68 / 39; K = 1536 (nine, -, six) 2.4 / 1.9 / -, 2.5 / 3.5 / 2.4, 38 / 56 / 26.
-  const cudaError_t e = k <= 256 * 5               ? DP_ROWS(1, 5)
-                        : k > 256 * 9 || M <= 512 ? DP_ROWS(kDaqThreads / 32, 5)
-                        : k <= 256 * 6            ? DP_ROWS(1, 6)
-                                                  : DP_ROWS(1, 9);
+  // Few registers, many CTAs to an SM, only from 4096 rows on. Up to there all rows are resident either way and more CTAs of
+  // them beside the GEMM before make the GEMM behind wait. Quantization and the GEMM of an 8-bit layer of 1152 channels on its codes,
+  // p = 99.9, CTAs of 256 threads and two or three to an SM / ten small ones (K = 2304: six) / this: K = 1152, M = 900 7.27 / 7.95 / 7.33 us,
+  // 2048 8.53 / 9.57 / 8.62, 3001 10.05 / 11.08 / 9.94; K = 1536, M = 2048 9.50 / 10.69 / 8.96; K = 2304, M = 2048 11.15 / 12.59 / 11.09.
+  // Beyond it the rate of the quantization itself counts: K = 1152, six / eight to an SM, M = 9000 8.61 / 8.06, layer 19.4 / 19.4.
+  const bool few = M < 4096;
+  const cudaError_t e = k <= 256 * 5               ? few ? DP_ROWS(1, 5, 6) : DP_ROWS(1, 5, 8)
+                        : k > 256 * 9 || M <= 512 ? DP_ROWS(kDaqThreads / 32, 5, 10)
+                        : k <= 256 * 6            ? few ? DP_ROWS(1, 6, 4) : DP_ROWS(1, 6, 8)
+                                                  : few ? DP_ROWS(1, 9, 4) : DP_ROWS(1, 9, 6);
 #undef DP_ROWS
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, "robust DAQ launch failed: %s", cudaGetErrorString(e));
   return DP_OK;

@@ -72,7 +72,8 @@ def test_repeats_sparse_rows_and_pitches():
         _same(_run(x, rank, bits, ldx=K + 8, ldq=K + 32), x, rank, bits)
 
 
-@pytest.mark.parametrize("M,K", [(9, 1280), (9, 1288), (512, 1536), (513, 1536), (513, 1544), (513, 2304), (9, 2312), (9, 4608)])
+@pytest.mark.parametrize("M,K", [(9, 1280), (9, 1288), (512, 1536), (513, 1536), (513, 1544), (513, 2304), (9, 2312), (9, 4608),
+                                 (4095, 1280), (4096, 1280), (4095, 1536), (4096, 1288), (4095, 2304), (4096, 2304)])
 def test_equal_magnitudes_across_the_warps_of_a_row(M, K):
     """Ranks that end inside, at and behind a run of equal magnitudes spread over the whole row, on both sides of the row
     lengths and counts at which one warp, with six or nine vectors a lane, or four warps take a row."""
