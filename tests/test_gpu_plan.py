@@ -389,8 +389,8 @@ def test_in_kernel_quantization_covers_packed_layers(M, autotune):
 @pytest.mark.parametrize("M", [300, 8200])
 @pytest.mark.parametrize("K", [256, 1408, 2816])
 def test_in_kernel_quantization_of_an_earlier_output(K, M):
-    """DP_FLAG_FUSED_DAQ with layers that read the output of the layer before, rows on both sides of one batch of loads (1280
-    elements) and of two: the bits of a plan that runs one kernel at a time."""
+    """DP_FLAG_FUSED_DAQ with layers that read the output of the layer before, rows shorter and longer than the five vectors a
+    lane that a pass over them unrolls: the bits of a plan that runs one kernel at a time."""
     dims, bits = (K, 384, K, 384), (4, 8, 3)
     dev = [DevLayer(*synth.weights(SEED, l, dims[l + 1], dims[l], b), synth.bias(SEED, l, dims[l + 1]), b)
            for l, b in enumerate(bits)]
